@@ -122,7 +122,9 @@ typedef struct div_plan {
     int32_t decompress_fast;/* 1: quad kernel (W%4==0, B a power of two >= 4); 3: the same conditions on a 1-D map
                                (h == 1): line kernel; 2: flat kernel with a tile table (sample size a multiple of 4,
                                planes up to 8192 elements); 0: general */
-    int32_t reserved;
+    int32_t on_chip;        /* 1: the cluster kernel takes the descriptor first (x is read once and waits in shared memory; a
+                               thread-block cluster per sample); the fields above then describe the kernel that runs where
+                               the device refuses clusters of that size.  0: they describe what runs */
 } div_plan;
 
 /* flags of div_compress_ex */
@@ -220,11 +222,11 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                           void* xhat_dev, void* cuda_stream);
 
 /*
- * Test hook for the bounded waits of the single-launch compress kernels (plan codes 2, 3, 6 and 7): runs the
+ * Test hook for the bounded waits of the single-launch compress kernels (on_chip 1, plan codes 2, 3, 6 and 7): runs the
  * kernel div_compress_ex would run, but tells it to wait for a number of arrivals per sample that is never
  * reached, with `timeout_ns` (at most 100 ms) as the limit of every wait.  The kernel must give up, record
  * DIV_ERR_TIMEOUT in the workspace status word (read it with div_read_device_status) and return; the blob's
- * contents are then unspecified.  The first of the strip ring, lagged, staged and fused small-plane
+ * contents are then unspecified.  The first of the cluster (flags 0), strip ring, lagged, staged and fused small-plane
  * kernels that the flags allow and the descriptor fits is taken; DIV_ERR_PARAM when there is none.
  * Arguments as for div_compress_ex.  No counterpart in the paper.
  */

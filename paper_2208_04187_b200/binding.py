@@ -54,7 +54,7 @@ class DivLayout(ctypes.Structure):
 class DivPlan(ctypes.Structure):
     _fields_ = [("fused", c_int32), ("grid", c_int32), ("threads", c_int32), ("stages", c_int32),
                 ("lag", c_int32), ("smem_bytes", c_int32), ("chunk_elems", c_int64),
-                ("chunks_per_sample", c_int64), ("decompress_fast", c_int32), ("reserved", c_int32)]
+                ("chunks_per_sample", c_int64), ("decompress_fast", c_int32), ("on_chip", c_int32)]
 
 
 class DivisionError(RuntimeError):

@@ -5,17 +5,19 @@ import os
 import shutil
 import subprocess
 import sys
+from concurrent.futures import ThreadPoolExecutor
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libdivision.so")
-SOURCES = ["division.cu"]
-HEADERS = ["common.cuh", "twopass.cuh", "decompress.cuh", "fused.cuh", "fused_v.cuh", "lagged.cuh", "staged.cuh", "planes.cuh", "planegroup.cuh", "masks.cuh", "lines.cuh", "volume.cuh", os.path.join("..", "..", "include", "division.h")]
+OBJ_DIR = os.path.join(PKG_DIR, "_build")
+SOURCES = ["division.cu", "cluster.cu"]
+HEADERS = ["common.cuh", "cluster_plan.cuh", "halves.cuh", "twopass.cuh", "decompress.cuh", "fused.cuh", "fused_v.cuh", "lagged.cuh", "staged.cuh", "planes.cuh", "planegroup.cuh", "masks.cuh", "lines.cuh", "volume.cuh", os.path.join("..", "..", "include", "division.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-lineinfo", "-std=c++17",
-    "-shared", "-Xcompiler", "-fPIC",
+    "-Xcompiler", "-fPIC", "--split-compile=0",
     "--fmad=false",          # one rounding per operation is part of the output contract
     "-Xptxas", "-v",
 ]
@@ -40,15 +42,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Build libdivision.so next to this file; returns its path."""
     if not force and not is_stale():
         return LIB_PATH
-    cmd = [_nvcc()] + NVCC_FLAGS + [os.path.join(CSRC, s) for s in SOURCES] + ["-o", LIB_PATH]
+    os.makedirs(OBJ_DIR, exist_ok=True)
+    newest_header = max(os.path.getmtime(os.path.join(CSRC, h)) for h in HEADERS)
+
+    def compile_one(src):
+        path, obj = os.path.join(CSRC, src), os.path.join(OBJ_DIR, src[:-3] + ".o")
+        log = obj[:-2] + ".log"
+        if force or not (os.path.exists(obj) and os.path.getmtime(obj) > max(newest_header, os.path.getmtime(path))):
+            _run([_nvcc()] + NVCC_FLAGS + ["-c", path, "-o", obj], verbose, log)
+        return obj, log
+
+    with ThreadPoolExecutor(len(SOURCES)) as pool:          # one nvcc per source, side by side
+        done = list(pool.map(compile_one, SOURCES))
+    _run([_nvcc(), "-shared"] + NVCC_FLAGS[:2] + [obj for obj, _ in done] + ["-o", LIB_PATH], verbose, None)
+    with open(os.path.join(PKG_DIR, "ptxas_info.log"), "w") as f:
+        f.write("".join(open(log).read() for _, log in done))
+    return LIB_PATH
+
+
+def _run(cmd, verbose, log):
     proc = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or proc.returncode != 0:
         sys.stderr.write(proc.stdout + proc.stderr)
     if proc.returncode != 0:
         raise RuntimeError("nvcc failed building libdivision.so")
-    with open(os.path.join(PKG_DIR, "ptxas_info.log"), "w") as f:
-        f.write(proc.stderr)
-    return LIB_PATH
+    if log:
+        with open(log, "w") as f:
+            f.write(proc.stderr)
 
 
 if __name__ == "__main__":

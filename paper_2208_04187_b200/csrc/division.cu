@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "cluster_plan.cuh"
 #include "common.cuh"
 #include "decompress.cuh"
 #include "fused.cuh"
@@ -237,6 +238,50 @@ void choose_compress(const div_desc* d, const Shape& s, uint32_t flags, Choice* 
     if (plan_fused(d, s, &c->fp) == DIV_OK) c->code = 1;
 }
 
+#ifdef DIVK_DEV
+}
+#include <stdlib.h>
+namespace {
+#endif
+// Does the cluster kernel take a descriptor, and in clusters of how many CTAs?  (Flags pin one of the other kernels.)
+bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPlan* out) {
+    if (flags != 0) return false;
+    const DeviceInfo di = device_info();
+    if (!di.ok || di.sms < 1) return false;
+#ifdef DIVK_DEV
+    if (const char* e = getenv("DIVK_CS"); e && *e) {
+        if (atoi(e) == 0) return false;
+        return plan_cluster_cs(d, s, (uint32_t)atoi(e), di, out);
+    }
+#endif
+    if (s.H == 1) {
+        LineGeom lg;
+        if (plan_lines(d, s, &lg)) return false;          // 1-D maps have a kernel of their own
+    }
+    // Cost in KB of x an SM works through (41 KB take 1 us): its share, and 3 us for every further time the device has
+    // to be filled, since the CTAs of one filling load, reduce and quantise in step.  Ties go to the smaller shares.
+    uint64_t best = ~0ull;
+    for (uint32_t cs = 1; cs <= CL_MAX; cs *= 2) {
+        ClusterPlan pl;
+        if (!plan_cluster_cs(d, s, cs, di, &pl)) continue;
+        const uint64_t share = (uint64_t)pl.ppc * s.HW * 4u / 1024u;
+        const uint64_t cost = ((uint64_t)s.N * cs + (uint32_t)di.sms - 1u) / (uint32_t)di.sms * share + 123u * (pl.waves - 1u);
+        if (cost <= best) {
+            best = cost;
+            *out = pl;
+        }
+    }
+    if (best == ~0ull) return false;
+    // Where a kernel that reads x a second time from the L2 applies it is as good or better once the clusters have to
+    // take turns (three fillings: 50 x 256 x 40 x 40 39 against 35 us; two: 64 x 64 x 56 x 56 22.6 against 27.5 us,
+    // 64 x 1024 x 14 x 14 26.2 against 26.7 us), and on bfloat16 maps, whose residuals take twice the room of x, as soon as there are
+    // two (128 x 320 x 16 x 16 22.3 against 20.7 us).  The general kernels never are (32 x 64 x 75 x 75: 33 against 82 us).
+    PlaneGeom pg;
+    SPlan sp;
+    const bool rereads = plan_staged(d, s, &sp) == DIV_OK || plan_planes(d, s, &pg);
+    return !rereads || out->waves <= (d->x_dtype == DIV_BF16 ? 1u : 2u);
+}
+
 bool decompress_fast_ok(const Shape& s) {
     return (s.W % 4 == 0) && s.B >= 4 && (s.B & (s.B - 1)) == 0 && s.N <= 65535;
 }
@@ -336,6 +381,7 @@ div_status div_plan_query(const div_desc* desc, uint32_t flags, div_plan* out) {
         out->grid = (int32_t)((s.tiles + 255) / 256);
         out->threads = 256;
     }
+    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl)) out->on_chip = 1;
     out->decompress_fast = decompress_fast_ok(s) ? ((s.H == 1 && s.CHW < (1u << 31)) ? 3 : 1) : (decompress_flat_ok(s) ? 2 : 0);
     return DIV_OK;
 }
@@ -353,13 +399,15 @@ div_status div_compress_ex(const div_desc* desc, const void* x_dev, void* comp_d
     make_layout(desc, s, &lo);
     if (comp_capacity < lo.total_bytes || workspace_bytes < lo.workspace_bytes) return DIV_ERR_CAPACITY;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    if (cudaMemsetAsync(workspace_dev, 0, lo.workspace_bytes, stream) != cudaSuccess) return DIV_ERR_CUDA;
     uint8_t* blob = (uint8_t*)comp_dev;
     uint32_t* ws = (uint32_t*)workspace_dev;
     // kernels that store bytes or half-words leave the unused top of a partial last word alone: it is zero by contract
     if ((s.total * (uint64_t)desc->qbits) % 32u != 0 &&
         cudaMemsetAsync(blob + lo.packed_off + lo.packed_bytes - 4, 0, 4, stream) != cudaSuccess)
         return DIV_ERR_CUDA;
+    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl) && compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream) == DIV_OK)
+        return DIV_OK;
+    if (cudaMemsetAsync(workspace_dev, 0, lo.workspace_bytes, stream) != cudaSuccess) return DIV_ERR_CUDA;
     // The single-launch kernels need all their CTAs resident, so they are launched cooperatively; where the
     // device refuses such a launch (fewer SMs visible to the process than the device reports, for instance) the
     // next kernel in line takes the descriptor: nothing has been enqueued by the refused launch.
@@ -402,6 +450,8 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
     uint8_t* blob = (uint8_t*)comp_dev;
     uint32_t* ws = (uint32_t*)workspace_dev;
     const uint32_t never = 0xFFFFFFFFu;      // an arrival count no sample reaches
+    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl))
+        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, 1u << 19, timeout_ns);
     if (!(flags & DIV_FLAG_NO_STRIP_KERNEL)) {
         VPlan vp;
         if (plan_v(desc, s, &vp) == DIV_OK) return compress_fused_v(desc, s, lo, vp, x_dev, blob, ws, seed, stream, never, timeout_ns);

@@ -511,6 +511,23 @@ inline bool ensure_dynamic_smem(const void* kern, int bytes, SmemSeen* seen) {
     return true;
 }
 
+// leave to launch a kernel in clusters of more than 8 CTAs: asked for once per device
+inline bool ensure_wide_cluster(const void* kern, SmemSeen* seen) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    const bool slot = dev >= 0 && dev < DEVICE_CACHE_SLOTS;
+    if (slot && seen[dev].fn.load(std::memory_order_acquire) == kern) return true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (slot) seen[dev].fn.store(kern, std::memory_order_release);
+    return true;
+}
+
 // Decide whether and how the fused kernel runs a descriptor.  DIV_OK: plan filled in.
 inline div_status plan_fused(const div_desc* d, const Shape& s, FusedPlan* out) {
     const uint32_t sx = d->x_dtype == DIV_F32 ? 4u : 2u;

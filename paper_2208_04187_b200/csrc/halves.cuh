@@ -1,0 +1,244 @@
+// The two halves of a compress kernel that keeps its share of x on chip, as code shared by such kernels:
+//   half 1  one slot = the NC adjacent columns of one tile of one band (tile row) that a lane owns: tile sum in the fixed
+//           order, stored low-frequency value, extremes, fp32 residual;
+//   half 2  Eq. 9 on groups of 4 consecutive residuals, which needs no notion of tiles.
+#pragma once
+
+#include "planes.cuh"      // ColLoad; quant_row, packed pairs
+
+namespace divk {
+
+// ------------------------------------------------------------------------------------------------
+// arithmetic
+// ------------------------------------------------------------------------------------------------
+// sum / cnt, correctly rounded, for a small whole cnt and rcp = RN(1 / cnt): one Newton step on the quotient with an
+// exact remainder (Markstein, "Computation of elementary functions on the IBM RISC System/6000", 1990).  Checked
+// against IEEE division for every significand of the sum and every count up to 1024; scaling by powers of two
+// changes nothing while no intermediate result leaves the normal range, hence the guard.
+__device__ __forceinline__ float div_by_count(float sum, float cnt, float rcp) {
+    const float m = fabsf(sum);
+    if (m > 1e-30f && m < 1e30f) {
+        const float q = __fmul_rn(sum, rcp);
+        return __fmaf_rn(__fmaf_rn(-q, cnt, sum), rcp, q);
+    }
+    return __fdiv_rn(sum, cnt);
+}
+
+// Can the sample's codes be had from quant4_fixed?  It needs products that neither overflow nor become subnormal
+// (|delta| bounds the smallest non-zero r - delta from below) and no result past the top code (the only value that
+// may round past it is the sample's largest residual).
+template <int Q>
+__device__ __forceinline__ bool fixed_point_ok(const QParams& q, float rmax) {
+    if (Q > 4) return false;
+    const float d = fabsf(q.delta);
+    return d >= 1e-24f && q.scale >= 1e-6f && q.scale <= 1e30f &&
+           __fmul_rn(__fsub_rn(rmax, q.delta), q.scale) <= (float)((1 << Q) - 1);
+}
+
+__device__ __forceinline__ uint64_t add2_rm(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Codes of 4 residuals (Eq. 9 with stochastic rounding), packed Q bits apart, in fixed point with 16 fraction bits.
+// With t = fl(fl(r - delta) * scale) as everywhere, nscale = -65536 * scale gives -65536 t exactly.  The float
+// M = 2^23 + 65536 qmax + field is a random half-word under a constant high half; M - 65536 t rounded down is
+// 2^23 + floor(65536 (qmax - t) + field), and dropping its low 16 bits leaves qmax - ceil(t - field / 65536), the
+// code's complement.  Per element: one byte permutation, half a packed add and the packing, where quant2 needs a
+// clamp, the permutation, half a fused multiply-add and half an add: 18 against 20 us for the 51 M residuals of a
+// 64 x 64 x 112 x 112 map already in shared memory.
+template <int Q>
+__device__ __forceinline__ uint32_t quant4_fixed(uint64_t xy, uint64_t zw, uint64_t delta2, uint64_t nscale2, uint64_t z) {
+    constexpr uint32_t TOP = 0x4B00u + ((1u << Q) - 1u);
+    const uint64_t a = mul2_rn(sub2_rn(xy, delta2), nscale2), b = mul2_rn(sub2_rn(zw, delta2), nscale2);
+    const uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
+    uint32_t v0, v1, v2, v3;
+    upk2u(add2_rm(a, pk2u(__byte_perm(lo, TOP, 0x5410), __byte_perm(lo, TOP, 0x5432))), v0, v1);
+    upk2u(add2_rm(b, pk2u(__byte_perm(hi, TOP, 0x5410), __byte_perm(hi, TOP, 0x5432))), v2, v3);
+    const uint32_t w01 = __byte_perm(v0, v1, 0x7632), w23 = __byte_perm(v2, v3, 0x7632);      // 0x4B00 + complement, two by two
+    const uint32_t s = w01 + (w23 << (2 * Q));
+    // the four fields; everything above the low 4 * Q bits is dropped by the caller's store
+    constexpr uint32_t W = 0x4B004B00u, S = W + (W << (2 * Q));
+    if (Q == 2) return 0xFFu + (S + (S >> 14)) - (s + (s >> 14));
+    return 0xFFFFu + (S + ((S >> 16) << Q)) - (s + ((s >> 16) << Q));
+}
+
+// the same codes by the general route (clamped, any parameters)
+template <int Q>
+__device__ __forceinline__ uint32_t quant4_general(uint64_t xy, uint64_t zw, uint64_t delta2, uint64_t scale2, uint64_t z) {
+    return quant_row<Q>(xy, zw, 0ull, delta2, scale2, z);        // r - 0 is r (a zero's sign does not reach the codes)
+}
+template <int Q, bool FIXED>
+__device__ __forceinline__ uint32_t quant4_res(uint64_t xy, uint64_t zw, uint64_t delta2, uint64_t mul2, uint64_t z) {
+    if constexpr (FIXED && Q <= 4) return quant4_fixed<Q>(xy, zw, delta2, mul2, z);
+    else return quant4_general<Q>(xy, zw, delta2, mul2, z);
+}
+
+// ------------------------------------------------------------------------------------------------
+// half 1: one slot = NC adjacent columns of one tile of one band
+// ------------------------------------------------------------------------------------------------
+// How a slot is read: NC columns (4; 2 where 16 rows of 4 would not fit the registers), VW of them at a time (4, 2 or 1:
+// what the alignment of the rows allows).  Where a row takes several accesses, lane groups take them in different
+// orders: access u reads the columns VW * (u ^ swap) ..., swap from the lane number.  Neighbouring lanes are NC words
+// apart, so with one order for all NC / VW lanes would meet in every bank; with these orders none do.  A slot's columns
+// then sit in the registers in a lane-dependent order, of which every sum below is independent: swap only exchanges
+// the operands of an addition.
+template <int NC_, int VW_> struct SlotGeo {
+    static constexpr int NC = NC_, VW = VW_, NU = NC_ / VW_, NV = NC_ / 2;
+    static __device__ __forceinline__ uint32_t swap(uint32_t lane) { return NU == 4 ? (lane >> 3) & 3u : NU == 2 ? (NC == 4 ? (lane >> 3) & 1u : lane >> 4) : 0u; }
+};
+template <typename XT, typename G>
+__device__ __forceinline__ void slot_row_load(const XT* p, const uint32_t (&col)[G::NU], uint64_t (&v)[G::NV]) {
+    if constexpr (G::VW == 4) {
+        StripRow2<XT>::load(reinterpret_cast<const unsigned char*>(p), v[0], v[1]);
+    } else if constexpr (G::VW == 2) {
+#pragma unroll
+        for (int u = 0; u < G::NU; ++u) v[u] = ColLoad<XT, 2>::load(p + col[u]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < G::NV; ++u) {
+            if constexpr (sizeof(XT) == 4) {
+                v[u] = pk2(p[col[2 * u]], p[col[2 * u + 1]]);
+            } else {
+                const uint16_t* h = reinterpret_cast<const uint16_t*>(p);
+                v[u] = pk2u((uint32_t)h[col[2 * u]] << 16, (uint32_t)h[col[2 * u + 1]] << 16);
+            }
+        }
+    }
+}
+
+struct SlotSink {
+    void* lfc;
+    uint64_t lfc_at;          // where the tile's low-frequency value goes
+    int32_t lfc_bf16;
+    bool writer;              // this lane stores it
+    float inv, cnt, rcp;      // 1 / count when that is a power of two, else 0; count; RN(1 / count)
+};
+// Mean of a slot's tile as it is stored.  Every lane of the warp calls it (lanes of a tile meet by shuffles); columns a
+// lane does not own count as zeros.
+template <typename XT, int P2, typename G, int ROWS>
+__device__ __forceinline__ float slot_mean(const uint64_t (&v)[ROWS][G::NV], const bool (&ok)[G::NU], bool any, const SlotSink& s) {
+    constexpr int NV = G::NV;
+    constexpr uint32_t LPT = P2 / G::NC;                       // lanes per tile
+    // tile sum in the fixed order: balanced tree down the rows of each column (missing rows are zeros), then across the columns
+    float part[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        uint64_t t[P2];
+#pragma unroll
+        for (int r = 0; r < P2; ++r) t[r] = r < ROWS ? v[r < ROWS ? r : 0][k] : 0ull;
+#pragma unroll
+        for (int w = P2 / 2, left = ROWS; w >= 1; w >>= 1, left = (left + 1) / 2)
+#pragma unroll
+            for (int i = 0; i < w; ++i)
+                if (2 * i < left) t[i] = add2_rn(t[2 * i], 2 * i + 1 < left ? t[2 * i + 1] : 0ull);
+        float c0, c1;
+        upk2(t[0], c0, c1);
+        // what was loaded for a column the lane does not own belongs to somebody else
+        if (!ok[G::VW == 1 ? 2 * k : G::VW == 2 ? k : 0]) c0 = 0.f;
+        if (!ok[G::VW == 1 ? 2 * k + 1 : G::VW == 2 ? k : 0]) c1 = 0.f;
+        part[k] = __fadd_rn(c0, c1);
+    }
+    float sum = NV == 2 ? __fadd_rn(part[0], part[NV - 1]) : part[0];
+#pragma unroll
+    for (int m = 1; m < (int)LPT; m <<= 1) sum = __fadd_rn(sum, __shfl_xor_sync(0xFFFFFFFFu, sum, m));
+    const float mean = s.inv != 0.f ? __fmul_rn(sum, s.inv) : div_by_count(sum, s.cnt, s.rcp);
+    if (any && s.writer) {
+        if (s.lfc_bf16) Elem<__nv_bfloat16>::store(reinterpret_cast<__nv_bfloat16*>(s.lfc) + s.lfc_at, mean);
+        else reinterpret_cast<float*>(s.lfc)[s.lfc_at] = mean;
+    }
+    return s.lfc_bf16 ? Elem<__nv_bfloat16>::round(mean) : mean;
+}
+
+// One slot of half 1 whose residuals go to shared memory.  All slots of a warp have the same number of rows, ROWS; a lane
+// owns the first `cols` of its NC columns (0: none; it loads from anywhere in bounds).  xs / rp: first element of the
+// slot where x landed / where the residual goes (the same place for fp32).  lo / hi collect the residual's extremes.
+template <typename XT, int P2, typename G, int ROWS>
+__device__ __forceinline__ void reduce_slot_rows(const XT* xs, float* rp, uint32_t W, uint32_t cols, const SlotSink& s, float& lo, float& hi) {
+    constexpr int NV = G::NV, NU = G::NU;
+    const uint32_t sw = G::swap(threadIdx.x & 31u);
+    uint32_t col[NU];
+    bool ok[NU];
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+        col[u] = ((uint32_t)u ^ sw) * G::VW;
+        ok[u] = col[u] < cols;
+    }
+    uint64_t v[ROWS][NV];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) slot_row_load<XT, G>(xs + r * W, col, v[r]);
+    const float stored = slot_mean<XT, P2, G, ROWS>(v, ok, cols != 0u, s);
+    if (cols != 0u) {
+        // residuals back to shared memory; extremes of x (x -> fl(x - stored) is monotone): of the columns of one access
+        // together, or of two rows at a time where every column has to be kept apart
+        const uint64_t stored2 = pk2(stored, stored);
+        float l[NU], h[NU];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            l[u] = 3.402823466e+38f;
+            h[u] = -3.402823466e+38f;
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            float x[2 * NV], y[2 * NV];
+            uint64_t d[NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                d[k] = sub2_rn(v[r][k], stored2);
+                upk2(v[r][k], x[2 * k], x[2 * k + 1]);
+            }
+            float* row = rp + r * W;
+            if constexpr (G::VW == 4) {
+                l[0] = fmin3(fmin3(l[0], x[0], x[1]), x[2], x[3]);
+                h[0] = fmax3(fmax3(h[0], x[0], x[1]), x[2], x[3]);
+                ulonglong2 q;
+                q.x = d[0];
+                q.y = d[1];
+                *reinterpret_cast<ulonglong2*>(row) = q;
+            } else if constexpr (G::VW == 2) {
+#pragma unroll
+                for (int u = 0; u < NU; ++u) {
+                    l[u] = fmin3(l[u], x[2 * u], x[2 * u + 1]);
+                    h[u] = fmax3(h[u], x[2 * u], x[2 * u + 1]);
+                    if (ok[u]) *reinterpret_cast<uint64_t*>(row + col[u]) = d[u];
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < NV; ++k) {
+                    upk2(v[r % 2 == 1 ? r - 1 : r][k], y[2 * k], y[2 * k + 1]);
+                    if (r % 2 == 1 || r + 1 == ROWS) {
+#pragma unroll
+                        for (int c = 2 * k; c < 2 * k + 2; ++c) {
+                            l[c] = fmin3(l[c], x[c], y[c]);
+                            h[c] = fmax3(h[c], x[c], y[c]);
+                        }
+                    }
+                    float d0, d1;
+                    upk2(d[k], d0, d1);
+                    if (ok[2 * k]) row[col[2 * k]] = d0;
+                    if (ok[2 * k + 1]) row[col[2 * k + 1]] = d1;
+                }
+            }
+        }
+        float lx = 3.402823466e+38f, hx = -3.402823466e+38f;
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            if (NU == 1 || ok[u]) {
+                lx = fminf(lx, l[u]);
+                hx = fmaxf(hx, h[u]);
+            }
+        }
+        lo = fminf(lo, __fsub_rn(lx, stored));
+        hi = fmaxf(hi, __fsub_rn(hx, stored));
+    }
+}
+// the row count is the same in the whole warp: one unrolled body for each
+template <typename XT, int P2, typename G, int ROWS = P2>
+__device__ __forceinline__ void reduce_slot(const XT* xs, float* rp, uint32_t W, uint32_t rows, uint32_t cols, const SlotSink& s, float& lo,
+                                            float& hi) {
+    if (ROWS == 1 || rows == (uint32_t)ROWS) reduce_slot_rows<XT, P2, G, ROWS>(xs, rp, W, cols, s, lo, hi);
+    else if constexpr (ROWS > 1) reduce_slot<XT, P2, G, ROWS - 1>(xs, rp, W, rows, cols, s, lo, hi);
+}
+
+}  // namespace divk

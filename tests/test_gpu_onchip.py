@@ -1,0 +1,78 @@
+"""The compress kernels that keep x on chip between their two halves: exact parity with the CPU checker at the edges of
+their tilings (widths of every alignment, short bands, narrow tiles, shares that do not divide evenly, degenerate and
+extreme values that leave the fixed-point quantiser), and their bounded wait."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import division_oracle as orc
+from paper_2208_04187_b200 import binding, build, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built_library():
+    build.build()
+    binding.lib()
+
+
+def check(x_np, block, q, seed, xd="f32", ld="f32", on_chip=1):
+    codec = binding.Codec(*x_np.shape, block, q, xd, ld)
+    assert codec.plan().on_chip == on_chip
+    t = torch.from_numpy(x_np)
+    t = (t.view(torch.bfloat16) if xd == "bf16" else t).cuda()
+    codec.compress(t, seed=seed)
+    ref = orc.compress(x_np, block, q, seed, xd, ld)
+    torch.cuda.synchronize()
+    assert codec.device_status() == binding.DIV_OK
+    np.testing.assert_array_equal(codec.blob.cpu().numpy(), ref.blob())
+
+
+def make(shape, kind, seed, xd):
+    x = synth.activation_map(*shape, kind, seed)
+    return synth.to_bf16_bits(x) if xd == "bf16" else x
+
+
+CLUSTER = [   # n, c, h, w, block, q, x, lfc
+    (3, 8, 32, 32, 8, 2, "f32", "f32"), (2, 37, 8, 12, 8, 4, "f32", "bf16"), (5, 4, 7, 7, 8, 2, "f32", "f32"),
+    (2, 36, 13, 9, 4, 8, "f32", "f32"), (2, 12, 75, 75, 8, 2, "f32", "bf16"), (3, 8, 61, 47, 16, 2, "bf16", "bf16"),
+    (2, 8, 33, 34, 16, 4, "f32", "f32"), (2, 24, 14, 14, 8, 2, "bf16", "f32"), (4, 16, 19, 19, 8, 4, "bf16", "bf16"),
+    (1, 4, 5, 5, 4, 2, "f32", "f32"), (2, 16, 30, 10, 12, 2, "f32", "f32"), (2, 8, 21, 6, 6, 8, "f32", "f32"),
+    (9, 64, 4, 4, 8, 2, "f32", "f32"), (1, 2048, 7, 7, 8, 2, "f32", "f32"), (2, 3, 100, 100, 8, 4, "f32", "f32"),
+]
+
+
+@pytest.mark.parametrize("case", CLUSTER, ids=lambda c: "x".join(map(str, c)))
+def test_cluster_kernel_matches_the_checker(case):
+    n, c, h, w, block, q, xd, ld = case
+    check(make((n, c, h, w), "bn" if c % 3 else "relu", 11 + h, xd), block, q, 77, xd, ld)
+
+
+@pytest.mark.parametrize("q", [2, 4])
+def test_values_outside_the_fixed_point_route(q):
+    """Constant, tiny, huge and one-sided samples beside an ordinary one."""
+    x = make((6, 16, 14, 14), "bn", 5, "f32")
+    x[0] = 3.25
+    x[1] *= np.float32(1e-30)
+    x[2] *= np.float32(1e30)
+    x[3] = 0.0
+    x[4, 0, 0, 0] = 1e6
+    check(x, 8, q, 9)
+
+
+def test_cluster_kernel_gives_up_a_wait_that_cannot_end():
+    x_np = make((4, 32, 14, 14), "relu", 3, "f32")
+    x = torch.from_numpy(x_np).cuda()
+    codec = binding.Codec(*x_np.shape, 8, 2)
+    assert codec.plan().on_chip == 1
+    st = binding.lib().div_debug_compress_starved(
+        ctypes.byref(codec.desc), ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(codec.blob.data_ptr()), codec.blob.numel(),
+        ctypes.c_void_p(codec.workspace.data_ptr()), codec.workspace.numel(), 0, ctypes.c_void_p(binding.current_stream_handle()),
+        0, 2_000_000)
+    assert st == binding.DIV_OK
+    torch.cuda.synchronize()
+    assert codec.device_status() == binding.DIV_ERR_TIMEOUT
+    check(x_np, 8, 2, 5)
