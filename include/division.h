@@ -121,7 +121,8 @@ typedef struct div_plan {
     int64_t chunks_per_sample;
     int32_t decompress_fast;/* 1: quad kernel (W%4==0, B a power of two >= 4); 3: the same conditions on a 1-D map
                                (h == 1): line kernel; 2: flat kernel with a tile table (sample size a multiple of 4,
-                               planes up to 8192 elements); 0: general */
+                               planes up to 8192 elements); 4: row kernel (sample size a multiple of 4, rows of at
+                               least 4 elements, planes too large for the table); 0: general */
     int32_t on_chip;        /* 1: the cluster kernel takes the descriptor first (x is read once and waits in shared memory; a
                                thread-block cluster per sample); the fields above then describe the kernel that runs where
                                the device refuses clusters of that size.  0: they describe what runs */

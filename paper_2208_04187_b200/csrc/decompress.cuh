@@ -331,4 +331,86 @@ decompress_flat_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ 
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// row kernel: any width >= 4, any B, any height, sample size a multiple of 4 elements.
+// A CTA produces 1024 * QPT consecutive elements.  The low-frequency values of the bands (tile rows) that it touches
+// stand in shared memory UPSAMPLED ALONG THE ROW, W values per band, so that element (band, w) finds its value at
+// band * W + w and a quad's 4 values follow each other, but for one possible step to the next row.  Lanes read their 4
+// values in different orders (element (i ^ lane / 8) first): at 4 words from lane to lane one order would meet in 8 banks.
+// The row of a quad is found by divisions once per thread; from one quad to the next (1024 elements on) it is stepped.
+// HBM writes bound it by its roofline (7.6 us for 32 x 64 x 75 x 75 fp32, 46 MB); it takes 15.4 us (3.2 TB/s), the general
+// kernel, a thread per packed word with stores 64 bytes apart, 51 us.
+// grid = (ceil(quads_per_sample / (256*QPT)), N), dynamic shared memory = 4 * bands * W bytes
+// ---------------------------------------------------------------------------------------------
+struct DecRows {
+    uint32_t qps;            // quads per sample
+    uint32_t tiles;          // low-frequency values of a sample
+    uint32_t H, W, Hb, Wb;
+    uint32_t bands;          // most bands that a CTA touches
+    uint32_t step_rows, step_cols;      // 1024 elements = step_rows rows and step_cols columns
+    FastDiv by_w, by_h, by_b;
+};
+template <typename XT, typename LT, int Q, int QPT>
+__global__ void __launch_bounds__(256)
+decompress_rows_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
+                       const float* __restrict__ stats, XT* __restrict__ xhat, const DecRows d) {
+    extern __shared__ __align__(16) float rows_smem[];
+    __shared__ DeqTable<Q> table;
+    const uint32_t n = blockIdx.y;
+    const uint64_t sample_quad0 = (uint64_t)n * d.qps;
+    const uint32_t q0 = blockIdx.x * (256u * QPT) + threadIdx.x;
+    uint32_t bits[QPT];
+#pragma unroll
+    for (int k = 0; k < QPT; ++k) bits[k] = q0 + k * 256u < d.qps ? quad_bits<Q>(packed, sample_quad0 + q0 + k * 256u) : 0u;
+    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
+    const uint32_t first_row = fdiv(blockIdx.x * (1024u * QPT), d.by_w);
+    const uint32_t first_plane = fdiv(first_row, d.by_h);
+    const uint32_t band0 = first_plane * d.Hb + fdiv(first_row - first_plane * d.H, d.by_b);      // bands counted through the sample
+    const LT* src = lfc + (uint64_t)n * d.tiles + (uint64_t)band0 * d.Wb;
+    const uint32_t left = d.tiles - band0 * d.Wb;
+    for (uint32_t i = threadIdx.x; i < d.bands * d.W; i += 256u) {
+        const uint32_t b = fdiv(i, d.by_w);
+        const uint32_t t = b * d.Wb + fdiv(i - b * d.W, d.by_b);
+        rows_smem[i] = t < left ? Elem<LT>::load(src + t) : 0.f;
+    }
+    __syncthreads();
+    uint32_t row = fdiv(4u * q0, d.by_w);
+    uint32_t w = 4u * q0 - row * d.W;
+    uint32_t plane = fdiv(row, d.by_h);
+    uint32_t h = row - plane * d.H;
+    const uint32_t swap = (threadIdx.x >> 3) & 3u;
+#pragma unroll
+    for (int k = 0; k < QPT; ++k) {
+        const uint32_t q = q0 + k * 256u;
+        if (q < d.qps) {
+            const uint32_t band = fdiv(h, d.by_b);
+            const uint32_t at = (plane * d.Hb + band - band0) * d.W + w;
+            // where the next row lies in the same band the walk along the row starts over, else it goes on into the next band
+            const uint32_t back = (h + 1u != d.H && fdiv(h + 1u, d.by_b) == band) ? d.W : 0u;
+            const float4 hq = table.quad(bits[k]);
+            float lf[4];
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) {
+                const uint32_t e = i ^ swap;
+                lf[i] = rows_smem[at + e - (w + e >= d.W ? back : 0u)];
+            }
+            // lf[i] is the value of element i ^ swap: undo the exchange
+            const bool s1 = swap & 1u, s2 = swap & 2u;
+            const float a0 = s2 ? lf[2] : lf[0], a1 = s2 ? lf[3] : lf[1], a2 = s2 ? lf[0] : lf[2], a3 = s2 ? lf[1] : lf[3];
+            Quad<XT>::store(xhat + (sample_quad0 + q) * 4u, __fadd_rn(s1 ? a1 : a0, hq.x), __fadd_rn(s1 ? a0 : a1, hq.y),
+                            __fadd_rn(s1 ? a3 : a2, hq.z), __fadd_rn(s1 ? a2 : a3, hq.w));
+        }
+        w += d.step_cols;
+        h += d.step_rows;
+        if (w >= d.W) {
+            w -= d.W;
+            ++h;
+        }
+        while (h >= d.H) {
+            h -= d.H;
+            ++plane;
+        }
+    }
+}
+
 }  // namespace divk

@@ -290,6 +290,22 @@ bool decompress_flat_ok(const Shape& s) {
            flat_smem_bytes(4u * 256u * FLAT_QPT, s.HW, s.TPP) <= 40000;
 }
 
+// bands that a run of `elems` elements can touch, and whether the row kernel takes the map: at most 40 KB of shared memory
+uint64_t rows_bands(const Shape& s, uint32_t elems) {
+    const uint64_t planes = elems / s.HW + 2u;             // whole or in part
+    const uint64_t by_rows = (uint64_t)(elems / s.W + 1u) / s.B + 2u + planes;
+    const uint64_t all = planes * s.Hb;
+    return by_rows < all ? by_rows : all;
+}
+// Against the flat kernel the row kernel wins once building the quad table shows (64 x 64 x 90 x 90 54 -> 35 us, 24 x 64 x 61 x 47
+// 13.5 -> 8.2 us, 35 x 35 13.3 -> 12.3 us) and loses on small planes, where its bands hold few rows (34 x 34 16.6 against
+// 26.7 us, 14 x 14 13.3 against 18.5 us): from 2048 elements per plane on.
+bool decompress_rows_ok(const Shape& s) {
+    if (decompress_flat_ok(s) && s.HW < 2048u) return false;
+    return s.W >= 4 && s.CHW % 4 == 0 && s.N <= 65535 && s.CHW < (1u << 31) &&
+           rows_bands(s, 1024u * FLAT_QPT) * s.W * 4u <= 40000u;
+}
+
 }  // namespace
 
 extern "C" {
@@ -382,7 +398,7 @@ div_status div_plan_query(const div_desc* desc, uint32_t flags, div_plan* out) {
         out->threads = 256;
     }
     if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl)) out->on_chip = 1;
-    out->decompress_fast = decompress_fast_ok(s) ? ((s.H == 1 && s.CHW < (1u << 31)) ? 3 : 1) : (decompress_flat_ok(s) ? 2 : 0);
+    out->decompress_fast = decompress_fast_ok(s) ? ((s.H == 1 && s.CHW < (1u << 31)) ? 3 : 1) : decompress_rows_ok(s) ? 4 : (decompress_flat_ok(s) ? 2 : 0);
     return DIV_OK;
 }
 
@@ -531,6 +547,22 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                     decompress_quad_kernel<XT, LT, Q, DEC_QPT, true><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
                 else
                     decompress_quad_kernel<XT, LT, Q, DEC_QPT, false><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+            } else if (decompress_rows_ok(s)) {
+                DecRows d;
+                d.qps = s.CHW / 4;
+                d.tiles = s.C * s.TPP;
+                d.H = s.H;
+                d.W = s.W;
+                d.Hb = s.Hb;
+                d.Wb = s.Wb;
+                d.bands = (uint32_t)rows_bands(s, 1024u * FLAT_QPT);
+                d.step_rows = 1024u / s.W;
+                d.step_cols = 1024u % s.W;
+                d.by_w = make_fastdiv(s.W);
+                d.by_h = make_fastdiv(s.H);
+                d.by_b = make_fastdiv(s.B);
+                dim3 grid((d.qps + 256u * FLAT_QPT - 1) / (256u * FLAT_QPT), s.N);
+                decompress_rows_kernel<XT, LT, Q, FLAT_QPT><<<grid, 256, 4u * d.bands * d.W, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
             } else if (decompress_flat_ok(s)) {
                 DecFlat d;
                 d.qps = s.CHW / 4;
