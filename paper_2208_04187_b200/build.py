@@ -11,7 +11,7 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libdivision.so")
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
-SOURCES = ["division.cu", "cluster.cu"]
+SOURCES = ["division.cu", "cluster.cu", "planeshare.cu"]
 HEADERS = ["common.cuh", "cluster_plan.cuh", "halves.cuh", "twopass.cuh", "decompress.cuh", "fused.cuh", "fused_v.cuh", "lagged.cuh", "staged.cuh", "planes.cuh", "planegroup.cuh", "masks.cuh", "lines.cuh", "volume.cuh", os.path.join("..", "..", "include", "division.h")]
 
 NVCC_FLAGS = [

@@ -18,23 +18,10 @@
 
 namespace divk {
 
-struct ClusterParams {
-    const void* x;
-    void* lfc;
-    void* packed;
+struct ClusterParams : ShareParams {
     float* stats;
-    uint32_t* ws;
-    uint64_t seed, timeout_ns;
-    uint32_t C, W, B, Hb, Wb, HW, TPP, qps;
-    uint32_t log2cs, ppc, ppp, res_bytes, expect_bytes;
-    uint32_t spb;             // slots per band (tile row) of a plane
-    uint32_t sppf;            // slots of full-height bands per plane
-    uint32_t sppt;            // slots of a short last band per plane (0: H % B == 0)
-    uint32_t tail_rows;
-    uint32_t partial;         // 1: the last tile of a row is narrower than B
-    int32_t qbits, lfc_bf16;
-    FastDiv by_sppf, by_spb, by_ppp;
-    float inv[4], cnt[4], rcp[4];     // [short band][narrow tile]: 1 / count when that is a power of two, else 0; count; RN(1 / count)
+    uint32_t log2cs, expect_bytes;
+    int32_t qbits;
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -57,20 +44,6 @@ __device__ __forceinline__ void st_async_u64(uint64_t* dst, uint64_t v, uint64_t
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(d), "l"(v), "r"(b) : "memory");
 }
 
-__device__ __forceinline__ bool cl_wait(uint64_t* bar, uint64_t timeout_ns) {
-    if (mbar_try_wait(bar, 0)) return true;
-    uint32_t polls = 0;
-    uint64_t t0 = 0;
-    while (!mbar_try_wait(bar, 0)) {
-        if ((++polls & 15u) == 0) {
-            const uint64_t t = now_ns();
-            if (t0 == 0) t0 = t;
-            if (t - t0 > timeout_ns) return false;
-        }
-    }
-    return true;
-}
-
 // ------------------------------------------------------------------------------------------------
 // half 2: the CTA's residuals, 4 consecutive elements per thread and step
 // ------------------------------------------------------------------------------------------------
@@ -82,18 +55,18 @@ __device__ __forceinline__ void cl_half2(const float* res, typename PackedUnit<Q
     const float m = FIXED ? -65536.0f * scale : scale;
     const uint64_t mul2 = pk2(m, m);
     constexpr int U = 4;
-    constexpr uint64_t STEP = K_GROUP * (uint64_t)CL_THREADS;
+    constexpr uint64_t STEP = K_GROUP * (uint64_t)SHARE_THREADS;
     uint32_t q = threadIdx.x;
-    for (; q + (U - 1) * CL_THREADS < nq; q += U * CL_THREADS) {
+    for (; q + (U - 1) * SHARE_THREADS < nq; q += U * SHARE_THREADS) {
         ulonglong2 v[U];
 #pragma unroll
-        for (int k = 0; k < U; ++k) v[k] = reinterpret_cast<const ulonglong2*>(res)[q + k * CL_THREADS];
+        for (int k = 0; k < U; ++k) v[k] = reinterpret_cast<const ulonglong2*>(res)[q + k * SHARE_THREADS];
 #pragma unroll
         for (int k = 0; k < U; ++k)
-            out[q + k * CL_THREADS] = (OutT)quant4_res<Q, FIXED>(v[k].x, v[k].y, delta2, mul2, rng_mix(ctr + STEP * (uint64_t)k));
+            out[q + k * SHARE_THREADS] = (OutT)quant4_res<Q, FIXED>(v[k].x, v[k].y, delta2, mul2, rng_mix(ctr + STEP * (uint64_t)k));
         ctr += STEP * U;
     }
-    for (; q < nq; q += CL_THREADS) {
+    for (; q < nq; q += SHARE_THREADS) {
         const ulonglong2 v = reinterpret_cast<const ulonglong2*>(res)[q];
         out[q] = (OutT)quant4_res<Q, FIXED>(v.x, v.y, delta2, mul2, rng_mix(ctr));
         ctr += STEP;
@@ -113,73 +86,23 @@ __device__ __forceinline__ void cl_half2_q(const ClusterParams& p, const float* 
     else cl_half2<Q, false>(res, out, nq, ctr, qp.delta, qp.scale);
 }
 
-// ------------------------------------------------------------------------------------------------
-// half 1
-// ------------------------------------------------------------------------------------------------
-// Slots of the CTA's share are numbered so that every warp holds slots of one height: the full-height bands of all planes
-// first, then, from the next multiple of 32, the short last bands.
 template <typename XT, int P2, typename G>
-__device__ __forceinline__ void cl_half1(const ClusterParams& p, float* res, const XT* land, uint64_t* full, uint32_t n, uint32_t plane0,
-                                         uint32_t nplanes, float& lo, float& hi) {
-    constexpr uint32_t NC = G::NC, LPT = P2 / NC;               // lanes per tile
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t nfull = nplanes * p.sppf, first_short = (nfull + 31u) & ~31u, total = first_short + nplanes * p.sppt;
-    const uint64_t lfc0 = ((uint64_t)n * p.C + plane0) * p.TPP;
-    uint32_t landed = 0;
-    for (uint32_t first = warp * 32u; first < total; first += CL_THREADS) {
-        const bool short_band = first >= first_short;          // the same in the whole warp
-        const uint32_t S = first + lane;
-        const bool valid = short_band ? S < total : S < nfull;
-        const uint32_t T = valid ? (short_band ? S - first_short : S) : 0u;
-        const uint32_t plane = fdiv(T, short_band ? p.by_spb : p.by_sppf);
-        const uint32_t rem = T - plane * (short_band ? p.spb : p.sppf);
-        const uint32_t bf = fdiv(rem, p.by_spb);
-        const uint32_t band = short_band ? p.Hb - 1u : bf;
-        const uint32_t q = rem - bf * p.spb;                   // slot inside the band (a short band's rem is below spb)
-        const uint32_t bw = q / LPT, cw = (q % LPT) * NC;
-        const bool narrow = p.partial && bw + 1u == p.Wb;
-        const uint32_t cols = narrow ? p.W - bw * p.B : p.B;
-        const uint32_t mine = valid && cw < cols ? min(cols - cw, NC) : 0u;
-        const uint32_t off = mine ? plane * p.HW + (band * p.B) * p.W + bw * p.B + cw : 0u;
-        // pieces land in order; the unit's last slot needs the latest one
-        {
-            const uint32_t last = __shfl_sync(0xFFFFFFFFu, valid ? plane : nplanes - 1u, 31);
-            const uint32_t need = fdiv(last, p.by_ppp) + 1u;
-            while (landed < need) {
-                if (!cl_wait(&full[landed], p.timeout_ns)) atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
-                ++landed;
-            }
-        }
-        const uint32_t which = (short_band ? 2u : 0u) + (narrow ? 1u : 0u);
-        SlotSink sink;
-        sink.lfc = p.lfc;
-        sink.lfc_at = lfc0 + (plane * p.TPP + band * p.Wb + bw);
-        sink.lfc_bf16 = p.lfc_bf16;
-        sink.writer = cw == 0;
-        sink.inv = p.inv[which];
-        sink.cnt = p.cnt[which];
-        sink.rcp = p.rcp[which];
-        reduce_slot<XT, P2, G>(land + off, res + off, p.W, short_band ? p.tail_rows : p.B, mine, sink, lo, hi);
-    }
-}
-
-template <typename XT, int P2, typename G>
-__global__ void __launch_bounds__(CL_THREADS, 3)
+__global__ void __launch_bounds__(SHARE_THREADS, 3)
 cluster_kernel(const __grid_constant__ ClusterParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     float* res = reinterpret_cast<float*>(smem);
     const XT* land = reinterpret_cast<const XT*>(sizeof(XT) == 4 ? smem : smem + p.res_bytes);
-    __shared__ __align__(8) uint64_t full[CL_PIECES];
+    __shared__ __align__(8) uint64_t full[SHARE_PIECES];
     __shared__ __align__(8) uint64_t xbar;
     __shared__ __align__(8) uint64_t xch[CL_MAX];
-    __shared__ uint32_t wkey[2][CL_WARPS];
+    __shared__ uint32_t wkey[2][SHARE_WARPS];
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank(), n = blockIdx.x >> p.log2cs;
     const uint32_t plane0 = rank * p.ppc;
     const uint32_t nplanes = plane0 < p.C ? min(p.ppc, p.C - plane0) : 0u;
     if (tid == 0) {
 #pragma unroll
-        for (uint32_t i = 0; i < CL_PIECES; ++i) mbar_init(&full[i], 1);
+        for (uint32_t i = 0; i < SHARE_PIECES; ++i) mbar_init(&full[i], 1);
         mbar_init(&xbar, 1);
         fence_barrier_init();
         mbar_arrive_expect_tx(&xbar, p.expect_bytes);
@@ -187,18 +110,13 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
             p.ws[0] = 0u;
             p.ws[1] = 0u;
         }
-        const XT* src = reinterpret_cast<const XT*>(p.x) + ((uint64_t)n * p.C + plane0) * p.HW;
-        for (uint32_t i = 0, a = 0; a < nplanes; ++i, a += p.ppp) {
-            const uint32_t bytes = min(p.ppp, nplanes - a) * p.HW * (uint32_t)sizeof(XT);
-            mbar_arrive_expect_tx(&full[i], bytes);
-            bulk_load(const_cast<XT*>(land) + (size_t)a * p.HW, src + (size_t)a * p.HW, bytes, &full[i]);
-        }
+        share_load(p, const_cast<XT*>(land), full, n, plane0, nplanes);
     }
     __syncthreads();
     cluster_arrive();                          // waited for below, before anything is sent to another CTA
 
     float lo = 3.402823466e+38f, hi = -3.402823466e+38f;
-    if (nplanes) cl_half1<XT, P2, G>(p, res, land, full, n, plane0, nplanes, lo, hi);
+    if (nplanes) share_half1<XT, P2, G, false>(p, res, land, full, n, plane0, nplanes, nullptr, lo, hi);
     {
         const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, ~float_key(lo));
         const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, float_key(hi));
@@ -210,11 +128,11 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
     __syncthreads();                           // also: every residual is in place
     cluster_wait();
     if (warp == 0) {
-        const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, lane < CL_WARPS ? wkey[0][lane] : 0u);
-        const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, lane < CL_WARPS ? wkey[1][lane] : 0u);
+        const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, lane < SHARE_WARPS ? wkey[0][lane] : 0u);
+        const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, lane < SHARE_WARPS ? wkey[1][lane] : 0u);
         if (lane < (1u << p.log2cs)) st_async_u64(&xch[rank], ((uint64_t)kmax << 32) | kmin, &xbar, lane);
     }
-    if (!__all_sync(0xFFFFFFFFu, cl_wait(&xbar, p.timeout_ns))) {
+    if (!__all_sync(0xFFFFFFFFu, share_wait(&xbar, p.timeout_ns))) {
         if (tid == 0) {
             atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
             atomicCAS(p.ws + 1, 0u, n + 1u);
@@ -246,7 +164,7 @@ inline div_status launch_cluster(const ClusterParams& prm, const ClusterPlan& pl
     if (pl.cs > 8 && !ensure_wide_cluster((const void*)kern, wide_set)) return DIV_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(N * pl.cs);
-    cfg.blockDim = dim3(CL_THREADS);
+    cfg.blockDim = dim3(SHARE_THREADS);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
@@ -289,30 +207,11 @@ div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout&
     p.ws = ws;
     p.seed = seed;
     p.timeout_ns = timeout_ns ? timeout_ns : 2000000000ull;
-    p.C = s.C; p.W = s.W; p.B = s.B; p.Hb = s.Hb; p.Wb = s.Wb; p.HW = s.HW; p.TPP = s.TPP; p.qps = s.CHW / 4;
+    fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
     p.log2cs = 0;
     while ((1u << p.log2cs) < pl.cs) ++p.log2cs;
-    p.ppc = pl.ppc; p.ppp = pl.ppp; p.res_bytes = pl.res_bytes;
     p.expect_bytes = expect_bytes ? expect_bytes : 8u * pl.cs;
-    const uint32_t nc = s.P2 == 16 ? 2u : 4u;                  // columns of a slot
-    p.spb = s.Wb * (s.P2 / nc);
-    const bool tail = s.H % s.B != 0;
-    p.sppf = (tail ? s.Hb - 1u : s.Hb) * p.spb;
-    p.sppt = tail ? p.spb : 0u;
-    p.tail_rows = s.H - (s.Hb - 1u) * s.B;
-    p.partial = s.W % s.B != 0 ? 1u : 0u;
     p.qbits = d->qbits;
-    p.lfc_bf16 = d->lfc_dtype == DIV_BF16 ? 1 : 0;
-    p.by_sppf = host_fastdiv(p.sppf ? p.sppf : 1u);
-    p.by_spb = host_fastdiv(p.spb);
-    p.by_ppp = host_fastdiv(p.ppp);
-    const uint32_t tail_cols = s.W - (s.Wb - 1u) * s.B;
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t cnt = ((i & 2) ? p.tail_rows : s.B) * ((i & 1) ? tail_cols : s.B);
-        p.cnt[i] = (float)cnt;
-        p.rcp[i] = 1.0f / (float)cnt;
-        p.inv[i] = (cnt & (cnt - 1u)) == 0 ? p.rcp[i] : 0.f;
-    }
     return d->x_dtype == DIV_F32 ? launch_cluster_p2<float>(p, pl, s, st) : launch_cluster_p2<__nv_bfloat16>(p, pl, s, st);
 }
 

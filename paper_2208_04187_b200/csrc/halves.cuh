@@ -4,7 +4,8 @@
 //   half 2  Eq. 9 on groups of 4 consecutive residuals, which needs no notion of tiles.
 #pragma once
 
-#include "planes.cuh"      // ColLoad; quant_row, packed pairs
+#include "cluster_plan.cuh" // SharePlan
+#include "planes.cuh"       // ColLoad; quant_row, packed pairs
 
 namespace divk {
 
@@ -239,6 +240,145 @@ __device__ __forceinline__ void reduce_slot(const XT* xs, float* rp, uint32_t W,
                                             float& hi) {
     if (ROWS == 1 || rows == (uint32_t)ROWS) reduce_slot_rows<XT, P2, G, ROWS>(xs, rp, W, cols, s, lo, hi);
     else if constexpr (ROWS > 1) reduce_slot<XT, P2, G, ROWS - 1>(xs, rp, W, rows, cols, s, lo, hi);
+}
+
+// ------------------------------------------------------------------------------------------------
+// a CTA's share: a run of whole planes of one sample in shared memory
+// ------------------------------------------------------------------------------------------------
+struct ShareParams {
+    const void* x;
+    void* lfc;
+    void* packed;
+    uint32_t* ws;             // where a wait that ran out is recorded
+    uint64_t seed, timeout_ns;
+    uint32_t C, W, B, Hb, Wb, HW, TPP, qps;
+    uint32_t ppc, ppp;        // planes per CTA, planes per piece
+    uint32_t res_bytes;       // bf16: where the landing place begins, behind the fp32 residuals
+    uint32_t spb;             // slots per band (tile row) of a plane
+    uint32_t sppf;            // slots of full-height bands per plane
+    uint32_t sppt;            // slots of a short last band per plane (0: H % B == 0)
+    uint32_t tail_rows;
+    uint32_t partial;         // 1: the last tile of a row is narrower than B
+    int32_t lfc_bf16;
+    FastDiv by_sppf, by_spb, by_ppp;
+    float inv[4], cnt[4], rcp[4];     // [short band][narrow tile]: 1 / count when that is a power of two, else 0; count; RN(1 / count)
+};
+__device__ __forceinline__ bool share_wait(uint64_t* bar, uint64_t timeout_ns) {
+    if (mbar_try_wait(bar, 0)) return true;
+    uint32_t polls = 0;
+    uint64_t t0 = 0;
+    while (!mbar_try_wait(bar, 0)) {
+        if ((++polls & 15u) == 0) {
+            const uint64_t t = now_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > timeout_ns) return false;
+        }
+    }
+    return true;
+}
+
+// the copies of the share, one thread: piece i completes on full[i]
+template <typename XT>
+__device__ __forceinline__ void share_load(const ShareParams& p, XT* land, uint64_t* full, uint32_t n, uint32_t plane0, uint32_t nplanes) {
+    const XT* src = reinterpret_cast<const XT*>(p.x) + ((uint64_t)n * p.C + plane0) * p.HW;
+    for (uint32_t i = 0, a = 0; a < nplanes; ++i, a += p.ppp) {
+        const uint32_t bytes = min(p.ppp, nplanes - a) * p.HW * (uint32_t)sizeof(XT);
+        mbar_arrive_expect_tx(&full[i], bytes);
+        bulk_load(land + (size_t)a * p.HW, src + (size_t)a * p.HW, bytes, &full[i]);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// half 1 of a CTA's share: planes [plane0, plane0 + nplanes) of sample n, which land in shared memory in SHARE_PIECES pieces
+// ------------------------------------------------------------------------------------------------
+// keys (PER_PLANE): ~key(min), key(max) of the residuals of each plane; else lo / hi collect the extremes of the thread.
+// Slots of the CTA's share are numbered so that every warp holds slots of one height: the full-height bands of all planes
+// first, then, from the next multiple of 32, the short last bands.
+template <typename XT, int P2, typename G, bool PER_PLANE>
+__device__ __forceinline__ void share_half1(const ShareParams& p, float* res, const XT* land, uint64_t* full, uint32_t n, uint32_t plane0,
+                                         uint32_t nplanes, uint32_t* keys, float& lo, float& hi) {
+    constexpr uint32_t NC = G::NC, LPT = P2 / NC;               // lanes per tile
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t nfull = nplanes * p.sppf, first_short = (nfull + 31u) & ~31u, total = first_short + nplanes * p.sppt;
+    const uint64_t lfc0 = ((uint64_t)n * p.C + plane0) * p.TPP;
+    uint32_t landed = 0;
+    for (uint32_t first = warp * 32u; first < total; first += SHARE_THREADS) {
+        const bool short_band = first >= first_short;          // the same in the whole warp
+        const uint32_t S = first + lane;
+        const bool valid = short_band ? S < total : S < nfull;
+        const uint32_t T = valid ? (short_band ? S - first_short : S) : 0u;
+        const uint32_t plane = fdiv(T, short_band ? p.by_spb : p.by_sppf);
+        const uint32_t rem = T - plane * (short_band ? p.spb : p.sppf);
+        const uint32_t bf = fdiv(rem, p.by_spb);
+        const uint32_t band = short_band ? p.Hb - 1u : bf;
+        const uint32_t q = rem - bf * p.spb;                   // slot inside the band (a short band's rem is below spb)
+        const uint32_t bw = q / LPT, cw = (q % LPT) * NC;
+        const bool narrow = p.partial && bw + 1u == p.Wb;
+        const uint32_t cols = narrow ? p.W - bw * p.B : p.B;
+        const uint32_t mine = valid && cw < cols ? min(cols - cw, NC) : 0u;
+        const uint32_t off = mine ? plane * p.HW + (band * p.B) * p.W + bw * p.B + cw : 0u;
+        // pieces land in order; the unit's last slot needs the latest one
+        {
+            const uint32_t last = __shfl_sync(0xFFFFFFFFu, valid ? plane : nplanes - 1u, 31);
+            const uint32_t need = fdiv(last, p.by_ppp) + 1u;
+            while (landed < need) {
+                if (!share_wait(&full[landed], p.timeout_ns)) atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
+                ++landed;
+            }
+        }
+        const uint32_t which = (short_band ? 2u : 0u) + (narrow ? 1u : 0u);
+        SlotSink sink;
+        sink.lfc = p.lfc;
+        sink.lfc_at = lfc0 + (plane * p.TPP + band * p.Wb + bw);
+        sink.lfc_bf16 = p.lfc_bf16;
+        sink.writer = cw == 0;
+        sink.inv = p.inv[which];
+        sink.cnt = p.cnt[which];
+        sink.rcp = p.rcp[which];
+        if constexpr (!PER_PLANE) {
+            reduce_slot<XT, P2, G>(land + off, res + off, p.W, short_band ? p.tail_rows : p.B, mine, sink, lo, hi);
+        } else {
+            float l = 3.402823466e+38f, h = -3.402823466e+38f;
+            reduce_slot<XT, P2, G>(land + off, res + off, p.W, short_band ? p.tail_rows : p.B, mine, sink, l, h);
+            // lanes without a slot bring neutral extremes (whose keys are not neutral)
+            uint32_t kmin = mine ? ~float_key(l) : 0u, kmax = mine ? float_key(h) : 0u;
+            const uint32_t first_plane = __shfl_sync(0xFFFFFFFFu, plane, 0);
+            if (__all_sync(0xFFFFFFFFu, plane == first_plane || mine == 0u)) {
+                kmin = __reduce_max_sync(0xFFFFFFFFu, kmin);
+                kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
+                if (lane == 0) {
+                    atomicMax(&keys[2u * first_plane], kmin);
+                    atomicMax(&keys[2u * first_plane + 1u], kmax);
+                }
+            } else if (mine) {
+                atomicMax(&keys[2u * plane], kmin);
+                atomicMax(&keys[2u * plane + 1u], kmax);
+            }
+        }
+    }
+}
+
+inline void fill_share(ShareParams* p, const Shape& s, const SharePlan& pl, bool lfc_bf16) {
+    p->C = s.C; p->W = s.W; p->B = s.B; p->Hb = s.Hb; p->Wb = s.Wb; p->HW = s.HW; p->TPP = s.TPP; p->qps = s.CHW / 4;
+    p->ppc = pl.ppc; p->ppp = pl.ppp; p->res_bytes = pl.res_bytes;
+    const uint32_t nc = s.P2 == 16 ? 2u : 4u;                  // columns of a slot
+    p->spb = s.Wb * (s.P2 / nc);
+    const bool tail = s.H % s.B != 0;
+    p->sppf = (tail ? s.Hb - 1u : s.Hb) * p->spb;
+    p->sppt = tail ? p->spb : 0u;
+    p->tail_rows = s.H - (s.Hb - 1u) * s.B;
+    p->partial = s.W % s.B != 0 ? 1u : 0u;
+    p->lfc_bf16 = lfc_bf16 ? 1 : 0;
+    p->by_sppf = host_fastdiv(p->sppf ? p->sppf : 1u);
+    p->by_spb = host_fastdiv(p->spb);
+    p->by_ppp = host_fastdiv(p->ppp);
+    const uint32_t tail_cols = s.W - (s.Wb - 1u) * s.B;
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t cnt = ((i & 2) ? p->tail_rows : s.B) * ((i & 1) ? tail_cols : s.B);
+        p->cnt[i] = (float)cnt;
+        p->rcp[i] = 1.0f / (float)cnt;
+        p->inv[i] = (cnt & (cnt - 1u)) == 0 ? p->rcp[i] : 0.f;
+    }
 }
 
 }  // namespace divk

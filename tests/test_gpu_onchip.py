@@ -76,3 +76,24 @@ def test_cluster_kernel_gives_up_a_wait_that_cannot_end():
     torch.cuda.synchronize()
     assert codec.device_status() == binding.DIV_ERR_TIMEOUT
     check(x_np, 8, 2, 5)
+
+
+PLANE_SHARE = [   # n, c, h, w, block, q, x, lfc: odd widths beyond a warp, blocks of 16, quads that straddle planes
+    (2, 8, 75, 75, 8, 2, "f32", "f32"), (3, 12, 35, 35, 8, 4, "f32", "bf16"), (2, 5, 40, 40, 16, 4, "f32", "f32"),
+    (2, 8, 39, 37, 4, 8, "bf16", "bf16"), (1, 44, 9, 41, 16, 2, "f32", "f32"), (2, 16, 17, 70, 12, 2, "bf16", "f32"),
+    (4, 8, 3, 50, 4, 2, "f32", "f32"),
+]
+
+
+@pytest.mark.parametrize("case", PLANE_SHARE, ids=lambda c: "x".join(map(str, c)))
+def test_plane_share_kernel_matches_the_checker(case):
+    n, c, h, w, block, q, xd, ld = case
+    x_np = make((n, c, h, w), "bn", 31 + h, xd)
+    if xd == "f32":
+        x_np[0, 1] = 0.0                        # a degenerate plane beside ordinary ones
+        x_np[-1, 2] *= np.float32(1e-28)        # and one outside the fixed-point route
+    codec = binding.PlaneGroupCodec(n, c, h, w, block, q, xd, ld)
+    assert codec.plan().on_chip == 1
+    t = torch.from_numpy(x_np)
+    codec.compress((t.view(torch.bfloat16) if xd == "bf16" else t).cuda(), seed=13)
+    np.testing.assert_array_equal(codec.blob.cpu().numpy(), orc.compress_planes(x_np, block, q, 13, xd, ld).blob())
