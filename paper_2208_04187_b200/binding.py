@@ -1,4 +1,5 @@
-"""ctypes binding of libdivision.so: the same entry points as include/division.h, argument marshalling only.
+"""Binding of libdivision.so: the same entry points as include/division.h by ctypes, argument marshalling only, and the
+codec classes on torch tensors, whose calls go through a small CPython extension (csrc/native.cpp).
 
 Every step of compress / decompress runs inside the CUDA library.  PyTorch appears here only as the
 owner of device memory and streams.  If the library has not been built the import of the symbols
@@ -64,6 +65,7 @@ class DivisionError(RuntimeError):
 
 
 _lib = None
+_U64 = 2 ** 64 - 1
 
 
 def lib() -> ctypes.CDLL:
@@ -154,10 +156,9 @@ def div_plan_query(desc: DivDesc, flags: int = 0) -> DivPlan:
 def div_compress(desc: DivDesc, x_ptr: int, comp_ptr: int, comp_capacity: int, ws_ptr: int, ws_bytes: int,
                  seed: int, stream: int = 0, flags: int = 0) -> None:
     """Raw-pointer call (device pointers as integers, stream as a cudaStream_t handle)."""
-    st = lib().div_compress_ex(ctypes.byref(desc), c_void_p(x_ptr), c_void_p(comp_ptr), comp_capacity,
-                               c_void_p(ws_ptr), ws_bytes, c_uint64(seed & (2 ** 64 - 1)), c_void_p(stream),
-                               int(flags))
-    _check(st, "div_compress")
+    st = (_lib or lib()).div_compress_ex(desc, x_ptr, comp_ptr, comp_capacity, ws_ptr, ws_bytes, seed & _U64, stream, flags)
+    if st:
+        _check(st, "div_compress")
 
 
 DIV_STATIC_MAX_SAMPLES = 1024
@@ -182,9 +183,9 @@ def div_read_static_status(stream: int = 0) -> int:
 
 
 def div_decompress(desc: DivDesc, comp_ptr: int, comp_bytes: int, xhat_ptr: int, stream: int = 0) -> None:
-    st = lib().div_decompress(ctypes.byref(desc), c_void_p(comp_ptr), comp_bytes, c_void_p(xhat_ptr),
-                              c_void_p(stream))
-    _check(st, "div_decompress")
+    st = (_lib or lib()).div_decompress(desc, comp_ptr, comp_bytes, xhat_ptr, stream)
+    if st:
+        _check(st, "div_decompress")
 
 
 def div_planegroup_bytes(desc: DivDesc) -> DivLayout:
@@ -203,15 +204,15 @@ def div_planegroup_plan_query(desc: DivDesc, flags: int = 0) -> DivPlan:
 
 def div_planegroup_compress(desc: DivDesc, x_ptr: int, comp_ptr: int, comp_capacity: int, seed: int,
                             stream: int = 0, flags: int = 0) -> None:
-    st = lib().div_planegroup_compress(ctypes.byref(desc), c_void_p(x_ptr), c_void_p(comp_ptr), comp_capacity,
-                                       c_uint64(seed & (2 ** 64 - 1)), c_void_p(stream), int(flags))
-    _check(st, "div_planegroup_compress")
+    st = (_lib or lib()).div_planegroup_compress(desc, x_ptr, comp_ptr, comp_capacity, seed & _U64, stream, flags)
+    if st:
+        _check(st, "div_planegroup_compress")
 
 
 def div_planegroup_decompress(desc: DivDesc, comp_ptr: int, comp_bytes: int, xhat_ptr: int, stream: int = 0) -> None:
-    st = lib().div_planegroup_decompress(ctypes.byref(desc), c_void_p(comp_ptr), comp_bytes, c_void_p(xhat_ptr),
-                                         c_void_p(stream))
-    _check(st, "div_planegroup_decompress")
+    st = (_lib or lib()).div_planegroup_decompress(desc, comp_ptr, comp_bytes, xhat_ptr, stream)
+    if st:
+        _check(st, "div_planegroup_decompress")
 
 
 def make_desc_3d(n, c, d, h, w, block, qbits, x_dtype="f32", lfc_dtype="f32") -> DivDesc3D:
@@ -226,13 +227,15 @@ def div_compressed_bytes_3d(desc: DivDesc3D) -> DivLayout:
 
 def div_compress_3d(desc: DivDesc3D, x_ptr: int, comp_ptr: int, comp_capacity: int, ws_ptr: int, ws_bytes: int,
                     seed: int, stream: int = 0) -> None:
-    _check(lib().div_compress_3d(ctypes.byref(desc), c_void_p(x_ptr), c_void_p(comp_ptr), comp_capacity, c_void_p(ws_ptr),
-                                 ws_bytes, c_uint64(seed & (2 ** 64 - 1)), c_void_p(stream)), "div_compress_3d")
+    st = (_lib or lib()).div_compress_3d(desc, x_ptr, comp_ptr, comp_capacity, ws_ptr, ws_bytes, seed & _U64, stream)
+    if st:
+        _check(st, "div_compress_3d")
 
 
 def div_decompress_3d(desc: DivDesc3D, comp_ptr: int, comp_bytes: int, xhat_ptr: int, stream: int = 0) -> None:
-    _check(lib().div_decompress_3d(ctypes.byref(desc), c_void_p(comp_ptr), comp_bytes, c_void_p(xhat_ptr), c_void_p(stream)),
-           "div_decompress_3d")
+    st = (_lib or lib()).div_decompress_3d(desc, comp_ptr, comp_bytes, xhat_ptr, stream)
+    if st:
+        _check(st, "div_decompress_3d")
 
 
 def div_mask_bytes(total: int) -> int:
@@ -283,10 +286,37 @@ def torch_dtype(name: str):
 def current_stream_handle() -> int:
     """cudaStream_t of torch's current stream on the current device, as an integer."""
     torch = _torch()
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # one C call instead of building a Stream object
-    if raw is not None:
-        return int(raw(torch.cuda.current_device()))
-    return int(torch.cuda.current_stream().cuda_stream)
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())      # two C calls instead of building a Stream object
+    except AttributeError:
+        return int(torch.cuda.current_stream().cuda_stream)
+
+
+_native = None
+
+
+def native():
+    """The CPython extension behind the codec classes; raises if it was never built."""
+    global _native
+    if _native is None:
+        lib()
+        _torch()                         # its libraries first
+        path = os.path.join(os.path.dirname(LIB_PATH), "_native.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build it with `python -m paper_2208_04187_b200.build`")
+        import importlib.machinery
+        import importlib.util
+        loader = importlib.machinery.ExtensionFileLoader("_native", path)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_native", loader))
+        loader.exec_module(module)
+        _native = module
+    return _native
+
+
+def _raise(status: int, where: str):
+    if status == -1:
+        raise ValueError("x must be a contiguous CUDA tensor matching the descriptor")
+    raise DivisionError(status, where)
 
 
 class Codec:
@@ -301,28 +331,25 @@ class Codec:
         self.device = torch.device(device)
         self.blob = torch.zeros(int(self.layout.total_bytes), dtype=torch.uint8, device=self.device)
         self.workspace = torch.zeros(int(self.layout.workspace_bytes), dtype=torch.uint8, device=self.device)
+        self._native, self._addr = native(), ctypes.addressof(self.desc)
 
     def plan(self, flags: int = 0) -> DivPlan:
         return div_plan_query(self.desc, flags)
 
     def compress(self, x, seed: int = 0, flags: int = 0, blob=None):
         """x: contiguous CUDA tensor of shape N x C x H x W in the descriptor's dtype."""
-        torch = _torch()
-        blob = self.blob if blob is None else blob
-        if not (x.is_cuda and x.is_contiguous() and tuple(x.shape) == self.shape
-                and x.dtype == torch_dtype(self.x_dtype)):
-            raise ValueError("x must be a contiguous CUDA tensor matching the descriptor")
-        div_compress(self.desc, x.data_ptr(), blob.data_ptr(), blob.numel(), self.workspace.data_ptr(),
-                     self.workspace.numel(), seed, current_stream_handle(), flags)
+        if blob is None:
+            blob = self.blob
+        status = self._native.compress(self._addr, x, blob, self.workspace, seed, flags)
+        if status:
+            _raise(status, "div_compress")
         return blob
 
     def decompress(self, blob=None, out=None):
-        torch = _torch()
-        blob = self.blob if blob is None else blob
-        if out is None:
-            out = torch.empty(self.shape, dtype=torch_dtype(self.x_dtype), device=self.device)
-        div_decompress(self.desc, blob.data_ptr(), blob.numel(), out.data_ptr(), current_stream_handle())
-        return out
+        got = self._native.decompress(self._addr, self.blob if blob is None else blob, out, False)
+        if got.__class__ is int:
+            _raise(got, "div_decompress")
+        return got
 
     def device_status(self) -> int:
         return div_read_device_status(self.workspace.data_ptr(), current_stream_handle())
@@ -339,24 +366,21 @@ class PlaneGroupCodec:
         self.shape = (n, c, h, w)
         self.device = torch.device(device)
         self.blob = torch.zeros(int(self.layout.total_bytes), dtype=torch.uint8, device=self.device)
+        self._native, self._addr = native(), ctypes.addressof(self.desc)
 
     def plan(self, flags: int = 0) -> DivPlan:
         return div_planegroup_plan_query(self.desc, flags)
 
     def compress(self, x, seed: int = 0, flags: int = 0, blob=None):
-        torch = _torch()
-        blob = self.blob if blob is None else blob
-        if not (x.is_cuda and x.is_contiguous() and tuple(x.shape) == self.shape
-                and x.dtype == torch_dtype(self.x_dtype)):
-            raise ValueError("x must be a contiguous CUDA tensor matching the descriptor")
-        div_planegroup_compress(self.desc, x.data_ptr(), blob.data_ptr(), blob.numel(), seed,
-                                current_stream_handle(), flags)
+        if blob is None:
+            blob = self.blob
+        status = self._native.compress(self._addr, x, blob, None, seed, flags)
+        if status:
+            _raise(status, "div_planegroup_compress")
         return blob
 
     def decompress(self, blob=None, out=None):
-        torch = _torch()
-        blob = self.blob if blob is None else blob
-        if out is None:
-            out = torch.empty(self.shape, dtype=torch_dtype(self.x_dtype), device=self.device)
-        div_planegroup_decompress(self.desc, blob.data_ptr(), blob.numel(), out.data_ptr(), current_stream_handle())
-        return out
+        got = self._native.decompress(self._addr, self.blob if blob is None else blob, out, True)
+        if got.__class__ is int:
+            _raise(got, "div_planegroup_decompress")
+        return got

@@ -10,6 +10,8 @@ from concurrent.futures import ThreadPoolExecutor
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libdivision.so")
+NATIVE_SRC = os.path.join(CSRC, "native.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")        # the calls on torch tensors, linked against the library
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
 SOURCES = ["division.cu", "cluster.cu", "planeshare.cu"]
 HEADERS = ["common.cuh", "cluster_plan.cuh", "halves.cuh", "twopass.cuh", "decompress.cuh", "fused.cuh", "fused_v.cuh", "lagged.cuh", "staged.cuh", "planes.cuh", "planegroup.cuh", "masks.cuh", "lines.cuh", "volume.cuh", os.path.join("..", "..", "include", "division.h")]
@@ -31,11 +33,11 @@ def _nvcc() -> str:
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
     deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS]
-    return any(os.path.getmtime(d) > t for d in deps)
+    return any(os.path.getmtime(d) > t for d in deps) or os.path.getmtime(NATIVE_SRC) > os.path.getmtime(NATIVE_PATH)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -55,9 +57,25 @@ def build(force: bool = False, verbose: bool = False) -> str:
     with ThreadPoolExecutor(len(SOURCES)) as pool:          # one nvcc per source, side by side
         done = list(pool.map(compile_one, SOURCES))
     _run([_nvcc(), "-shared"] + NVCC_FLAGS[:2] + [obj for obj, _ in done] + ["-o", LIB_PATH], verbose, None)
+    _build_native(verbose)
     with open(os.path.join(PKG_DIR, "ptxas_info.log"), "w") as f:
         f.write("".join(open(log).read() for _, log in done))
     return LIB_PATH
+
+
+def _build_native(verbose):
+    """The CPython extension: host C++ only, needs torch's headers and libraries."""
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    includes = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    _run([shutil.which("g++") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC",
+          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + i for i in includes] +
+         [NATIVE_SRC, "-o", NATIVE_PATH, "-L" + os.path.join(root, "lib"), "-L" + PKG_DIR, "-ltorch_python", "-ltorch_cpu", "-lc10",
+          "-lc10_cuda", "-l:libdivision.so", "-Wl,-rpath,$ORIGIN"], verbose, None)
 
 
 def _run(cmd, verbose, log):
@@ -65,7 +83,7 @@ def _run(cmd, verbose, log):
     if verbose or proc.returncode != 0:
         sys.stderr.write(proc.stdout + proc.stderr)
     if proc.returncode != 0:
-        raise RuntimeError("nvcc failed building libdivision.so")
+        raise RuntimeError("building the library failed: " + os.path.basename(cmd[0]))
     if log:
         with open(log, "w") as f:
             f.write(proc.stderr)
