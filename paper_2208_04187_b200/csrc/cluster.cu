@@ -106,6 +106,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
         mbar_init(&xbar, 1);
         fence_barrier_init();
         mbar_arrive_expect_tx(&xbar, p.expect_bytes);
+        griddep_wait();
         if (blockIdx.x == 0) {
             p.ws[0] = 0u;
             p.ws[1] = 0u;
@@ -113,6 +114,8 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
         share_load(p, const_cast<XT*>(land), full, n, plane0, nplanes);
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
     cluster_arrive();                          // waited for below, before anything is sent to another CTA
 
     float lo = 3.402823466e+38f, hi = -3.402823466e+38f;
@@ -167,12 +170,14 @@ inline div_status launch_cluster(const ClusterParams& prm, const ClusterPlan& pl
     cfg.blockDim = dim3(SHARE_THREADS);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = pl.cs;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, kern, prm) != cudaSuccess) {
         cudaGetLastError();
         return DIV_ERR_CUDA;

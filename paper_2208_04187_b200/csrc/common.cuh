@@ -143,6 +143,10 @@ __device__ __forceinline__ float reconstruct(uint32_t code, float step, float de
     return __fadd_rn(lfc, __fadd_rn(__fmul_rn(step, cf), delta));
 }
 
+// programmatic dependent launch (see launch_pdl)
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // division of a 31-bit number by a runtime constant: q = (n * mul) >> shift, exact for n < 2^31
 struct FastDiv {
     uint32_t d, mul, shift;

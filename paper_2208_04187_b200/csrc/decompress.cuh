@@ -137,12 +137,13 @@ template <> struct DeqTable<8> {
 };
 
 // the packed bits of quad number `quad` (global numbering) of the code stream
+// (plain loads: in a kernel that may start before its predecessor ends, the read-only path is not for what that one writes)
 template <int Q>
-__device__ __forceinline__ uint32_t quad_bits(const uint32_t* __restrict__ packed, uint64_t quad) {
-    if (Q == 2) return __ldg(reinterpret_cast<const uint8_t*>(packed) + quad);
-    if (Q == 4) return __ldg(reinterpret_cast<const uint16_t*>(packed) + quad);
-    if (Q == 8) return __ldg(packed + quad);
-    return (__ldg(reinterpret_cast<const uint8_t*>(packed) + (quad >> 1)) >> (4u * (uint32_t)(quad & 1u))) & 15u;
+__device__ __forceinline__ uint32_t quad_bits(const uint32_t* packed, uint64_t quad) {
+    if (Q == 2) return *(reinterpret_cast<const uint8_t*>(packed) + quad);
+    if (Q == 4) return *(reinterpret_cast<const uint16_t*>(packed) + quad);
+    if (Q == 8) return *(packed + quad);
+    return (*(reinterpret_cast<const uint8_t*>(packed) + (quad >> 1)) >> (4u * (uint32_t)(quad & 1u))) & 15u;
 }
 
 // SPREAD: where a row is not a whole number of 32-byte sectors (28 fp32 columns: 112 bytes) the 4 rows of a work
@@ -151,12 +152,14 @@ __device__ __forceinline__ uint32_t quad_bits(const uint32_t* __restrict__ packe
 // different tiles, each with its own low-frequency value.
 template <typename XT, typename LT, int Q, int QPT, bool SPREAD>
 __global__ void __launch_bounds__(256)
-decompress_quad_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
-                       const float* __restrict__ stats, XT* __restrict__ xhat, DecFast d) {
+decompress_quad_kernel(const LT* lfc, const uint32_t* packed,
+                       const float* stats, XT* xhat, DecFast d) {
     static_assert(QPT == 4, "a work item is 4 rows high");
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
-    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
+    griddep_wait();
+    griddep_launch();
+    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
     __syncthreads();
     const uint32_t item = blockIdx.x * 256u + threadIdx.x;
     if (item >= d.items) return;
@@ -206,11 +209,13 @@ struct DecLine {
 };
 template <typename XT, typename LT, int Q, int QPT>
 __global__ void __launch_bounds__(256)
-decompress_line_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
-                       const float* __restrict__ stats, XT* __restrict__ xhat, DecLine d) {
+decompress_line_kernel(const LT* lfc, const uint32_t* packed,
+                       const float* stats, XT* xhat, DecLine d) {
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
-    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
+    griddep_wait();
+    griddep_launch();
+    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
     __syncthreads();
     const uint64_t sample_quad0 = (uint64_t)n * d.qps;
     const LT* lfc_n = lfc + (size_t)n * d.C * d.Wb;
@@ -286,14 +291,18 @@ __device__ __forceinline__ uint2 quad_table_entry(uint32_t idx, uint32_t HW, uin
 
 template <typename XT, typename LT, int Q, int QPT>
 __global__ void __launch_bounds__(256)
-decompress_flat_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
-                       const float* __restrict__ stats, XT* __restrict__ xhat, DecFlat d) {
+decompress_flat_kernel(const LT* lfc, const uint32_t* packed,
+                       const float* stats, XT* xhat, DecFlat d) {
     extern __shared__ __align__(16) uint32_t flat_smem[];
     uint2* quad_of = reinterpret_cast<uint2*>(flat_smem);            // quad inside a period -> where its 4 low-frequency values sit
     float* lfc_s = reinterpret_cast<float*>(flat_smem + d.table_words);   // low-frequency values of this CTA's planes
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
-    // the codes of this thread's quads are asked for first: their trip to memory overlaps the set-up below
+    for (uint32_t idx = threadIdx.x; idx < d.period; idx += 256u)
+        quad_of[idx] = quad_table_entry(idx, d.HW, d.W, d.Wb, d.TPP, d.by_hw, d.by_w, d.by_b);
+    griddep_wait();
+    griddep_launch();
+    // the codes of this thread's quads are asked for first: their trip to memory overlaps the rest of the set-up
     const uint64_t sample_quad0 = (uint64_t)n * d.qps;
     const uint32_t q0 = blockIdx.x * (256u * QPT) + threadIdx.x;
     uint32_t bits[QPT];
@@ -302,9 +311,7 @@ decompress_flat_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ 
         const uint32_t q = q0 + k * 256u;
         bits[k] = q < d.qps ? quad_bits<Q>(packed, sample_quad0 + q) : 0u;
     }
-    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
-    for (uint32_t idx = threadIdx.x; idx < d.period; idx += 256u)
-        quad_of[idx] = quad_table_entry(idx, d.HW, d.W, d.Wb, d.TPP, d.by_hw, d.by_w, d.by_b);
+    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
     const uint32_t e_first = blockIdx.x * (1024u * QPT);
     const uint32_t plane0 = fdiv(e_first, d.by_hw);
     const uint32_t nplanes = min(d.planes_per_cta, d.C - plane0);
@@ -352,17 +359,19 @@ struct DecRows {
 };
 template <typename XT, typename LT, int Q, int QPT>
 __global__ void __launch_bounds__(256)
-decompress_rows_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
-                       const float* __restrict__ stats, XT* __restrict__ xhat, const DecRows d) {
+decompress_rows_kernel(const LT* lfc, const uint32_t* packed,
+                       const float* stats, XT* xhat, const DecRows d) {
     extern __shared__ __align__(16) float rows_smem[];
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
     const uint64_t sample_quad0 = (uint64_t)n * d.qps;
     const uint32_t q0 = blockIdx.x * (256u * QPT) + threadIdx.x;
+    griddep_wait();
+    griddep_launch();
     uint32_t bits[QPT];
 #pragma unroll
     for (int k = 0; k < QPT; ++k) bits[k] = q0 + k * 256u < d.qps ? quad_bits<Q>(packed, sample_quad0 + q0 + k * 256u) : 0u;
-    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
+    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
     const uint32_t first_row = fdiv(blockIdx.x * (1024u * QPT), d.by_w);
     const uint32_t first_plane = fdiv(first_row, d.by_h);
     const uint32_t band0 = first_plane * d.Hb + fdiv(first_row - first_plane * d.H, d.by_b);      // bands counted through the sample

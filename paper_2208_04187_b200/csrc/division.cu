@@ -524,7 +524,7 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                 d.by_qpr = make_fastdiv(d.qpr);
                 const uint32_t per_block = 256u * DEC_QPT;
                 dim3 grid((d.qps + per_block - 1) / per_block, s.N);
-                decompress_line_kernel<XT, LT, Q, DEC_QPT><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+                return launch_pdl(decompress_line_kernel<XT, LT, Q, DEC_QPT>, grid, 256, 0, stream, lfc, packed, stats, (XT*)xhat_dev, d);
             } else if (decompress_fast_ok(s)) {
                 DecFast d;
                 d.qps = s.CHW / 4;
@@ -544,9 +544,9 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                 dim3 grid((d.items + 255u) / 256u, s.N);
                 // rows that are not whole 32-byte sectors: the 4 rows of an item spread over the plane (see the kernel)
                 if ((s.W * (uint32_t)sizeof(XT)) % 32u != 0 && s.H >= 8u)
-                    decompress_quad_kernel<XT, LT, Q, DEC_QPT, true><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+                    return launch_pdl(decompress_quad_kernel<XT, LT, Q, DEC_QPT, true>, grid, 256, 0, stream, lfc, packed, stats, (XT*)xhat_dev, d);
                 else
-                    decompress_quad_kernel<XT, LT, Q, DEC_QPT, false><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+                    return launch_pdl(decompress_quad_kernel<XT, LT, Q, DEC_QPT, false>, grid, 256, 0, stream, lfc, packed, stats, (XT*)xhat_dev, d);
             } else if (decompress_rows_ok(s)) {
                 DecRows d;
                 d.qps = s.CHW / 4;
@@ -562,7 +562,7 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                 d.by_h = make_fastdiv(s.H);
                 d.by_b = make_fastdiv(s.B);
                 dim3 grid((d.qps + 256u * FLAT_QPT - 1) / (256u * FLAT_QPT), s.N);
-                decompress_rows_kernel<XT, LT, Q, FLAT_QPT><<<grid, 256, 4u * d.bands * d.W, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+                return launch_pdl(decompress_rows_kernel<XT, LT, Q, FLAT_QPT>, grid, 256, 4u * d.bands * d.W, stream, lfc, packed, stats, (XT*)xhat_dev, d);
             } else if (decompress_flat_ok(s)) {
                 DecFlat d;
                 d.qps = s.CHW / 4;
@@ -582,8 +582,8 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                 d.by_period = make_fastdiv(d.period);
                 d.planes_per_cta = flat_planes_per_cta(4u * per_block, s.HW);
                 dim3 grid((d.qps + per_block - 1) / per_block, s.N);
-                decompress_flat_kernel<XT, LT, Q, FLAT_QPT><<<grid, 256, flat_smem_bytes(4u * per_block, s.HW, s.TPP), stream>>>(
-                    lfc, packed, stats, (XT*)xhat_dev, d);
+                return launch_pdl(decompress_flat_kernel<XT, LT, Q, FLAT_QPT>, grid, 256, flat_smem_bytes(4u * per_block, s.HW, s.TPP), stream,
+                                  lfc, packed, stats, (XT*)xhat_dev, d);
             } else {
                 const uint64_t g = (nwords + 255) / 256;
                 if (g > 0x7FFFFFFFull) return DIV_ERR_SHAPE;
@@ -777,9 +777,9 @@ div_status div_planegroup_decompress(const div_desc* desc, const void* comp_dev,
                 d.by_wq = make_fastdiv(d.wq);
                 dim3 grid((d.items + 255u) / 256u, s.N);
                 if ((s.W * (uint32_t)sizeof(XT)) % 32u != 0 && s.H >= 8u)
-                    pg_decompress_quad_kernel<XT, LT, Q, DEC_QPT, true><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+                    return launch_pdl(pg_decompress_quad_kernel<XT, LT, Q, DEC_QPT, true>, grid, 256, 0, stream, lfc, packed, stats, (XT*)xhat_dev, d);
                 else
-                    pg_decompress_quad_kernel<XT, LT, Q, DEC_QPT, false><<<grid, 256, 0, stream>>>(lfc, packed, stats, (XT*)xhat_dev, d);
+                    return launch_pdl(pg_decompress_quad_kernel<XT, LT, Q, DEC_QPT, false>, grid, 256, 0, stream, lfc, packed, stats, (XT*)xhat_dev, d);
             } else if (pg_decompress_flat_ok(s)) {
                 PgDecFlat d;
                 d.quads = s.total / 4;

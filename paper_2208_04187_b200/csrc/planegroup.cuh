@@ -110,6 +110,8 @@ pg_strip_kernel(const PgParams p) {
     const uint32_t W4 = s.W >> 2;
     const uint32_t plane0 = blockIdx.x * p.G;
     for (uint32_t i = tid; i < 2u * p.G; i += PG_THREADS) s_key[i] = 0u;
+    griddep_wait();
+    griddep_launch();
 
     // ---- where this thread's slots are, and their loads (everything a thread reads is requested at once)
     uint32_t rows[PG_K], pl[PG_K], first[PG_K], tile[PG_K], which[PG_K];
@@ -277,6 +279,8 @@ pg_small_kernel(const PgSmall g) {
         }
     }
     for (uint32_t i = tid; i < 2u * g.G; i += 256u) s_key[i] = 0u;
+    griddep_wait();
+    griddep_launch();
     __syncthreads();
 
     // ---- first half: lane = two adjacent columns of one tile (packed adds; CPL says how they are loaded, see load_cols)
@@ -506,13 +510,15 @@ __device__ __forceinline__ void pg_unpack_stats(uint32_t w, float& delta, float&
 // hq_count rows apart, each with its own tile's low-frequency value)
 template <typename XT, typename LT, int Q, int QPT, bool SPREAD>
 __global__ void __launch_bounds__(256)
-pg_decompress_quad_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
-                          const uint32_t* __restrict__ stats, XT* __restrict__ xhat, DecFast d) {
+pg_decompress_quad_kernel(const LT* lfc, const uint32_t* packed,
+                          const uint32_t* stats, XT* xhat, DecFast d) {
     static_assert(QPT == 4, "a work item is 4 rows high");
     constexpr uint32_t MASK = (1u << Q) - 1u;
     const uint32_t n = blockIdx.y;
     const uint32_t item = blockIdx.x * 256u + threadIdx.x;
     if (item >= d.items) return;
+    griddep_wait();
+    griddep_launch();
     const uint32_t plane = fdiv(item, d.by_ipp);
     const uint32_t rem = item - plane * d.ipp;
     const uint32_t hq = fdiv(rem, d.by_wq);
@@ -522,7 +528,7 @@ pg_decompress_quad_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict
     const size_t gp = (size_t)n * d.C + plane;
     const LT* lfc_p = lfc + gp * d.TPP + ((wq * 4u) >> d.log2B);
     float delta, step;
-    pg_unpack_stats(__ldg(stats + gp), delta, step);
+    pg_unpack_stats(stats[gp], delta, step);
     const uint64_t quad0 = (uint64_t)n * d.qps + plane * d.hwq + h0 * d.wq + wq;
     const uint32_t qstep = hstep * d.wq;
     uint32_t bits[4];
@@ -691,7 +697,7 @@ inline bool plan_pg_strip(const div_desc* d, const Shape& s, PgPlan* out) {
 template <typename XT, typename LT>
 inline div_status launch_pg_strip(int qbits, uint32_t p2, const PgParams& prm, const PgPlan& pl, cudaStream_t st) {
 #define DIVK_PG_CASE(QQ, PP) \
-    if (qbits == QQ && p2 == PP) { pg_strip_kernel<XT, LT, QQ, PP><<<pl.grid, pl.threads, 0, st>>>(prm); return DIV_OK; }
+    if (qbits == QQ && p2 == PP) return launch_pdl(pg_strip_kernel<XT, LT, QQ, PP>, dim3(pl.grid), pl.threads, 0, st, prm);
     DIVK_PG_CASE(2, 8)
     DIVK_PG_CASE(4, 8)
     DIVK_PG_CASE(8, 8)
@@ -777,9 +783,8 @@ inline div_status launch_pg_small(int qbits, uint32_t p2, const PgSmall& g, cuda
     const size_t smem = pg_small_smem_bytes(g);
 #define DIVK_PGS_CASE(QQ, PP) \
     if (qbits == QQ && p2 == PP) {                                                      \
-        if (g.cpl == 2) pg_small_kernel<XT, LT, QQ, PP, 2><<<grid, 256, smem, st>>>(g); \
-        else pg_small_kernel<XT, LT, QQ, PP, 3><<<grid, 256, smem, st>>>(g);            \
-        return DIV_OK;                                                                  \
+        if (g.cpl == 2) return launch_pdl(pg_small_kernel<XT, LT, QQ, PP, 2>, dim3(grid), 256, smem, st, g); \
+        return launch_pdl(pg_small_kernel<XT, LT, QQ, PP, 3>, dim3(grid), 256, smem, st, g);                 \
     }
     DIVK_PGS_CASE(2, 4)
     DIVK_PGS_CASE(4, 4)

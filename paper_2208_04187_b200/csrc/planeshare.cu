@@ -33,10 +33,13 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
 #pragma unroll
         for (uint32_t i = 0; i < SHARE_PIECES; ++i) mbar_init(&full[i], 1);
         fence_barrier_init();
+        griddep_wait();
         share_load(p, land, full, n, plane0, nplanes);
     }
     for (uint32_t i = tid; i < 2u * nplanes; i += SHARE_THREADS) keys[i] = 0u;
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
     float lo, hi;
     share_half1<XT, P2, G, true>(p, res, land, full, n, plane0, nplanes, keys, lo, hi);
     __syncthreads();
@@ -113,8 +116,7 @@ inline div_status launch_plane_share(const PlaneShareParams& prm, const SharePla
     auto kern = plane_share_kernel<XT, P2, G, Q>;
     static SmemSeen smem_set[DEVICE_CACHE_SLOTS];
     if (!ensure_dynamic_smem((const void*)kern, (int)pl.smem_bytes, smem_set)) return DIV_ERR_CUDA;
-    kern<<<dim3((prm.C + pl.ppc - 1u) / pl.ppc, N), SHARE_THREADS, pl.smem_bytes, st>>>(prm);
-    return cudaGetLastError() == cudaSuccess ? DIV_OK : DIV_ERR_CUDA;
+    return launch_pdl(kern, dim3((prm.C + pl.ppc - 1u) / pl.ppc, N), SHARE_THREADS, pl.smem_bytes, st, prm);
 }
 template <typename XT, int P2, typename G>
 inline div_status launch_plane_share_q(int qbits, const PlaneShareParams& prm, const SharePlan& pl, uint32_t N, cudaStream_t st) {
