@@ -19,7 +19,7 @@ HEADERS = ["common.cuh", "cluster_plan.cuh", "halves.cuh", "twopass.cuh", "decom
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-lineinfo", "-std=c++17",
-    "-Xcompiler", "-fPIC", "--split-compile=0",
+    "-Xcompiler", "-fPIC",
     "--fmad=false",          # one rounding per operation is part of the output contract
     "-Xptxas", "-v",
 ]
