@@ -423,7 +423,7 @@ div_status div_compress_ex(const div_desc* desc, const void* x_dev, void* comp_d
         return DIV_ERR_CUDA;
     if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl) && compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream) == DIV_OK)
         return DIV_OK;
-    if (cudaMemsetAsync(workspace_dev, 0, lo.workspace_bytes, stream) != cudaSuccess) return DIV_ERR_CUDA;
+    if (clear_scratch(workspace_dev, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
     // The single-launch kernels need all their CTAs resident, so they are launched cooperatively; where the
     // device refuses such a launch (fewer SMs visible to the process than the device reports, for instance) the
     // next kernel in line takes the descriptor: nothing has been enqueued by the refused launch.
@@ -462,7 +462,7 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
     make_layout(desc, s, &lo);
     if (comp_capacity < lo.total_bytes || workspace_bytes < lo.workspace_bytes) return DIV_ERR_CAPACITY;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    if (cudaMemsetAsync(workspace_dev, 0, lo.workspace_bytes, stream) != cudaSuccess) return DIV_ERR_CUDA;
+    if (clear_scratch(workspace_dev, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
     uint8_t* blob = (uint8_t*)comp_dev;
     uint32_t* ws = (uint32_t*)workspace_dev;
     const uint32_t never = 0xFFFFFFFFu;      // an arrival count no sample reaches
@@ -906,7 +906,7 @@ div_status div_compress_3d(const div_desc3d* desc, const void* x_dev, void* comp
     make_layout3(desc, s, &lo);
     if (comp_capacity < lo.total_bytes || workspace_bytes < lo.workspace_bytes) return DIV_ERR_CAPACITY;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    if (cudaMemsetAsync(workspace_dev, 0, lo.workspace_bytes, stream) != cudaSuccess) return DIV_ERR_CUDA;
+    if (clear_scratch(workspace_dev, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
     uint8_t* blob = (uint8_t*)comp_dev;
     uint32_t* ws = (uint32_t*)workspace_dev;
     // kernels that store bytes or half-words leave the unused top of a partial last word alone: it is zero by contract
@@ -927,32 +927,33 @@ div_status div_compress_3d(const div_desc3d* desc, const void* x_dev, void* comp
         // W % 4 == 0 and B = 4 or 8: a lane per strip of 4 columns (16-byte loads)
         const uint64_t strip_slots = (uint64_t)s.N * s.C * s.Db * s.Hb * s.Wb * (s.B / 4u) * 2u;      // two lanes per strip
         const uint64_t gs = (strip_slots + 127u) / 128u;
+        div_status st1 = DIV_OK;
         if (s.W % 4u == 0 && (s.B == 4u || s.B == 8u) && s.P2 == s.B && gs <= 0x7FFFFFFFull) {
             const XT* xs = (const XT*)x_dev;
             LT* lf = (LT*)(blob + lo.lfc_off);
-            if (s.B == 8u) lfc_stats3d_strip_kernel<XT, LT, 8><<<(unsigned)gs, 128, 0, stream>>>(xs, lf, ws, s, strip_slots);
-            else lfc_stats3d_strip_kernel<XT, LT, 4><<<(unsigned)gs, 128, 0, stream>>>(xs, lf, ws, s, strip_slots);
+            if (s.B == 8u) st1 = launch_pdl(lfc_stats3d_strip_kernel<XT, LT, 8>, dim3((unsigned)gs), 128, 0, stream, xs, lf, ws, s, strip_slots);
+            else st1 = launch_pdl(lfc_stats3d_strip_kernel<XT, LT, 4>, dim3((unsigned)gs), 128, 0, stream, xs, lf, ws, s, strip_slots);
         } else if (bpw && gw <= 0x7FFFFFFFull) {
             const XT* xs = (const XT*)x_dev;
             LT* lf = (LT*)(blob + lo.lfc_off);
             switch (s.P2) {
-                case 1: lfc_stats3d_warp_kernel<XT, LT, 1><<<(unsigned)gw, 256, 0, stream>>>(xs, lf, ws, s, gpr, groups); break;
-                case 2: lfc_stats3d_warp_kernel<XT, LT, 2><<<(unsigned)gw, 256, 0, stream>>>(xs, lf, ws, s, gpr, groups); break;
-                case 4: lfc_stats3d_warp_kernel<XT, LT, 4><<<(unsigned)gw, 256, 0, stream>>>(xs, lf, ws, s, gpr, groups); break;
-                case 8: lfc_stats3d_warp_kernel<XT, LT, 8><<<(unsigned)gw, 256, 0, stream>>>(xs, lf, ws, s, gpr, groups); break;
-                case 16: lfc_stats3d_warp_kernel<XT, LT, 16><<<(unsigned)gw, 256, 0, stream>>>(xs, lf, ws, s, gpr, groups); break;
-                default: lfc_stats3d_warp_kernel<XT, LT, 32><<<(unsigned)gw, 256, 0, stream>>>(xs, lf, ws, s, gpr, groups); break;
+                case 1: st1 = launch_pdl(lfc_stats3d_warp_kernel<XT, LT, 1>, dim3((unsigned)gw), 256, 0, stream, xs, lf, ws, s, gpr, groups); break;
+                case 2: st1 = launch_pdl(lfc_stats3d_warp_kernel<XT, LT, 2>, dim3((unsigned)gw), 256, 0, stream, xs, lf, ws, s, gpr, groups); break;
+                case 4: st1 = launch_pdl(lfc_stats3d_warp_kernel<XT, LT, 4>, dim3((unsigned)gw), 256, 0, stream, xs, lf, ws, s, gpr, groups); break;
+                case 8: st1 = launch_pdl(lfc_stats3d_warp_kernel<XT, LT, 8>, dim3((unsigned)gw), 256, 0, stream, xs, lf, ws, s, gpr, groups); break;
+                case 16: st1 = launch_pdl(lfc_stats3d_warp_kernel<XT, LT, 16>, dim3((unsigned)gw), 256, 0, stream, xs, lf, ws, s, gpr, groups); break;
+                default: st1 = launch_pdl(lfc_stats3d_warp_kernel<XT, LT, 32>, dim3((unsigned)gw), 256, 0, stream, xs, lf, ws, s, gpr, groups); break;
             }
         } else {
             lfc_stats3d_kernel<XT, LT><<<(unsigned)g1, 128, 0, stream>>>((const XT*)x_dev, (LT*)(blob + lo.lfc_off), ws, s);
         }
-        if (launch_status() != DIV_OK) return DIV_ERR_CUDA;
+        if (st1 != DIV_OK || launch_status() != DIV_OK) return DIV_ERR_CUDA;
         if (s.W % 4u == 0 && (s.B == 4u || s.B == 8u) && s.P2 == s.B && gs <= 0x7FFFFFFFull && desc->qbits != 1) {
             void* packed = blob + lo.packed_off;
             float* stats = (float*)(blob + lo.stats_off);
             const XT* xs = (const XT*)x_dev;
             const LT* lf = (const LT*)(blob + lo.lfc_off);
-#define DIVK_Q3(QQ, PP) quant3d_strip_kernel<XT, LT, QQ, PP><<<(unsigned)gs, 128, 0, stream>>>(xs, lf, ws, packed, stats, s, seed, strip_slots)
+#define DIVK_Q3(QQ, PP) return launch_pdl(quant3d_strip_kernel<XT, LT, QQ, PP>, dim3((unsigned)gs), 128, 0, stream, xs, lf, ws, packed, stats, s, seed, strip_slots)
             if (s.B == 8u) {
                 if (desc->qbits == 2) DIVK_Q3(2, 8); else if (desc->qbits == 4) DIVK_Q3(4, 8); else DIVK_Q3(8, 8);
             } else {
@@ -969,9 +970,9 @@ div_status div_compress_3d(const div_desc3d* desc, const void* x_dev, void* comp
             const XT* xs = (const XT*)x_dev;
             const LT* lf = (const LT*)(blob + lo.lfc_off);
             switch (desc->qbits) {
-                case 2: quant3d_quad_kernel<XT, LT, 2, DEC_QPT><<<grid, 256, 0, stream>>>(xs, lf, ws, packed, stats, g, seed); break;
-                case 4: quant3d_quad_kernel<XT, LT, 4, DEC_QPT><<<grid, 256, 0, stream>>>(xs, lf, ws, packed, stats, g, seed); break;
-                default: quant3d_quad_kernel<XT, LT, 8, DEC_QPT><<<grid, 256, 0, stream>>>(xs, lf, ws, packed, stats, g, seed); break;
+                case 2: return launch_pdl(quant3d_quad_kernel<XT, LT, 2, DEC_QPT>, grid, 256, 0, stream, xs, lf, ws, packed, stats, g, seed);
+                case 4: return launch_pdl(quant3d_quad_kernel<XT, LT, 4, DEC_QPT>, grid, 256, 0, stream, xs, lf, ws, packed, stats, g, seed);
+                default: return launch_pdl(quant3d_quad_kernel<XT, LT, 8, DEC_QPT>, grid, 256, 0, stream, xs, lf, ws, packed, stats, g, seed);
             }
             return launch_status();
         }
@@ -1009,7 +1010,7 @@ div_status div_decompress_3d(const div_desc3d* desc, const void* comp_dev, size_
             const LT* lf = (const LT*)(blob + lo.lfc_off);
             const uint32_t* pk = (const uint32_t*)(blob + lo.packed_off);
             const float* stt = (const float*)(blob + lo.stats_off);
-#define DIVK_D3(QQ, PP) decompress3d_strip_kernel<XT, LT, QQ, PP><<<grid, 256, 0, stream>>>(lf, pk, stt, (XT*)xhat_dev, s, (uint32_t)sps)
+#define DIVK_D3(QQ, PP) return launch_pdl(decompress3d_strip_kernel<XT, LT, QQ, PP>, grid, 256, 0, stream, lf, pk, stt, (XT*)xhat_dev, s, (uint32_t)sps)
             if (s.B == 8u) {
                 if (desc->qbits == 2) DIVK_D3(2, 8); else if (desc->qbits == 4) DIVK_D3(4, 8); else DIVK_D3(8, 8);
             } else {
@@ -1022,10 +1023,9 @@ div_status div_decompress_3d(const div_desc3d* desc, const void* comp_dev, size_
             const Quad3 g3 = make_quad3(s);
             const dim3 grid((g3.qps + 256u * DEC_QPT - 1) / (256u * DEC_QPT), s.N);
             return dispatch_q(desc->qbits, [&](auto q) -> div_status {
-                decompress3d_quad_kernel<XT, LT, decltype(q)::value, DEC_QPT><<<grid, 256, 0, stream>>>(
-                    (const LT*)(blob + lo.lfc_off), (const uint32_t*)(blob + lo.packed_off), (const float*)(blob + lo.stats_off),
-                    (XT*)xhat_dev, g3);
-                return launch_status();
+                return launch_pdl(decompress3d_quad_kernel<XT, LT, decltype(q)::value, DEC_QPT>, grid, 256, 0, stream,
+                                  (const LT*)(blob + lo.lfc_off), (const uint32_t*)(blob + lo.packed_off),
+                                  (const float*)(blob + lo.stats_off), (XT*)xhat_dev, g3);
             });
         }
         return dispatch_q(desc->qbits, [&](auto q) -> div_status {

@@ -231,6 +231,8 @@ lagged_kernel(const LParams p) {
     OutT* packed = reinterpret_cast<OutT*>(p.packed);
     uint32_t* claim_word = p.ws + WS_CLAIM_WORD;
 
+    griddep_wait();
+    griddep_launch();
     bool gave_up = false;
     uint32_t next = 0;
     if (lane == 0) next = atomicAdd(claim_word, 1u);
@@ -549,12 +551,7 @@ inline div_status plan_lagged(const div_desc* d, const Shape& s, LPlan* out) {
 template <typename XT, typename LT, int Q, int P2>
 inline div_status launch_lagged(const LParams& prm, cudaStream_t st) {
     void* args[] = {(void*)&prm};
-    if (cudaLaunchCooperativeKernel((const void*)lagged_kernel<XT, LT, Q, P2>, dim3(prm.pl.grid), dim3(prm.pl.threads), args,
-                                    0, st) != cudaSuccess) {
-        cudaGetLastError();
-        return DIV_ERR_CUDA;
-    }
-    return DIV_OK;
+    return launch_coop((const void*)lagged_kernel<XT, LT, Q, P2>, dim3(prm.pl.grid), prm.pl.threads, 0, st, args) ? DIV_OK : DIV_ERR_CUDA;
 }
 
 template <typename XT, typename LT>

@@ -162,6 +162,8 @@ line_fused_kernel(const XT* __restrict__ x, LT* __restrict__ lfc, uint32_t* __re
         s_ok = 0;
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
 
     // ---------------- half 1: a lane owns a segment of EQ quads of one block ----------------
     // Slot j of a row: block j >> log2spb, part j & (spb - 1) of it; the parts of a block sit in neighbouring lanes
@@ -387,12 +389,7 @@ inline bool launch_line_fused(const Shape& s, const div_layout& lo, const LineGe
     float* stats = (float*)(blob + lo.stats_off);
     LineGeom gg = g;
     void* args[] = {(void*)&xt, (void*)&lfc, (void*)&ws, (void*)&packed, (void*)&stats, (void*)&gg, (void*)&f, (void*)&seed};
-    if (cudaLaunchCooperativeKernel((const void*)line_fused_kernel<XT, LT, Q, EQ>, dim3(f.ctas_per_sample, s.N), dim3(256), args, 0, st) !=
-        cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return true;
+    return launch_coop((const void*)line_fused_kernel<XT, LT, Q, EQ>, dim3(f.ctas_per_sample, s.N), 256, 0, st, args);
 }
 
 template <typename XT, typename LT>

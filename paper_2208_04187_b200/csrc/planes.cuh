@@ -260,6 +260,8 @@ plane_fused_kernel(const XT* __restrict__ x, LT* __restrict__ lfc, uint32_t* __r
         s_ok = 0;
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
 
     // ---------------- half 1: a lane owns one or two tile columns of one plane ----------------
     {
@@ -448,12 +450,7 @@ inline bool launch_plane_fused(const Shape& s, const div_layout& lo, const Plane
     float* stats = (float*)(blob + lo.stats_off);
     PlaneGeom gg = g;
     void* args[] = {(void*)&xt, (void*)&lfc, (void*)&ws, (void*)&packed, (void*)&stats, (void*)&gg, (void*)&f, (void*)&seed};
-    if (cudaLaunchCooperativeKernel((const void*)plane_fused_kernel<XT, LT, Q, P2, CPL>, dim3(pf.ctas_per_sample, s.N), dim3(256), args,
-                                    pf.smem, st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return true;
+    return launch_coop((const void*)plane_fused_kernel<XT, LT, Q, P2, CPL>, dim3(pf.ctas_per_sample, s.N), 256, pf.smem, st, args);
 }
 
 template <typename XT, typename LT>

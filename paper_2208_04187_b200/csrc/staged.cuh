@@ -363,6 +363,8 @@ staged_kernel(const SParams p) {
         fence_barrier_init();
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
 
     if (warp == 2) {
         // ================= watcher (one thread).  Two duties, taken in turns:
@@ -793,12 +795,7 @@ inline div_status launch_staged(const SParams& prm, cudaStream_t st) {
     static SmemSeen smem_set[DEVICE_CACHE_SLOTS];
     if (!ensure_dynamic_smem((const void*)kern, prm.pl.smem_bytes, smem_set)) return DIV_ERR_CUDA;
     void* args[] = {(void*)&prm};
-    if (cudaLaunchCooperativeKernel((const void*)kern, dim3(prm.pl.grid), dim3(prm.pl.threads), args,
-                                    (size_t)prm.pl.smem_bytes, st) != cudaSuccess) {
-        cudaGetLastError();
-        return DIV_ERR_CUDA;
-    }
-    return DIV_OK;
+    return launch_coop((const void*)kern, dim3(prm.pl.grid), prm.pl.threads, (size_t)prm.pl.smem_bytes, st, args) ? DIV_OK : DIV_ERR_CUDA;
 }
 
 template <typename XT, typename LT>

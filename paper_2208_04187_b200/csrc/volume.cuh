@@ -72,6 +72,8 @@ template <typename XT, typename LT, int P2>
 __global__ void __launch_bounds__(256)
 lfc_stats3d_warp_kernel(const XT* __restrict__ x, LT* __restrict__ lfc, uint32_t* __restrict__ ws, Shape3 s,
                         uint32_t groups_per_row, uint64_t groups) {
+    griddep_wait();
+    griddep_launch();
     constexpr uint32_t BPW = 32 / P2;                         // blocks per warp
     const uint64_t grp = (uint64_t)blockIdx.x * 8u + (threadIdx.x >> 5);
     if (grp >= groups) return;                                // whole warps leave together
@@ -133,6 +135,8 @@ lfc_stats3d_warp_kernel(const XT* __restrict__ x, LT* __restrict__ lfc, uint32_t
 template <typename XT, typename LT, int P2>
 __global__ void __launch_bounds__(128)
 lfc_stats3d_strip_kernel(const XT* __restrict__ x, LT* __restrict__ lfc, uint32_t* __restrict__ ws, Shape3 s, uint64_t slots) {
+    griddep_wait();
+    griddep_launch();
     constexpr uint32_t LPB = P2 / 4;                                   // lanes per block
     const uint32_t lane = threadIdx.x & 31;
     constexpr uint32_t HR = P2 / 2;                                    // rows per lane
@@ -259,7 +263,7 @@ lfc_stats3d_strip_kernel(const XT* __restrict__ x, LT* __restrict__ lfc, uint32_
 // Eq. 9 on packed pairs, one byte / half-word / word of codes.  x is read a second time.
 template <typename XT, typename LT, int Q, int P2>
 __global__ void __launch_bounds__(128)
-quant3d_strip_kernel(const XT* __restrict__ x, const LT* __restrict__ lfc, const uint32_t* __restrict__ ws,
+quant3d_strip_kernel(const XT* __restrict__ x, const LT* lfc, const uint32_t* ws,
                      void* __restrict__ packed_v, float* __restrict__ stats, Shape3 s, uint64_t seed, uint64_t slots) {
     typedef typename PackedUnit<Q>::type OutT;
     constexpr uint32_t LPB = P2 / 4;
@@ -280,8 +284,10 @@ quant3d_strip_kernel(const XT* __restrict__ x, const LT* __restrict__ lfc, const
     const uint32_t c = (uint32_t)(vol - (uint64_t)n * s.C);
     const uint32_t d0 = bd * s.B, h0 = bh * s.B, w0 = bw * s.B;
     const uint32_t nd = min(s.B, s.D - d0), nh = min(s.B, s.H - h0), nw = min(s.B, s.W - w0);
+    griddep_wait();
+    griddep_launch();
     const uint32_t* slot_n = ws + WS_HEADER_WORDS + (size_t)n * WS_SLOT_WORDS;
-    const QParams qp = make_qparams(key_float(~__ldg(slot_n + 0)), key_float(__ldg(slot_n + 1)), Q);
+    const QParams qp = make_qparams(key_float(~slot_n[0]), key_float(slot_n[1]), Q);
     if (c == 0 && rowid == vol * s.Db * s.Hb && sq == 0) {             // the first slot of the sample
         stats[2 * (size_t)n + 0] = qp.delta;
         stats[2 * (size_t)n + 1] = qp.step;
@@ -323,12 +329,14 @@ quant3d_strip_kernel(const XT* __restrict__ x, const LT* __restrict__ lfc, const
 // grid = (ceil(slots per sample / 256), N)
 template <typename XT, typename LT, int Q, int P2>
 __global__ void __launch_bounds__(256)
-decompress3d_strip_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed, const float* __restrict__ stats,
-                          XT* __restrict__ xhat, Shape3 s, uint32_t slots_per_sample) {
+decompress3d_strip_kernel(const LT* lfc, const uint32_t* packed, const float* stats,
+                          XT* xhat, Shape3 s, uint32_t slots_per_sample) {
     constexpr uint32_t LPB = P2 / 4;
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
-    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
+    griddep_wait();
+    griddep_launch();
+    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
     __syncthreads();
     const uint32_t slot = blockIdx.x * 256u + threadIdx.x;
     if (slot >= slots_per_sample) return;
@@ -492,12 +500,14 @@ __device__ __forceinline__ float quad3_lfc(const LT* __restrict__ lfc_n, const Q
 
 template <typename XT, typename LT, int Q, int QPT>
 __global__ void __launch_bounds__(256)
-quant3d_quad_kernel(const XT* __restrict__ x, const LT* __restrict__ lfc, const uint32_t* __restrict__ ws,
+quant3d_quad_kernel(const XT* __restrict__ x, const LT* lfc, const uint32_t* ws,
                     void* __restrict__ packed_v, float* __restrict__ stats, Quad3 g, uint64_t seed) {
     typedef typename PackedUnit<Q>::type OutT;
     const uint32_t n = blockIdx.y;
+    griddep_wait();
+    griddep_launch();
     const uint32_t* slot = ws + WS_HEADER_WORDS + (size_t)n * WS_SLOT_WORDS;
-    const QParams qp = make_qparams(key_float(~__ldg(slot + 0)), key_float(__ldg(slot + 1)), Q);
+    const QParams qp = make_qparams(key_float(~slot[0]), key_float(slot[1]), Q);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         stats[2 * (size_t)n + 0] = qp.delta;
         stats[2 * (size_t)n + 1] = qp.step;
@@ -528,11 +538,13 @@ quant3d_quad_kernel(const XT* __restrict__ x, const LT* __restrict__ lfc, const 
 
 template <typename XT, typename LT, int Q, int QPT>
 __global__ void __launch_bounds__(256)
-decompress3d_quad_kernel(const LT* __restrict__ lfc, const uint32_t* __restrict__ packed,
-                         const float* __restrict__ stats, XT* __restrict__ xhat, Quad3 g) {
+decompress3d_quad_kernel(const LT* lfc, const uint32_t* packed,
+                         const float* stats, XT* xhat, Quad3 g) {
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
-    table.build(__ldg(stats + 2 * (size_t)n + 1), __ldg(stats + 2 * (size_t)n));
+    griddep_wait();
+    griddep_launch();
+    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
     __syncthreads();
     const uint64_t sample_quad0 = (uint64_t)n * g.qps;
     const LT* lfc_n = lfc + (size_t)n * g.C * g.Db * g.Hb * g.Wb;
