@@ -47,7 +47,7 @@ __device__ __forceinline__ void st_async_u64(uint64_t* dst, uint64_t v, uint64_t
 // ------------------------------------------------------------------------------------------------
 // half 2: the CTA's residuals, 4 consecutive elements per thread and step
 // ------------------------------------------------------------------------------------------------
-template <int Q, bool FIXED>
+template <int Q, bool FIXED, uint32_t THREADS>
 __device__ __forceinline__ void cl_half2(const float* res, typename PackedUnit<Q>::type* out, uint32_t nq, uint64_t ctr, float delta,
                                          float scale) {
     typedef typename PackedUnit<Q>::type OutT;
@@ -55,47 +55,95 @@ __device__ __forceinline__ void cl_half2(const float* res, typename PackedUnit<Q
     const float m = FIXED ? -65536.0f * scale : scale;
     const uint64_t mul2 = pk2(m, m);
     constexpr int U = 4;
-    constexpr uint64_t STEP = K_GROUP * (uint64_t)SHARE_THREADS;
+    constexpr uint64_t STEP = K_GROUP * (uint64_t)THREADS;
     uint32_t q = threadIdx.x;
-    for (; q + (U - 1) * SHARE_THREADS < nq; q += U * SHARE_THREADS) {
+    for (; q + (U - 1) * THREADS < nq; q += U * THREADS) {
         ulonglong2 v[U];
 #pragma unroll
-        for (int k = 0; k < U; ++k) v[k] = reinterpret_cast<const ulonglong2*>(res)[q + k * SHARE_THREADS];
+        for (int k = 0; k < U; ++k) v[k] = reinterpret_cast<const ulonglong2*>(res)[q + k * THREADS];
 #pragma unroll
         for (int k = 0; k < U; ++k)
-            out[q + k * SHARE_THREADS] = (OutT)quant4_res<Q, FIXED>(v[k].x, v[k].y, delta2, mul2, rng_mix(ctr + STEP * (uint64_t)k));
+            out[q + k * THREADS] = (OutT)quant4_res<Q, FIXED>(v[k].x, v[k].y, delta2, mul2, rng_mix(ctr + STEP * (uint64_t)k));
         ctr += STEP * U;
     }
-    for (; q < nq; q += SHARE_THREADS) {
+    for (; q < nq; q += THREADS) {
         const ulonglong2 v = reinterpret_cast<const ulonglong2*>(res)[q];
         out[q] = (OutT)quant4_res<Q, FIXED>(v.x, v.y, delta2, mul2, rng_mix(ctr));
         ctr += STEP;
     }
 }
-template <int Q>
-__device__ __forceinline__ void cl_half2_q(const ClusterParams& p, const float* res, uint32_t n, uint32_t qfirst, uint32_t nq,
-                                           float rmin, float rmax, bool write_stats) {
+// The same where x stayed in place (bfloat16, rows read 4 columns at a time): slot by slot as in half 1, the residual formed
+// once more from x and the tile's stored low-frequency value.
+template <typename XT, int P2, typename G, int Q, bool FIXED, uint32_t THREADS>
+__device__ __forceinline__ void cl_half2_slots(const ShareParams& p, const float* stored_of, const XT* land,
+                                               typename PackedUnit<Q>::type* out, uint32_t nplanes, uint64_t ctr0, float delta, float scale) {
+    typedef typename PackedUnit<Q>::type OutT;
+    const uint64_t delta2 = pk2(delta, delta);
+    const float m = FIXED ? -65536.0f * scale : scale;
+    const uint64_t mul2 = pk2(m, m);
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W4 = p.W >> 2;
+    const uint32_t nfull = nplanes * p.sppf, first_short = (nfull + 31u) & ~31u, total = first_short + nplanes * p.sppt;
+    const uint64_t row_step = K_GROUP * (uint64_t)W4;
+    for (uint32_t first = warp * 32u; first < total; first += THREADS) {
+        const ShareSlot t = share_slot<P2, G::NC>(p, first, lane, nfull, first_short, total);
+        if (t.cols == 0u) continue;
+        const float stored = stored_of[t.tile];
+        const uint64_t stored2 = pk2(stored, stored);
+        const unsigned char* xs = reinterpret_cast<const unsigned char*>(land + t.off);
+        const uint32_t row_bytes = p.W * (uint32_t)sizeof(XT);
+        OutT* o = out + (t.off >> 2);
+        uint64_t ctr = ctr0 + K_GROUP * (uint64_t)(t.off >> 2);
+        if (t.rows == (uint32_t)P2) {
+            uint64_t xy[P2], zw[P2];
+#pragma unroll
+            for (int r = 0; r < P2; ++r) StripRow2<XT>::load(xs + r * row_bytes, xy[r], zw[r]);
+#pragma unroll
+            for (int r = 0; r < P2; ++r) {
+                o[r * W4] = (OutT)quant4_res<Q, FIXED>(sub2_rn(xy[r], stored2), sub2_rn(zw[r], stored2), delta2, mul2, rng_mix(ctr));
+                ctr += row_step;
+            }
+        } else {
+            for (uint32_t r = 0; r < t.rows; ++r) {
+                uint64_t xy, zw;
+                StripRow2<XT>::load(xs + r * row_bytes, xy, zw);
+                o[r * W4] = (OutT)quant4_res<Q, FIXED>(sub2_rn(xy, stored2), sub2_rn(zw, stored2), delta2, mul2, rng_mix(ctr));
+                ctr += row_step;
+            }
+        }
+    }
+}
+template <typename XT, int P2, typename G, int Q, bool IN_PLACE, uint32_t THREADS>
+__device__ __forceinline__ void cl_half2_q(const ClusterParams& p, const float* res, const XT* land, uint32_t n, uint32_t qfirst,
+                                           uint32_t nplanes, float rmin, float rmax, bool write_stats) {
     const QParams qp = make_qparams(rmin, rmax, Q);
     if (write_stats) {
         p.stats[2 * (size_t)n + 0] = qp.delta;
         p.stats[2 * (size_t)n + 1] = qp.step;
     }
     typename PackedUnit<Q>::type* out = reinterpret_cast<typename PackedUnit<Q>::type*>(p.packed) + ((uint64_t)n * p.qps + qfirst);
-    const uint64_t ctr = rng_sample_base(p.seed, n) + K_GROUP * (uint64_t)(qfirst + threadIdx.x + 1u);
-    if (Q <= 4 && fixed_point_ok<Q>(qp, rmax)) cl_half2<Q, true>(res, out, nq, ctr, qp.delta, qp.scale);
-    else cl_half2<Q, false>(res, out, nq, ctr, qp.delta, qp.scale);
+    if constexpr (IN_PLACE) {
+        const uint64_t ctr = rng_sample_base(p.seed, n) + K_GROUP * (uint64_t)(qfirst + 1u);
+        if (Q <= 4 && fixed_point_ok<Q>(qp, rmax)) cl_half2_slots<XT, P2, G, Q, true, THREADS>(p, res, land, out, nplanes, ctr, qp.delta, qp.scale);
+        else cl_half2_slots<XT, P2, G, Q, false, THREADS>(p, res, land, out, nplanes, ctr, qp.delta, qp.scale);
+    } else {
+        const uint32_t nq = (nplanes * p.HW) >> 2;
+        const uint64_t ctr = rng_sample_base(p.seed, n) + K_GROUP * (uint64_t)(qfirst + threadIdx.x + 1u);
+        if (Q <= 4 && fixed_point_ok<Q>(qp, rmax)) cl_half2<Q, true, THREADS>(res, out, nq, ctr, qp.delta, qp.scale);
+        else cl_half2<Q, false, THREADS>(res, out, nq, ctr, qp.delta, qp.scale);
+    }
 }
 
-template <typename XT, int P2, typename G>
-__global__ void __launch_bounds__(SHARE_THREADS, 3)
+template <typename XT, int P2, typename G, uint32_t THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS > SHARE_THREADS ? 2 : share_by_regs(P2, G::VW, sizeof(XT)))
 cluster_kernel(const __grid_constant__ ClusterParams p) {
+    constexpr bool IN_PLACE = share_in_place(G::VW, sizeof(XT));
     extern __shared__ __align__(128) unsigned char smem[];
     float* res = reinterpret_cast<float*>(smem);
     const XT* land = reinterpret_cast<const XT*>(sizeof(XT) == 4 ? smem : smem + p.res_bytes);
     __shared__ __align__(8) uint64_t full[SHARE_PIECES];
     __shared__ __align__(8) uint64_t xbar;
     __shared__ __align__(8) uint64_t xch[CL_MAX];
-    __shared__ uint32_t wkey[2][SHARE_WARPS];
+    __shared__ uint32_t wkey[2][THREADS / 32];
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank(), n = blockIdx.x >> p.log2cs;
     const uint32_t plane0 = rank * p.ppc;
@@ -119,7 +167,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
     cluster_arrive();                          // waited for below, before anything is sent to another CTA
 
     float lo = 3.402823466e+38f, hi = -3.402823466e+38f;
-    if (nplanes) share_half1<XT, P2, G, false>(p, res, land, full, n, plane0, nplanes, nullptr, lo, hi);
+    if (nplanes) share_half1<XT, P2, G, false, IN_PLACE, THREADS>(p, res, land, full, n, plane0, nplanes, nullptr, lo, hi);
     {
         const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, ~float_key(lo));
         const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, float_key(hi));
@@ -131,8 +179,8 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
     __syncthreads();                           // also: every residual is in place
     cluster_wait();
     if (warp == 0) {
-        const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, lane < SHARE_WARPS ? wkey[0][lane] : 0u);
-        const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, lane < SHARE_WARPS ? wkey[1][lane] : 0u);
+        const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, lane < THREADS / 32 ? wkey[0][lane] : 0u);
+        const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, lane < THREADS / 32 ? wkey[1][lane] : 0u);
         if (lane < (1u << p.log2cs)) st_async_u64(&xch[rank], ((uint64_t)kmax << 32) | kmin, &xbar, lane);
     }
     if (!__all_sync(0xFFFFFFFFu, share_wait(&xbar, p.timeout_ns))) {
@@ -149,25 +197,25 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
     const float rmin = key_float(~__reduce_max_sync(0xFFFFFFFFu, (uint32_t)w));
     const float rmax = key_float(__reduce_max_sync(0xFFFFFFFFu, (uint32_t)(w >> 32)));
     if (nplanes == 0) return;
-    const uint32_t qfirst = (plane0 * p.HW) >> 2, nq = (nplanes * p.HW) >> 2;
+    const uint32_t qfirst = (plane0 * p.HW) >> 2;
     const bool stats = rank == 0 && tid == 0;
-    if (p.qbits == 2) cl_half2_q<2>(p, res, n, qfirst, nq, rmin, rmax, stats);
-    else if (p.qbits == 4) cl_half2_q<4>(p, res, n, qfirst, nq, rmin, rmax, stats);
-    else cl_half2_q<8>(p, res, n, qfirst, nq, rmin, rmax, stats);
+    if (p.qbits == 2) cl_half2_q<XT, P2, G, 2, IN_PLACE, THREADS>(p, res, land, n, qfirst, nplanes, rmin, rmax, stats);
+    else if (p.qbits == 4) cl_half2_q<XT, P2, G, 4, IN_PLACE, THREADS>(p, res, land, n, qfirst, nplanes, rmin, rmax, stats);
+    else cl_half2_q<XT, P2, G, 8, IN_PLACE, THREADS>(p, res, land, n, qfirst, nplanes, rmin, rmax, stats);
 }
 
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-template <typename XT, int P2, typename G>
-inline div_status launch_cluster(const ClusterParams& prm, const ClusterPlan& pl, uint32_t N, cudaStream_t st) {
-    auto kern = cluster_kernel<XT, P2, G>;
+template <typename XT, int P2, typename G, uint32_t THREADS>
+inline div_status launch_cluster_t(const ClusterParams& prm, const ClusterPlan& pl, uint32_t N, cudaStream_t st) {
+    auto kern = cluster_kernel<XT, P2, G, THREADS>;
     static SmemSeen smem_set[DEVICE_CACHE_SLOTS], wide_set[DEVICE_CACHE_SLOTS];
     if (!ensure_dynamic_smem((const void*)kern, (int)pl.smem_bytes, smem_set)) return DIV_ERR_CUDA;
     if (pl.cs > 8 && !ensure_wide_cluster((const void*)kern, wide_set)) return DIV_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(N * pl.cs);
-    cfg.blockDim = dim3(SHARE_THREADS);
+    cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
@@ -183,6 +231,12 @@ inline div_status launch_cluster(const ClusterParams& prm, const ClusterPlan& pl
         return DIV_ERR_CUDA;
     }
     return DIV_OK;
+}
+template <typename XT, int P2, typename G>
+inline div_status launch_cluster(const ClusterParams& prm, const ClusterPlan& pl, uint32_t N, cudaStream_t st) {
+    // as many threads as the registers allow where only two shares fit an SM
+    if (pl.wide) return launch_cluster_t<XT, P2, G, share_wide_threads(P2, G::VW)>(prm, pl, N, st);
+    return launch_cluster_t<XT, P2, G, SHARE_THREADS>(prm, pl, N, st);
 }
 template <typename XT, int P2>
 inline div_status launch_cluster_geo(const ClusterParams& prm, const ClusterPlan& pl, uint32_t N, cudaStream_t st) {

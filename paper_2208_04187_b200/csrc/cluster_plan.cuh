@@ -7,6 +7,15 @@ namespace divk {
 
 constexpr uint32_t SHARE_THREADS = 256;
 constexpr uint32_t SHARE_WARPS = SHARE_THREADS / 32;
+// threads where at most two CTAs fit an SM and clusters take turns (32 x 64 x 75 x 75 28.6 -> 27.0 us, 64 x 1024 x 14 x 14
+// 23.6 -> 23.0 us; where all of x fits at once more threads cost a little, 64 x 2048 x 7 x 7 11.5 -> 12.1 us): 64 registers a thread suffice where rows are read 4 columns at a time or have 4 rows
+__host__ __device__ constexpr uint32_t share_wide_threads(uint32_t p2, uint32_t vw) { return vw == 4 || p2 == 4 ? 512u : 384u; }
+// resident CTAs per SM that the registers allow: up to 80 a thread, 64 (48) where they suffice (128 x 64 x 32 x 32: three of
+// 78 registers 14.5 us, four of 64 12.8 us)
+__host__ __device__ constexpr uint32_t share_by_regs(uint32_t p2, uint32_t vw, uint32_t sx) { return vw == 4 && p2 == 4 && sx == 2 ? 5u : vw == 4 || p2 == 4 ? 4u : 3u; }
+// bfloat16 read 4 columns at a time: x stays as it is and half 2 forms the residual again, which would take twice its room
+// (128 x 160 x 32 x 32 with B = 4, 42 MB: 126 MB of landing place and residuals 36 us, 47 MB 29.8 us)
+__host__ __device__ constexpr bool share_in_place(uint32_t vw, uint32_t sx) { return sx == 2 && vw == 4; }
 constexpr uint32_t SHARE_PIECES = 8;       // bulk copies a CTA's share arrives in
 constexpr uint32_t CL_MAX = 16;            // CTAs of the largest cluster
 
@@ -14,12 +23,13 @@ constexpr uint32_t CL_MAX = 16;            // CTAs of the largest cluster
 struct SharePlan {
     uint32_t ppc;             // planes per CTA
     uint32_t ppp;             // planes per piece
-    uint32_t res_bytes;       // fp32 residuals of a CTA's share (fp32 input lands in the same place)
+    uint32_t res_bytes;       // fp32 residuals of a CTA's share (fp32 input lands in the same place), or its tiles' stored values
     uint32_t smem_bytes;
     uint32_t vw;              // columns a lane can read at once: 4, 2 or 1
 };
 struct ClusterPlan : SharePlan {
     uint32_t cs;              // CTAs per cluster (and per sample)
+    uint32_t wide;            // 1: share_wide_threads a CTA, else SHARE_THREADS
     uint32_t waves;           // times the device has to be filled
 };
 
@@ -34,20 +44,22 @@ inline bool share_takes(const div_desc* d, const Shape& s) {
            ((uint64_t)s.CHW * sx) % 16u == 0 && s.CHW < (1u << 31);
 }
 // a share of `ppc` planes (a multiple of share_step); false when it does not fit
-inline bool plan_share(const div_desc* d, const Shape& s, uint64_t ppc, uint32_t extra_smem, const DeviceInfo& di, SharePlan* out) {
+inline bool plan_share(const div_desc* d, const Shape& s, uint64_t ppc, uint32_t extra_smem, bool in_place, const DeviceInfo& di, SharePlan* out) {
     const uint32_t sx = d->x_dtype == DIV_F32 ? 4u : 2u, step = share_step(d, s);
     const uint64_t elems = ppc * s.HW;
     if (elems > (1u << 16)) return false;
     out->ppc = (uint32_t)ppc;
     out->ppp = (uint32_t)(((ppc + SHARE_PIECES - 1) / SHARE_PIECES + step - 1) / step * step);
-    out->res_bytes = (uint32_t)((elems * 4u + 16u + 127u) & ~127ull);                 // + 16: a slot may read up to 3 elements past a row
-    out->smem_bytes = out->res_bytes + (sx == 2u ? (uint32_t)((elems * 2u + 16u + 127u) & ~127ull) : 0u) + extra_smem;
-    out->vw = (s.W % 4 == 0 && s.B % 4 == 0) ? 4u : (s.W % 2 == 0 && s.B % 2 == 0) ? 2u : 1u;
+    out->vw = (s.W % 4 == 0 && s.B % 4 == 0 && s.P2 < 16) ? 4u : (s.W % 2 == 0 && s.B % 2 == 0) ? 2u : 1u;
+    // + 16: a slot may read up to 3 elements past a row
+    const uint32_t res = (uint32_t)((elems * 4u + 16u + 127u) & ~127ull), land = (uint32_t)((elems * sx + 16u + 127u) & ~127ull);
+    out->res_bytes = in_place && share_in_place(out->vw, sx) ? (uint32_t)((ppc * s.TPP * 4u + 127u) & ~127ull) : res;
+    out->smem_bytes = out->res_bytes + (sx == 2u ? land : 0u) + extra_smem;
     return out->smem_bytes + 1024u <= (uint32_t)di.smem_optin;
 }
-// resident CTAs per SM: shared memory, and registers (64 a thread where rows are read 4 columns at a time, else up to 80)
-inline uint32_t share_per_sm(const SharePlan& pl, const DeviceInfo& di) {
-    const uint32_t by_smem = (uint32_t)di.smem_optin / (pl.smem_bytes + 2048u), by_regs = pl.vw == 4u ? 4u : 3u;
+// resident CTAs per SM: shared memory, and registers
+inline uint32_t share_per_sm(const SharePlan& pl, const DeviceInfo& di, uint32_t by_regs) {
+    const uint32_t by_smem = (uint32_t)di.smem_optin / (pl.smem_bytes + 2048u);
     return by_smem < 1u ? 1u : by_smem < by_regs ? by_smem : by_regs;
 }
 
@@ -57,9 +69,14 @@ inline bool plan_cluster_cs(const div_desc* d, const Shape& s, uint32_t cs, cons
     ClusterPlan pl;
     const uint32_t step = share_step(d, s);
     pl.cs = cs;
-    if (!plan_share(d, s, ((uint64_t)(s.C + cs - 1) / cs + step - 1) / step * step, 0u, di, &pl)) return false;
-    const uint64_t places = (uint64_t)share_per_sm(pl, di) * (uint32_t)di.sms * 95u / 100u;      // clusters leave about 5 % of the places empty
+    if (!plan_share(d, s, ((uint64_t)(s.C + cs - 1) / cs + step - 1) / step * step, 0u, true, di, &pl)) return false;
+    const uint32_t per_sm = share_per_sm(pl, di, share_by_regs(s.P2, pl.vw, d->x_dtype == DIV_F32 ? 4u : 2u));
+    const uint64_t places = (uint64_t)per_sm * (uint32_t)di.sms * 95u / 100u;      // clusters leave about 5 % of the places empty
     pl.waves = (uint32_t)(((uint64_t)s.N * cs + places - 1) / (places ? places : 1u));
+    pl.wide = pl.waves > 1u && per_sm <= 2u ? 1u : 0u;
+#ifdef DIVK_DEV
+    if (const char* e = getenv("DIVK_WIDE"); e && *e) pl.wide = atoi(e);
+#endif
     *out = pl;
     return true;
 }

@@ -274,12 +274,14 @@ bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPl
     if (best == ~0ull) return false;
     // Where a kernel that reads x a second time from the L2 applies it is as good or better once the clusters have to
     // take turns (three fillings: 50 x 256 x 40 x 40 39 against 35 us; two: 64 x 64 x 56 x 56 22.6 against 27.5 us,
-    // 64 x 1024 x 14 x 14 26.2 against 26.7 us), and on bfloat16 maps, whose residuals take twice the room of x, as soon as there are
-    // two (128 x 320 x 16 x 16 22.3 against 20.7 us).  The general kernels never are (32 x 64 x 75 x 75: 33 against 82 us).
+    // 64 x 1024 x 14 x 14 23.0 against 24.6 us).  bfloat16 that stays in place the same (128 x 160 x 32 x 32 29.8 against 33.0 us,
+    // 64 x 512 x 28 x 28 36.5 against 53.3 us) while three shares fit an SM (with two, 32 x 64 x 112 x 112 37.5 against 36.4 us);
+    // other bfloat16, whose residuals take twice the room of x, one filling.  The general kernels never are (32 x 64 x 75 x 75:
+    // 26.8 against 82 us).
     PlaneGeom pg;
     SPlan sp;
     const bool rereads = plan_staged(d, s, &sp) == DIV_OK || plan_planes(d, s, &pg);
-    return !rereads || out->waves <= (d->x_dtype == DIV_BF16 ? 1u : 2u);
+    return !rereads || out->waves <= (d->x_dtype == DIV_F32 || (share_in_place(out->vw, 2u) && !out->wide) ? 2u : 1u);
 }
 
 bool decompress_fast_ok(const Shape& s) {

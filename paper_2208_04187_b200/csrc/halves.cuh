@@ -154,8 +154,9 @@ __device__ __forceinline__ float slot_mean(const uint64_t (&v)[ROWS][G::NV], con
 
 // One slot of half 1 whose residuals go to shared memory.  All slots of a warp have the same number of rows, ROWS; a lane
 // owns the first `cols` of its NC columns (0: none; it loads from anywhere in bounds).  xs / rp: first element of the
-// slot where x landed / where the residual goes (the same place for fp32).  lo / hi collect the residual's extremes.
-template <typename XT, int P2, typename G, int ROWS>
+// slot where x landed / where the residual goes (the same place for fp32).  IN_PLACE (VW = 4): no residuals, rp takes the
+// tile's stored low-frequency value.  lo / hi collect the residual's extremes.
+template <typename XT, int P2, typename G, bool IN_PLACE, int ROWS>
 __device__ __forceinline__ void reduce_slot_rows(const XT* xs, float* rp, uint32_t W, uint32_t cols, const SlotSink& s, float& lo, float& hi) {
     constexpr int NV = G::NV, NU = G::NU;
     const uint32_t sw = G::swap(threadIdx.x & 31u);
@@ -170,6 +171,7 @@ __device__ __forceinline__ void reduce_slot_rows(const XT* xs, float* rp, uint32
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) slot_row_load<XT, G>(xs + r * W, col, v[r]);
     const float stored = slot_mean<XT, P2, G, ROWS>(v, ok, cols != 0u, s);
+    if (IN_PLACE && cols != 0u && s.writer) *rp = stored;
     if (cols != 0u) {
         // residuals back to shared memory; extremes of x (x -> fl(x - stored) is monotone): of the columns of one access
         // together, or of two rows at a time where every column has to be kept apart
@@ -193,10 +195,12 @@ __device__ __forceinline__ void reduce_slot_rows(const XT* xs, float* rp, uint32
             if constexpr (G::VW == 4) {
                 l[0] = fmin3(fmin3(l[0], x[0], x[1]), x[2], x[3]);
                 h[0] = fmax3(fmax3(h[0], x[0], x[1]), x[2], x[3]);
-                ulonglong2 q;
-                q.x = d[0];
-                q.y = d[1];
-                *reinterpret_cast<ulonglong2*>(row) = q;
+                if constexpr (!IN_PLACE) {
+                    ulonglong2 q;
+                    q.x = d[0];
+                    q.y = d[1];
+                    *reinterpret_cast<ulonglong2*>(row) = q;
+                }
             } else if constexpr (G::VW == 2) {
 #pragma unroll
                 for (int u = 0; u < NU; ++u) {
@@ -235,11 +239,11 @@ __device__ __forceinline__ void reduce_slot_rows(const XT* xs, float* rp, uint32
     }
 }
 // the row count is the same in the whole warp: one unrolled body for each
-template <typename XT, int P2, typename G, int ROWS = P2>
+template <typename XT, int P2, typename G, bool IN_PLACE, int ROWS = P2>
 __device__ __forceinline__ void reduce_slot(const XT* xs, float* rp, uint32_t W, uint32_t rows, uint32_t cols, const SlotSink& s, float& lo,
                                             float& hi) {
-    if (ROWS == 1 || rows == (uint32_t)ROWS) reduce_slot_rows<XT, P2, G, ROWS>(xs, rp, W, cols, s, lo, hi);
-    else if constexpr (ROWS > 1) reduce_slot<XT, P2, G, ROWS - 1>(xs, rp, W, rows, cols, s, lo, hi);
+    if (ROWS == 1 || rows == (uint32_t)ROWS) reduce_slot_rows<XT, P2, G, IN_PLACE, ROWS>(xs, rp, W, cols, s, lo, hi);
+    else if constexpr (ROWS > 1) reduce_slot<XT, P2, G, IN_PLACE, ROWS - 1>(xs, rp, W, rows, cols, s, lo, hi);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -288,71 +292,88 @@ __device__ __forceinline__ void share_load(const ShareParams& p, XT* land, uint6
     }
 }
 
+// Slots of the CTA's share are numbered so that every warp holds slots of one height: the full-height bands of all planes
+// first, then, from the next multiple of 32, the short last bands.
+struct ShareSlot {
+    bool valid, short_band, narrow, writer;
+    uint32_t plane, tile;     // plane and tile inside the share
+    uint32_t off, rows, cols; // first element inside the share; rows; columns this lane owns (0: none)
+};
+template <int P2, int NC>
+__device__ __forceinline__ ShareSlot share_slot(const ShareParams& p, uint32_t first, uint32_t lane, uint32_t nfull, uint32_t first_short,
+                                                uint32_t total) {
+    constexpr uint32_t LPT = P2 / NC;                          // lanes per tile
+    ShareSlot t;
+    t.short_band = first >= first_short;                       // the same in the whole warp
+    const uint32_t S = first + lane;
+    t.valid = t.short_band ? S < total : S < nfull;
+    const uint32_t T = t.valid ? (t.short_band ? S - first_short : S) : 0u;
+    t.plane = fdiv(T, t.short_band ? p.by_spb : p.by_sppf);
+    const uint32_t rem = T - t.plane * (t.short_band ? p.spb : p.sppf);
+    const uint32_t bf = fdiv(rem, p.by_spb);
+    const uint32_t band = t.short_band ? p.Hb - 1u : bf;
+    const uint32_t q = rem - bf * p.spb;                       // slot inside the band (a short band's rem is below spb)
+    const uint32_t bw = q / LPT, cw = (q % LPT) * NC;
+    t.narrow = p.partial && bw + 1u == p.Wb;
+    const uint32_t cols = t.narrow ? p.W - bw * p.B : p.B;
+    t.cols = t.valid && cw < cols ? min(cols - cw, (uint32_t)NC) : 0u;
+    t.off = t.cols ? t.plane * p.HW + (band * p.B) * p.W + bw * p.B + cw : 0u;
+    t.tile = t.plane * p.TPP + band * p.Wb + bw;
+    t.writer = cw == 0;
+    t.rows = t.short_band ? p.tail_rows : p.B;
+    return t;
+}
+
 // ------------------------------------------------------------------------------------------------
 // half 1 of a CTA's share: planes [plane0, plane0 + nplanes) of sample n, which land in shared memory in SHARE_PIECES pieces
 // ------------------------------------------------------------------------------------------------
+// IN_PLACE: x stays as it is and res takes the stored low-frequency values of the tiles instead of the residuals.
 // keys (PER_PLANE): ~key(min), key(max) of the residuals of each plane; else lo / hi collect the extremes of the thread.
-// Slots of the CTA's share are numbered so that every warp holds slots of one height: the full-height bands of all planes
-// first, then, from the next multiple of 32, the short last bands.
-template <typename XT, int P2, typename G, bool PER_PLANE>
+template <typename XT, int P2, typename G, bool PER_PLANE, bool IN_PLACE, uint32_t THREADS>
 __device__ __forceinline__ void share_half1(const ShareParams& p, float* res, const XT* land, uint64_t* full, uint32_t n, uint32_t plane0,
                                          uint32_t nplanes, uint32_t* keys, float& lo, float& hi) {
-    constexpr uint32_t NC = G::NC, LPT = P2 / NC;               // lanes per tile
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nfull = nplanes * p.sppf, first_short = (nfull + 31u) & ~31u, total = first_short + nplanes * p.sppt;
     const uint64_t lfc0 = ((uint64_t)n * p.C + plane0) * p.TPP;
     uint32_t landed = 0;
-    for (uint32_t first = warp * 32u; first < total; first += SHARE_THREADS) {
-        const bool short_band = first >= first_short;          // the same in the whole warp
-        const uint32_t S = first + lane;
-        const bool valid = short_band ? S < total : S < nfull;
-        const uint32_t T = valid ? (short_band ? S - first_short : S) : 0u;
-        const uint32_t plane = fdiv(T, short_band ? p.by_spb : p.by_sppf);
-        const uint32_t rem = T - plane * (short_band ? p.spb : p.sppf);
-        const uint32_t bf = fdiv(rem, p.by_spb);
-        const uint32_t band = short_band ? p.Hb - 1u : bf;
-        const uint32_t q = rem - bf * p.spb;                   // slot inside the band (a short band's rem is below spb)
-        const uint32_t bw = q / LPT, cw = (q % LPT) * NC;
-        const bool narrow = p.partial && bw + 1u == p.Wb;
-        const uint32_t cols = narrow ? p.W - bw * p.B : p.B;
-        const uint32_t mine = valid && cw < cols ? min(cols - cw, NC) : 0u;
-        const uint32_t off = mine ? plane * p.HW + (band * p.B) * p.W + bw * p.B + cw : 0u;
+    for (uint32_t first = warp * 32u; first < total; first += THREADS) {
+        const ShareSlot t = share_slot<P2, G::NC>(p, first, lane, nfull, first_short, total);
         // pieces land in order; the unit's last slot needs the latest one
         {
-            const uint32_t last = __shfl_sync(0xFFFFFFFFu, valid ? plane : nplanes - 1u, 31);
+            const uint32_t last = __shfl_sync(0xFFFFFFFFu, t.valid ? t.plane : nplanes - 1u, 31);
             const uint32_t need = fdiv(last, p.by_ppp) + 1u;
             while (landed < need) {
                 if (!share_wait(&full[landed], p.timeout_ns)) atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
                 ++landed;
             }
         }
-        const uint32_t which = (short_band ? 2u : 0u) + (narrow ? 1u : 0u);
+        const uint32_t which = (t.short_band ? 2u : 0u) + (t.narrow ? 1u : 0u);
         SlotSink sink;
         sink.lfc = p.lfc;
-        sink.lfc_at = lfc0 + (plane * p.TPP + band * p.Wb + bw);
+        sink.lfc_at = lfc0 + t.tile;
         sink.lfc_bf16 = p.lfc_bf16;
-        sink.writer = cw == 0;
+        sink.writer = t.writer;
         sink.inv = p.inv[which];
         sink.cnt = p.cnt[which];
         sink.rcp = p.rcp[which];
         if constexpr (!PER_PLANE) {
-            reduce_slot<XT, P2, G>(land + off, res + off, p.W, short_band ? p.tail_rows : p.B, mine, sink, lo, hi);
+            reduce_slot<XT, P2, G, IN_PLACE>(land + t.off, res + (IN_PLACE ? t.tile : t.off), p.W, t.rows, t.cols, sink, lo, hi);
         } else {
             float l = 3.402823466e+38f, h = -3.402823466e+38f;
-            reduce_slot<XT, P2, G>(land + off, res + off, p.W, short_band ? p.tail_rows : p.B, mine, sink, l, h);
+            reduce_slot<XT, P2, G, IN_PLACE>(land + t.off, res + (IN_PLACE ? t.tile : t.off), p.W, t.rows, t.cols, sink, l, h);
             // lanes without a slot bring neutral extremes (whose keys are not neutral)
-            uint32_t kmin = mine ? ~float_key(l) : 0u, kmax = mine ? float_key(h) : 0u;
-            const uint32_t first_plane = __shfl_sync(0xFFFFFFFFu, plane, 0);
-            if (__all_sync(0xFFFFFFFFu, plane == first_plane || mine == 0u)) {
+            uint32_t kmin = t.cols ? ~float_key(l) : 0u, kmax = t.cols ? float_key(h) : 0u;
+            const uint32_t first_plane = __shfl_sync(0xFFFFFFFFu, t.plane, 0);
+            if (__all_sync(0xFFFFFFFFu, t.plane == first_plane || t.cols == 0u)) {
                 kmin = __reduce_max_sync(0xFFFFFFFFu, kmin);
                 kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
                 if (lane == 0) {
                     atomicMax(&keys[2u * first_plane], kmin);
                     atomicMax(&keys[2u * first_plane + 1u], kmax);
                 }
-            } else if (mine) {
-                atomicMax(&keys[2u * plane], kmin);
-                atomicMax(&keys[2u * plane + 1u], kmax);
+            } else if (t.cols) {
+                atomicMax(&keys[2u * t.plane], kmin);
+                atomicMax(&keys[2u * t.plane + 1u], kmax);
             }
         }
     }

@@ -41,7 +41,7 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
     griddep_wait();
     griddep_launch();
     float lo, hi;
-    share_half1<XT, P2, G, true>(p, res, land, full, n, plane0, nplanes, keys, lo, hi);
+    share_half1<XT, P2, G, true, false, SHARE_THREADS>(p, res, land, full, n, plane0, nplanes, keys, lo, hi);
     __syncthreads();
     for (uint32_t i = tid; i < nplanes; i += SHARE_THREADS) {
         const float rmax = key_float(keys[2u * i + 1u]);
@@ -97,7 +97,7 @@ bool plan_plane_share(const div_desc* d, const Shape& s, SharePlan* out) {
     double best = 0;
     for (uint64_t ppc = step; ppc <= 2048u; ppc += step) {
         SharePlan pl;
-        if (!plan_share(d, s, ppc, (uint32_t)(24u * ppc + 32u), di, &pl)) break;
+        if (!plan_share(d, s, ppc, (uint32_t)(24u * ppc + 32u), false, di, &pl)) break;
         if (ppc > step && pl.smem_bytes > 72u * 1024u) break;
         const uint64_t units = (ppc * full + 31u) / 32u + (ppc * shrt + 31u) / 32u;
         const double lanes = (double)(ppc * (full + shrt)) / (32.0 * ((units + SHARE_WARPS - 1u) / SHARE_WARPS * SHARE_WARPS));

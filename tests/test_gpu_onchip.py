@@ -51,6 +51,39 @@ def test_cluster_kernel_matches_the_checker(case):
     check(make((n, c, h, w), "bn" if c % 3 else "relu", 11 + h, xd), block, q, 77, xd, ld)
 
 
+IN_PLACE = [   # bfloat16, W % 4 == 0, B = 4 or 8: x stays as it is
+    (2, 8, 32, 32, 8, 2, "bf16"), (3, 16, 28, 28, 8, 4, "f32"), (2, 40, 20, 12, 4, 8, "bf16"), (2, 24, 5, 36, 8, 2, "f32"),
+    (5, 2, 9, 4, 4, 4, "bf16"), (1, 512, 7, 8, 8, 8, "f32"),
+]
+
+
+@pytest.mark.parametrize("case", IN_PLACE, ids=lambda c: "x".join(map(str, c)))
+def test_cluster_kernel_with_bfloat16_in_place(case):
+    n, c, h, w, block, q, ld = case
+    x = make((n, c, h, w), "bn", 21 + h, "bf16")
+    check(x, block, q, 78, "bf16", ld)
+    x[0] = 0x4050                              # a constant sample leaves the fixed-point route
+    check(x, block, q, 79, "bf16", ld)
+
+
+@pytest.mark.parametrize("case", [(32, 64, 75, 75, 8, "f32"), (64, 1024, 14, 14, 8, "f32"), (24, 512, 28, 28, 8, "f32"),
+                                  (30, 64, 90, 90, 16, "bf16")], ids=lambda c: "x".join(map(str, c)))
+def test_cluster_kernel_in_wide_blocks(case):
+    """Shares of which two fit an SM, more of them than fit at once: the same bytes as the kernel with a pass per half."""
+    n, c, h, w, block, xd = case
+    x = torch.randn((n, c, h, w), device="cuda", generator=torch.Generator("cuda").manual_seed(4)).to(torch.bfloat16 if xd == "bf16" else torch.float32)
+    codec = binding.Codec(n, c, h, w, block, 2, xd, "f32")
+    assert codec.plan().on_chip == 1
+    blobs = []
+    for flags in (0, binding.DIV_FLAG_FORCE_TWO_PASS):
+        codec.blob.zero_()
+        codec.compress(x, seed=6, flags=flags)
+        torch.cuda.synchronize()
+        assert codec.device_status() == binding.DIV_OK
+        blobs.append(codec.blob.clone())
+    assert torch.equal(*blobs)
+
+
 @pytest.mark.parametrize("q", [2, 4])
 def test_values_outside_the_fixed_point_route(q):
     """Constant, tiny, huge and one-sided samples beside an ordinary one."""
