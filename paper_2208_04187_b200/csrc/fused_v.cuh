@@ -32,6 +32,8 @@
 // cooperative only to be certain that all CTAs are resident (no grid-wide barrier is used).
 #pragma once
 
+#include <type_traits>
+
 #include "fused.cuh"
 
 namespace divk {
@@ -291,6 +293,67 @@ __device__ __forceinline__ uint64_t rng_mix(uint64_t z) {
     z *= K_MIX;
     z ^= z >> 32;
     return z;
+}
+
+// Can the sample's codes be had from quant4_fixed?  It needs products that neither overflow nor become subnormal
+// (|delta| bounds the smallest non-zero r - delta from below) and no result past the top code (the only value that
+// may round past it is the sample's largest residual).
+template <int Q>
+__device__ __forceinline__ bool fixed_point_ok(const QParams& q, float rmax) {
+    if (Q > 4) return false;
+    const float d = fabsf(q.delta);
+    return d >= 1e-24f && q.scale >= 1e-6f && q.scale <= 1e30f &&
+           __fmul_rn(__fsub_rn(rmax, q.delta), q.scale) <= (float)((1 << Q) - 1);
+}
+
+__device__ __forceinline__ uint64_t add2_rm(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Codes of 4 residuals (Eq. 9 with stochastic rounding), packed Q bits apart, in fixed point with 16 fraction bits.
+// With t = fl(fl(r - delta) * scale) as everywhere, nscale = -65536 * scale gives -65536 t exactly.  The float
+// M = 2^23 + 65536 qmax + field is a random half-word under a constant high half; M - 65536 t rounded down is
+// 2^23 + floor(65536 (qmax - t) + field), and dropping its low 16 bits leaves qmax - ceil(t - field / 65536), the
+// code's complement.  Per element: one byte permutation, half a packed add and the packing, where quant2 needs a
+// clamp, the permutation, half a fused multiply-add and half an add: 18 against 20 us for the 51 M residuals of a
+// 64 x 64 x 112 x 112 map already in shared memory.
+template <int Q>
+__device__ __forceinline__ uint32_t quant4_fixed(uint64_t xy, uint64_t zw, uint64_t delta2, uint64_t nscale2, uint64_t z) {
+    constexpr uint32_t TOP = 0x4B00u + ((1u << Q) - 1u);
+    const uint64_t a = mul2_rn(sub2_rn(xy, delta2), nscale2), b = mul2_rn(sub2_rn(zw, delta2), nscale2);
+    const uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
+    uint32_t v0, v1, v2, v3;
+    upk2u(add2_rm(a, pk2u(__byte_perm(lo, TOP, 0x5410), __byte_perm(lo, TOP, 0x5432))), v0, v1);
+    upk2u(add2_rm(b, pk2u(__byte_perm(hi, TOP, 0x5410), __byte_perm(hi, TOP, 0x5432))), v2, v3);
+    const uint32_t w01 = __byte_perm(v0, v1, 0x7632), w23 = __byte_perm(v2, v3, 0x7632);      // 0x4B00 + complement, two by two
+    const uint32_t s = w01 + (w23 << (2 * Q));
+    // the four fields; everything above the low 4 * Q bits is dropped by the caller's store
+    constexpr uint32_t W = 0x4B004B00u, S = W + (W << (2 * Q));
+    if (Q == 2) return 0xFFu + (S + (S >> 14)) - (s + (s >> 14));
+    return 0xFFFFu + (S + ((S >> 16) << Q)) - (s + ((s >> 16) << Q));
+}
+
+// Scale as it travels with a sample's parameters: negative where quant4_fixed applies (a scale is never negative itself).
+template <int Q>
+__device__ __forceinline__ float tagged_scale(const QParams& q, float rmax) { return fixed_point_ok<Q>(q, rmax) ? -q.scale : q.scale; }
+// the multiplier of quant4_x
+__device__ __forceinline__ uint64_t tagged_mul2(float tagged) {
+    const float m = tagged < 0.f ? 65536.0f * tagged : tagged;
+    return pk2(m, m);
+}
+// four elements of one strip row -> their codes, by the route that the sample's tag names
+template <int Q, bool FIXED>
+__device__ __forceinline__ uint32_t quant4_x(uint64_t xy, uint64_t zw, uint64_t stored2, uint64_t delta2, uint64_t mul2, uint64_t z) {
+    if constexpr (FIXED && Q <= 4) return quant4_fixed<Q>(sub2_rn(xy, stored2), sub2_rn(zw, stored2), delta2, mul2, z);
+    else return quant_row<Q>(xy, zw, stored2, delta2, mul2, z);
+}
+// run body(fixed) for the tag
+template <int Q, typename F>
+__device__ __forceinline__ void by_tag(float tagged, F&& body) {
+    if (Q <= 4 && tagged < 0.f) body(std::true_type());
+    else body(std::false_type());
 }
 
 // per-slot record, written by the reduce half for the quantise half

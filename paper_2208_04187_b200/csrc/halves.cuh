@@ -25,46 +25,6 @@ __device__ __forceinline__ float div_by_count(float sum, float cnt, float rcp) {
     return __fdiv_rn(sum, cnt);
 }
 
-// Can the sample's codes be had from quant4_fixed?  It needs products that neither overflow nor become subnormal
-// (|delta| bounds the smallest non-zero r - delta from below) and no result past the top code (the only value that
-// may round past it is the sample's largest residual).
-template <int Q>
-__device__ __forceinline__ bool fixed_point_ok(const QParams& q, float rmax) {
-    if (Q > 4) return false;
-    const float d = fabsf(q.delta);
-    return d >= 1e-24f && q.scale >= 1e-6f && q.scale <= 1e30f &&
-           __fmul_rn(__fsub_rn(rmax, q.delta), q.scale) <= (float)((1 << Q) - 1);
-}
-
-__device__ __forceinline__ uint64_t add2_rm(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
-// Codes of 4 residuals (Eq. 9 with stochastic rounding), packed Q bits apart, in fixed point with 16 fraction bits.
-// With t = fl(fl(r - delta) * scale) as everywhere, nscale = -65536 * scale gives -65536 t exactly.  The float
-// M = 2^23 + 65536 qmax + field is a random half-word under a constant high half; M - 65536 t rounded down is
-// 2^23 + floor(65536 (qmax - t) + field), and dropping its low 16 bits leaves qmax - ceil(t - field / 65536), the
-// code's complement.  Per element: one byte permutation, half a packed add and the packing, where quant2 needs a
-// clamp, the permutation, half a fused multiply-add and half an add: 18 against 20 us for the 51 M residuals of a
-// 64 x 64 x 112 x 112 map already in shared memory.
-template <int Q>
-__device__ __forceinline__ uint32_t quant4_fixed(uint64_t xy, uint64_t zw, uint64_t delta2, uint64_t nscale2, uint64_t z) {
-    constexpr uint32_t TOP = 0x4B00u + ((1u << Q) - 1u);
-    const uint64_t a = mul2_rn(sub2_rn(xy, delta2), nscale2), b = mul2_rn(sub2_rn(zw, delta2), nscale2);
-    const uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
-    uint32_t v0, v1, v2, v3;
-    upk2u(add2_rm(a, pk2u(__byte_perm(lo, TOP, 0x5410), __byte_perm(lo, TOP, 0x5432))), v0, v1);
-    upk2u(add2_rm(b, pk2u(__byte_perm(hi, TOP, 0x5410), __byte_perm(hi, TOP, 0x5432))), v2, v3);
-    const uint32_t w01 = __byte_perm(v0, v1, 0x7632), w23 = __byte_perm(v2, v3, 0x7632);      // 0x4B00 + complement, two by two
-    const uint32_t s = w01 + (w23 << (2 * Q));
-    // the four fields; everything above the low 4 * Q bits is dropped by the caller's store
-    constexpr uint32_t W = 0x4B004B00u, S = W + (W << (2 * Q));
-    if (Q == 2) return 0xFFu + (S + (S >> 14)) - (s + (s >> 14));
-    return 0xFFFFu + (S + ((S >> 16) << Q)) - (s + ((s >> 16) << Q));
-}
-
 // the same codes by the general route (clamped, any parameters)
 template <int Q>
 __device__ __forceinline__ uint32_t quant4_general(uint64_t xy, uint64_t zw, uint64_t delta2, uint64_t scale2, uint64_t z) {

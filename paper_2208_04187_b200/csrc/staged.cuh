@@ -24,7 +24,7 @@
 //     the chunk as arrived (the count is sent by the CTA's watcher thread, behind a release fence).  The
 //     watcher also polls the counts of the samples blockIdx.x, blockIdx.x + gridDim.x, ...; when a sample is
 //     complete it derives (delta, Delta, scale), writes the first two to the blob and publishes delta and
-//     scale as one 64-bit word in the slot.
+//     scale as one 64-bit word in the slot (scale negative: the fixed-point quantiser applies; 0: not there yet).
 //   * quantise unit: the tile mean is computed again from the staged rows, then the 4 codes of each strip
 //     row are emitted as one byte (Q = 2), half-word (Q = 4) or word (Q = 8); lanes of a warp write
 //     consecutive bytes.  The quantise producer reads the sample's published word before it issues the
@@ -58,7 +58,7 @@ namespace divk {
 #define DIVK_S_Q_STAGES_PER_8 4
 #endif
 #ifndef DIVK_S_REDUCE_WARPS
-#define DIVK_S_REDUCE_WARPS 14
+#define DIVK_S_REDUCE_WARPS 13
 #endif
 #ifndef DIVK_S_TARGET_BYTES
 #define DIVK_S_TARGET_BYTES (28 * 1024)
@@ -67,7 +67,9 @@ namespace divk {
 #define DIVK_S_LAG_BYTES (48u << 20)
 #endif
 constexpr int S_WORKER_WARPS = DIVK_S_WORKER_WARPS;
-constexpr int S_REDUCE_WARPS = DIVK_S_REDUCE_WARPS;      // of the worker warps
+// of the worker warps.  64 x 64 x 112 x 112, 64 x 512 x 28 x 28 with the fixed-point quantiser: 10 warps 61.7, 43.2 us; 12 59.5,
+// 41.1; 13 58.5, 40.9; 14 58.9, 41.8; 15 60.4, 45.9 (general quantiser, 14 warps: 59.5, 41.1).
+constexpr int S_REDUCE_WARPS = DIVK_S_REDUCE_WARPS;
 static_assert(S_REDUCE_WARPS >= 1 && S_REDUCE_WARPS < S_WORKER_WARPS, "both worker classes need a warp");
 constexpr int S_SERVICE_WARPS = 3;          // reduce producer, quantise producer, watcher
 constexpr int S_THREADS = 32 * (S_SERVICE_WARPS + S_WORKER_WARPS);
@@ -397,10 +399,12 @@ staged_kernel(const SParams p) {
             if (n < s.N) {
                 uint32_t* slot = p.ws + WS_HEADER_WORDS + (size_t)n * WS_SLOT_WORDS;
                 if (ld_acquire_u32(slot + 2) == p.expected_chunks) {
-                    const QParams qp = make_qparams(key_float(~ld_relaxed_u32(slot + 0)), key_float(ld_relaxed_u32(slot + 1)), Q);
+                    const float rmax = key_float(ld_relaxed_u32(slot + 1));
+                    const QParams qp = make_qparams(key_float(~ld_relaxed_u32(slot + 0)), rmax, Q);
                     p.stats[2 * (size_t)n + 0] = qp.delta;
                     p.stats[2 * (size_t)n + 1] = qp.step;
-                    const uint64_t word = ((uint64_t)(__float_as_uint(qp.scale) | 0x80000000u) << 32) | (uint64_t)__float_as_uint(qp.delta);
+                    uint64_t word = ((uint64_t)__float_as_uint(tagged_scale<Q>(qp, rmax)) << 32) | (uint64_t)__float_as_uint(qp.delta);
+                    if (word == 0ull) word = 0x80000000ull;      // nothing published reads as zero; a zero's sign does not reach the codes
                     st_release_u64(reinterpret_cast<uint64_t*>(slot + 4), word);
                     n += G;
                     progress = true;
@@ -471,13 +475,13 @@ staged_kernel(const SParams p) {
                 }
                 if (!ok) break;
             }
-            if (quant && !(word >> 63)) {
+            if (quant && word == 0ull) {
                 const uint64_t* pw = reinterpret_cast<const uint64_t*>(p.ws + WS_HEADER_WORDS + (size_t)n * WS_SLOT_WORDS + 4);
                 uint32_t polls = 0;
                 SWait w = {0, 0};
                 while (true) {
                     word = ld_relaxed_u64(pw);
-                    if (word >> 63) break;
+                    if (word != 0ull) break;
                     if ((++polls & 7u) == 0 && s_give_up(p, ctl, w)) {
                         s_record_failure(p, ctl, n + 1u);
                         ok = false;
@@ -498,7 +502,7 @@ staged_kernel(const SParams p) {
             d.quad0 = ((uint64_t)n * s.CHW + e0) >> 2;
             d.ctr0 = rng_sample_base(p.seed, n) + K_GROUP * (uint64_t)((e0 >> 2) + 1u);
             d.delta = __uint_as_float((uint32_t)word);
-            d.scale = __uint_as_float((uint32_t)(word >> 32) & 0x7FFFFFFFu);
+            d.scale = __uint_as_float((uint32_t)(word >> 32));
             desc[st] = d;
             const uint32_t bytes = nelem * (uint32_t)sizeof(XT);
             const XT* src = reinterpret_cast<const XT*>(p.x) + ((size_t)n * s.CHW + e0);
@@ -668,28 +672,29 @@ staged_kernel(const SParams p) {
             if (active) {
                 const float delta = ctl->desc_q[st].delta, scale = ctl->desc_q[st].scale;
                 const uint64_t stored2 = pk2(stored, stored);
-                const uint64_t delta2 = pk2(delta, delta), scale2 = pk2(scale, scale);
+                const uint64_t delta2 = pk2(delta, delta), mul2 = tagged_mul2(scale);
                 uint64_t ctr = ctl->desc_q[st].ctr0 + K_GROUP * (uint64_t)quad;
                 OutT* out = packed + ctl->desc_q[st].quad0 + quad;
-                if (full) {
+                by_tag<Q>(scale, [&](auto fixed) {                       // the same in the whole warp: a chunk has one sample
+                    constexpr bool FIXED = decltype(fixed)::value;
+                    if (full) {
 #pragma unroll
-                    for (int r = 0; r < P2; ++r) {
-                        *out = (OutT)quant_row<Q>(vxy[r], vzw[r], stored2, delta2, scale2, rng_mix(ctr));
-                        out += W4;
-                        ctr += p.rng_row_step;
-                    }
-                } else {
+                        for (int r = 0; r < P2; ++r) {
+                            *out = (OutT)quant4_x<Q, FIXED>(vxy[r], vzw[r], stored2, delta2, mul2, rng_mix(ctr));
+                            out += W4;
+                            ctr += p.rng_row_step;
+                        }
+                    } else {
 #pragma unroll
-                    for (int r = 0; r < P2; ++r) {
-                        if ((uint32_t)r < rmax) {
-                            if ((uint32_t)r < rows) {
-                                *out = (OutT)quant_row<Q>(vxy[r], vzw[r], stored2, delta2, scale2, rng_mix(ctr));
+                        for (int r = 0; r < P2; ++r) {
+                            if ((uint32_t)r < rmax && (uint32_t)r < rows) {
+                                *out = (OutT)quant4_x<Q, FIXED>(vxy[r], vzw[r], stored2, delta2, mul2, rng_mix(ctr));
                                 out += W4;
                                 ctr += p.rng_row_step;
                             }
                         }
                     }
-                }
+                });
             }
         }
         __syncwarp();
