@@ -53,6 +53,10 @@ def ncu_traffic(kernel: str, map_label: str):
         return None
 
 
+def compress_name(names, plan):
+    return "cluster_kernel" if plan.on_chip else names[int(plan.fused)]
+
+
 def measured_peak():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
@@ -327,7 +331,7 @@ def measure_configs(device, ev, barrier, configs, peak, names, dec_names):
             d_us = a.elapsed_time(b) * 1e3 / reps
             rows.append({"map": "x".join(map(str, spec.shape)) + f" {spec.x_dtype} {spec.kind} B{spec.block} Q{spec.qbits}",
                          "MB": round(nbytes / 1e6, 1), "pool": pool, "calls": reps,
-                         "compress_kernel": names[int(plan.fused)], "compress_us": round(c_us, 1),
+                         "compress_kernel": compress_name(names, plan), "compress_us": round(c_us, 1),
                          "compress_GBps": round(algo / c_us / 1e3, 1), "compress_frac": round(algo / c_us / 1e3 / peak, 3),
                          "decompress_kernel": dec_names[int(plan.decompress_fast)], "decompress_us": round(d_us, 1),
                          "decompress_GBps": round(algo / d_us / 1e3, 1), "decompress_frac": round(algo / d_us / 1e3 / peak, 3)})
@@ -545,6 +549,7 @@ def run_ours(args):
                    for i in range(len(pg))]
         pg_dec = [statistics.mean(pg_rec[k][1][i][0].elapsed_time(pg_rec[k][1][i][1]) for k in range(pg_steps))
                   for i in range(len(pg))]
+        pg_name = lambda pl: "plane_share_kernel" if pl.on_chip else pg_names[int(pl.fused)]
         pg_names = {1: "pg_strip_kernel", 2: "pg_small_kernel", 0: "pg_general_kernel"}
         pg_dec_names = {1: "pg_decompress_quad_kernel", 2: "pg_decompress_flat_kernel", 0: "pg_decompress_general_kernel"}
         pg_algo = [int(c.layout.raw_bytes) + int(c.layout.closed_form_bytes) for c in pg]
@@ -557,15 +562,15 @@ def run_ours(args):
             "value": raw_bytes / (pg_ms * 1e-3) / 1e9, "unit": UNIT, "steps": pg_steps, "ms_per_step": pg_ms,
             "compression_ratio": raw_bytes / sum(int(c.layout.closed_form_bytes) for c in pg),
             "gpu_launches": 2 * len(pg) * pg_steps,
-            "per_map": [{"map": "x".join(map(str, s.shape)), "compress_kernel": pg_names[int(p.fused)],
+            "per_map": [{"map": "x".join(map(str, s.shape)), "compress_kernel": pg_name(p),
                          "decompress_kernel": pg_dec_names[int(p.decompress_fast)],
                          "compress_us": round(cm * 1e3, 2), "compress_GBps": round(b / cm / 1e6, 1),
                          "decompress_us": round(dm * 1e3, 2), "decompress_GBps": round(b / dm / 1e6, 1)}
                         for s, p, cm, dm, b in zip(specs, pg_plans, pg_comp, pg_dec, pg_algo)],
-            "roofline": {"bound": "hbm", "kernel": pg_names[int(pg_plans[pg_dom].fused)] + " on " +
+            "roofline": {"bound": "hbm", "kernel": pg_name(pg_plans[pg_dom]) + " on " +
                          "x".join(map(str, specs[pg_dom].shape)), "achieved": pg_dom_gbs, "peak": pg_peak,
                          "unit": "GB/s", "frac": pg_dom_gbs / pg_peak, "peak_kind": f"of {pg_peak_kind}",
-                         "traffic": ncu_traffic(pg_names[int(pg_plans[pg_dom].fused)], "x".join(map(str, specs[pg_dom].shape))),
+                         "traffic": ncu_traffic(pg_name(pg_plans[pg_dom]), "x".join(map(str, specs[pg_dom].shape))),
                          "algorithmic_bytes_per_launch": pg_algo[pg_dom]},
         }
 
@@ -655,7 +660,7 @@ def run_ours(args):
             cm = statistics.mean(t_rec[k][0][i][0].elapsed_time(t_rec[k][0][i][1]) for k in range(t_steps))
             dm = statistics.mean(t_rec[k][1][i][0].elapsed_time(t_rec[k][1][i][1]) for k in range(t_steps))
             b = int(t_codec[i].layout.raw_bytes) + int(t_codec[i].layout.closed_form_bytes)
-            rows.append({"map": name, "compress_kernel": kernel_names_all[int(t_codec[i].plan().fused)],
+            rows.append({"map": name, "compress_kernel": compress_name(kernel_names_all, t_codec[i].plan()),
                          "compress_us": round(cm * 1e3, 2), "compress_GBps": round(b / cm / 1e6, 1),
                          "compress_frac_of_peak": round(b / cm / 1e6 / t_peak, 3),
                          "decompress_us": round(dm * 1e3, 2), "decompress_GBps": round(b / dm / 1e6, 1),
@@ -743,7 +748,7 @@ def run_ours(args):
     comp_gbs = sum(algo_bytes) / (sum(comp_ms) * 1e-3) / 1e9
     dec_gbs = sum(algo_bytes) / (sum(dec_ms) * 1e-3) / 1e9
     kernel_names = kernel_names_all
-    per_map = [{"map": "x".join(map(str, s.shape)), "compress_kernel": kernel_names[int(p.fused)],
+    per_map = [{"map": "x".join(map(str, s.shape)), "compress_kernel": compress_name(kernel_names, p),
                 "compress_us": round(cm * 1e3, 2), "compress_GBps": round(b / cm / 1e6, 1),
                 "decompress_us": round(dm * 1e3, 2), "decompress_GBps": round(b / dm / 1e6, 1)}
                for s, p, cm, dm, b in zip(specs, plans, comp_ms, dec_ms, algo_bytes)]
@@ -776,12 +781,12 @@ def run_ours(args):
                    "ms_per_step_min": min(rep_ms) / args.steps, "ms_per_step_max": max(rep_ms) / args.steps, "repeats": len(rep_ms),
                    "multi_gpu": "replicas only: each rank runs the same set on its own GPU, no collective",
                    "compression_ratio": raw_bytes / comp_bytes, "per_map": per_map},
-        "roofline": {"bound": "hbm", "kernel": kernel_names[int(plans[dom].fused)] + " on " + per_map[dom]["map"] +
+        "roofline": {"bound": "hbm", "kernel": compress_name(kernel_names, plans[dom]) + " on " + per_map[dom]["map"] +
                      f" ({dom_n} back-to-back calls between two CUDA events on its stream, two inputs alternating; "
                      "the span includes the 2-us workspace clear)",
                      "achieved": dom_gbs, "peak": peak, "unit": "GB/s", "frac": dom_gbs / peak, "us_per_launch": dom_ms * 1e3,
                      "peak_kind": f"of {peak_kind}", "frac_of_nominal_8TBps": dom_gbs / NOMINAL_HBM_GBS,
-                     "traffic": ncu_traffic(kernel_names[int(plans[dom].fused)], per_map[dom]["map"]),
+                     "traffic": ncu_traffic(compress_name(kernel_names, plans[dom]), per_map[dom]["map"]),
                      "algorithmic_bytes_per_launch": algo_bytes[dom]},
         "roofline_all_compress": {"bound": "hbm", "kernel": "all compress calls of the step", "achieved": comp_gbs,
                                   "peak": peak, "unit": "GB/s", "frac": comp_gbs / peak, "peak_kind": f"of {peak_kind}"},
