@@ -74,9 +74,6 @@ inline bool plan_cluster_cs(const div_desc* d, const Shape& s, uint32_t cs, cons
     const uint64_t places = (uint64_t)per_sm * (uint32_t)di.sms * 95u / 100u;      // clusters leave about 5 % of the places empty
     pl.waves = (uint32_t)(((uint64_t)s.N * cs + places - 1) / (places ? places : 1u));
     pl.wide = pl.waves > 1u && per_sm <= 2u ? 1u : 0u;
-#ifdef DIVK_DEV
-    if (const char* e = getenv("DIVK_WIDE"); e && *e) pl.wide = atoi(e);
-#endif
     *out = pl;
     return true;
 }

@@ -238,22 +238,11 @@ void choose_compress(const div_desc* d, const Shape& s, uint32_t flags, Choice* 
     if (plan_fused(d, s, &c->fp) == DIV_OK) c->code = 1;
 }
 
-#ifdef DIVK_DEV
-}
-#include <stdlib.h>
-namespace {
-#endif
 // Does the cluster kernel take a descriptor, and in clusters of how many CTAs?  (Flags pin one of the other kernels.)
 bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPlan* out) {
     if (flags != 0) return false;
     const DeviceInfo di = device_info();
     if (!di.ok || di.sms < 1) return false;
-#ifdef DIVK_DEV
-    if (const char* e = getenv("DIVK_CS"); e && *e) {
-        if (atoi(e) == 0) return false;
-        return plan_cluster_cs(d, s, (uint32_t)atoi(e), di, out);
-    }
-#endif
     if (s.H == 1) {
         LineGeom lg;
         if (plan_lines(d, s, &lg)) return false;          // 1-D maps have a kernel of their own
