@@ -19,60 +19,69 @@ bool tensor_arg(PyObject* o, const at::Tensor** out) {
     *out = &THPVariable_Unpack(o);
     return true;
 }
-bool desc_arg(PyObject* o, const div_desc** out) {
-    *out = reinterpret_cast<const div_desc*>(PyLong_AsVoidPtr(o));
-    return !PyErr_Occurred();
+bool desc_arg(PyObject* o, div_desc* out) {
+    const void* at = PyLong_AsVoidPtr(o);
+    if (at) *out = *reinterpret_cast<const div_desc*>(at);
+    return at && !PyErr_Occurred();
 }
-at::ScalarType scalar(const div_desc* d) { return d->x_dtype == DIV_F32 ? at::kFloat : at::kBFloat16; }
+at::ScalarType scalar(const div_desc& d) { return d.x_dtype == DIV_F32 ? at::kFloat : at::kBFloat16; }
 void* stream() { return reinterpret_cast<void*>(c10::cuda::getCurrentCUDAStream().stream()); }
-bool matches(const at::Tensor& x, const div_desc* d) {
-    return x.is_cuda() && x.scalar_type() == scalar(d) && x.dim() == 4 && x.size(0) == d->n && x.size(1) == d->c && x.size(2) == d->h &&
-           x.size(3) == d->w && x.is_contiguous();
+bool matches(const at::Tensor& x, const div_desc& d) {
+    return x.is_cuda() && x.scalar_type() == scalar(d) && x.dim() == 4 && x.size(0) == d.n && x.size(1) == d.c && x.size(2) == d.h &&
+           x.size(3) == d.w && x.is_contiguous();
 }
 
 // compress(desc address, x, blob, workspace or None (per-plane groups), seed, flags) -> status, or -1: x does not match
+// (What a tensor may answer with an exception, its sizes, layout and storage, is asked before the interpreter is released.)
 PyObject* compress(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 6) {
         PyErr_SetString(PyExc_TypeError, "compress takes 6 arguments");
         return nullptr;
     }
-    const div_desc* d;
+    div_desc d;
     const at::Tensor *x, *blob, *ws = nullptr;
     if (!desc_arg(a[0], &d) || !tensor_arg(a[1], &x) || !tensor_arg(a[2], &blob) || (a[3] != Py_None && !tensor_arg(a[3], &ws))) return nullptr;
     const uint64_t seed = PyLong_AsUnsignedLongLongMask(a[4]);
     const uint32_t flags = (uint32_t)PyLong_AsUnsignedLongMask(a[5]);
     if (PyErr_Occurred()) return nullptr;
     if (!matches(*x, d)) return PyLong_FromLong(-1);
-    div_status st;
+    const void* from = x->data_ptr();
+    void *to = blob->data_ptr(), *scratch = ws ? ws->data_ptr() : nullptr, *st = stream();
+    const size_t room = (size_t)blob->numel(), scratch_room = ws ? (size_t)ws->numel() : 0;
+    div_status got;
     Py_BEGIN_ALLOW_THREADS              // a full launch queue blocks
-    st = ws ? div_compress_ex(d, x->data_ptr(), blob->data_ptr(), (size_t)blob->numel(), ws->data_ptr(), (size_t)ws->numel(), seed, stream(), flags)
-            : div_planegroup_compress(d, x->data_ptr(), blob->data_ptr(), (size_t)blob->numel(), seed, stream(), flags);
+    got = ws ? div_compress_ex(&d, from, to, room, scratch, scratch_room, seed, st, flags) : div_planegroup_compress(&d, from, to, room, seed, st, flags);
     Py_END_ALLOW_THREADS
-    return PyLong_FromLong((long)st);
+    return PyLong_FromLong((long)got);
+    END_HANDLE_TH_ERRORS
 }
 
 // decompress(desc address, blob, out or None, per-plane groups?) -> the output tensor (a new one on the blob's device
 // where out is None), or a status
 PyObject* decompress(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 4) {
         PyErr_SetString(PyExc_TypeError, "decompress takes 4 arguments");
         return nullptr;
     }
-    const div_desc* d;
+    div_desc d;
     const at::Tensor *blob, *given = nullptr;
     if (!desc_arg(a[0], &d) || !tensor_arg(a[1], &blob) || (a[2] != Py_None && !tensor_arg(a[2], &given))) return nullptr;
-    HANDLE_TH_ERRORS
     at::Tensor made;
     if (!given) {
-        made = at::empty({d->n, d->c, d->h, d->w}, blob->options().dtype(scalar(d)).requires_grad(false));
+        made = at::empty({d.n, d.c, d.h, d.w}, blob->options().dtype(scalar(d)).requires_grad(false));
         given = &made;
     }
     const auto call = a[3] == Py_True ? div_planegroup_decompress : div_decompress;
-    div_status st;
+    const void* from = blob->data_ptr();
+    void *to = given->data_ptr(), *st = stream();
+    const size_t bytes = (size_t)blob->numel();
+    div_status got;
     Py_BEGIN_ALLOW_THREADS
-    st = call(d, blob->data_ptr(), (size_t)blob->numel(), given->data_ptr(), stream());
+    got = call(&d, from, bytes, to, st);
     Py_END_ALLOW_THREADS
-    if (st != DIV_OK) return PyLong_FromLong((long)st);
+    if (got != DIV_OK) return PyLong_FromLong((long)got);
     if (made.defined()) return THPVariable_Wrap(std::move(made));
     Py_INCREF(a[2]);
     return a[2];
