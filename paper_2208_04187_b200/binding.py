@@ -331,7 +331,6 @@ class Codec:
         self.device = torch.device(device)
         self.blob = torch.zeros(int(self.layout.total_bytes), dtype=torch.uint8, device=self.device)
         self.workspace = torch.zeros(int(self.layout.workspace_bytes), dtype=torch.uint8, device=self.device)
-        self._native, self._addr = native(), ctypes.addressof(self.desc)
 
     def plan(self, flags: int = 0) -> DivPlan:
         return div_plan_query(self.desc, flags)
@@ -340,13 +339,13 @@ class Codec:
         """x: contiguous CUDA tensor of shape N x C x H x W in the descriptor's dtype."""
         if blob is None:
             blob = self.blob
-        status = self._native.compress(self._addr, x, blob, self.workspace, seed, flags)
+        status = (_native or native()).compress(self.desc, x, blob, self.workspace, seed, flags)
         if status:
             _raise(status, "div_compress")
         return blob
 
     def decompress(self, blob=None, out=None):
-        got = self._native.decompress(self._addr, self.blob if blob is None else blob, out, False)
+        got = (_native or native()).decompress(self.desc, self.blob if blob is None else blob, out, False)
         if got.__class__ is int:
             _raise(got, "div_decompress")
         return got
@@ -366,7 +365,6 @@ class PlaneGroupCodec:
         self.shape = (n, c, h, w)
         self.device = torch.device(device)
         self.blob = torch.zeros(int(self.layout.total_bytes), dtype=torch.uint8, device=self.device)
-        self._native, self._addr = native(), ctypes.addressof(self.desc)
 
     def plan(self, flags: int = 0) -> DivPlan:
         return div_planegroup_plan_query(self.desc, flags)
@@ -374,13 +372,13 @@ class PlaneGroupCodec:
     def compress(self, x, seed: int = 0, flags: int = 0, blob=None):
         if blob is None:
             blob = self.blob
-        status = self._native.compress(self._addr, x, blob, None, seed, flags)
+        status = (_native or native()).compress(self.desc, x, blob, None, seed, flags)
         if status:
             _raise(status, "div_planegroup_compress")
         return blob
 
     def decompress(self, blob=None, out=None):
-        got = self._native.decompress(self._addr, self.blob if blob is None else blob, out, True)
+        got = (_native or native()).decompress(self.desc, self.blob if blob is None else blob, out, True)
         if got.__class__ is int:
             _raise(got, "div_planegroup_decompress")
         return got

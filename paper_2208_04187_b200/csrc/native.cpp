@@ -19,10 +19,15 @@ bool tensor_arg(PyObject* o, const at::Tensor** out) {
     *out = &THPVariable_Unpack(o);
     return true;
 }
+// the descriptor's fields, copied: the object may be replaced or changed while the interpreter is released
 bool desc_arg(PyObject* o, div_desc* out) {
-    const void* at = PyLong_AsVoidPtr(o);
-    if (at) *out = *reinterpret_cast<const div_desc*>(at);
-    return at && !PyErr_Occurred();
+    Py_buffer view;
+    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return false;
+    const bool ok = view.len == (Py_ssize_t)sizeof(*out);
+    if (ok) memcpy(out, view.buf, sizeof(*out));
+    PyBuffer_Release(&view);
+    if (!ok) PyErr_SetString(PyExc_TypeError, "expected a DivDesc");
+    return ok;
 }
 at::ScalarType scalar(const div_desc& d) { return d.x_dtype == DIV_F32 ? at::kFloat : at::kBFloat16; }
 void* stream() { return reinterpret_cast<void*>(c10::cuda::getCurrentCUDAStream().stream()); }
@@ -31,7 +36,7 @@ bool matches(const at::Tensor& x, const div_desc& d) {
            x.size(3) == d.w && x.is_contiguous();
 }
 
-// compress(desc address, x, blob, workspace or None (per-plane groups), seed, flags) -> status, or -1: x does not match
+// compress(descriptor, x, blob, workspace or None (per-plane groups), seed, flags) -> status, or -1: x does not match
 // (What a tensor may answer with an exception, its sizes, layout and storage, is asked before the interpreter is released.)
 PyObject* compress(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
@@ -57,7 +62,7 @@ PyObject* compress(PyObject*, PyObject* const* a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
-// decompress(desc address, blob, out or None, per-plane groups?) -> the output tensor (a new one on the blob's device
+// decompress(descriptor, blob, out or None, per-plane groups?) -> the output tensor (a new one on the blob's device
 // where out is None), or a status
 PyObject* decompress(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS

@@ -1,12 +1,15 @@
 """The codec's calls through the CPython extension, as far as they need no GPU: tensors that cannot answer end in a
-Python exception."""
+Python exception, and a codec is an ordinary object (it can be copied, sent to another process, given another descriptor)."""
+import copy
 import os
+import pickle
 import subprocess
 import sys
 
 import pytest
+import torch
 
-from paper_2208_04187_b200 import build
+from paper_2208_04187_b200 import binding, build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -18,7 +21,7 @@ def built_library():
 
 # `without` has no storage to ask for; `x` stands for a CUDA tensor on a machine without one
 STORAGELESS = """
-import ctypes, torch
+import torch
 from torch._subclasses.fake_tensor import FakeTensorMode
 from paper_2208_04187_b200 import binding
 without = torch.zeros(4096, dtype=torch.uint8).to_sparse()
@@ -26,8 +29,7 @@ with FakeTensorMode():
     x = torch.empty(2, 3, 8, 8, device="cuda")
 desc = binding.make_desc(2, 3, 8, 8, 8, 2)
 codec = object.__new__(binding.{cls})
-codec.__dict__.update(desc=desc, blob=without, workspace=torch.zeros(4096, dtype=torch.uint8), device=torch.device("cpu"),
-                      _native=binding.native(), _addr=ctypes.addressof(desc))
+codec.__dict__.update(desc=desc, blob=without, workspace=torch.zeros(4096, dtype=torch.uint8), device=torch.device("cpu"))
 for call in (lambda: codec.compress(x), codec.decompress, lambda: codec.decompress(out=without)):
     try:
         call()
@@ -42,3 +44,36 @@ def test_a_tensor_without_storage_is_an_exception(cls):
     got = subprocess.run([sys.executable, "-c", STORAGELESS.format(cls=cls)], cwd=ROOT, capture_output=True, text=True,
                          env=dict(os.environ, PYTHONPATH=ROOT), timeout=300)
     assert got.returncode == 0 and got.stdout.split() == ["raised"] * 3, (got.returncode, got.stderr[-2000:])
+
+
+def codec_on_the_host(cls):
+    """A codec whose buffers are on the host, through its own constructor: the library refuses its calls by the
+    buffers' sizes, before any of them is touched."""
+    return cls(2, 3, 8, 8, 8, 2, device="cpu")
+
+
+@pytest.mark.parametrize("cls", [binding.Codec, binding.PlaneGroupCodec])
+def test_codecs_can_be_copied_and_pickled(cls):
+    codec = codec_on_the_host(cls)
+    for twin in (copy.deepcopy(codec), pickle.loads(pickle.dumps(codec)), copy.copy(codec)):
+        assert bytes(twin.desc) == bytes(codec.desc) and twin.shape == codec.shape and twin.blob.numel() == codec.blob.numel()
+        assert not any(isinstance(v, type(os)) for v in vars(twin).values())
+
+
+@pytest.mark.parametrize("cls", [binding.Codec, binding.PlaneGroupCodec])
+def test_a_codec_follows_its_descriptor(cls, monkeypatch):
+    """The call is made with the descriptor that the codec has now, not with one that it had when it was made."""
+    codec = codec_on_the_host(cls)
+    codec.blob = torch.zeros(16, dtype=torch.uint8)[:1]                # too small for either descriptor
+    seen = []
+
+    class Spy:
+        def decompress(self, desc, *rest):
+            seen.append(bytes(desc))
+            return binding.DIV_ERR_CAPACITY
+    monkeypatch.setattr(binding, "_native", Spy())
+    for w in (8, 24):
+        codec.desc = binding.make_desc(2, 3, 8, w, 8, 2)
+        with pytest.raises(binding.DivisionError):
+            codec.decompress()
+        assert seen[-1] == bytes(codec.desc)
