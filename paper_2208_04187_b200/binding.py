@@ -345,7 +345,7 @@ class Codec:
         return blob
 
     def decompress(self, blob=None, out=None):
-        got = (_native or native()).decompress(self.desc, self.blob if blob is None else blob, out, False)
+        got = (_native or native()).decompress(self.desc, self.blob if blob is None else blob, out, self.device, False)
         if got.__class__ is int:
             _raise(got, "div_decompress")
         return got
@@ -378,7 +378,7 @@ class PlaneGroupCodec:
         return blob
 
     def decompress(self, blob=None, out=None):
-        got = (_native or native()).decompress(self.desc, self.blob if blob is None else blob, out, True)
+        got = (_native or native()).decompress(self.desc, self.blob if blob is None else blob, out, self.device, True)
         if got.__class__ is int:
             _raise(got, "div_planegroup_decompress")
         return got

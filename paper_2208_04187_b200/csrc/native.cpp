@@ -2,10 +2,14 @@
 // call into libdivision.so, without a Python interpreter step in between.  (The ctypes route costs 2.3 us of marshalling per
 // compress call and 5 us per decompress call, 2.8 us of it to parse the arguments of torch.empty: more than the 2.5 us that
 // the launch itself takes.)  Plain CPython extension, vector calls; all arithmetic stays in the CUDA library.
+#include <torch/csrc/Device.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+
+#include <cstring>
 
 #include "../../include/division.h"
 
@@ -62,23 +66,27 @@ PyObject* compress(PyObject*, PyObject* const* a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
-// decompress(descriptor, blob, out or None, per-plane groups?) -> the output tensor (a new one on the blob's device
-// where out is None), or a status
+// decompress(descriptor, blob, out or None, device, per-plane groups?) -> the output tensor (where out is None a new one on
+// the device: the blob may be elsewhere, in pinned host memory for instance), or a status
 PyObject* decompress(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
-    if (n != 4) {
-        PyErr_SetString(PyExc_TypeError, "decompress takes 4 arguments");
+    if (n != 5) {
+        PyErr_SetString(PyExc_TypeError, "decompress takes 5 arguments");
         return nullptr;
     }
     div_desc d;
     const at::Tensor *blob, *given = nullptr;
     if (!desc_arg(a[0], &d) || !tensor_arg(a[1], &blob) || (a[2] != Py_None && !tensor_arg(a[2], &given))) return nullptr;
+    if (!THPDevice_Check(a[3])) {
+        PyErr_SetString(PyExc_TypeError, "expected a device");
+        return nullptr;
+    }
     at::Tensor made;
     if (!given) {
-        made = at::empty({d.n, d.c, d.h, d.w}, blob->options().dtype(scalar(d)).requires_grad(false));
+        made = at::empty({d.n, d.c, d.h, d.w}, at::TensorOptions(reinterpret_cast<THPDevice*>(a[3])->device).dtype(scalar(d)));
         given = &made;
     }
-    const auto call = a[3] == Py_True ? div_planegroup_decompress : div_decompress;
+    const auto call = a[4] == Py_True ? div_planegroup_decompress : div_decompress;
     const void* from = blob->data_ptr();
     void *to = given->data_ptr(), *st = stream();
     const size_t bytes = (size_t)blob->numel();

@@ -8,6 +8,7 @@ import sys
 
 import pytest
 import torch
+from torch.utils._python_dispatch import TorchDispatchMode
 
 from paper_2208_04187_b200 import binding, build
 
@@ -22,6 +23,7 @@ def built_library():
 # `without` has no storage to ask for; `x` stands for a CUDA tensor on a machine without one
 STORAGELESS = """
 import torch
+from torch.utils._python_dispatch import TorchDispatchMode
 from torch._subclasses.fake_tensor import FakeTensorMode
 from paper_2208_04187_b200 import binding
 without = torch.zeros(4096, dtype=torch.uint8).to_sparse()
@@ -77,3 +79,38 @@ def test_a_codec_follows_its_descriptor(cls, monkeypatch):
         with pytest.raises(binding.DivisionError):
             codec.decompress()
         assert seen[-1] == bytes(codec.desc)
+
+
+class Takes(Exception):
+    pass
+
+
+@pytest.mark.parametrize("cls", [binding.Codec, binding.PlaneGroupCodec])
+def test_the_output_is_made_on_the_codec_s_device(cls):
+    """Not on the blob's: a blob in pinned host memory, which the GPU reads in place, is rebuilt on the GPU."""
+    codec = codec_on_the_host(cls)
+    codec.device = torch.device("meta")
+    made = []
+
+    class Watch(TorchDispatchMode):
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            if func is torch.ops.aten.empty.memory_format:
+                made.append((list(args[0]), kwargs.get("device"), kwargs.get("dtype")))
+                raise Takes                     # before the call itself
+            return func(*args, **(kwargs or {}))
+
+    with Watch(), pytest.raises(Takes):
+        codec.decompress()
+    assert made == [([2, 3, 8, 8], torch.device("meta"), torch.float32)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("cls", [binding.Codec, binding.PlaneGroupCodec])
+def test_a_blob_in_pinned_host_memory_is_rebuilt_on_the_gpu(cls):
+    x = torch.randn(2, 16, 28, 28, device="cuda")
+    codec = cls(2, 16, 28, 28, 8, 2)
+    codec.compress(x, seed=3)
+    want = codec.decompress()
+    host = codec.blob.cpu().pin_memory()
+    got = codec.decompress(blob=host)
+    assert got.device == want.device and torch.equal(got, want)
