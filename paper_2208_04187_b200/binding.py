@@ -156,7 +156,8 @@ def div_plan_query(desc: DivDesc, flags: int = 0) -> DivPlan:
 def div_compress(desc: DivDesc, x_ptr: int, comp_ptr: int, comp_capacity: int, ws_ptr: int, ws_bytes: int,
                  seed: int, stream: int = 0, flags: int = 0) -> None:
     """Raw-pointer call (device pointers as integers, stream as a cudaStream_t handle)."""
-    st = (_lib or lib()).div_compress_ex(desc, x_ptr, comp_ptr, comp_capacity, ws_ptr, ws_bytes, seed & _U64, stream, flags)
+    st = (_lib or lib()).div_compress_ex(desc, x_ptr, comp_ptr, comp_capacity, ws_ptr, ws_bytes, seed & _U64, stream,
+                                        int(flags))
     if st:
         _check(st, "div_compress")
 
@@ -204,7 +205,7 @@ def div_planegroup_plan_query(desc: DivDesc, flags: int = 0) -> DivPlan:
 
 def div_planegroup_compress(desc: DivDesc, x_ptr: int, comp_ptr: int, comp_capacity: int, seed: int,
                             stream: int = 0, flags: int = 0) -> None:
-    st = (_lib or lib()).div_planegroup_compress(desc, x_ptr, comp_ptr, comp_capacity, seed & _U64, stream, flags)
+    st = (_lib or lib()).div_planegroup_compress(desc, x_ptr, comp_ptr, comp_capacity, seed & _U64, stream, int(flags))
     if st:
         _check(st, "div_planegroup_compress")
 

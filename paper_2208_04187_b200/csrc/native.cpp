@@ -52,7 +52,10 @@ PyObject* compress(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor *x, *blob, *ws = nullptr;
     if (!desc_arg(a[0], &d) || !tensor_arg(a[1], &x) || !tensor_arg(a[2], &blob) || (a[3] != Py_None && !tensor_arg(a[3], &ws))) return nullptr;
     const uint64_t seed = PyLong_AsUnsignedLongLongMask(a[4]);
-    const uint32_t flags = (uint32_t)PyLong_AsUnsignedLongMask(a[5]);
+    PyObject* whole = PyNumber_Long(a[5]);                 // whatever int() takes
+    if (!whole) return nullptr;
+    const uint32_t flags = (uint32_t)PyLong_AsUnsignedLongMask(whole);
+    Py_DECREF(whole);
     if (PyErr_Occurred()) return nullptr;
     if (!matches(*x, d)) return PyLong_FromLong(-1);
     const void* from = x->data_ptr();

@@ -4,6 +4,7 @@ import ctypes
 import os
 import re
 
+import numpy as np
 import pytest
 
 from oracle import division_oracle as orc
@@ -147,6 +148,17 @@ def test_null_and_misaligned_pointers_are_refused_before_any_launch():
     assert L.div_decompress(ctypes.byref(d), None, cap, 512, None) == binding.DIV_ERR_NULL
     assert L.div_decompress(ctypes.byref(d), 256, cap, 520, None) == binding.DIV_ERR_ALIGN
     assert L.div_decompress(ctypes.byref(d), 256, cap - 1, 512, None) == binding.DIV_ERR_CAPACITY
+
+
+@pytest.mark.parametrize("flags", [0x80, np.int64(0x80), np.uint8(0x80), 128.0, "128"])
+def test_flags_are_whatever_int_takes(flags):
+    """(0x80 is no flag: the library refuses it before it looks at the pointers.)"""
+    d = binding.make_desc(2, 3, 8, 8, 8, 2)
+    for call in (lambda: binding.div_compress(d, 256, 512, 1 << 20, 1024, 1 << 20, 0, 0, flags),
+                 lambda: binding.div_planegroup_compress(d, 256, 512, 1 << 20, 0, 0, flags)):
+        with pytest.raises(binding.DivisionError) as e:
+            call()
+        assert e.value.status == binding.DIV_ERR_PARAM
 
 
 def test_status_strings():
