@@ -44,6 +44,22 @@ __device__ __forceinline__ void st_async_u64(uint64_t* dst, uint64_t v, uint64_t
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(d), "l"(v), "r"(b) : "memory");
 }
 
+// a word that another CTA of the cluster sent is read behind this wait: acquire for the cluster (the plain form acquires for
+// the CTA alone)
+struct ClusterScope {
+    static __device__ __forceinline__ bool try_wait(uint64_t* bar) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar))
+            : "memory");
+        return ok != 0;
+    }
+};
+
 // ------------------------------------------------------------------------------------------------
 // half 2: the CTA's residuals, 4 consecutive elements per thread and step
 // ------------------------------------------------------------------------------------------------
@@ -183,7 +199,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
         const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, lane < THREADS / 32 ? wkey[1][lane] : 0u);
         if (lane < (1u << p.log2cs)) st_async_u64(&xch[rank], ((uint64_t)kmax << 32) | kmin, &xbar, lane);
     }
-    if (!__all_sync(0xFFFFFFFFu, share_wait(&xbar, p.timeout_ns))) {
+    if (!__all_sync(0xFFFFFFFFu, share_wait<ClusterScope>(&xbar, p.timeout_ns))) {
         if (tid == 0) {
             atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
             atomicCAS(p.ws + 1, 0u, n + 1u);

@@ -227,11 +227,15 @@ struct ShareParams {
     FastDiv by_sppf, by_spb, by_ppp;
     float inv[4], cnt[4], rcp[4];     // [short band][narrow tile]: 1 / count when that is a power of two, else 0; count; RN(1 / count)
 };
+struct CtaScope {
+    static __device__ __forceinline__ bool try_wait(uint64_t* bar) { return mbar_try_wait(bar, 0); }
+};
+template <typename Scope = CtaScope>
 __device__ __forceinline__ bool share_wait(uint64_t* bar, uint64_t timeout_ns) {
-    if (mbar_try_wait(bar, 0)) return true;
+    if (Scope::try_wait(bar)) return true;
     uint32_t polls = 0;
     uint64_t t0 = 0;
-    while (!mbar_try_wait(bar, 0)) {
+    while (!Scope::try_wait(bar)) {
         if ((++polls & 15u) == 0) {
             const uint64_t t = now_ns();
             if (t0 == 0) t0 = t;
