@@ -236,6 +236,18 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
                                       uint32_t flags, uint64_t timeout_ns);
 
 /*
+ * Test hook for what the kernels that keep x on chip (on_chip 1) do when something goes wrong: runs the kernel that
+ * div_compress_ex would run with flags 0, with `timeout_ns` (1 ns to 100 ms) as the limit of every wait, `fault` as below
+ * and 1 as the number of the call.  The status word is not cleared ahead of the kernel: what an earlier call recorded
+ * there (status, and in the word behind it the call's number) is cleared by the kernel itself, unless the number is that
+ * of the call.  DIV_ERR_PARAM where no such kernel takes the descriptor.  No counterpart in the paper.
+ */
+#define DIV_FAULT_NONE 0
+div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
+                             void* workspace_dev, size_t workspace_bytes, uint64_t seed, void* cuda_stream,
+                             int32_t fault, uint64_t timeout_ns);
+
+/*
  * Per-plane quantisation groups: the same pair of operations with one (delta, Delta) pair per
  * (sample, channel) plane, stored as two bfloat16 numbers.  This is the grouping behind the paper's count of
  * N^2*Q/8 + 4 bytes per channel for the high-frequency component (Sec. 4.1; proof of Theorem 3A), and

@@ -27,7 +27,7 @@ DTYPE_CODES = {"f32": DIV_F32, "bf16": DIV_BF16}
 
 EXPORTED_SYMBOLS = (
     "div_compressed_bytes", "div_compress", "div_compress_ex", "div_compress_static", "div_read_static_status",
-    "div_debug_compress_starved",
+    "div_debug_compress_starved", "div_debug_on_chip",
     "div_decompress", "div_plan_query",
     "div_compressed_bytes_3d", "div_compress_3d", "div_decompress_3d",
     "div_mask_bytes", "div_relu_forward", "div_dropout_forward", "div_mask_backward",
@@ -90,6 +90,8 @@ def lib() -> ctypes.CDLL:
         L.div_read_static_status.restype = c_int32
         L.div_debug_compress_starved.argtypes = L.div_compress_ex.argtypes + [c_uint64]
         L.div_debug_compress_starved.restype = c_int32
+        L.div_debug_on_chip.argtypes = L.div_compress.argtypes + [c_int32, c_uint64]
+        L.div_debug_on_chip.restype = c_int32
         L.div_decompress.argtypes = [ctypes.POINTER(DivDesc), c_void_p, c_size_t, c_void_p, c_void_p]
         L.div_decompress.restype = c_int32
         L.div_plan_query.argtypes = [ctypes.POINTER(DivDesc), c_uint32, ctypes.POINTER(DivPlan)]

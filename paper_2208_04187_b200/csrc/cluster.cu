@@ -13,6 +13,8 @@
 //     grid-wide co-residency: clusters that do not fit at once run one after the other.
 // Waits are bounded: when a limit runs out DIV_ERR_TIMEOUT is recorded in the workspace status word and the cluster
 // leaves together.
+#include <chrono>
+
 #include "cluster_plan.cuh"
 #include "halves.cuh"
 
@@ -171,16 +173,13 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
         fence_barrier_init();
         mbar_arrive_expect_tx(&xbar, p.expect_bytes);
         griddep_wait();
-        if (blockIdx.x == 0) {
-            p.ws[0] = 0u;
-            p.ws[1] = 0u;
-        }
         share_load(p, const_cast<XT*>(land), full, n, plane0, nplanes);
     }
     __syncthreads();
     griddep_wait();
     griddep_launch();
     cluster_arrive();                          // waited for below, before anything is sent to another CTA
+    if (blockIdx.x == 0 && tid == THREADS - 1) share_clear_status(p);
 
     float lo = 3.402823466e+38f, hi = -3.402823466e+38f;
     if (nplanes) share_half1<XT, P2, G, false, IN_PLACE, THREADS>(p, res, land, full, n, plane0, nplanes, nullptr, lo, hi);
@@ -200,10 +199,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
         if (lane < (1u << p.log2cs)) st_async_u64(&xch[rank], ((uint64_t)kmax << 32) | kmin, &xbar, lane);
     }
     if (!__all_sync(0xFFFFFFFFu, share_wait<ClusterScope>(&xbar, p.timeout_ns))) {
-        if (tid == 0) {
-            atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
-            atomicCAS(p.ws + 1, 0u, n + 1u);
-        }
+        if (tid == 0) share_record(p);
         __syncthreads();
         cluster_arrive();                      // nobody leaves while a word may still be on its way to it
         cluster_wait();
@@ -273,19 +269,22 @@ inline div_status launch_cluster_p2(const ClusterParams& prm, const ClusterPlan&
 }
 
 div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& pl, const void* x, uint8_t* blob,
-                            uint32_t* ws, uint64_t seed, cudaStream_t st, uint32_t expect_bytes, uint64_t timeout_ns) {
+                            uint32_t* ws, uint64_t seed, cudaStream_t st, const ShareFault& fault) {
     ClusterParams p;
     p.x = x;
     p.lfc = blob + lo.lfc_off;
     p.packed = blob + lo.packed_off;
     p.stats = reinterpret_cast<float*>(blob + lo.stats_off);
-    p.ws = ws;
+    p.status = reinterpret_cast<uint64_t*>(ws);
+    // a number that no earlier call on this workspace is likely to have had: 4 s of nanoseconds
+    const uint32_t number = fault.number ? fault.number : (uint32_t)std::chrono::steady_clock::now().time_since_epoch().count();
+    p.failure = ((uint64_t)number << 32) | (uint64_t)DIV_ERR_TIMEOUT;
     p.seed = seed;
-    p.timeout_ns = timeout_ns ? timeout_ns : 2000000000ull;
+    p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000ull;
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
     p.log2cs = 0;
     while ((1u << p.log2cs) < pl.cs) ++p.log2cs;
-    p.expect_bytes = expect_bytes ? expect_bytes : 8u * pl.cs;
+    p.expect_bytes = fault.expect_bytes ? fault.expect_bytes : 8u * pl.cs;
     p.qbits = d->qbits;
     return d->x_dtype == DIV_F32 ? launch_cluster_p2<float>(p, pl, s, st) : launch_cluster_p2<__nv_bfloat16>(p, pl, s, st);
 }

@@ -78,9 +78,14 @@ inline bool plan_cluster_cs(const div_desc* d, const Shape& s, uint32_t cs, cons
     return true;
 }
 
-// `expect_bytes`: what a CTA waits to receive (0: what its cluster sends; a test may ask for more than ever arrives)
+// What a test may ask of a call beyond the ordinary (zeros: nothing).
+struct ShareFault {
+    uint32_t expect_bytes;    // what a CTA waits to receive, more than ever arrives, instead of what its cluster sends
+    uint32_t number;          // the call's number (see ShareParams::failure)
+    uint64_t timeout_ns;      // limit of every wait
+};
 div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& pl, const void* x, uint8_t* blob,
-                            uint32_t* ws, uint64_t seed, cudaStream_t st, uint32_t expect_bytes = 0, uint64_t timeout_ns = 0);
+                            uint32_t* ws, uint64_t seed, cudaStream_t st, const ShareFault& fault = ShareFault());
 
 // per-plane groups (planeshare.cu)
 bool plan_plane_share(const div_desc* d, const Shape& s, SharePlan* out);

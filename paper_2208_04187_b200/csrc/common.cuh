@@ -14,7 +14,7 @@ namespace divk {
 // ---------------------------------------------------------------------------------------------
 // workspace layout (device scratch owned by the caller)
 //   word 0          : device status (0 = ok, 7 = a bounded wait ran out)
-//   word 1          : detail of the first failure (sample index)
+//   word 1          : detail of the first failure (sample index; of the cluster kernel the number of the call)
 //   words 16 + 32n.. : per-sample slot of 128 bytes (one cache line each, so that the slots of
 //                      neighbouring samples do not share an L2 line): { ~key(min), key(max), arrivals,
 //                      unused, 64-bit parameter word (general fused kernel), unused ... }

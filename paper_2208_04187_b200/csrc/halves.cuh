@@ -213,7 +213,8 @@ struct ShareParams {
     const void* x;
     void* lfc;
     void* packed;
-    uint32_t* ws;             // where a wait that ran out is recorded
+    uint64_t* status;         // where a wait that ran out is recorded (share_record)
+    uint64_t failure;         // what is recorded: DIV_ERR_TIMEOUT, above it the call's number
     uint64_t seed, timeout_ns;
     uint32_t C, W, B, Hb, Wb, HW, TPP, qps;
     uint32_t ppc, ppp;        // planes per CTA, planes per piece
@@ -227,6 +228,20 @@ struct ShareParams {
     FastDiv by_sppf, by_spb, by_ppp;
     float inv[4], cnt[4], rcp[4];     // [short band][narrow tile]: 1 / count when that is a power of two, else 0; count; RN(1 / count)
 };
+// The status words, as one 64-bit word: zero, or the failure of a call with the call's number.  One CTA clears what an earlier
+// call (or nobody) left there, in no order with the other CTAs of the launch, which may have failed already: it leaves
+// alone what carries the number of its own call.  (The replays of a captured call share its number: a failure that one of
+// them recorded stays.)
+__device__ __forceinline__ void share_record(const ShareParams& p) { atomicExch(reinterpret_cast<unsigned long long*>(p.status), p.failure); }
+__device__ __forceinline__ void share_clear_status(const ShareParams& p) {
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(p.status);
+    unsigned long long seen = ld_relaxed_u64(p.status);
+    while (seen != 0ull && seen != p.failure) {              // at most twice: from here on only p.failure is written
+        const unsigned long long old = atomicCAS(w, seen, 0ull);
+        if (old == seen) break;
+        seen = old;
+    }
+}
 struct CtaScope {
     static __device__ __forceinline__ bool try_wait(uint64_t* bar) { return mbar_try_wait(bar, 0); }
 };
@@ -307,7 +322,7 @@ __device__ __forceinline__ void share_half1(const ShareParams& p, float* res, co
             const uint32_t last = __shfl_sync(0xFFFFFFFFu, t.valid ? t.plane : nplanes - 1u, 31);
             const uint32_t need = fdiv(last, p.by_ppp) + 1u;
             while (landed < need) {
-                if (!share_wait(&full[landed], p.timeout_ns)) atomicCAS(p.ws, 0u, (uint32_t)DIV_ERR_TIMEOUT);
+                if (!share_wait(&full[landed], p.timeout_ns)) share_record(p);
                 ++landed;
             }
         }

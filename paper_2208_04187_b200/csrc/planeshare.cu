@@ -153,7 +153,8 @@ div_status compress_plane_share(const div_desc* d, const Shape& s, const div_lay
     p.lfc = blob + lo.lfc_off;
     p.packed = blob + lo.packed_off;
     p.stats = reinterpret_cast<uint32_t*>(blob + lo.stats_off);
-    p.ws = nullptr;
+    p.status = nullptr;
+    p.failure = 0;
     p.seed = seed;
     p.timeout_ns = ~0ull;             // the only wait is for the CTA's own copies
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);

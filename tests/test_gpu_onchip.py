@@ -111,6 +111,28 @@ def test_cluster_kernel_gives_up_a_wait_that_cannot_end():
     check(x_np, 8, 2, 5)
 
 
+def debug_call(codec, x, fault, timeout_ns):
+    return binding.lib().div_debug_on_chip(codec.desc, x.data_ptr(), codec.blob.data_ptr(), codec.blob.numel(), codec.workspace.data_ptr(),
+                                           codec.workspace.numel(), 5, binding.current_stream_handle(), fault, timeout_ns)
+
+
+def test_a_failure_of_the_same_call_is_not_cleared():
+    """The CTA that clears the status word runs in no order with the others, one of which may have failed before it: what
+    stands there under the call's own number (1) stays; a failure of another call goes."""
+    x_np = make((4, 32, 14, 14), "relu", 3, "f32")
+    x = torch.from_numpy(x_np).cuda()
+    codec = binding.Codec(*x_np.shape, 8, 2)
+    words = codec.workspace.view(torch.int32)
+    for status, number, want in ((binding.DIV_ERR_TIMEOUT, 1, binding.DIV_ERR_TIMEOUT), (binding.DIV_ERR_TIMEOUT, 2, binding.DIV_OK),
+                                 (-1, -1, binding.DIV_OK), (0, 0, binding.DIV_OK)):
+        words[0], words[1] = status, number
+        assert debug_call(codec, x, 0, 100_000_000) == binding.DIV_OK
+        torch.cuda.synchronize()
+        assert codec.device_status() == want
+        np.testing.assert_array_equal(codec.blob.cpu().numpy(), orc.compress(x_np, 8, 2, 5).blob())
+    assert debug_call(codec, x, 9, 100_000_000) == binding.DIV_ERR_PARAM
+
+
 PLANE_SHARE = [   # n, c, h, w, block, q, x, lfc: odd widths beyond a warp, blocks of 16, quads that straddle planes
     (2, 8, 75, 75, 8, 2, "f32", "f32"), (3, 12, 35, 35, 8, 4, "f32", "bf16"), (2, 5, 40, 40, 16, 4, "f32", "f32"),
     (2, 8, 39, 37, 4, 8, "bf16", "bf16"), (1, 44, 9, 41, 16, 2, "f32", "f32"), (2, 16, 17, 70, 12, 2, "bf16", "f32"),
