@@ -243,6 +243,8 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
  * of the call.  DIV_ERR_PARAM where no such kernel takes the descriptor.  No counterpart in the paper.
  */
 #define DIV_FAULT_NONE 0
+#define DIV_FAULT_COPIES 1   /* the waits for x never end: the kernel gives up, records DIV_ERR_TIMEOUT and returns; the blob's
+                                contents are then unspecified */
 div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
                              void* workspace_dev, size_t workspace_bytes, uint64_t seed, void* cuda_stream,
                              int32_t fault, uint64_t timeout_ns);

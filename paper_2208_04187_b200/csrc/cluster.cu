@@ -11,8 +11,9 @@
 //   * the sample's extremes meet in distributed shared memory: every CTA sends one 8-byte word to each CTA of the
 //     cluster, counted by an mbarrier there.  No scratch memory, hence nothing to clear before the launch, and no
 //     grid-wide co-residency: clusters that do not fit at once run one after the other.
-// Waits are bounded: when a limit runs out DIV_ERR_TIMEOUT is recorded in the workspace status word and the cluster
-// leaves together.
+// Waits are bounded.  A warp whose wait runs out records DIV_ERR_TIMEOUT in the workspace status word; if it waited for x its
+// CTA quantises nothing.  The CTA's word is sent all the same (nobody else has to wait for its limit), and no CTA
+// leaves before what is on its way to it has come or SHARE_DRAIN_NS have passed.
 #include <chrono>
 
 #include "cluster_plan.cuh"
@@ -162,6 +163,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
     __shared__ __align__(8) uint64_t xbar;
     __shared__ __align__(8) uint64_t xch[CL_MAX];
     __shared__ uint32_t wkey[2][THREADS / 32];
+    __shared__ uint32_t gave_up;              // a warp's wait for a piece ran out
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank(), n = blockIdx.x >> p.log2cs;
     const uint32_t plane0 = rank * p.ppc;
@@ -170,6 +172,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
 #pragma unroll
         for (uint32_t i = 0; i < SHARE_PIECES; ++i) mbar_init(&full[i], 1);
         mbar_init(&xbar, 1);
+        gave_up = 0u;
         fence_barrier_init();
         mbar_arrive_expect_tx(&xbar, p.expect_bytes);
         griddep_wait();
@@ -182,7 +185,7 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
     if (blockIdx.x == 0 && tid == THREADS - 1) share_clear_status(p);
 
     float lo = 3.402823466e+38f, hi = -3.402823466e+38f;
-    if (nplanes) share_half1<XT, P2, G, false, IN_PLACE, THREADS>(p, res, land, full, n, plane0, nplanes, nullptr, lo, hi);
+    if (nplanes) share_half1<XT, P2, G, false, IN_PLACE, THREADS>(p, res, land, full, n, plane0, nplanes, nullptr, &gave_up, lo, hi);
     {
         const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, ~float_key(lo));
         const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, float_key(hi));
@@ -198,11 +201,11 @@ cluster_kernel(const __grid_constant__ ClusterParams p) {
         const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, lane < THREADS / 32 ? wkey[1][lane] : 0u);
         if (lane < (1u << p.log2cs)) st_async_u64(&xch[rank], ((uint64_t)kmax << 32) | kmin, &xbar, lane);
     }
-    if (!__all_sync(0xFFFFFFFFu, share_wait<ClusterScope>(&xbar, p.timeout_ns))) {
-        if (tid == 0) share_record(p);
-        __syncthreads();
-        cluster_arrive();                      // nobody leaves while a word may still be on its way to it
-        cluster_wait();
+    const bool all_came = __all_sync(0xFFFFFFFFu, share_wait<ClusterScope>(&xbar, p.timeout_ns));
+    if (!all_came || gave_up) {                // gave_up: the same in the whole CTA, written before the barrier above
+        if (lane == 0) share_record(p);
+        if (!all_came) share_wait<ClusterScope>(&xbar, SHARE_DRAIN_NS);
+        if (warp == 0 && gave_up) share_drain(p, full, nplanes);
         return;
     }
     const uint64_t w = lane < (1u << p.log2cs) ? xch[lane] : 0ull;
@@ -268,6 +271,15 @@ inline div_status launch_cluster_p2(const ClusterParams& prm, const ClusterPlan&
     return DIV_ERR_PARAM;
 }
 
+// a number that the failed call before on this workspace is not likely to have had: the low bits of a clock
+static inline uint32_t call_number() {
+#if defined(__x86_64__)
+    return (uint32_t)__builtin_ia32_rdtsc();                   // (no call into the system)
+#else
+    return (uint32_t)std::chrono::steady_clock::now().time_since_epoch().count();
+#endif
+}
+
 div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& pl, const void* x, uint8_t* blob,
                             uint32_t* ws, uint64_t seed, cudaStream_t st, const ShareFault& fault) {
     ClusterParams p;
@@ -276,10 +288,10 @@ div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout&
     p.packed = blob + lo.packed_off;
     p.stats = reinterpret_cast<float*>(blob + lo.stats_off);
     p.status = reinterpret_cast<uint64_t*>(ws);
-    // a number that no earlier call on this workspace is likely to have had: 4 s of nanoseconds
-    const uint32_t number = fault.number ? fault.number : (uint32_t)std::chrono::steady_clock::now().time_since_epoch().count();
+    const uint32_t number = fault.number ? fault.number : call_number();
     p.failure = ((uint64_t)number << 32) | (uint64_t)DIV_ERR_TIMEOUT;
     p.seed = seed;
+    p.never_bytes = fault.never_bytes;
     p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000ull;
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
     p.log2cs = 0;

@@ -458,7 +458,7 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
     uint32_t* ws = (uint32_t*)workspace_dev;
     const uint32_t never = 0xFFFFFFFFu;      // an arrival count no sample reaches
     if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl))
-        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, timeout_ns});
+        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, timeout_ns});
     if (!(flags & DIV_FLAG_NO_STRIP_KERNEL)) {
         VPlan vp;
         if (plan_v(desc, s, &vp) == DIV_OK) return compress_fused_v(desc, s, lo, vp, x_dev, blob, ws, seed, stream, never, timeout_ns);
@@ -483,7 +483,7 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     if (!desc || !x_dev || !comp_dev || !workspace_dev) return DIV_ERR_NULL;
     const div_status st = check_desc(desc);
     if (st != DIV_OK) return st;
-    if (fault != DIV_FAULT_NONE || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
+    if (!(fault == DIV_FAULT_NONE || fault == DIV_FAULT_COPIES) || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
     if (!aligned16(x_dev) || !aligned16(comp_dev) || !aligned16(workspace_dev)) return DIV_ERR_ALIGN;
     const Shape s = make_shape(desc);
     div_layout lo;
@@ -491,6 +491,7 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     if (comp_capacity < lo.total_bytes || workspace_bytes < lo.workspace_bytes) return DIV_ERR_CAPACITY;
     ShareFault f = {};
     f.number = 1;
+    f.never_bytes = fault == DIV_FAULT_COPIES ? 16u : 0u;
     f.timeout_ns = timeout_ns;
     ClusterPlan cl;
     if (!choose_cluster(desc, s, 0u, &cl)) return DIV_ERR_PARAM;

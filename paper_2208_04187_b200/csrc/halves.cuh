@@ -216,6 +216,7 @@ struct ShareParams {
     uint64_t* status;         // where a wait that ran out is recorded (share_record)
     uint64_t failure;         // what is recorded: DIV_ERR_TIMEOUT, above it the call's number
     uint64_t seed, timeout_ns;
+    uint32_t never_bytes;     // a test has the waits for pieces wait for more than is copied (0)
     uint32_t C, W, B, Hb, Wb, HW, TPP, qps;
     uint32_t ppc, ppp;        // planes per CTA, planes per piece
     uint32_t res_bytes;       // bf16: where the landing place begins, behind the fp32 residuals
@@ -254,11 +255,13 @@ __device__ __forceinline__ bool share_wait(uint64_t* bar, uint64_t timeout_ns) {
         if ((++polls & 15u) == 0) {
             const uint64_t t = now_ns();
             if (t0 == 0) t0 = t;
-            if (t - t0 > timeout_ns) return false;
+            if (t - t0 > timeout_ns) return Scope::try_wait(bar);      // the clock may have jumped past the limit
         }
     }
     return true;
 }
+// what a CTA that gives up still waits for what is on its way into its shared memory, which is somebody else's once it has left
+constexpr uint64_t SHARE_DRAIN_NS = 20000000;
 
 // the copies of the share, one thread: piece i completes on full[i]
 template <typename XT>
@@ -266,9 +269,16 @@ __device__ __forceinline__ void share_load(const ShareParams& p, XT* land, uint6
     const XT* src = reinterpret_cast<const XT*>(p.x) + ((uint64_t)n * p.C + plane0) * p.HW;
     for (uint32_t i = 0, a = 0; a < nplanes; ++i, a += p.ppp) {
         const uint32_t bytes = min(p.ppp, nplanes - a) * p.HW * (uint32_t)sizeof(XT);
-        mbar_arrive_expect_tx(&full[i], bytes);
+        mbar_arrive_expect_tx(&full[i], bytes + p.never_bytes);
         bulk_load(land + (size_t)a * p.HW, src + (size_t)a * p.HW, bytes, &full[i]);
     }
+}
+// before a CTA leaves with a wait for a piece that ran out: one warp, until every piece has landed or the limit has passed
+__device__ __forceinline__ void share_drain(const ShareParams& p, uint64_t* full, uint32_t nplanes) {
+    const uint64_t t0 = now_ns();
+    for (uint32_t i = 0, a = 0; a < nplanes; ++i, a += p.ppp)
+        while (!mbar_try_wait(&full[i], 0))
+            if (now_ns() - t0 > SHARE_DRAIN_NS) return;
 }
 
 // Slots of the CTA's share are numbered so that every warp holds slots of one height: the full-height bands of all planes
@@ -308,9 +318,11 @@ __device__ __forceinline__ ShareSlot share_slot(const ShareParams& p, uint32_t f
 // ------------------------------------------------------------------------------------------------
 // IN_PLACE: x stays as it is and res takes the stored low-frequency values of the tiles instead of the residuals.
 // keys (PER_PLANE): ~key(min), key(max) of the residuals of each plane; else lo / hi collect the extremes of the thread.
+// A wait for a piece that runs out is noted in *gave_up, in shared memory; the warp then works on with whatever is there and waits for
+// no further piece (a way out of the loop costs the ordinary case 1 %), and the caller lets nothing of it out.
 template <typename XT, int P2, typename G, bool PER_PLANE, bool IN_PLACE, uint32_t THREADS>
 __device__ __forceinline__ void share_half1(const ShareParams& p, float* res, const XT* land, uint64_t* full, uint32_t n, uint32_t plane0,
-                                         uint32_t nplanes, uint32_t* keys, float& lo, float& hi) {
+                                         uint32_t nplanes, uint32_t* keys, uint32_t* gave_up, float& lo, float& hi) {
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nfull = nplanes * p.sppf, first_short = (nfull + 31u) & ~31u, total = first_short + nplanes * p.sppt;
     const uint64_t lfc0 = ((uint64_t)n * p.C + plane0) * p.TPP;
@@ -322,7 +334,10 @@ __device__ __forceinline__ void share_half1(const ShareParams& p, float* res, co
             const uint32_t last = __shfl_sync(0xFFFFFFFFu, t.valid ? t.plane : nplanes - 1u, 31);
             const uint32_t need = fdiv(last, p.by_ppp) + 1u;
             while (landed < need) {
-                if (!share_wait(&full[landed], p.timeout_ns)) share_record(p);
+                if (!share_wait(&full[landed], p.timeout_ns)) {
+                    *gave_up = 1u;
+                    landed = SHARE_PIECES - 1u;
+                }
                 ++landed;
             }
         }

@@ -26,6 +26,7 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
     float4* par = reinterpret_cast<float4*>(smem + p.res_bytes + land_bytes);      // per plane: delta_b, 1 / Delta_b, -65536 / Delta_b (0: general route)
     uint32_t* keys = reinterpret_cast<uint32_t*>(par + p.ppc);
     __shared__ __align__(8) uint64_t full[SHARE_PIECES];
+    __shared__ uint32_t gave_up;              // (no limit here)
     const uint32_t tid = threadIdx.x;
     const uint32_t n = blockIdx.y, plane0 = blockIdx.x * p.ppc;
     const uint32_t nplanes = min(p.ppc, p.C - plane0);
@@ -41,7 +42,7 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
     griddep_wait();
     griddep_launch();
     float lo, hi;
-    share_half1<XT, P2, G, true, false, SHARE_THREADS>(p, res, land, full, n, plane0, nplanes, keys, lo, hi);
+    share_half1<XT, P2, G, true, false, SHARE_THREADS>(p, res, land, full, n, plane0, nplanes, keys, &gave_up, lo, hi);
     __syncthreads();
     for (uint32_t i = tid; i < nplanes; i += SHARE_THREADS) {
         const float rmax = key_float(keys[2u * i + 1u]);
@@ -155,6 +156,7 @@ div_status compress_plane_share(const div_desc* d, const Shape& s, const div_lay
     p.stats = reinterpret_cast<uint32_t*>(blob + lo.stats_off);
     p.status = nullptr;
     p.failure = 0;
+    p.never_bytes = 0;
     p.seed = seed;
     p.timeout_ns = ~0ull;             // the only wait is for the CTA's own copies
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);

@@ -133,6 +133,29 @@ def test_a_failure_of_the_same_call_is_not_cleared():
     assert debug_call(codec, x, 9, 100_000_000) == binding.DIV_ERR_PARAM
 
 
+@pytest.mark.parametrize("case", [(4, 32, 14, 14, "f32"), (3, 24, 75, 75, "f32"), (4, 32, 32, 32, "bf16"), (40, 64, 75, 75, "f32")],
+                         ids=lambda c: "x".join(map(str, c)))
+@pytest.mark.parametrize("timeout_ns", [1, 1_000_000])
+def test_a_wait_for_x_that_cannot_end(case, timeout_ns):
+    """Every warp gives up on its first piece (or, with a limit of 1 ns, some of them on the exchange): the failure is
+    recorded, nothing behind the blob is written, and the next call on the same buffers is an ordinary one.  The last
+    case takes several turns."""
+    n, c, h, w, xd = case
+    x = torch.randn((n, c, h, w), device="cuda").to(binding.torch_dtype(xd))
+    codec = binding.Codec(n, c, h, w, 8, 2, xd, "f32")
+    assert codec.plan().on_chip == 1
+    room = torch.full((codec.blob.numel() + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    whole, codec.blob = codec.blob, room[:codec.blob.numel()]
+    codec.compress(x, seed=5)
+    want = codec.blob.clone()
+    assert debug_call(codec, x, 1, timeout_ns) == binding.DIV_OK
+    torch.cuda.synchronize()
+    assert codec.device_status() == binding.DIV_ERR_TIMEOUT
+    assert bool((room[whole.numel():] == 0xA5).all())
+    codec.compress(x, seed=5)
+    assert codec.device_status() == binding.DIV_OK and torch.equal(codec.blob, want)
+
+
 PLANE_SHARE = [   # n, c, h, w, block, q, x, lfc: odd widths beyond a warp, blocks of 16, quads that straddle planes
     (2, 8, 75, 75, 8, 2, "f32", "f32"), (3, 12, 35, 35, 8, 4, "f32", "bf16"), (2, 5, 40, 40, 16, 4, "f32", "f32"),
     (2, 8, 39, 37, 4, 8, "bf16", "bf16"), (1, 44, 9, 41, 16, 2, "f32", "f32"), (2, 16, 17, 70, 12, 2, "bf16", "f32"),
