@@ -237,14 +237,15 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
 
 /*
  * Test hook for what the kernels that keep x on chip (on_chip 1) do when something goes wrong: runs the kernel that
- * div_compress_ex would run with flags 0, with `timeout_ns` (1 ns to 100 ms) as the limit of every wait, `fault` as below
- * and 1 as the number of the call.  The status word is not cleared ahead of the kernel: what an earlier call recorded
- * there (status, and in the word behind it the call's number) is cleared by the kernel itself, unless the number is that
- * of the call.  DIV_ERR_PARAM where no such kernel takes the descriptor.  No counterpart in the paper.
+ * div_compress_ex (workspace_dev NULL: div_planegroup_compress) would run with flags 0, with `timeout_ns` (1 ns to
+ * 100 ms) as the limit of every wait, `fault` as below and 1 as the number of the call.  The status word is not cleared
+ * ahead of the kernel: what an earlier call recorded there (status, and in the word behind it the call's number) is
+ * cleared by the kernel itself, unless the number is that of the call.  DIV_ERR_PARAM where no such kernel takes the
+ * descriptor.  No counterpart in the paper.
  */
 #define DIV_FAULT_NONE 0
-#define DIV_FAULT_COPIES 1   /* the waits for x never end: the kernel gives up, records DIV_ERR_TIMEOUT and returns; the blob's
-                                contents are then unspecified */
+#define DIV_FAULT_COPIES 1   /* the waits for x never end: the kernel gives up, records DIV_ERR_TIMEOUT (per-plane groups: NaN as
+                                the parameters of its planes) and returns; the rest of the blob is then unspecified */
 div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
                              void* workspace_dev, size_t workspace_bytes, uint64_t seed, void* cuda_stream,
                              int32_t fault, uint64_t timeout_ns);
@@ -260,7 +261,8 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
  *     Delta_b = smallest bfloat16 number >= (max H^H - delta_b)/(2^Q - 1); both sides use the stored pair:
  *     t = (H^H - delta_b) * (1/Delta_b), H^H_hat = Delta_b * V^H + delta_b.  A plane whose Delta_b or
  *     1/Delta_b would be zero or not finite stores Delta_b = 0 and all codes 0;
- *   - a plane's extremes stay inside one CTA, so compress needs no scratch and no device-side waiting;
+ *   - a plane's extremes stay inside one CTA, so compress needs no scratch and no CTA waits for another.  A kernel that
+ *     waits for its own copies of x longer than 2 s gives up: its planes get NaN for both parameters and rebuild as NaN;
  *   - n*c < 2^31 (else DIV_ERR_SHAPE).
  * Everything else (pooling grid, residual against the stored value, stochastic rounding, random stream,
  * packing order, argument meaning, ownership, error codes) is as documented above.

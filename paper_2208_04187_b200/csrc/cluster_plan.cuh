@@ -91,6 +91,6 @@ div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout&
 // per-plane groups (planeshare.cu)
 bool plan_plane_share(const div_desc* d, const Shape& s, SharePlan* out);
 div_status compress_plane_share(const div_desc* d, const Shape& s, const div_layout& lo, const SharePlan& pl, const void* x, uint8_t* blob,
-                                uint64_t seed, cudaStream_t st);
+                                uint64_t seed, cudaStream_t st, const ShareFault& fault = ShareFault());
 
 }  // namespace divk

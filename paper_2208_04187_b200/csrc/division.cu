@@ -480,19 +480,27 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
 
 div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity, void* workspace_dev,
                              size_t workspace_bytes, uint64_t seed, void* cuda_stream, int32_t fault, uint64_t timeout_ns) {
-    if (!desc || !x_dev || !comp_dev || !workspace_dev) return DIV_ERR_NULL;
+    if (!desc || !x_dev || !comp_dev) return DIV_ERR_NULL;
     const div_status st = check_desc(desc);
     if (st != DIV_OK) return st;
     if (!(fault == DIV_FAULT_NONE || fault == DIV_FAULT_COPIES) || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
     if (!aligned16(x_dev) || !aligned16(comp_dev) || !aligned16(workspace_dev)) return DIV_ERR_ALIGN;
     const Shape s = make_shape(desc);
+    const bool planes = workspace_dev == nullptr;
+    if (planes && !pg_shape_ok(s)) return DIV_ERR_SHAPE;
     div_layout lo;
-    make_layout(desc, s, &lo);
+    if (planes) make_layout_pg(desc, s, &lo);
+    else make_layout(desc, s, &lo);
     if (comp_capacity < lo.total_bytes || workspace_bytes < lo.workspace_bytes) return DIV_ERR_CAPACITY;
     ShareFault f = {};
     f.number = 1;
-    f.never_bytes = fault == DIV_FAULT_COPIES ? 16u : 0u;
     f.timeout_ns = timeout_ns;
+    f.never_bytes = fault == DIV_FAULT_COPIES ? 16u : 0u;
+    if (planes) {
+        SharePlan ps;
+        if (!plan_plane_share(desc, s, &ps)) return DIV_ERR_PARAM;
+        return compress_plane_share(desc, s, lo, ps, x_dev, (uint8_t*)comp_dev, seed, (cudaStream_t)cuda_stream, f);
+    }
     ClusterPlan cl;
     if (!choose_cluster(desc, s, 0u, &cl)) return DIV_ERR_PARAM;
     return compress_cluster(desc, s, lo, cl, x_dev, (uint8_t*)comp_dev, (uint32_t*)workspace_dev, seed, (cudaStream_t)cuda_stream, f);

@@ -5,6 +5,10 @@
 // shapes that the register-resident strip kernel cannot: odd widths beyond a warp and blocks of 16, where the general kernel
 // (a thread per tile, then per packed word) is bound by scalar uncoalesced loads: 50 x 256 x 40 x 40 with B = 16 515 -> 37 us,
 // 64 x 96 x 35 x 35 106 -> 21 us, 32 x 64 x 75 x 75 88 -> 29 us.
+//
+// The only wait is for the CTA's own copies.  It is bounded all the same; there is no status word to record it in, so a CTA that
+// gives up stores NaN as the parameters of its planes (which rebuild as NaN), and leaves when the copies have landed or
+// SHARE_DRAIN_NS have passed.
 #include "halves.cuh"
 #include "planegroup.cuh"
 
@@ -26,13 +30,14 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
     float4* par = reinterpret_cast<float4*>(smem + p.res_bytes + land_bytes);      // per plane: delta_b, 1 / Delta_b, -65536 / Delta_b (0: general route)
     uint32_t* keys = reinterpret_cast<uint32_t*>(par + p.ppc);
     __shared__ __align__(8) uint64_t full[SHARE_PIECES];
-    __shared__ uint32_t gave_up;              // (no limit here)
+    __shared__ uint32_t gave_up;              // a warp's wait for a piece ran out
     const uint32_t tid = threadIdx.x;
     const uint32_t n = blockIdx.y, plane0 = blockIdx.x * p.ppc;
     const uint32_t nplanes = min(p.ppc, p.C - plane0);
     if (tid == 0) {
 #pragma unroll
         for (uint32_t i = 0; i < SHARE_PIECES; ++i) mbar_init(&full[i], 1);
+        gave_up = 0u;
         fence_barrier_init();
         griddep_wait();
         share_load(p, land, full, n, plane0, nplanes);
@@ -44,6 +49,11 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
     float lo, hi;
     share_half1<XT, P2, G, true, false, SHARE_THREADS>(p, res, land, full, n, plane0, nplanes, keys, &gave_up, lo, hi);
     __syncthreads();
+    if (gave_up) {                            // the same in the whole CTA
+        for (uint32_t i = tid; i < nplanes; i += SHARE_THREADS) p.stats[(uint64_t)n * p.C + plane0 + i] = 0x7FC07FC0u;
+        if (tid < 32u) share_drain(p, full, nplanes);
+        return;
+    }
     for (uint32_t i = tid; i < nplanes; i += SHARE_THREADS) {
         const float rmax = key_float(keys[2u * i + 1u]);
         const PgQ q = pg_params(key_float(~keys[2u * i]), rmax, Q);
@@ -148,7 +158,7 @@ inline div_status launch_plane_share_p2(uint32_t p2, int qbits, const PlaneShare
 }
 
 div_status compress_plane_share(const div_desc* d, const Shape& s, const div_layout& lo, const SharePlan& pl, const void* x, uint8_t* blob,
-                                uint64_t seed, cudaStream_t st) {
+                                uint64_t seed, cudaStream_t st, const ShareFault& fault) {
     PlaneShareParams p;
     p.x = x;
     p.lfc = blob + lo.lfc_off;
@@ -156,9 +166,9 @@ div_status compress_plane_share(const div_desc* d, const Shape& s, const div_lay
     p.stats = reinterpret_cast<uint32_t*>(blob + lo.stats_off);
     p.status = nullptr;
     p.failure = 0;
-    p.never_bytes = 0;
+    p.never_bytes = fault.never_bytes;
     p.seed = seed;
-    p.timeout_ns = ~0ull;             // the only wait is for the CTA's own copies
+    p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000ull;
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
     p.by_hw = host_fastdiv(s.HW);
     return d->x_dtype == DIV_F32 ? launch_plane_share_p2<float>(s.P2, d->qbits, p, pl, s.N, st)

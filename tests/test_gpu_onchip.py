@@ -175,3 +175,25 @@ def test_plane_share_kernel_matches_the_checker(case):
     t = torch.from_numpy(x_np)
     codec.compress((t.view(torch.bfloat16) if xd == "bf16" else t).cuda(), seed=13)
     np.testing.assert_array_equal(codec.blob.cpu().numpy(), orc.compress_planes(x_np, block, q, 13, xd, ld).blob())
+
+
+@pytest.mark.parametrize("case", [(3, 12, 35, 35, "f32"), (40, 64, 39, 75, "bf16")], ids=lambda c: "x".join(map(str, c)))
+@pytest.mark.parametrize("timeout_ns", [1, 1_000_000])
+def test_plane_share_kernel_gives_up_a_wait_that_cannot_end(case, timeout_ns):
+    """The planes rebuild as NaN, nothing behind the blob is written, and the next call on the same buffers is an ordinary one."""
+    n, c, h, w, xd = case
+    x = torch.randn((n, c, h, w), device="cuda").to(binding.torch_dtype(xd))
+    codec = binding.PlaneGroupCodec(n, c, h, w, 8, 2, xd, "f32")
+    assert codec.plan().on_chip == 1
+    size = codec.blob.numel()
+    room = torch.full((size + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    codec.blob = room[:size]
+    codec.compress(x, seed=5)
+    want = codec.blob.clone()
+    st = binding.lib().div_debug_on_chip(codec.desc, x.data_ptr(), codec.blob.data_ptr(), size, None, 0, 5, binding.current_stream_handle(), 1, timeout_ns)
+    assert st == binding.DIV_OK
+    torch.cuda.synchronize()
+    assert bool(torch.isnan(codec.decompress()).all())
+    assert bool((room[size:] == 0xA5).all())
+    codec.compress(x, seed=5)
+    assert torch.equal(codec.blob, want)

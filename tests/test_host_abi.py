@@ -150,6 +150,20 @@ def test_null_and_misaligned_pointers_are_refused_before_any_launch():
     assert L.div_decompress(ctypes.byref(d), 256, cap - 1, 512, None) == binding.DIV_ERR_CAPACITY
 
 
+def test_the_on_chip_test_hook_checks_its_arguments():
+    L = binding.lib()
+    d = binding.make_desc(2, 3, 8, 8, 8, 2)
+    cap = ws = 1 << 20
+    call = lambda *a: L.div_debug_on_chip(ctypes.byref(d), *a)  # noqa: E731
+    assert call(None, 256, cap, 512, ws, 0, None, 0, 1) == binding.DIV_ERR_NULL
+    assert call(256, 512, cap, 1024, ws, 0, None, 7, 1) == binding.DIV_ERR_PARAM
+    assert call(256, 512, cap, 1024, ws, 0, None, 0, 0) == binding.DIV_ERR_PARAM
+    assert call(256, 512, cap, 1024, ws, 0, None, 0, 100_000_001) == binding.DIV_ERR_PARAM
+    assert call(256, 512, cap, 1028, ws, 0, None, 0, 1) == binding.DIV_ERR_ALIGN
+    assert call(256, 512, cap, 1024, 64, 0, None, 0, 1) == binding.DIV_ERR_CAPACITY
+    assert call(256, 512, 64, None, 0, 0, None, 0, 1) == binding.DIV_ERR_CAPACITY
+
+
 @pytest.mark.parametrize("flags", [0x80, np.int64(0x80), np.uint8(0x80), 128.0, "128"])
 def test_flags_are_whatever_int_takes(flags):
     """(0x80 is no flag: the library refuses it before it looks at the pointers.)"""
