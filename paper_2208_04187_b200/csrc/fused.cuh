@@ -485,33 +485,35 @@ inline DeviceInfo device_info() {
     return di;
 }
 
-// cudaFuncAttributeMaxDynamicSharedMemorySize of one kernel: set once per device and size, not once per launch.
-// `seen` is the per-kernel table of what has been set on each device; an entry also names the kernel it is
-// about, so that a table shared by accident (two copies of the library in one process) is never trusted for
-// another copy's kernel.
+// cudaFuncAttributeMaxDynamicSharedMemorySize of one kernel: set once per device, to all that the device has beside the
+// kernel's static share.  (Not to the size at hand: threads that launch different sizes would set different values, and the
+// one that sets the smaller value last would have the larger size refused.)  `seen` is the per-kernel table of what has
+// been set on each device; an entry also names the kernel it is about, so that a table shared by accident (two copies of
+// the library in one process) is never trusted for another copy's kernel.
 struct SmemSeen {
     std::atomic<const void*> fn;
     std::atomic<int> bytes;
 };
 inline bool ensure_dynamic_smem(const void* kern, int bytes, SmemSeen* seen) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
+    const DeviceInfo di = device_info();
+    if (!di.ok) return false;
+    const bool slot = di.dev >= 0 && di.dev < DEVICE_CACHE_SLOTS;
+    if (slot && seen[di.dev].fn.load(std::memory_order_acquire) == kern) return bytes <= seen[di.dev].bytes.load(std::memory_order_acquire);
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, kern) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    const bool slot = dev >= 0 && dev < DEVICE_CACHE_SLOTS;
-    if (slot && seen[dev].fn.load(std::memory_order_acquire) == kern && seen[dev].bytes.load(std::memory_order_acquire) >= bytes)
-        return true;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+    const int all = di.smem_optin - (int)a.sharedSizeBytes;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, all) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     if (slot) {
-        seen[dev].fn.store(nullptr, std::memory_order_release);
-        seen[dev].bytes.store(bytes, std::memory_order_release);
-        seen[dev].fn.store(kern, std::memory_order_release);
+        seen[di.dev].bytes.store(all, std::memory_order_release);
+        seen[di.dev].fn.store(kern, std::memory_order_release);
     }
-    return true;
+    return bytes <= all;
 }
 
 // Programmatic dependent launch: a kernel launched this way may start while the kernel before it in the stream is still
