@@ -246,6 +246,7 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
 #define DIV_FAULT_NONE 0
 #define DIV_FAULT_COPIES 1   /* the waits for x never end: the kernel gives up, records DIV_ERR_TIMEOUT (per-plane groups: NaN as
                                 the parameters of its planes) and returns; the rest of the blob is then unspecified */
+#define DIV_FAULT_REFUSED 2  /* the launch asks for more shared memory than the device has: the next kernel in line runs */
 div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
                              void* workspace_dev, size_t workspace_bytes, uint64_t seed, void* cuda_stream,
                              int32_t fault, uint64_t timeout_ns);

@@ -280,8 +280,10 @@ static inline uint32_t call_number() {
 #endif
 }
 
-div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& pl, const void* x, uint8_t* blob,
+div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& plan, const void* x, uint8_t* blob,
                             uint32_t* ws, uint64_t seed, cudaStream_t st, const ShareFault& fault) {
+    ClusterPlan pl = plan;
+    pl.smem_bytes += fault.more_smem;
     ClusterParams p;
     p.x = x;
     p.lfc = blob + lo.lfc_off;

@@ -297,6 +297,76 @@ bool decompress_rows_ok(const Shape& s) {
            rows_bands(s, 1024u * FLAT_QPT) * s.W * 4u <= 40000u;
 }
 
+// the launches of div_compress_ex, whose arguments have been checked
+div_status compress_map(const div_desc* desc, const Shape& s, const div_layout& lo, const void* x_dev, uint8_t* blob, uint32_t* ws,
+                        uint64_t seed, cudaStream_t stream, uint32_t flags, const ShareFault& fault) {
+    // kernels that store bytes or half-words leave the unused top of a partial last word alone: it is zero by contract
+    if ((s.total * (uint64_t)desc->qbits) % 32u != 0 &&
+        cudaMemsetAsync(blob + lo.packed_off + lo.packed_bytes - 4, 0, 4, stream) != cudaSuccess)
+        return DIV_ERR_CUDA;
+    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl) && compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, fault) == DIV_OK)
+        return DIV_OK;
+    if (clear_scratch(ws, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
+    // The single-launch kernels need all their CTAs resident, so they are launched cooperatively; where the
+    // device refuses such a launch (fewer SMs visible to the process than the device reports, for instance) the
+    // next kernel in line takes the descriptor: nothing has been enqueued by the refused launch.
+    for (uint32_t f = flags;;) {
+        Choice ch;
+        choose_compress(desc, s, f, &ch);
+        div_status r = DIV_OK;
+        uint32_t drop = 0;
+        switch (ch.code) {
+            case 8: return compress_lines(desc, s, lo, ch.lg, x_dev, blob, ws, seed, stream, true);
+            case 5: return compress_lines(desc, s, lo, ch.lg, x_dev, blob, ws, seed, stream, false);
+            case 6: r = compress_staged(desc, s, lo, ch.sp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_NO_STAGED_KERNEL; break;
+            case 3: r = compress_lagged(desc, s, lo, ch.lp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_NO_LAGGED_KERNEL; break;
+            case 2: r = compress_fused_v(desc, s, lo, ch.vp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_NO_STRIP_KERNEL; break;
+            case 7: return compress_planes(desc, s, lo, ch.pg, x_dev, blob, ws, seed, stream, true);
+            case 4: return compress_planes(desc, s, lo, ch.pg, x_dev, blob, ws, seed, stream, false);
+            case 1: r = compress_fused(desc, s, lo, ch.fp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_FORCE_TWO_PASS; break;
+            default: return compress_two_pass(desc, s, lo, x_dev, blob, ws, seed, stream);
+        }
+        if (r != DIV_ERR_CUDA) return r;
+        f |= drop;
+    }
+    return compress_two_pass(desc, s, lo, x_dev, blob, ws, seed, stream);
+}
+
+// the same for div_planegroup_compress
+div_status compress_planegroup(const div_desc* desc, const Shape& s, const div_layout& lo, const void* x_dev, uint8_t* blob, uint64_t seed,
+                               cudaStream_t stream, uint32_t flags, const ShareFault& fault) {
+    // kernels that store bytes or half-words leave the unused top of a partial last word alone: it is zero by contract
+    if ((s.total * (uint64_t)desc->qbits) % 32u != 0 &&
+        cudaMemsetAsync(blob + lo.packed_off + lo.packed_bytes - 4, 0, 4, stream) != cudaSuccess)
+        return DIV_ERR_CUDA;
+    PgPlan pl;
+    if (!(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_pg_strip(desc, s, &pl))
+        return compress_pg_strip(desc, s, lo, pl, x_dev, blob, seed, stream);
+    if (PgSmall g; !(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_pg_small(desc, s, &g))
+        return compress_pg_small(desc, s, lo, g, x_dev, blob, seed, stream);
+    // Everything else that fits shared memory.  (Where the two kernels above apply they are faster or as good: 64 x 256 x 56 x 56 53
+    // against 70 us, 64 x 2048 x 7 x 7 18.6 against 20.0 us, 64 x 1024 x 14 x 14 30.8 against 28.8 us.)
+    // Where the launch is refused the general kernel takes the map.
+    if (SharePlan ps; !(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_plane_share(desc, s, &ps) &&
+                      compress_plane_share(desc, s, lo, ps, x_dev, blob, seed, stream, fault) == DIV_OK)
+        return DIV_OK;
+    // general kernel: words shared by two planes (and the zero-padded last word) are merged with atomic ORs
+    // into a cleared buffer
+    if (((uint64_t)s.HW * (uint64_t)desc->qbits) % 32u != 0 &&
+        cudaMemsetAsync(blob + lo.packed_off, 0, lo.packed_bytes, stream) != cudaSuccess)
+        return DIV_ERR_CUDA;
+    return dispatch_types(desc->x_dtype, desc->lfc_dtype, [&](auto* xt, auto* lt) -> div_status {
+        typedef std::remove_pointer_t<decltype(xt)> XT;
+        typedef std::remove_pointer_t<decltype(lt)> LT;
+        return dispatch_q(desc->qbits, [&](auto q) -> div_status {
+            pg_general_kernel<XT, LT, decltype(q)::value><<<s.N * s.C, 256, 0, stream>>>(
+                (const XT*)x_dev, (LT*)(blob + lo.lfc_off), (uint32_t*)(blob + lo.packed_off),
+                (uint32_t*)(blob + lo.stats_off), s, seed);
+            return launch_status();
+        });
+    });
+}
+
 }  // namespace
 
 extern "C" {
@@ -408,36 +478,7 @@ div_status div_compress_ex(const div_desc* desc, const void* x_dev, void* comp_d
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     uint8_t* blob = (uint8_t*)comp_dev;
     uint32_t* ws = (uint32_t*)workspace_dev;
-    // kernels that store bytes or half-words leave the unused top of a partial last word alone: it is zero by contract
-    if ((s.total * (uint64_t)desc->qbits) % 32u != 0 &&
-        cudaMemsetAsync(blob + lo.packed_off + lo.packed_bytes - 4, 0, 4, stream) != cudaSuccess)
-        return DIV_ERR_CUDA;
-    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl) && compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream) == DIV_OK)
-        return DIV_OK;
-    if (clear_scratch(workspace_dev, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
-    // The single-launch kernels need all their CTAs resident, so they are launched cooperatively; where the
-    // device refuses such a launch (fewer SMs visible to the process than the device reports, for instance) the
-    // next kernel in line takes the descriptor: nothing has been enqueued by the refused launch.
-    for (uint32_t f = flags;;) {
-        Choice ch;
-        choose_compress(desc, s, f, &ch);
-        div_status r = DIV_OK;
-        uint32_t drop = 0;
-        switch (ch.code) {
-            case 8: return compress_lines(desc, s, lo, ch.lg, x_dev, blob, ws, seed, stream, true);
-            case 5: return compress_lines(desc, s, lo, ch.lg, x_dev, blob, ws, seed, stream, false);
-            case 6: r = compress_staged(desc, s, lo, ch.sp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_NO_STAGED_KERNEL; break;
-            case 3: r = compress_lagged(desc, s, lo, ch.lp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_NO_LAGGED_KERNEL; break;
-            case 2: r = compress_fused_v(desc, s, lo, ch.vp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_NO_STRIP_KERNEL; break;
-            case 7: return compress_planes(desc, s, lo, ch.pg, x_dev, blob, ws, seed, stream, true);
-            case 4: return compress_planes(desc, s, lo, ch.pg, x_dev, blob, ws, seed, stream, false);
-            case 1: r = compress_fused(desc, s, lo, ch.fp, x_dev, blob, ws, seed, stream); drop = DIV_FLAG_FORCE_TWO_PASS; break;
-            default: return compress_two_pass(desc, s, lo, x_dev, blob, ws, seed, stream);
-        }
-        if (r != DIV_ERR_CUDA) return r;
-        f |= drop;
-    }
-    return compress_two_pass(desc, s, lo, x_dev, blob, ws, seed, stream);
+    return compress_map(desc, s, lo, x_dev, blob, ws, seed, stream, flags, ShareFault());
 }
 
 div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
@@ -458,7 +499,7 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
     uint32_t* ws = (uint32_t*)workspace_dev;
     const uint32_t never = 0xFFFFFFFFu;      // an arrival count no sample reaches
     if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl))
-        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, timeout_ns});
+        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, 0u, timeout_ns});
     if (!(flags & DIV_FLAG_NO_STRIP_KERNEL)) {
         VPlan vp;
         if (plan_v(desc, s, &vp) == DIV_OK) return compress_fused_v(desc, s, lo, vp, x_dev, blob, ws, seed, stream, never, timeout_ns);
@@ -483,7 +524,7 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     if (!desc || !x_dev || !comp_dev) return DIV_ERR_NULL;
     const div_status st = check_desc(desc);
     if (st != DIV_OK) return st;
-    if (!(fault == DIV_FAULT_NONE || fault == DIV_FAULT_COPIES) || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
+    if (fault < DIV_FAULT_NONE || fault > DIV_FAULT_REFUSED || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
     if (!aligned16(x_dev) || !aligned16(comp_dev) || !aligned16(workspace_dev)) return DIV_ERR_ALIGN;
     const Shape s = make_shape(desc);
     const bool planes = workspace_dev == nullptr;
@@ -496,14 +537,16 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     f.number = 1;
     f.timeout_ns = timeout_ns;
     f.never_bytes = fault == DIV_FAULT_COPIES ? 16u : 0u;
+    f.more_smem = fault == DIV_FAULT_REFUSED ? 1u << 20 : 0u;
+    const cudaStream_t stream = (cudaStream_t)cuda_stream;
     if (planes) {
-        SharePlan ps;
-        if (!plan_plane_share(desc, s, &ps)) return DIV_ERR_PARAM;
-        return compress_plane_share(desc, s, lo, ps, x_dev, (uint8_t*)comp_dev, seed, (cudaStream_t)cuda_stream, f);
+        div_plan plan;
+        if (div_planegroup_plan_query(desc, 0u, &plan) != DIV_OK || !plan.on_chip) return DIV_ERR_PARAM;
+        return compress_planegroup(desc, s, lo, x_dev, (uint8_t*)comp_dev, seed, stream, 0u, f);
     }
     ClusterPlan cl;
     if (!choose_cluster(desc, s, 0u, &cl)) return DIV_ERR_PARAM;
-    return compress_cluster(desc, s, lo, cl, x_dev, (uint8_t*)comp_dev, (uint32_t*)workspace_dev, seed, (cudaStream_t)cuda_stream, f);
+    return compress_map(desc, s, lo, x_dev, (uint8_t*)comp_dev, (uint32_t*)workspace_dev, seed, stream, 0u, f);
 }
 
 div_status div_compress(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
@@ -726,34 +769,7 @@ div_status div_planegroup_compress(const div_desc* desc, const void* x_dev, void
     if (comp_capacity < lo.total_bytes) return DIV_ERR_CAPACITY;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     uint8_t* blob = (uint8_t*)comp_dev;
-    // kernels that store bytes or half-words leave the unused top of a partial last word alone: it is zero by contract
-    if ((s.total * (uint64_t)desc->qbits) % 32u != 0 &&
-        cudaMemsetAsync(blob + lo.packed_off + lo.packed_bytes - 4, 0, 4, stream) != cudaSuccess)
-        return DIV_ERR_CUDA;
-    PgPlan pl;
-    if (!(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_pg_strip(desc, s, &pl))
-        return compress_pg_strip(desc, s, lo, pl, x_dev, blob, seed, stream);
-    if (PgSmall g; !(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_pg_small(desc, s, &g))
-        return compress_pg_small(desc, s, lo, g, x_dev, blob, seed, stream);
-    // Everything else that fits shared memory.  (Where the two kernels above apply they are faster or as good: 64 x 256 x 56 x 56 53
-    // against 70 us, 64 x 2048 x 7 x 7 18.6 against 20.0 us, 64 x 1024 x 14 x 14 30.8 against 28.8 us.)
-    if (SharePlan ps; !(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_plane_share(desc, s, &ps))
-        return compress_plane_share(desc, s, lo, ps, x_dev, blob, seed, stream);
-    // general kernel: words shared by two planes (and the zero-padded last word) are merged with atomic ORs
-    // into a cleared buffer
-    if (((uint64_t)s.HW * (uint64_t)desc->qbits) % 32u != 0 &&
-        cudaMemsetAsync(blob + lo.packed_off, 0, lo.packed_bytes, stream) != cudaSuccess)
-        return DIV_ERR_CUDA;
-    return dispatch_types(desc->x_dtype, desc->lfc_dtype, [&](auto* xt, auto* lt) -> div_status {
-        typedef std::remove_pointer_t<decltype(xt)> XT;
-        typedef std::remove_pointer_t<decltype(lt)> LT;
-        return dispatch_q(desc->qbits, [&](auto q) -> div_status {
-            pg_general_kernel<XT, LT, decltype(q)::value><<<s.N * s.C, 256, 0, stream>>>(
-                (const XT*)x_dev, (LT*)(blob + lo.lfc_off), (uint32_t*)(blob + lo.packed_off),
-                (uint32_t*)(blob + lo.stats_off), s, seed);
-            return launch_status();
-        });
-    });
+    return compress_planegroup(desc, s, lo, x_dev, blob, seed, stream, flags, ShareFault());
 }
 
 div_status div_planegroup_decompress(const div_desc* desc, const void* comp_dev, size_t comp_bytes, void* xhat_dev,

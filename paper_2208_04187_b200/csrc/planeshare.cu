@@ -157,8 +157,10 @@ inline div_status launch_plane_share_p2(uint32_t p2, int qbits, const PlaneShare
     return DIV_ERR_PARAM;
 }
 
-div_status compress_plane_share(const div_desc* d, const Shape& s, const div_layout& lo, const SharePlan& pl, const void* x, uint8_t* blob,
+div_status compress_plane_share(const div_desc* d, const Shape& s, const div_layout& lo, const SharePlan& plan, const void* x, uint8_t* blob,
                                 uint64_t seed, cudaStream_t st, const ShareFault& fault) {
+    SharePlan pl = plan;
+    pl.smem_bytes += fault.more_smem;
     PlaneShareParams p;
     p.x = x;
     p.lfc = blob + lo.lfc_off;

@@ -197,3 +197,31 @@ def test_plane_share_kernel_gives_up_a_wait_that_cannot_end(case, timeout_ns):
     assert bool((room[size:] == 0xA5).all())
     codec.compress(x, seed=5)
     assert torch.equal(codec.blob, want)
+
+
+@pytest.mark.parametrize("case", [(4, 32, 14, 14, 8, "f32"), (3, 16, 39, 39, 8, "bf16"), (2, 8, 32, 32, 8, "f32"), (20, 16, 19, 19, 4, "f32")],
+                         ids=lambda c: "x".join(map(str, c)))
+def test_a_refused_cluster_launch_leaves_the_map_to_the_next_kernel(case):
+    """... over a workspace full of leftovers, which that kernel has to find cleared."""
+    n, c, h, w, block, xd = case
+    x_np = make((n, c, h, w), "bn", 17, xd)
+    t = torch.from_numpy(x_np)
+    x = (t.view(torch.bfloat16) if xd == "bf16" else t).cuda()
+    codec = binding.Codec(n, c, h, w, block, 2, xd, "f32")
+    assert codec.plan().on_chip == 1
+    codec.workspace.fill_(0xFF)
+    assert debug_call(codec, x, 2, 100_000_000) == binding.DIV_OK
+    assert codec.device_status() == binding.DIV_OK
+    np.testing.assert_array_equal(codec.blob.cpu().numpy(), orc.compress(x_np, block, 2, 5, xd, "f32").blob())
+    assert bool((codec.workspace[64:80] != 0xFF).any())        # the slots were cleared and used: another kernel ran
+
+
+def test_a_refused_plane_share_launch_leaves_the_map_to_the_general_kernel():
+    x_np = make((2, 8, 75, 75), "bn", 17, "f32")
+    x = torch.from_numpy(x_np).cuda()
+    codec = binding.PlaneGroupCodec(2, 8, 75, 75, 8, 2)
+    assert codec.plan().on_chip == 1
+    st = binding.lib().div_debug_on_chip(codec.desc, x.data_ptr(), codec.blob.data_ptr(), codec.blob.numel(), None, 0, 5, binding.current_stream_handle(),
+                                         2, 100_000_000)
+    assert st == binding.DIV_OK
+    np.testing.assert_array_equal(codec.blob.cpu().numpy(), orc.compress_planes(x_np, 8, 2, 5).blob())

@@ -156,7 +156,7 @@ def test_the_on_chip_test_hook_checks_its_arguments():
     cap = ws = 1 << 20
     call = lambda *a: L.div_debug_on_chip(ctypes.byref(d), *a)  # noqa: E731
     assert call(None, 256, cap, 512, ws, 0, None, 0, 1) == binding.DIV_ERR_NULL
-    assert call(256, 512, cap, 1024, ws, 0, None, 7, 1) == binding.DIV_ERR_PARAM
+    assert call(256, 512, cap, 1024, ws, 0, None, 3, 1) == binding.DIV_ERR_PARAM
     assert call(256, 512, cap, 1024, ws, 0, None, 0, 0) == binding.DIV_ERR_PARAM
     assert call(256, 512, cap, 1024, ws, 0, None, 0, 100_000_001) == binding.DIV_ERR_PARAM
     assert call(256, 512, cap, 1028, ws, 0, None, 0, 1) == binding.DIV_ERR_ALIGN
