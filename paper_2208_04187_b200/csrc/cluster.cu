@@ -26,6 +26,7 @@ struct ClusterParams : ShareParams {
     uint32_t log2cs, expect_bytes;
     int32_t qbits;
 };
+static_assert(sizeof(ClusterParams) <= SHARE_PARAM_BYTES, "dearer launches");
 
 // ------------------------------------------------------------------------------------------------
 // cluster and distributed shared memory
@@ -290,11 +291,10 @@ div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout&
     p.packed = blob + lo.packed_off;
     p.stats = reinterpret_cast<float*>(blob + lo.stats_off);
     p.status = reinterpret_cast<uint64_t*>(ws);
-    const uint32_t number = fault.number ? fault.number : call_number();
-    p.failure = ((uint64_t)number << 32) | (uint64_t)DIV_ERR_TIMEOUT;
+    p.number = fault.number ? fault.number : call_number();
     p.seed = seed;
     p.never_bytes = fault.never_bytes;
-    p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000ull;
+    p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000u;
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
     p.log2cs = 0;
     while ((1u << p.log2cs) < pl.cs) ++p.log2cs;

@@ -83,8 +83,8 @@ struct ShareFault {
     uint32_t expect_bytes;    // what a CTA waits to receive, more than ever arrives, instead of what its cluster sends
     uint32_t never_bytes;     // what every wait for a piece of x waits for beyond the copy
     uint32_t more_smem;       // shared memory that the launch asks for beyond what it needs
-    uint32_t number;          // the call's number (see ShareParams::failure)
-    uint64_t timeout_ns;      // limit of every wait
+    uint32_t number;          // the call's number (see share_record)
+    uint32_t timeout_ns;      // limit of every wait
 };
 div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& pl, const void* x, uint8_t* blob,
                             uint32_t* ws, uint64_t seed, cudaStream_t st, const ShareFault& fault = ShareFault());

@@ -499,7 +499,7 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
     uint32_t* ws = (uint32_t*)workspace_dev;
     const uint32_t never = 0xFFFFFFFFu;      // an arrival count no sample reaches
     if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl))
-        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, 0u, timeout_ns});
+        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, 0u, (uint32_t)timeout_ns});
     if (!(flags & DIV_FLAG_NO_STRIP_KERNEL)) {
         VPlan vp;
         if (plan_v(desc, s, &vp) == DIV_OK) return compress_fused_v(desc, s, lo, vp, x_dev, blob, ws, seed, stream, never, timeout_ns);
@@ -535,7 +535,7 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     if (comp_capacity < lo.total_bytes || workspace_bytes < lo.workspace_bytes) return DIV_ERR_CAPACITY;
     ShareFault f = {};
     f.number = 1;
-    f.timeout_ns = timeout_ns;
+    f.timeout_ns = (uint32_t)timeout_ns;
     f.never_bytes = fault == DIV_FAULT_COPIES ? 16u : 0u;
     f.more_smem = fault == DIV_FAULT_REFUSED ? 1u << 20 : 0u;
     const cudaStream_t stream = (cudaStream_t)cuda_stream;

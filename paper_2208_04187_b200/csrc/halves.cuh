@@ -74,7 +74,7 @@ struct SlotSink {
     uint64_t lfc_at;          // where the tile's low-frequency value goes
     int32_t lfc_bf16;
     bool writer;              // this lane stores it
-    float inv, cnt, rcp;      // 1 / count when that is a power of two, else 0; count; RN(1 / count)
+    float cnt, rcp;           // count (0: a power of two, multiply), RN(1 / count)
 };
 // Mean of a slot's tile as it is stored.  Every lane of the warp calls it (lanes of a tile meet by shuffles); columns a
 // lane does not own count as zeros.
@@ -104,7 +104,7 @@ __device__ __forceinline__ float slot_mean(const uint64_t (&v)[ROWS][G::NV], con
     float sum = NV == 2 ? __fadd_rn(part[0], part[NV - 1]) : part[0];
 #pragma unroll
     for (int m = 1; m < (int)LPT; m <<= 1) sum = __fadd_rn(sum, __shfl_xor_sync(0xFFFFFFFFu, sum, m));
-    const float mean = s.inv != 0.f ? __fmul_rn(sum, s.inv) : div_by_count(sum, s.cnt, s.rcp);
+    const float mean = s.cnt == 0.f ? __fmul_rn(sum, s.rcp) : div_by_count(sum, s.cnt, s.rcp);
     if (any && s.writer) {
         if (s.lfc_bf16) Elem<__nv_bfloat16>::store(reinterpret_cast<__nv_bfloat16*>(s.lfc) + s.lfc_at, mean);
         else reinterpret_cast<float*>(s.lfc)[s.lfc_at] = mean;
@@ -214,8 +214,9 @@ struct ShareParams {
     void* lfc;
     void* packed;
     uint64_t* status;         // where a wait that ran out is recorded (share_record)
-    uint64_t failure;         // what is recorded: DIV_ERR_TIMEOUT, above it the call's number
-    uint64_t seed, timeout_ns;
+    uint64_t seed;
+    uint32_t number;          // of the call, recorded with a failure
+    uint32_t timeout_ns;
     uint32_t never_bytes;     // a test has the waits for pieces wait for more than is copied (0)
     uint32_t C, W, B, Hb, Wb, HW, TPP, qps;
     uint32_t ppc, ppp;        // planes per CTA, planes per piece
@@ -227,17 +228,21 @@ struct ShareParams {
     uint32_t partial;         // 1: the last tile of a row is narrower than B
     int32_t lfc_bf16;
     FastDiv by_sppf, by_spb, by_ppp;
-    float inv[4], cnt[4], rcp[4];     // [short band][narrow tile]: 1 / count when that is a power of two, else 0; count; RN(1 / count)
+    float cnt[4], rcp[4];     // [short band][narrow tile]: count (0: a power of two, the mean is a product), RN(1 / count)
+    __host__ __device__ uint64_t failure() const { return (uint64_t)number << 32 | (uint64_t)DIV_ERR_TIMEOUT; }
 };
+// Launching a kernel with more than 224 bytes of parameters costs the host 0.4 us more: 8 x 64 x 32 x 32, compress and decompress
+// 7.0 us with 224 bytes, 7.4 with 232.
+constexpr size_t SHARE_PARAM_BYTES = 224;
 // The status words, as one 64-bit word: zero, or the failure of a call with the call's number.  One CTA clears what an earlier
 // call (or nobody) left there, in no order with the other CTAs of the launch, which may have failed already: it leaves
 // alone what carries the number of its own call.  (The replays of a captured call share its number: a failure that one of
 // them recorded stays.)
-__device__ __forceinline__ void share_record(const ShareParams& p) { atomicExch(reinterpret_cast<unsigned long long*>(p.status), p.failure); }
+__device__ __forceinline__ void share_record(const ShareParams& p) { atomicExch(reinterpret_cast<unsigned long long*>(p.status), p.failure()); }
 __device__ __forceinline__ void share_clear_status(const ShareParams& p) {
     unsigned long long* w = reinterpret_cast<unsigned long long*>(p.status);
     unsigned long long seen = ld_relaxed_u64(p.status);
-    while (seen != 0ull && seen != p.failure) {              // at most twice: from here on only p.failure is written
+    while (seen != 0ull && seen != p.failure()) {            // at most twice: from here on only failure() is written
         const unsigned long long old = atomicCAS(w, seen, 0ull);
         if (old == seen) break;
         seen = old;
@@ -347,7 +352,6 @@ __device__ __forceinline__ void share_half1(const ShareParams& p, float* res, co
         sink.lfc_at = lfc0 + t.tile;
         sink.lfc_bf16 = p.lfc_bf16;
         sink.writer = t.writer;
-        sink.inv = p.inv[which];
         sink.cnt = p.cnt[which];
         sink.rcp = p.rcp[which];
         if constexpr (!PER_PLANE) {
@@ -390,9 +394,8 @@ inline void fill_share(ShareParams* p, const Shape& s, const SharePlan& pl, bool
     const uint32_t tail_cols = s.W - (s.Wb - 1u) * s.B;
     for (int i = 0; i < 4; ++i) {
         const uint32_t cnt = ((i & 2) ? p->tail_rows : s.B) * ((i & 1) ? tail_cols : s.B);
-        p->cnt[i] = (float)cnt;
+        p->cnt[i] = (cnt & (cnt - 1u)) == 0 ? 0.f : (float)cnt;
         p->rcp[i] = 1.0f / (float)cnt;
-        p->inv[i] = (cnt & (cnt - 1u)) == 0 ? p->rcp[i] : 0.f;
     }
 }
 

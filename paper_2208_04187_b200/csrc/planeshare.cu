@@ -18,6 +18,7 @@ struct PlaneShareParams : ShareParams {
     uint32_t* stats;
     FastDiv by_hw;
 };
+static_assert(sizeof(PlaneShareParams) <= SHARE_PARAM_BYTES, "dearer launches");
 
 template <typename XT, int P2, typename G, int Q>
 __global__ void __launch_bounds__(SHARE_THREADS, 3)
@@ -167,10 +168,10 @@ div_status compress_plane_share(const div_desc* d, const Shape& s, const div_lay
     p.packed = blob + lo.packed_off;
     p.stats = reinterpret_cast<uint32_t*>(blob + lo.stats_off);
     p.status = nullptr;
-    p.failure = 0;
+    p.number = 0;
     p.never_bytes = fault.never_bytes;
     p.seed = seed;
-    p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000ull;
+    p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000u;
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
     p.by_hw = host_fastdiv(s.HW);
     return d->x_dtype == DIV_F32 ? launch_plane_share_p2<float>(s.P2, d->qbits, p, pl, s.N, st)
