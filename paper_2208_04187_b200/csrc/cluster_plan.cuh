@@ -81,7 +81,7 @@ inline bool plan_cluster_cs(const div_desc* d, const Shape& s, uint32_t cs, cons
 // What a test may ask of a call beyond the ordinary (zeros: nothing).
 struct ShareFault {
     uint32_t expect_bytes;    // what a CTA waits to receive, more than ever arrives, instead of what its cluster sends
-    uint32_t never_bytes;     // what every wait for a piece of x waits for beyond the copy
+    uint32_t no_copies;       // the waits for x never end
     uint32_t more_smem;       // shared memory that the launch asks for beyond what it needs
     uint32_t number;          // the call's number (see share_record)
     uint32_t timeout_ns;      // limit of every wait

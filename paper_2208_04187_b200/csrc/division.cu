@@ -536,7 +536,7 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     ShareFault f = {};
     f.number = 1;
     f.timeout_ns = (uint32_t)timeout_ns;
-    f.never_bytes = fault == DIV_FAULT_COPIES ? 16u : 0u;
+    f.no_copies = fault == DIV_FAULT_COPIES;
     f.more_smem = fault == DIV_FAULT_REFUSED ? 1u << 20 : 0u;
     const cudaStream_t stream = (cudaStream_t)cuda_stream;
     if (planes) {

@@ -37,7 +37,7 @@ plane_share_kernel(const __grid_constant__ PlaneShareParams p) {
     const uint32_t nplanes = min(p.ppc, p.C - plane0);
     if (tid == 0) {
 #pragma unroll
-        for (uint32_t i = 0; i < SHARE_PIECES; ++i) mbar_init(&full[i], 1);
+        for (uint32_t i = 0; i < SHARE_PIECES; ++i) mbar_init(&full[i], p.arrivals);
         gave_up = 0u;
         fence_barrier_init();
         griddep_wait();
@@ -169,7 +169,7 @@ div_status compress_plane_share(const div_desc* d, const Shape& s, const div_lay
     p.stats = reinterpret_cast<uint32_t*>(blob + lo.stats_off);
     p.status = nullptr;
     p.number = 0;
-    p.never_bytes = fault.never_bytes;
+    p.arrivals = fault.no_copies ? 2u : 1u;
     p.seed = seed;
     p.timeout_ns = fault.timeout_ns ? fault.timeout_ns : 2000000000u;
     fill_share(&p, s, pl, d->lfc_dtype == DIV_BF16);
