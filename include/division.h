@@ -124,8 +124,10 @@ typedef struct div_plan {
                                planes up to 8192 elements); 4: row kernel (sample size a multiple of 4, rows of at
                                least 4 elements, planes too large for the table); 0: general */
     int32_t on_chip;        /* 1: the cluster kernel takes the descriptor first (x is read once and waits in shared memory; a
-                               thread-block cluster per sample); the fields above then describe the kernel that runs where
-                               the device refuses clusters of that size.  0: they describe what runs */
+                               thread-block cluster per sample).  grid, threads and smem_bytes are then those of its launch,
+                               chunks_per_sample the CTAs of a cluster, chunk_elems the elements of a CTA's share and stages the
+                               times that the device has to be filled; fused names the kernel that runs where the device
+                               refuses the launch.  0: all fields describe what runs */
 } div_plan;
 
 /* flags of div_compress_ex */
@@ -279,7 +281,8 @@ div_status div_planegroup_decompress(const div_desc* desc, const void* comp_dev,
 /* plan.fused: 1 strip kernel, 2 small-plane kernel (tile row of at most 32 padded columns, B up to 16, Q in
    {2,4,8}, sample size a multiple of 4), 0 general kernel;
    plan.on_chip: 1 where the share kernel runs instead of the general one (a CTA keeps a run of planes of any width in shared
-   memory; B up to 16, Q in {2,4,8}, samples of whole 16-byte groups); plan.decompress_fast: 1 quad kernel, 2 flat kernel
+   memory; B up to 16, Q in {2,4,8}, samples of whole 16-byte groups): grid, threads, smem_bytes, chunk_elems and
+   chunks_per_sample are then those of its launch; plan.decompress_fast: 1 quad kernel, 2 flat kernel
    (total size a multiple of 4, planes up to 8192 elements), 0 general. */
 div_status div_planegroup_plan_query(const div_desc* desc, uint32_t flags, div_plan* out);
 

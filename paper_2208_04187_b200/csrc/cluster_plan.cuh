@@ -32,6 +32,7 @@ struct ClusterPlan : SharePlan {
     uint32_t wide;            // 1: share_wide_threads a CTA, else SHARE_THREADS
     uint32_t waves;           // times the device has to be filled
 };
+inline uint32_t cluster_threads(uint32_t p2, const ClusterPlan& pl) { return pl.wide ? share_wide_threads(p2, pl.vw) : SHARE_THREADS; }
 
 // planes that are whole groups of 4 elements and 16-byte groups (bulk copies)
 inline uint32_t share_step(const div_desc* d, const Shape& s) {

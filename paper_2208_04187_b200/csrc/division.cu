@@ -458,7 +458,15 @@ div_status div_plan_query(const div_desc* desc, uint32_t flags, div_plan* out) {
         out->grid = (int32_t)((s.tiles + 255) / 256);
         out->threads = 256;
     }
-    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl)) out->on_chip = 1;
+    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl)) {
+        out->on_chip = 1;
+        out->grid = (int32_t)(s.N * cl.cs);
+        out->threads = (int32_t)cluster_threads(s.P2, cl);
+        out->stages = (int32_t)cl.waves;
+        out->smem_bytes = (int32_t)cl.smem_bytes;
+        out->chunk_elems = (int64_t)cl.ppc * s.HW;
+        out->chunks_per_sample = cl.cs;
+    }
     out->decompress_fast = decompress_fast_ok(s) ? ((s.H == 1 && s.CHW < (1u << 31)) ? 3 : 1) : decompress_rows_ok(s) ? 4 : (decompress_flat_ok(s) ? 2 : 0);
     return DIV_OK;
 }
@@ -749,7 +757,14 @@ div_status div_planegroup_plan_query(const div_desc* desc, uint32_t flags, div_p
         out->threads = 256;
         out->chunk_elems = s.HW;
         out->chunks_per_sample = s.C;
-        if (SharePlan ps; !(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_plane_share(desc, s, &ps)) out->on_chip = 1;
+        if (SharePlan ps; !(flags & DIV_FLAG_FORCE_TWO_PASS) && plan_plane_share(desc, s, &ps)) {
+            out->on_chip = 1;
+            out->chunks_per_sample = (s.C + ps.ppc - 1) / ps.ppc;
+            out->grid = (int32_t)(s.N * out->chunks_per_sample);
+            out->threads = (int32_t)SHARE_THREADS;
+            out->smem_bytes = (int32_t)ps.smem_bytes;
+            out->chunk_elems = (int64_t)ps.ppc * s.HW;
+        }
     }
     out->decompress_fast = decompress_fast_ok(s) ? 1 : (pg_decompress_flat_ok(s) ? 2 : 0);
     return DIV_OK;

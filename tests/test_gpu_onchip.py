@@ -45,6 +45,25 @@ CLUSTER = [   # n, c, h, w, block, q, x, lfc
 ]
 
 
+PLANE_SHARE = [   # n, c, h, w, block, q, x, lfc: odd widths beyond a warp, blocks of 16, quads that straddle planes
+    (2, 8, 75, 75, 8, 2, "f32", "f32"), (3, 12, 35, 35, 8, 4, "f32", "bf16"), (2, 5, 40, 40, 16, 4, "f32", "f32"),
+    (2, 8, 39, 37, 4, 8, "bf16", "bf16"), (1, 44, 9, 41, 16, 2, "f32", "f32"), (2, 16, 17, 70, 12, 2, "bf16", "f32"),
+    (4, 8, 3, 50, 4, 2, "f32", "f32"),
+]
+
+
+@pytest.mark.parametrize("case", CLUSTER + PLANE_SHARE, ids=lambda c: "x".join(map(str, c)))
+def test_the_plan_describes_the_launch(case):
+    """What runs, not what would run in its place: shares of whole planes that cover the sample, and room for them."""
+    n, c, h, w, block, q, xd, ld = case
+    plan = (binding.Codec if case in CLUSTER else binding.PlaneGroupCodec)(*case).plan()
+    assert plan.on_chip == 1 and plan.grid == n * plan.chunks_per_sample and plan.threads in (256, 384, 512)
+    assert plan.chunk_elems % (h * w) == 0 and plan.chunks_per_sample * plan.chunk_elems >= c * h * w
+    assert plan.chunk_elems * (4 if xd == "f32" else 2) <= plan.smem_bytes <= 232448
+    if case in CLUSTER:
+        assert plan.chunks_per_sample in (1, 2, 4, 8, 16) and plan.stages >= 1
+
+
 @pytest.mark.parametrize("case", CLUSTER, ids=lambda c: "x".join(map(str, c)))
 def test_cluster_kernel_matches_the_checker(case):
     n, c, h, w, block, q, xd, ld = case
@@ -154,13 +173,6 @@ def test_a_wait_for_x_that_cannot_end(case, timeout_ns):
     assert bool((room[whole.numel():] == 0xA5).all())
     codec.compress(x, seed=5)
     assert codec.device_status() == binding.DIV_OK and torch.equal(codec.blob, want)
-
-
-PLANE_SHARE = [   # n, c, h, w, block, q, x, lfc: odd widths beyond a warp, blocks of 16, quads that straddle planes
-    (2, 8, 75, 75, 8, 2, "f32", "f32"), (3, 12, 35, 35, 8, 4, "f32", "bf16"), (2, 5, 40, 40, 16, 4, "f32", "f32"),
-    (2, 8, 39, 37, 4, 8, "bf16", "bf16"), (1, 44, 9, 41, 16, 2, "f32", "f32"), (2, 16, 17, 70, 12, 2, "bf16", "f32"),
-    (4, 8, 3, 50, 4, 2, "f32", "f32"),
-]
 
 
 @pytest.mark.parametrize("case", PLANE_SHARE, ids=lambda c: "x".join(map(str, c)))
