@@ -275,6 +275,39 @@ inline div_status launch_cluster_p2(const ClusterParams& prm, const ClusterPlan&
     return DIV_ERR_PARAM;
 }
 
+static __global__ void place_kernel() {}                       // stands for any kernel in clusters_at_once
+
+uint32_t clusters_at_once(const DeviceInfo& di, uint32_t log2cs, uint32_t per_sm) {
+    constexpr uint32_t FORMS = 5, MOST = 8;
+    static std::atomic<int> known[DEVICE_CACHE_SLOTS][FORMS][MOST];      // the answer + 1
+    if (log2cs >= FORMS || per_sm < 1u || per_sm > MOST) return 0u;
+    const bool slot = di.dev >= 0 && di.dev < DEVICE_CACHE_SLOTS;
+    if (slot) {
+        const int got = known[di.dev][log2cs][per_sm - 1u].load(std::memory_order_relaxed);
+        if (got > 0) return (uint32_t)got - 1u;
+    }
+    static SmemSeen smem_set[DEVICE_CACHE_SLOTS], wide_set[DEVICE_CACHE_SLOTS];
+    const int smem = di.smem_optin / (int)per_sm - 2048;                  // per_sm such CTAs fit an SM, one more does not
+    if (!ensure_dynamic_smem((const void*)place_kernel, smem, smem_set) || !ensure_wide_cluster((const void*)place_kernel, wide_set)) return 0u;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << log2cs);
+    cfg.blockDim = dim3(SHARE_THREADS);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1u << log2cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, (const void*)place_kernel, &cfg) != cudaSuccess || n < 0) {
+        cudaGetLastError();
+        return 0u;
+    }
+    if (slot) known[di.dev][log2cs][per_sm - 1u].store(n + 1, std::memory_order_relaxed);
+    return (uint32_t)n;
+}
+
 // a number that the failed call before on this workspace is not likely to have had: the low bits of a clock
 static inline uint32_t call_number() {
 #if defined(__x86_64__)

@@ -8,7 +8,9 @@ namespace divk {
 constexpr uint32_t SHARE_THREADS = 256;
 constexpr uint32_t SHARE_WARPS = SHARE_THREADS / 32;
 // threads where at most two CTAs fit an SM and clusters take turns (32 x 64 x 75 x 75 28.6 -> 27.0 us, 64 x 1024 x 14 x 14
-// 23.6 -> 23.0 us; where all of x fits at once more threads cost a little, 64 x 2048 x 7 x 7 11.5 -> 12.1 us): 64 registers a thread suffice where rows are read 4 columns at a time or have 4 rows
+// 23.6 -> 23.0 us; where all of x fits at once more threads cost a little, 64 x 2048 x 7 x 7 11.5 -> 12.1 us), and where a CTA has
+// an SM to itself (1 x 64 x 112 x 112 10.8 -> 9.7 us, 1 x 128 x 56 x 56 7.4 -> 6.4 us): 64 registers a thread suffice where rows are
+// read 4 columns at a time or have 4 rows
 __host__ __device__ constexpr uint32_t share_wide_threads(uint32_t p2, uint32_t vw) { return vw == 4 || p2 == 4 ? 512u : 384u; }
 // resident CTAs per SM that the registers allow: up to 80 a thread, 64 (48) where they suffice (128 x 64 x 32 x 32: three of
 // 78 registers 14.5 us, four of 64 12.8 us)
@@ -30,9 +32,18 @@ struct SharePlan {
 struct ClusterPlan : SharePlan {
     uint32_t cs;              // CTAs per cluster (and per sample)
     uint32_t wide;            // 1: share_wide_threads a CTA, else SHARE_THREADS
-    uint32_t waves;           // times the device has to be filled
+    uint32_t turns64;         // 64ths of the times that the device has to be filled: whole times up to two, and where an SM holds one
+                              // CTA (the clusters of a turn then end together); beyond that what the clusters make up
+    uint32_t per_sm;          // CTAs that fit an SM
+    uint32_t load;            // CTAs at once on the busiest SM
 };
+
 inline uint32_t cluster_threads(uint32_t p2, const ClusterPlan& pl) { return pl.wide ? share_wide_threads(p2, pl.vw) : SHARE_THREADS; }
+
+// Clusters of 2^log2cs CTAs that the device holds at once where `per_sm` such CTAs fit an SM (a cluster stays within a group of
+// SMs, so that some places stay empty: with one CTA per SM 7 clusters of 16, 112 of 148 places; two, 33 of 8, 264 of 296).
+// Asked of the driver once per device and form; 0 where it has none.
+uint32_t clusters_at_once(const DeviceInfo& di, uint32_t log2cs, uint32_t per_sm);
 
 // planes that are whole groups of 4 elements and 16-byte groups (bulk copies)
 inline uint32_t share_step(const div_desc* d, const Shape& s) {
@@ -65,16 +76,23 @@ inline uint32_t share_per_sm(const SharePlan& pl, const DeviceInfo& di, uint32_t
 }
 
 // shape of the launch for clusters of cs CTAs; false when a share does not fit
-inline bool plan_cluster_cs(const div_desc* d, const Shape& s, uint32_t cs, const DeviceInfo& di, ClusterPlan* out) {
+inline bool plan_cluster_cs(const div_desc* d, const Shape& s, uint32_t log2cs, const DeviceInfo& di, ClusterPlan* out) {
+    const uint32_t cs = 1u << log2cs;
     if (!share_takes(d, s) || (uint64_t)s.N * cs >= (1ull << 31)) return false;
     ClusterPlan pl;
     const uint32_t step = share_step(d, s);
     pl.cs = cs;
     if (!plan_share(d, s, ((uint64_t)(s.C + cs - 1) / cs + step - 1) / step * step, 0u, true, di, &pl)) return false;
     const uint32_t per_sm = share_per_sm(pl, di, share_by_regs(s.P2, pl.vw, d->x_dtype == DIV_F32 ? 4u : 2u));
-    const uint64_t places = (uint64_t)per_sm * (uint32_t)di.sms * 95u / 100u;      // clusters leave about 5 % of the places empty
-    pl.waves = (uint32_t)(((uint64_t)s.N * cs + places - 1) / (places ? places : 1u));
-    pl.wide = pl.waves > 1u && per_sm <= 2u ? 1u : 0u;
+    const uint32_t at_once = clusters_at_once(di, log2cs, per_sm);
+    if (at_once == 0u) return false;
+    const uint64_t turns64 = per_sm == 1u || s.N <= 2u * at_once ? 64ull * ((s.N + at_once - 1u) / at_once) : 64ull * s.N / at_once;
+    if (turns64 >= (1ull << 31)) return false;
+    const uint32_t spread = (uint32_t)(((uint64_t)s.N * cs + (uint32_t)di.sms - 1u) / (uint32_t)di.sms);
+    pl.turns64 = (uint32_t)turns64;
+    pl.per_sm = per_sm;
+    pl.load = per_sm < spread ? per_sm : spread;
+    pl.wide = per_sm <= 2u && (pl.turns64 > 64u || spread == 1u) ? 1u : 0u;
     *out = pl;
     return true;
 }

@@ -238,6 +238,39 @@ void choose_compress(const div_desc* d, const Shape& s, uint32_t flags, Choice* 
     if (plan_fused(d, s, &c->fp) == DIV_OK) c->code = 1;
 }
 
+// Where the clusters of a map have to take turns, or keep much of the device idle (a single large sample), a kernel that
+// spreads the map over the whole device and reads x a second time may be faster.  Both measured on 1217 maps (1 to 192 samples of
+// 3 x 224 x 224 to 2048 x 7 x 7, up to 52 M elements, both types):
+//   * kernels for planes a warp wide (7, 4) are not within 2 turns (0.45 - 0.97 of their time), nor in any number of them for fp32 blocks
+//     up to 8 of which two shares fit an SM (192 x 512 x 19 x 19 0.76).  Else they are: 64 x 1984 x 32 x 8 with B = 16 120 against 71 us in 10;
+//     bfloat16, whose residuals take three times the room of x where it is not read 4 columns at a time, 64 x 1024 x 14 x 14 31.3 against
+//     26.9 us in 5.  With one share of fp32 per SM blocks of 4 are not (8 x 760 x 31 x 31 23 against 33 us), nor those of 8 in one turn (2 x
+//     936 x 32 x 23 11.2 against 14.1 us); in more, and for large shares of blocks of 16, it depends (128 x 1880 x 7 x 7 24 against 27 us in 2,
+//     24 x 2048 x 17 x 17 53 against 43 us in 4, 1 x 1064 x 28 x 28 with B = 16 12.8 against 10.4 us): both times are estimated, in ns;
+//   * the strip kernels (2, 3, 6) are not within 2 turns of which every SM holds two shares (or one of fp32), but where a share is large and
+//     the batch small (1 x 64 x 112 x 112 bfloat16 9.9 against 8.4 us) or the turns are many (64 x 64 x 112 x 112 89 against 60 us).  There
+//     both times are estimated; of 453 maps the estimates give 2 to the cluster that it takes 3 - 4 % longer for, and 10 to the others that
+//     these take 6 - 23 % longer for;
+//   * the general kernels never were (32 x 64 x 75 x 75 27 against 82 us).
+bool cluster_pays(const div_desc* d, const Shape& s, const ClusterPlan& pl) {
+    const uint64_t share = (uint64_t)pl.ppc * s.HW, wider = pl.vw == 4u ? 10u : pl.vw == 2u ? 12u : 13u;      // narrow accesses take longer
+    const bool f32 = d->x_dtype == DIV_F32, one_turn = pl.turns64 <= 64u, two_turns = pl.turns64 <= 128u;
+    if (one_turn && share < 40000u) return true;
+    const uint64_t own = 2400u + pl.turns64 * (1500u + share * (115u * pl.load + 30u) * wider / 10000u) / 64u;
+    Choice ch;
+    choose_compress(d, s, 0u, &ch);
+    switch (ch.code) {
+        case 7:
+        case 4:
+            if (f32 && pl.per_sm == 1u) return s.P2 <= 4u || (s.P2 <= 8u && one_turn) || own <= 8000u + s.total * 14u / 10000u;
+            return two_turns || (f32 && s.P2 <= 8u);
+        case 2: return (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) || own <= 7600u + s.total * 15u / 10000u;
+        case 3: return (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) || own <= 15500u + s.total * 105u / 100000u;
+        case 6: return (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) || own <= 14800u + s.total * 87u / 100000u;
+    }
+    return true;
+}
+
 // Does the cluster kernel take a descriptor, and in clusters of how many CTAs?  (Flags pin one of the other kernels.)
 bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPlan* out) {
     if (flags != 0) return false;
@@ -248,29 +281,20 @@ bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPl
         if (plan_lines(d, s, &lg)) return false;          // 1-D maps have a kernel of their own
     }
     // Cost in KB of x an SM works through (41 KB take 1 us): its share, and 3 us for every further time the device has
-    // to be filled, since the CTAs of one filling load, reduce and quantise in step.  Ties go to the smaller shares.
+    // to be filled, since the CTAs of one filling load, reduce and quantise in step.  Ties go to the smaller shares, and among
+    // equal ones to the smaller clusters (3 planes are 4 CTAs with work and none without: 8 x 3 x 224 x 224 17.9 -> 9.0 us).
     uint64_t best = ~0ull;
-    for (uint32_t cs = 1; cs <= CL_MAX; cs *= 2) {
+    for (uint32_t log2cs = 0; (1u << log2cs) <= CL_MAX; ++log2cs) {
         ClusterPlan pl;
-        if (!plan_cluster_cs(d, s, cs, di, &pl)) continue;
+        if (!plan_cluster_cs(d, s, log2cs, di, &pl)) continue;
         const uint64_t share = (uint64_t)pl.ppc * s.HW * 4u / 1024u;
-        const uint64_t cost = ((uint64_t)s.N * cs + (uint32_t)di.sms - 1u) / (uint32_t)di.sms * share + 123u * (pl.waves - 1u);
-        if (cost <= best) {
+        const uint64_t cost = ((uint64_t)s.N * pl.cs + (uint32_t)di.sms - 1u) / (uint32_t)di.sms * share + 123u * (pl.turns64 - 64u) / 64u;
+        if (cost < best || (cost == best && pl.ppc < out->ppc)) {
             best = cost;
             *out = pl;
         }
     }
-    if (best == ~0ull) return false;
-    // Where a kernel that reads x a second time from the L2 applies it is as good or better once the clusters have to
-    // take turns (three fillings: 50 x 256 x 40 x 40 39 against 35 us; two: 64 x 64 x 56 x 56 22.6 against 27.5 us,
-    // 64 x 1024 x 14 x 14 23.0 against 24.6 us).  bfloat16 that stays in place the same (128 x 160 x 32 x 32 29.8 against 33.0 us,
-    // 64 x 512 x 28 x 28 36.5 against 53.3 us) while three shares fit an SM (with two, 32 x 64 x 112 x 112 37.5 against 36.4 us);
-    // other bfloat16, whose residuals take twice the room of x, one filling.  The general kernels never are (32 x 64 x 75 x 75:
-    // 26.8 against 82 us).
-    PlaneGeom pg;
-    SPlan sp;
-    const bool rereads = plan_staged(d, s, &sp) == DIV_OK || plan_planes(d, s, &pg);
-    return !rereads || out->waves <= (d->x_dtype == DIV_F32 || (share_in_place(out->vw, 2u) && !out->wide) ? 2u : 1u);
+    return best != ~0ull && cluster_pays(d, s, *out);
 }
 
 bool decompress_fast_ok(const Shape& s) {
@@ -462,7 +486,7 @@ div_status div_plan_query(const div_desc* desc, uint32_t flags, div_plan* out) {
         out->on_chip = 1;
         out->grid = (int32_t)(s.N * cl.cs);
         out->threads = (int32_t)cluster_threads(s.P2, cl);
-        out->stages = (int32_t)cl.waves;
+        out->stages = (int32_t)((cl.turns64 + 63u) / 64u);
         out->smem_bytes = (int32_t)cl.smem_bytes;
         out->chunk_elems = (int64_t)cl.ppc * s.HW;
         out->chunks_per_sample = cl.cs;

@@ -103,6 +103,42 @@ def test_cluster_kernel_in_wide_blocks(case):
     assert torch.equal(*blobs)
 
 
+# A share per SM in a single turn: more threads.
+LONELY = [(1, 128, 56, 56, "f32"), (2, 64, 112, 112, "f32"), (1, 512, 28, 28, "f32"), (8, 3, 224, 224, "f32"), (4, 64, 112, 112, "bf16"), (1, 64, 75, 75, "f32")]
+
+
+@pytest.mark.parametrize("case", LONELY, ids=lambda c: "x".join(map(str, c)))
+def test_cluster_kernel_on_small_batches_of_large_samples(case):
+    n, c, h, w, xd = case
+    x = torch.randn((n, c, h, w), device="cuda", generator=torch.Generator("cuda").manual_seed(4)).to(binding.torch_dtype(xd))
+    codec = binding.Codec(n, c, h, w, 8, 2, xd, "f32")
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        plan = codec.plan()
+        assert not plan.on_chip or (plan.threads > 256 and plan.stages == 1)
+    blobs = []
+    for flags in (0, binding.DIV_FLAG_FORCE_TWO_PASS):
+        codec.blob.zero_()
+        codec.compress(x, seed=6, flags=flags)
+        assert codec.device_status() == binding.DIV_OK
+        blobs.append(codec.blob.clone())
+    assert torch.equal(*blobs)
+
+
+def test_turns_are_those_of_the_device():
+    """148 SMs hold 7 clusters of 16 CTAs with a share per SM each, and 33 clusters of 8 with two: the next sample takes another
+    turn.  Where that, or the batch, leaves the device to too few CTAs a kernel that spreads the map runs instead."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the figures are those of 148 SMs")
+
+    def plan(*a):
+        return binding.div_plan_query(binding.make_desc(*a))
+    assert [plan(n, 64, 112, 112, 8, 2).stages for n in (7, 8)] == [1, 2]
+    assert [plan(n, 1024, 14, 14, 8, 2).stages for n in (33, 34)] == [1, 2]
+    assert plan(16, 3, 150, 150, 8, 2).chunks_per_sample == 4              # a plane per CTA: no more CTAs than planes
+    for spread in ((1, 64, 112, 112, 8, 2, "bf16", "bf16"), (8, 64, 100, 152, 8, 2, "bf16", "bf16"), (64, 64, 112, 112, 8, 2), (64, 1024, 14, 14, 8, 2, "bf16", "bf16")):
+        assert plan(*spread).on_chip == 0, spread
+
+
 @pytest.mark.parametrize("q", [2, 4])
 def test_values_outside_the_fixed_point_route(q):
     """Constant, tiny, huge and one-sided samples beside an ordinary one."""
