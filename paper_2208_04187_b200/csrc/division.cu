@@ -264,9 +264,13 @@ bool cluster_pays(const div_desc* d, const Shape& s, const ClusterPlan& pl) {
         case 4:
             if (f32 && pl.per_sm == 1u) return s.P2 <= 4u || (s.P2 <= 8u && one_turn) || own <= 8000u + s.total * 14u / 10000u;
             return two_turns || (f32 && s.P2 <= 8u);
-        case 2: return (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) || own <= 7600u + s.total * 15u / 10000u;
-        case 3: return (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) || own <= 15500u + s.total * 105u / 100000u;
-        case 6: return (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) || own <= 14800u + s.total * 87u / 100000u;
+        case 2:
+        case 3:
+        case 6: {
+            if (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) return true;
+            const uint64_t other = ch.code == 2 ? 7600u + s.total * 15u / 10000u : ch.code == 3 ? 15500u + s.total * 105u / 100000u : 14800u + s.total * 87u / 100000u;
+            return own <= (two_turns ? other : other * 95u / 100u);
+        }
     }
     return true;
 }
