@@ -198,6 +198,26 @@ def test_fused_path_is_taken_where_expected():
         assert binding.div_plan_query(d).decompress_fast == (1 if spec.w % 4 == 0 else 2)
 
 
+def test_cluster_kernel_is_the_default_where_a_sample_is_whole_16_byte_groups():
+    """`fused` above names the kernel behind the cluster kernel; by default (flags 0) this one runs, for these small maps wherever
+    it can.  Flags other than 0 exclude it, which is how the tests here reach the others."""
+    count = 0
+    for case in SMALL:
+        n, c, h, w, block, q, xd, ld = case
+        b = min(block, max(h, w))
+        p2 = 1
+        while p2 < b:
+            p2 *= 2
+        lines = h == 1 and w % 4 == 0 and q != 1 and b & (b - 1) == 0 and b >= 4
+        takes = q != 1 and p2 in (4, 8, 16) and (c * h * w * (4 if xd == "f32" else 2)) % 16 == 0 and not lines
+        d = binding.make_desc(*case)
+        assert binding.div_plan_query(d).on_chip == int(takes), case
+        for flags in (RING, LAGGED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS):
+            assert binding.div_plan_query(d, flags).on_chip == 0
+        count += takes
+    assert count >= 20
+
+
 def test_decompress_reads_a_checker_blob():
     """The two directions are independent: the GPU decodes a buffer the CPU checker wrote."""
     for (shape, block, q, xd, ld) in [((2, 4, 28, 28), 8, 2, "f32", "f32"), ((2, 6, 14, 14), 8, 4, "bf16", "bf16"),

@@ -58,8 +58,8 @@ def _assert_equals_checker(blob, layout, x_np, block, qbits, seed, samples):
 
 def test_static_scratch_matches_the_checker_and_div_compress_on_calls_in_a_row():
     stream = binding.current_stream_handle()
-    # four maps of different shapes, one per compress path that keeps state in the scratch, so that every call
-    # finds another kernel's leftovers in the shared array
+    # four maps of different shapes, named after the kernels that take them where clusters are not to be had (the next test has
+    # a map for each kernel that keeps state in the scratch); the large one is the staged kernel's
     cases = [
         ("strip ring kernel", synth.activation_map(8, 16, 64, 64, "relu", 4246), 8, 2, 2),           # planes too wide for the small-plane kernel
         ("fused small-plane kernel", synth.activation_map(5, 24, 14, 14, "relu", 4242), 8, 2, 7),
@@ -97,6 +97,41 @@ def test_static_scratch_matches_the_checker_and_div_compress_on_calls_in_a_row()
     xref = codec.decompress(blob=want)
     torch.cuda.synchronize()
     assert torch.equal(xhat, xref)
+
+
+# Maps that the kernels with state in the scratch take by default, and one for the kernel that uses its status words alone: so
+# large that their number of CTAs is what decides (on 148 SMs).
+BY_DEFAULT = [
+    ("strip ring kernel", (1, 64, 112, 112), "bf16", 0, 2), ("cluster kernel", (16, 64, 14, 14), "f32", 1, None),
+    ("lagged kernel", (16, 64, 128, 128), "bf16", 0, 3), ("fused small-plane kernel", (24, 2048, 17, 17), "f32", 0, 7),
+    ("staged kernel", (20, 64, 112, 112), "f32", 0, 6), ("line kernel", (8, 64, 1, 768), "f32", 0, 8),
+]
+
+
+def test_static_scratch_between_the_kernels_that_keep_state_in_it():
+    """Every kernel finds the leftovers of each of the others: all ordered pairs, on one stream."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("which kernel takes a map is stated for 148 SMs")
+    stream = binding.current_stream_handle()
+    prepared = []
+    for name, shape, xd, on_chip, code in BY_DEFAULT:
+        x = torch.randn(shape, device="cuda", generator=torch.Generator("cuda").manual_seed(8)).to(binding.torch_dtype(xd))
+        codec, want = _reference_blob(x, (*shape, 8, 2, xd, "f32"), seed=11)
+        plan = codec.plan()
+        assert plan.on_chip == on_chip and code in (None, plan.fused), name
+        two_pass = binding.Codec(*shape, 8, 2, xd, "f32")
+        two_pass.compress(x, seed=11, flags=binding.DIV_FLAG_FORCE_TWO_PASS)
+        for g, w in zip(_sections(want, codec.layout), _sections(two_pass.blob, codec.layout)):
+            assert torch.equal(g, w), name
+        prepared.append((name, x, codec, want))
+    order = [k for i in range(len(prepared)) for j in range(len(prepared)) if i != j for k in (i, j)]
+    for i in order:
+        name, x, codec, want = prepared[i]
+        codec.blob.fill_(0xEE)
+        binding.div_compress_static(codec.desc, x.data_ptr(), codec.blob.data_ptr(), codec.blob.numel(), 11, stream)
+        for g, w in zip(_sections(codec.blob, codec.layout), _sections(want, codec.layout)):
+            assert torch.equal(g, w), name
+    assert binding.div_read_static_status(stream) == binding.DIV_OK
 
 
 def test_static_status_word_is_readable_through_its_accessor():
