@@ -14,8 +14,9 @@ namespace divk {
 // ------------------------------------------------------------------------------------------------
 // sum / cnt, correctly rounded, for a small whole cnt and rcp = RN(1 / cnt): one Newton step on the quotient with an
 // exact remainder (Markstein, "Computation of elementary functions on the IBM RISC System/6000", 1990).  Checked
-// against IEEE division for every significand of the sum and every count up to 1024; scaling by powers of two
-// changes nothing while no intermediate result leaves the normal range, hence the guard.
+// against IEEE division for every significand of the sum and every count that a tile of up to 16 x 16 can have
+// (tests/test_gpu_mean_division.py); scaling by powers of two changes nothing while no intermediate result leaves the
+// normal range, hence the guard.
 __device__ __forceinline__ float div_by_count(float sum, float cnt, float rcp) {
     const float m = fabsf(sum);
     if (m > 1e-30f && m < 1e30f) {
