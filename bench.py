@@ -7,7 +7,7 @@ every map is decompressed (Algorithm 1, backward loop).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints ONE JSON line.  `value` is GB of activation taken through the pair per second
+Prints ONE JSON line on stdout (and everything measured beside it, as another, on stderr).  `value` is GB of activation taken through the pair per second
 (raw activation bytes / (compress time + decompress time)), inputs resident in HBM.
 `--impl reference` times the CPU checker (oracle/) on host cores instead.
 """
@@ -783,7 +783,7 @@ def run_ours(args):
                    "compression_ratio": raw_bytes / comp_bytes, "per_map": per_map},
         "roofline": {"bound": "hbm", "kernel": compress_name(kernel_names, plans[dom]) + " on " + per_map[dom]["map"] +
                      f" ({dom_n} back-to-back calls between two CUDA events on its stream, two inputs alternating; "
-                     "the span includes the 2-us workspace clear)",
+                     "the span includes the clearing of the workspace)",
                      "achieved": dom_gbs, "peak": peak, "unit": "GB/s", "frac": dom_gbs / peak, "us_per_launch": dom_ms * 1e3,
                      "peak_kind": f"of {peak_kind}", "frac_of_nominal_8TBps": dom_gbs / NOMINAL_HBM_GBS,
                      "traffic": ncu_traffic(compress_name(kernel_names, plans[dom]), per_map[dom]["map"]),
@@ -807,9 +807,37 @@ def run_ours(args):
         "gpu_launches": kernels_per_step * args.steps * len(rep_ms),
         "clocks": clocks,
     }
-    print(json.dumps(line))
+    report(line)
     if world > 1:
         dist.destroy_process_group()
+
+
+DETAIL = os.path.join("gpurun_out", "bench_detail.json")
+
+
+def report(line):
+    """The result line on stdout, short enough that the tail of a log holds all of it; everything measured beside it goes to
+    stderr, and to a file where its folder exists."""
+    detail = json.dumps(line)
+    sys.stderr.write(detail + "\n")
+    if os.path.isdir(os.path.dirname(DETAIL)):
+        with open(DETAIL, "w") as f:
+            f.write(detail)
+
+    def short(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    out = {k: short(line[k]) for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                                       "vs_baseline", "dtype", "data")}
+    c, r, e, cpu = line["config"], line["roofline"], line["e2e"], line["cpu_baseline"]
+    out["config"] = {"workload": c["workload"], "parallelism": f"dp{line['n_gpus']}", "l2": "1.2 GB per step, each buffer touched once",
+                     "repeats": c["repeats"], "compression_ratio": short(c["compression_ratio"])}
+    out["roofline"] = {"bound": r["bound"], "kernel": r["kernel"].split(" (")[0], "us": short(r["us_per_launch"]), "achieved": short(r["achieved"]),
+                       "peak": r["peak"], "unit": r["unit"], "frac": short(r["frac"]), "traffic": r["traffic"]}
+    out["cpu_baseline"] = cpu and {"value": short(cpu["value"]), "unit": cpu["unit"], "cores": cpu["cores"], "kind": cpu["kind"]}
+    out["e2e"] = {k: short(e[k]) for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps")}
+    out["gpu_launches"], out["clocks"] = line["gpu_launches"], line["clocks"]
+    print(json.dumps(out))
 
 
 def main():
