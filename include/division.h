@@ -120,9 +120,11 @@ typedef struct div_plan {
     int64_t chunk_elems;    /* elements per full chunk (ring kernels) or per unit (3)         */
     int64_t chunks_per_sample;
     int32_t decompress_fast;/* 1: quad kernel (W%4==0, B a power of two >= 4); 3: the same conditions on a 1-D map
-                               (h == 1): line kernel; 2: flat kernel with a tile table (sample size a multiple of 4,
-                               planes up to 8192 elements); 4: row kernel (sample size a multiple of 4, rows of at
-                               least 4 elements, planes too large for the table); 0: general */
+                               (h == 1): line kernel; 4: row kernel (sample size a multiple of 4, rows of at least 4
+                               elements, the rows that 8192 elements touch in at most 40 KB; planes from 2048 elements
+                               up, smaller ones where 2 does not apply); 2: flat kernel with a tile table (sample size
+                               a multiple of 4, planes up to 8192 elements, at most 40000 bytes of shared memory);
+                               0: general */
     int32_t on_chip;        /* 1: the cluster kernel takes the descriptor first (x is read once and waits in shared memory; a
                                thread-block cluster per sample).  grid, threads and smem_bytes are then those of its launch,
                                chunks_per_sample the CTAs of a cluster, chunk_elems the elements of a CTA's share and stages the

@@ -345,8 +345,9 @@ decompress_flat_kernel(const LT* lfc, const uint32_t* packed,
 // band * W + w and a quad's 4 values follow each other, but for one possible step to the next row.  Lanes read their 4
 // values in different orders (element (i ^ lane / 8) first): at 4 words from lane to lane one order would meet in 8 banks.
 // The row of a quad is found by divisions once per thread; from one quad to the next (1024 elements on) it is stepped.
-// HBM writes bound it by its roofline (7.6 us for 32 x 64 x 75 x 75 fp32, 46 MB); it takes 15.4 us (3.2 TB/s), the general
-// kernel, a thread per packed word with stores 64 bytes apart, 51 us.
+// HBM writes bound it by its roofline (7.6 us for 32 x 64 x 75 x 75 fp32, 46 MB); it takes 13.6 us (3.7 TB/s) back to back and 17.8 us
+// alone on cold caches, 71 % of the issue slots busy; the general kernel, a thread per packed word with stores 64 bytes apart,
+// 51 us.  Taken from 2048 elements per plane on, and for smaller planes that the flat kernel cannot take.
 // grid = (ceil(quads_per_sample / (256*QPT)), N), dynamic shared memory = 4 * bands * W bytes
 // ---------------------------------------------------------------------------------------------
 struct DecRows {

@@ -164,7 +164,8 @@ constexpr int DEC_QPT = 4;
 #endif
 constexpr int FLAT_QPT = DIVK_FLAT_QPT;       // quads per thread of the flat decompress kernel
 
-// Which compress kernels run a descriptor.  Measured on the ResNet / WRN / DenseNet-shaped maps: from about
+// Which compress kernels run a descriptor that the cluster kernel (choose_cluster below, asked first) leaves to them, and all
+// descriptors where flags exclude it.  Measured on the ResNet / WRN / DenseNet-shaped maps: from about
 // 56 MB up with 8 x 8 blocks the staged kernel is fastest (both reads of x staged through shared memory by bulk
 // copies), from about 20 MB up the lagged kernel (plain loads, several bands per lane, cheap for small strips),
 // below that the strip ring kernel (shorter start-up); the general kernels take what those three cannot.

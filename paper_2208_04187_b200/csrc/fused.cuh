@@ -519,8 +519,10 @@ inline bool ensure_dynamic_smem(const void* kern, int bytes, SmemSeen* seen) {
 // Programmatic dependent launch: a kernel launched this way may start while the kernel before it in the stream is still
 // running; it does its set-up, and griddep_wait() holds it until that kernel is complete and its writes are visible.
 // Every kernel so launched calls griddep_wait() before it touches global memory, and griddep_launch() right after it so
-// that the next one can do the same.  Back to back it hides most of a launch and a kernel's ramp: compress + decompress of
-// 8 x 64 x 32 x 32 10.2 -> 7.0 us, 64 x 1024 x 14 x 14 40.6 -> 35.5 us, 128 x 64 x 32 x 32 24.1 -> 21.2 us.
+// that the next one can do the same.  What the kernel directly before it may write is read by plain loads.  The read-only
+// path (const __restrict__) is open to a kernel that follows clear_scratch_kernel, for everything but the scratch: that kernel has
+// waited for whatever ran before it, so its successor starts when all of that is complete.  Back to back it hides most of a
+// launch and a kernel's ramp: compress + decompress of 8 x 64 x 32 x 32 10.2 -> 7.0 us, 64 x 1024 x 14 x 14 40.6 -> 35.5 us, 128 x 64 x 32 x 32 24.1 -> 21.2 us.
 template <typename... Params, typename... Args>
 inline div_status launch_pdl(void (*kern)(Params...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -493,7 +493,7 @@ struct Quad3 {
 };
 // low-frequency value of quad q (inside sample n's map lfc_n)
 template <typename LT>
-__device__ __forceinline__ float quad3_lfc(const LT* __restrict__ lfc_n, const Quad3& g, uint32_t q) {
+__device__ __forceinline__ float quad3_lfc(const LT* lfc_n, const Quad3& g, uint32_t q) {
     const uint32_t vol = fdiv(q, g.by_qpv);
     uint32_t rem = q - vol * g.qpv;
     const uint32_t d = fdiv(rem, g.by_qpp);

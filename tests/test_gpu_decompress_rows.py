@@ -1,5 +1,5 @@
-"""The row decompress kernel (planes too large for the flat kernel's table, any width and block): exact parity with the
-CPU checker where quads straddle rows, bands and planes, and at the smallest width it takes."""
+"""The row decompress kernel (planes of 2048 elements and more, or too large for the flat kernel's table; any width and block):
+exact parity with the CPU checker where quads straddle rows, bands and planes, and at the smallest width it takes."""
 import numpy as np
 import pytest
 import torch
