@@ -812,17 +812,10 @@ def run_ours(args):
         dist.destroy_process_group()
 
 
-DETAIL = os.path.join("gpurun_out", "bench_detail.json")
-
-
 def report(line):
     """The result line on stdout, short enough that the tail of a log holds all of it; everything measured beside it goes to
-    stderr, and to a file where its folder exists."""
-    detail = json.dumps(line)
-    sys.stderr.write(detail + "\n")
-    if os.path.isdir(os.path.dirname(DETAIL)):
-        with open(DETAIL, "w") as f:
-            f.write(detail)
+    stderr."""
+    sys.stderr.write(json.dumps(line) + "\n")
 
     def short(v):
         return float(f"{v:.6g}") if isinstance(v, float) else v
