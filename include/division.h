@@ -93,9 +93,9 @@ typedef struct div_layout {
 /* How div_compress will run a descriptor (introspection for tests and benchmarks). */
 typedef struct div_plan {
     int32_t fused;          /* for W%4==0, B in {4,8}, Q in {2,4,8}, one launch:
-                               6: x read from HBM once and re-read from L2 a little later, both reads staged through
-                                  shared-memory rings by bulk copies (staged kernel; first choice from 56 MB up
-                                  with B = 8);
+                               6: bulk copies into shared-memory rings (first choice from 56 MB up with B = 8): x read once, its
+                                  residuals wait in tensor memory (parking kernel, lag 0), or, where the parts of a sample do
+                                  not fit there, x read from HBM once and re-read from L2 a little later (staged kernel);
                                3: as 6, with plain global loads (lagged kernel; first choice from 20 MB up);
                                2: chunks wait in a shared-memory ring (strip ring kernel; first choice below 20 MB);
                                7: small planes of any width (tile side 4, 8 or 16 after padding, at most 32 lanes per
@@ -129,7 +129,11 @@ typedef struct div_plan {
                                thread-block cluster per sample).  grid, threads and smem_bytes are then those of its launch,
                                chunks_per_sample the CTAs of a cluster, chunk_elems the elements of a CTA's share and stages the
                                times that the device has to be filled; fused names the kernel that runs where the device
-                               refuses the launch.  0: all fields describe what runs */
+                               refuses the launch.  0: all fields describe what runs.
+                               Either way threads 1024 and lag 0 say that the parking kernel (see fused, 6) takes the
+                               descriptor before all others: grid, threads, smem_bytes, chunk_elems and chunks_per_sample are
+                               those of its launch (with on_chip 0 stages too), fused and on_chip name what runs where the
+                               device refuses it */
 } div_plan;
 
 /* flags of div_compress_ex */
@@ -227,11 +231,11 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                           void* xhat_dev, void* cuda_stream);
 
 /*
- * Test hook for the bounded waits of the single-launch compress kernels (on_chip 1, plan codes 2, 3, 6 and 7): runs the
+ * Test hook for the bounded waits of the single-launch compress kernels (the parking kernel, on_chip 1, plan codes 2, 3, 6 and 7): runs the
  * kernel div_compress_ex would run, but tells it to wait for a number of arrivals per sample that is never
  * reached, with `timeout_ns` (at most 100 ms) as the limit of every wait.  The kernel must give up, record
  * DIV_ERR_TIMEOUT in the workspace status word (read it with div_read_device_status) and return; the blob's
- * contents are then unspecified.  The first of the cluster (flags 0), strip ring, lagged, staged and fused small-plane
+ * contents are then unspecified.  The first of the parking, cluster (flags 0), strip ring, lagged, staged and fused small-plane
  * kernels that the flags allow and the descriptor fits is taken; DIV_ERR_PARAM when there is none.
  * Arguments as for div_compress_ex.  No counterpart in the paper.
  */

@@ -13,8 +13,8 @@ LIB_PATH = os.path.join(PKG_DIR, "libdivision.so")
 NATIVE_SRC = os.path.join(CSRC, "native.cpp")
 NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")        # the calls on torch tensors, linked against the library
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
-SOURCES = ["division.cu", "cluster.cu", "planeshare.cu"]
-HEADERS = ["common.cuh", "cluster_plan.cuh", "halves.cuh", "twopass.cuh", "decompress.cuh", "fused.cuh", "fused_v.cuh", "lagged.cuh", "staged.cuh", "planes.cuh", "planegroup.cuh", "masks.cuh", "lines.cuh", "volume.cuh", os.path.join("..", "..", "include", "division.h")]
+SOURCES = ["division.cu", "cluster.cu", "planeshare.cu", "park.cu"]
+HEADERS = ["common.cuh", "cluster_plan.cuh", "halves.cuh", "park_plan.cuh", "twopass.cuh", "decompress.cuh", "fused.cuh", "fused_v.cuh", "lagged.cuh", "staged.cuh", "planes.cuh", "planegroup.cuh", "masks.cuh", "lines.cuh", "volume.cuh", os.path.join("..", "..", "include", "division.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",

@@ -14,6 +14,7 @@
 #include "lagged.cuh"
 #include "lines.cuh"
 #include "masks.cuh"
+#include "park_plan.cuh"
 #include "planegroup.cuh"
 #include "planes.cuh"
 #include "staged.cuh"
@@ -253,23 +254,31 @@ void choose_compress(const div_desc* d, const Shape& s, uint32_t flags, Choice* 
 //     both times are estimated; of 453 maps the estimates give 2 to the cluster that it takes 3 - 4 % longer for, and 10 to the others that
 //     these take 6 - 23 % longer for;
 //   * the general kernels never were (32 x 64 x 75 x 75 27 against 82 us).
-bool cluster_pays(const div_desc* d, const Shape& s, const ClusterPlan& pl) {
+uint64_t cluster_ns(const Shape& s, const ClusterPlan& pl) {
     const uint64_t share = (uint64_t)pl.ppc * s.HW, wider = pl.vw == 4u ? 10u : pl.vw == 2u ? 12u : 13u;      // narrow accesses take longer
+    return 2400u + pl.turns64 * (1500u + share * (115u * pl.load + 30u) * wider / 10000u) / 64u;
+}
+uint64_t other_ns(const Shape& s, int code) {
+    return code == 7 || code == 4 ? 8000u + s.total * 14u / 10000u : code == 2 ? 7600u + s.total * 15u / 10000u
+         : code == 3 ? 15500u + s.total * 105u / 100000u : 14800u + s.total * 87u / 100000u;
+}
+bool cluster_pays(const div_desc* d, const Shape& s, const ClusterPlan& pl) {
+    const uint64_t share = (uint64_t)pl.ppc * s.HW;
     const bool f32 = d->x_dtype == DIV_F32, one_turn = pl.turns64 <= 64u, two_turns = pl.turns64 <= 128u;
     if (one_turn && share < 40000u) return true;
-    const uint64_t own = 2400u + pl.turns64 * (1500u + share * (115u * pl.load + 30u) * wider / 10000u) / 64u;
+    const uint64_t own = cluster_ns(s, pl);
     Choice ch;
     choose_compress(d, s, 0u, &ch);
     switch (ch.code) {
         case 7:
         case 4:
-            if (f32 && pl.per_sm == 1u) return s.P2 <= 4u || (s.P2 <= 8u && one_turn) || own <= 8000u + s.total * 14u / 10000u;
+            if (f32 && pl.per_sm == 1u) return s.P2 <= 4u || (s.P2 <= 8u && one_turn) || own <= other_ns(s, 7);
             return two_turns || (f32 && s.P2 <= 8u);
         case 2:
         case 3:
         case 6: {
             if (!one_turn && two_turns && (f32 || pl.per_sm >= 2u)) return true;
-            const uint64_t other = ch.code == 2 ? 7600u + s.total * 15u / 10000u : ch.code == 3 ? 15500u + s.total * 105u / 100000u : 14800u + s.total * 87u / 100000u;
+            const uint64_t other = other_ns(s, ch.code);
             return own <= (two_turns ? other : other * 95u / 100u);
         }
     }
@@ -300,6 +309,35 @@ bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPl
         }
     }
     return best != ~0ull && cluster_pays(d, s, *out);
+}
+
+// Does the parking kernel take a descriptor that the rules above give to clusters (cl) or to kernel `code`?  Measured against both on 800
+// random maps (0.1 to 205 MB, both types, all blocks and bit widths that it takes): clusters in one turn are not asked to give way
+// (0.8 of its time in the geometric mean); clusters in turns and the kernels that read x twice where the estimated time is shorter:
+// 1.3 times faster in the geometric mean there (50 x 2048 x 16 x 16 with B = 4 49.5 -> 27.8 us, 96 x 432 x 15 x 56 with B = 4 74.9 -> 37.2 us).
+// The strip kernel's time is fitted once more over its small maps (1 x 56 x 112 x 112 5.9 against 7.2 us, 4.8 MB on the parking kernel's).
+// The staged kernel keeps samples of which less than two and a half fit the parked units (8 x 1840 x 56 x 56 58.5 against 68.1 us).
+bool choose_park(const div_desc* d, const Shape& s, uint32_t flags, const ClusterPlan* cl, int code, ParkPlan* out) {
+    if (flags != 0u) return code == 6 && plan_park(d, s, out);
+    if ((cl && cl->turns64 <= 64u) || !plan_park(d, s, out)) return false;
+    if (cl) return out->sets >= 2u && park_ns(*out) <= cluster_ns(s, *cl);      // (a chunk at a time: 96 x 16 x 100 x 100 bfloat16 21.8 -> 24.6 us)
+    if (code == 6) return 5u * out->per_cta <= 2u * PARK_DEPTH * out->sets && park_ns(*out) <= other_ns(s, code);
+    return park_ns(*out) <= (code == 2 ? 4600u + s.total * 155u / 100000u : other_ns(s, code));
+}
+
+// What runs a descriptor: the parking kernel, clusters, or kernel ch.code (which also follows where one of the others is refused).
+struct Route {
+    bool park, cluster;
+    ParkPlan pk;
+    ClusterPlan cl;
+};
+void choose_route(const div_desc* d, const Shape& s, uint32_t flags, Route* r) {
+    r->cluster = choose_cluster(d, s, flags, &r->cl);
+    r->park = false;
+    if (r->cluster && r->cl.turns64 <= 64u) return;
+    Choice ch;
+    choose_compress(d, s, flags, &ch);
+    r->park = choose_park(d, s, flags, r->cluster ? &r->cl : nullptr, ch.code, &r->pk);
 }
 
 bool decompress_fast_ok(const Shape& s) {
@@ -333,9 +371,11 @@ div_status compress_map(const div_desc* desc, const Shape& s, const div_layout& 
     if ((s.total * (uint64_t)desc->qbits) % 32u != 0 &&
         cudaMemsetAsync(blob + lo.packed_off + lo.packed_bytes - 4, 0, 4, stream) != cudaSuccess)
         return DIV_ERR_CUDA;
-    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl) && compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, fault) == DIV_OK)
-        return DIV_OK;
+    Route rt;
+    choose_route(desc, s, flags, &rt);
+    if (!rt.park && rt.cluster && compress_cluster(desc, s, lo, rt.cl, x_dev, blob, ws, seed, stream, fault) == DIV_OK) return DIV_OK;
     if (clear_scratch(ws, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
+    if (rt.park && compress_park(desc, s, lo, rt.pk, x_dev, blob, ws, seed, stream) == DIV_OK) return DIV_OK;
     // The single-launch kernels need all their CTAs resident, so they are launched cooperatively; where the
     // device refuses such a launch (fewer SMs visible to the process than the device reports, for instance) the
     // next kernel in line takes the descriptor: nothing has been enqueued by the refused launch.
@@ -487,8 +527,19 @@ div_status div_plan_query(const div_desc* desc, uint32_t flags, div_plan* out) {
         out->grid = (int32_t)((s.tiles + 255) / 256);
         out->threads = 256;
     }
-    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl)) {
-        out->on_chip = 1;
+    Route rt;
+    choose_route(desc, s, flags, &rt);
+    out->on_chip = rt.cluster ? 1 : 0;
+    if (rt.park) {
+        out->grid = (int32_t)rt.pk.grid;
+        out->threads = PARK_THREADS;
+        out->stages = rt.cluster ? (int32_t)((rt.cl.turns64 + 63u) / 64u) : (int32_t)rt.pk.stages;
+        out->lag = 0;
+        out->smem_bytes = (int32_t)rt.pk.smem_bytes;
+        out->chunk_elems = rt.pk.chunk_elems;
+        out->chunks_per_sample = rt.pk.chunks_per_sample;
+    } else if (rt.cluster) {
+        const ClusterPlan& cl = rt.cl;
         out->grid = (int32_t)(s.N * cl.cs);
         out->threads = (int32_t)cluster_threads(s.P2, cl);
         out->stages = (int32_t)((cl.turns64 + 63u) / 64u);
@@ -535,8 +586,11 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
     uint8_t* blob = (uint8_t*)comp_dev;
     uint32_t* ws = (uint32_t*)workspace_dev;
     const uint32_t never = 0xFFFFFFFFu;      // an arrival count no sample reaches
-    if (ClusterPlan cl; choose_cluster(desc, s, flags, &cl))
-        return compress_cluster(desc, s, lo, cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, 0u, (uint32_t)timeout_ns});
+    Route rt;
+    choose_route(desc, s, flags, &rt);
+    if (rt.park) return compress_park(desc, s, lo, rt.pk, x_dev, blob, ws, seed, stream, never, timeout_ns);
+    if (rt.cluster)
+        return compress_cluster(desc, s, lo, rt.cl, x_dev, blob, ws, seed, stream, ShareFault{1u << 19, 0u, 0u, 0u, (uint32_t)timeout_ns});
     if (!(flags & DIV_FLAG_NO_STRIP_KERNEL)) {
         VPlan vp;
         if (plan_v(desc, s, &vp) == DIV_OK) return compress_fused_v(desc, s, lo, vp, x_dev, blob, ws, seed, stream, never, timeout_ns);
@@ -581,8 +635,9 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
         if (div_planegroup_plan_query(desc, 0u, &plan) != DIV_OK || !plan.on_chip) return DIV_ERR_PARAM;
         return compress_planegroup(desc, s, lo, x_dev, (uint8_t*)comp_dev, seed, stream, 0u, f);
     }
-    ClusterPlan cl;
-    if (!choose_cluster(desc, s, 0u, &cl)) return DIV_ERR_PARAM;
+    Route rt;
+    choose_route(desc, s, 0u, &rt);
+    if (rt.park || !rt.cluster) return DIV_ERR_PARAM;
     return compress_map(desc, s, lo, x_dev, (uint8_t*)comp_dev, (uint32_t*)workspace_dev, seed, stream, 0u, f);
 }
 

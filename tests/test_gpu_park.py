@@ -1,0 +1,63 @@
+"""The compress kernel that parks residuals in tensor memory: the same bytes as the kernels with a pass per half, where its tilings end
+(last chunks, short bands, narrow tiles, planes larger than a chunk) and where a sample just fits what is parked, or just does not.
+(Small maps of every form against the CPU checker: test_gpu_parity, flags that leave the staged kernels alone.)"""
+import pytest
+import torch
+
+from paper_2208_04187_b200 import binding, build
+
+pytestmark = pytest.mark.gpu
+
+STAGED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built_library():
+    build.build()
+    binding.lib()
+
+
+def same_bytes(case, flags):
+    n, c, h, w, block, q, xd, ld = case
+    gen = torch.Generator("cuda").manual_seed(h * w)
+    x = torch.randn((n, c, h, w), device="cuda", generator=gen)
+    x[n // 2] *= 1e30                         # one sample off the fixed-point route
+    x = x.to(binding.torch_dtype(xd))
+    codec = binding.Codec(n, c, h, w, block, q, xd, ld)
+    blobs = []
+    for f in (flags, binding.DIV_FLAG_FORCE_TWO_PASS, flags):
+        codec.blob.zero_()
+        codec.compress(x, seed=11, flags=f)
+        assert codec.device_status() == binding.DIV_OK
+        blobs.append(codec.blob.clone())
+    assert torch.equal(blobs[0], blobs[1]) and torch.equal(blobs[0], blobs[2])
+    return codec.plan(flags)
+
+
+PARK = [  # n, c, h, w, block, q, x, lfc
+    (5, 64, 112, 112, 8, 2, "f32", "f32"),       # whole units, whole chunks
+    (3, 37, 28, 28, 8, 4, "f32", "bf16"),        # short bands, single-strip tiles side by side, a last chunk of few planes
+    (2, 19, 36, 36, 8, 8, "bf16", "bf16"),       # strips that do not fill their units
+    (300, 8, 4, 4, 4, 2, "f32", "f32"),          # a sample per unit
+    (9, 16, 14, 60, 4, 4, "bf16", "f32"),        # two strips a lane, short bands
+    (2, 512, 112, 112, 8, 2, "bf16", "f32"),     # a CTA has several chunks of a sample
+]
+
+
+@pytest.mark.parametrize("case", PARK, ids=lambda c: "x".join(map(str, c)))
+def test_parking_kernel_matches_the_two_pass_kernels(case):
+    plan = same_bytes(case, STAGED)
+    assert plan.fused == 6 and plan.threads == 1024 and plan.lag == 0
+
+
+# the last one's planes are more than a chunk
+@pytest.mark.parametrize("case", [(64, 64, 112, 112, 8, 2, "f32", "f32"), (128, 160, 32, 32, 4, 4, "bf16", "bf16"), (64, 24, 100, 112, 8, 2, "f32", "f32")], ids=lambda c: "x".join(map(str, c)))
+def test_parking_kernel_by_default(case):
+    plan = same_bytes(case, 0)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert plan.lag == 0 and plan.threads == 1024 and plan.grid == 148
+
+
+def test_samples_that_do_not_fit_go_to_the_staged_kernel():
+    plan = same_bytes((2, 64, 400, 400, 8, 2, "f32", "f32"), STAGED)          # 41 MB a sample, 38 MB of tensor memory
+    assert plan.fused == 6 and plan.lag > 0
