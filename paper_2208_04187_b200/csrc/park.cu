@@ -167,7 +167,7 @@ __device__ __forceinline__ void park_reduce(const ParkParams& p, ParkCtl* ctl, c
             if (FULL || (uint32_t)r < rows) StripRow2<XT>::load(xs + r * row_bytes, vxy[m][r], vzw[m][r]);
         }
     }
-    float lo = 3.402823466e+38f, hi = -3.402823466e+38f;
+    uint32_t kmin = 0u, kmax = 0u;                              // (keys, so that a NaN that came in stays one)
     uint32_t res[32];
 #pragma unroll
     for (int m = 0; m < MS; ++m) {
@@ -198,13 +198,13 @@ __device__ __forceinline__ void park_reduce(const ParkParams& p, ParkCtl* ctl, c
             upk2u(sub2_rn(vzw[m][r], stored2), res[i + 2], res[i + 3]);
         }
         if (active) {
-            lo = fminf(lo, __fsub_rn(blo, stored));
-            hi = fmaxf(hi, __fsub_rn(bhi, stored));
+            kmin = max(kmin, ~float_key(__fsub_rn(blo, stored)));
+            kmax = max(kmax, float_key(__fsub_rn(bhi, stored)));
         }
     }
     tmem_store32(at, res);
-    const uint32_t kmin = __reduce_max_sync(0xFFFFFFFFu, ~float_key(lo));
-    const uint32_t kmax = __reduce_max_sync(0xFFFFFFFFu, float_key(hi));
+    kmin = __reduce_max_sync(0xFFFFFFFFu, kmin);
+    kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
     if (lane == 0) {
         atomicMax(&ctl->kmin[slot], kmin);
         atomicMax(&ctl->kmax[slot], kmax);

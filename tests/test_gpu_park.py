@@ -61,3 +61,15 @@ def test_parking_kernel_by_default(case):
 def test_samples_that_do_not_fit_go_to_the_staged_kernel():
     plan = same_bytes((2, 64, 400, 400, 8, 2, "f32", "f32"), STAGED)          # 41 MB a sample, 38 MB of tensor memory
     assert plan.fused == 6 and plan.lag > 0
+
+
+def test_a_nan_reaches_the_sample_as_it_does_in_the_two_pass_kernels():
+    x = torch.randn((5, 64, 112, 112), device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    x[1, 7, 30, 50] = float("nan")
+    codec = binding.Codec(5, 64, 112, 112, 8, 2, "f32", "f32")
+    rebuilt = []
+    for f in (STAGED, binding.DIV_FLAG_FORCE_TWO_PASS):
+        codec.compress(x, seed=11, flags=f)
+        rebuilt.append(codec.decompress().clone())
+    assert codec.plan(STAGED).lag == 0
+    torch.testing.assert_close(rebuilt[0], rebuilt[1], rtol=0, atol=0, equal_nan=True)
