@@ -69,6 +69,17 @@ struct DecFast {
     uint32_t items;      // work items per sample = C * ipp
     FastDiv by_ipp;      // / ipp
     FastDiv by_wq;       // / (W/4)
+    __device__ __forceinline__ uint32_t lfc_plane(uint32_t plane) const { return plane; }
+};
+// The same for 3-D maps, a slice of a volume for a plane: C counts low-frequency planes (channels * Db), `planes` of a work item are
+// slices, and the B slices of a block share a low-frequency plane.
+struct DecFast3 : DecFast {
+    uint32_t D, Db;
+    FastDiv by_depth;    // / D
+    __device__ __forceinline__ uint32_t lfc_plane(uint32_t slice) const {
+        const uint32_t vol = fdiv(slice, by_depth);
+        return vol * Db + ((slice - vol * D) >> log2B);
+    }
 };
 
 template <typename XT> struct Quad;
@@ -150,10 +161,10 @@ __device__ __forceinline__ uint32_t quad_bits(const uint32_t* packed, uint64_t q
 // item are taken hq_count rows apart instead of next to each other, so that the lanes of a warp write consecutive
 // rows with one store instruction (whole sectors) instead of pieces 4 rows apart; the rows of an item then lie in
 // different tiles, each with its own low-frequency value.
-template <typename XT, typename LT, int Q, int QPT, bool SPREAD>
+template <typename XT, typename LT, int Q, int QPT, bool SPREAD, typename GEOM>
 __global__ void __launch_bounds__(256)
 decompress_quad_kernel(const LT* lfc, const uint32_t* packed,
-                       const float* stats, XT* xhat, DecFast d) {
+                       const float* stats, XT* xhat, GEOM d) {
     static_assert(QPT == 4, "a work item is 4 rows high");
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
@@ -169,7 +180,7 @@ decompress_quad_kernel(const LT* lfc, const uint32_t* packed,
     const uint32_t wq = rem - hq * d.wq;
     const uint32_t h0 = SPREAD ? hq : hq * 4u;
     const uint32_t hstep = SPREAD ? d.hq_count : 1u;
-    const LT* lfc_p = lfc + ((size_t)n * d.C + plane) * d.TPP + ((wq * 4u) >> d.log2B);
+    const LT* lfc_p = lfc + ((size_t)n * d.C + d.lfc_plane(plane)) * d.TPP + ((wq * 4u) >> d.log2B);
     const uint64_t quad0 = (uint64_t)n * d.qps + plane * d.hwq + h0 * d.wq + wq;      // first row's quad
     const uint32_t qstep = hstep * d.wq;
     float lf[4];

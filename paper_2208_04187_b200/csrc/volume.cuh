@@ -5,7 +5,7 @@
 //                        axis, then down the rows, then across the columns), stored low-frequency value,
 //                        residual extremes -> per-sample min / max keys in the scratch slots
 //   lfc_stats3d_warp_kernel  the same with a lane per block column (blocks of padded side <= 32): coalesced loads
-//   lfc_stats3d_strip_kernel, quant3d_strip_kernel, decompress3d_strip_kernel
+//   lfc_stats3d_strip_kernel, quant3d_strip_kernel
 //                        W % 4 == 0 and B = 4 or 8: a lane per strip of 4 adjacent columns of one block (16-byte
 //                        accesses), the default for such shapes
 //   quant_pack3d_kernel  one thread per packed 32-bit word
@@ -326,58 +326,6 @@ quant3d_strip_kernel(const XT* __restrict__ x, const LT* lfc, const uint32_t* ws
             }
         }
     });
-}
-
-// Decompress with the lane-per-strip layout (W % 4 == 0, B = 4 or 8, Q in {2,4,8}): the lane reads its block's
-// low-frequency value once, then per row of 4 elements one byte / half-word / word of codes, one look-up in the
-// sample's dequantisation table and one 16-byte (fp32) store.  Two lanes per strip (upper and lower rows).
-// grid = (ceil(slots per sample / 256), N)
-template <typename XT, typename LT, int Q, int P2>
-__global__ void __launch_bounds__(256)
-decompress3d_strip_kernel(const LT* lfc, const uint32_t* packed, const float* stats,
-                          XT* xhat, Shape3 s, uint32_t slots_per_sample) {
-    constexpr uint32_t LPB = P2 / 4;
-    __shared__ DeqTable<Q> table;
-    const uint32_t n = blockIdx.y;
-    griddep_wait();
-    griddep_launch();
-    table.build(stats[2 * (size_t)n + 1], stats[2 * (size_t)n]);
-    __syncthreads();
-    const uint32_t slot = blockIdx.x * 256u + threadIdx.x;
-    if (slot >= slots_per_sample) return;
-    const uint32_t spr = s.Wb * LPB * 2u;
-    const uint32_t rowid = slot / spr;                                 // (c * Db + bd) * Hb + bh
-    const uint32_t sq = slot - rowid * spr;
-    const uint32_t half = sq & 1u, strip = sq >> 1;
-    const uint32_t bw = strip / LPB, cw = (strip % LPB) * 4u;
-    const uint32_t vd = rowid / s.Hb, bh = rowid - vd * s.Hb;
-    const uint32_t c = vd / s.Db, bd = vd - c * s.Db;
-    const uint32_t d0 = bd * s.B, h0 = bh * s.B, w0 = bw * s.B;
-    const uint32_t nd = min(s.B, s.D - d0), nh = min(s.B, s.H - h0), nw = min(s.B, s.W - w0);
-    if (cw >= nw) return;
-    const float lf = Elem<LT>::load(lfc + (size_t)n * s.C * s.TPV + (size_t)rowid * s.Wb + bw);
-    const uint32_t e0 = c * s.DHW + (d0 * s.H + h0) * s.W + w0 + cw;   // in-sample index of the strip's first element
-    const uint64_t quad0 = ((uint64_t)n * s.CDHW + e0) >> 2;
-    XT* out = xhat + (size_t)n * s.CDHW + e0;
-    const uint32_t W4 = s.W >> 2, HW4 = s.HW >> 2;
-    const bool full = nd == (uint32_t)P2;
-    const uint32_t r_end = min(nh, (half + 1u) * (P2 / 2u));
-    for (uint32_t r = half * (P2 / 2u); r < r_end; ++r) {
-        uint32_t bits[P2];
-#pragma unroll
-        for (int k = 0; k < P2; ++k) {
-            bits[k] = 0u;
-            if (full || (uint32_t)k < nd) bits[k] = quad_bits<Q>(packed, quad0 + (uint64_t)r * W4 + (uint64_t)k * HW4);
-        }
-#pragma unroll
-        for (int k = 0; k < P2; ++k) {
-            if (full || (uint32_t)k < nd) {
-                const float4 hq = table.quad(bits[k]);
-                Quad<XT>::store(out + (size_t)r * s.W + (size_t)k * s.HW, __fadd_rn(lf, hq.x), __fadd_rn(lf, hq.y), __fadd_rn(lf, hq.z),
-                                __fadd_rn(lf, hq.w));
-            }
-        }
-    }
 }
 
 // position of a flat in-sample index

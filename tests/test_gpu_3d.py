@@ -52,6 +52,8 @@ CASES = [
     # warps that straddle volumes and samples
     ((3, 5, 6, 10, 12), 4, 2, "f32", "f32"), ((2, 3, 9, 7, 16), 4, 4, "bf16", "bf16"), ((5, 1, 4, 4, 8), 4, 2, "f32", "f32"),
     ((7, 3, 3, 5, 12), 8, 8, "f32", "bf16"), ((2, 2, 17, 9, 40), 8, 2, "bf16", "f32"),
+    # decompress by slices: rows that are no whole sectors, ragged heights and depths, a block of 16, a block per slice
+    ((2, 3, 12, 20, 28), 16, 4, "f32", "f32"), ((2, 3, 9, 13, 20), 8, 1, "bf16", "bf16"), ((3, 2, 33, 3, 8), 4, 8, "f32", "f32"),
 ]
 
 
