@@ -300,17 +300,38 @@ __device__ __forceinline__ uint2 quad_table_entry(uint32_t idx, uint32_t HW, uin
     return make_uint2(o[0] | (o[1] << 16), o[2] | (o[3] << 16));
 }
 
-template <typename XT, typename LT, int Q, int QPT>
+// 3-D maps, a volume for a plane (HW, TPP count a volume's elements and blocks, by_hw divides by them)
+struct DecFlat3 : DecFlat {
+    uint32_t slice, tiles;   // elements and blocks of a slice
+    FastDiv by_slice;
+};
+__device__ __forceinline__ uint2 flat_entry(const DecFlat& d, uint32_t idx) {
+    return quad_table_entry(idx, d.HW, d.W, d.Wb, d.TPP, d.by_hw, d.by_w, d.by_b);
+}
+__device__ __forceinline__ uint2 flat_entry(const DecFlat3& d, uint32_t idx) {
+    uint32_t o[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t e = 4u * idx + (uint32_t)i;
+        const uint32_t dp = fdiv(e, d.by_hw), pos = e - dp * d.HW;
+        const uint32_t z = fdiv(pos, d.by_slice), at = pos - z * d.slice;
+        const uint32_t h = fdiv(at, d.by_w), w = at - h * d.W;
+        o[i] = dp * d.TPP + fdiv(z, d.by_b) * d.tiles + fdiv(h, d.by_b) * d.Wb + fdiv(w, d.by_b);
+    }
+    return make_uint2(o[0] | (o[1] << 16), o[2] | (o[3] << 16));
+}
+
+template <typename XT, typename LT, int Q, int QPT, typename GEOM>
 __global__ void __launch_bounds__(256)
 decompress_flat_kernel(const LT* lfc, const uint32_t* packed,
-                       const float* stats, XT* xhat, DecFlat d) {
+                       const float* stats, XT* xhat, GEOM d) {
     extern __shared__ __align__(16) uint32_t flat_smem[];
     uint2* quad_of = reinterpret_cast<uint2*>(flat_smem);            // quad inside a period -> where its 4 low-frequency values sit
     float* lfc_s = reinterpret_cast<float*>(flat_smem + d.table_words);   // low-frequency values of this CTA's planes
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
     for (uint32_t idx = threadIdx.x; idx < d.period; idx += 256u)
-        quad_of[idx] = quad_table_entry(idx, d.HW, d.W, d.Wb, d.TPP, d.by_hw, d.by_w, d.by_b);
+        quad_of[idx] = flat_entry(d, idx);
     griddep_wait();
     griddep_launch();
     // the codes of this thread's quads are asked for first: their trip to memory overlaps the rest of the set-up

@@ -736,7 +736,7 @@ div_status div_decompress(const div_desc* desc, const void* comp_dev, size_t com
                 d.by_period = make_fastdiv(d.period);
                 d.planes_per_cta = flat_planes_per_cta(4u * per_block, s.HW);
                 dim3 grid((d.qps + per_block - 1) / per_block, s.N);
-                return launch_pdl(decompress_flat_kernel<XT, LT, Q, FLAT_QPT>, grid, 256, flat_smem_bytes(4u * per_block, s.HW, s.TPP), stream,
+                return launch_pdl(decompress_flat_kernel<XT, LT, Q, FLAT_QPT, DecFlat>, grid, 256, flat_smem_bytes(4u * per_block, s.HW, s.TPP), stream,
                                   lfc, packed, stats, (XT*)xhat_dev, d);
             } else {
                 const uint64_t g = (nwords + 255) / 256;
@@ -1176,6 +1176,37 @@ div_status div_decompress_3d(const div_desc3d* desc, const void* comp_dev, size_
                 return launch_pdl(decompress3d_quad_kernel<XT, LT, decltype(q)::value, DEC_QPT>, grid, 256, 0, stream,
                                   (const LT*)(blob + lo.lfc_off), (const uint32_t*)(blob + lo.packed_off),
                                   (const float*)(blob + lo.stats_off), (XT*)xhat_dev, g3);
+            });
+        }
+        // other widths and blocks: volumes as the flat 2-D kernel takes planes, where one's quad table and block values fit (up to 8192
+        // elements, about twice what a CTA rebuilds).  16 x 56 x 8 x 21 x 21 bfloat16 23.8 -> 5.6 us, 6 x 64 x 13 x 7 x 7 5.9 -> 2.6.
+        if (s.CDHW % 4u == 0 && s.CDHW < (1u << 31) && s.DHW <= FLAT_MAX_HW && s.N <= 65535u &&
+            flat_smem_bytes(4u * 256u * FLAT_QPT, s.DHW, s.TPV) <= 40000) {
+            DecFlat3 d;
+            d.qps = s.CDHW / 4u;
+            d.C = s.C;
+            d.TPP = s.TPV;
+            d.Wb = s.Wb;
+            d.HW = s.DHW;
+            d.W = s.W;
+            d.B = s.B;
+            d.by_hw = make_fastdiv(s.DHW);
+            d.by_w = make_fastdiv(s.W);
+            d.by_b = make_fastdiv(s.B);
+            const uint32_t per_block = 256u * FLAT_QPT;
+            d.table_words = quad_table_words(s.DHW);
+            d.period = quad_period(s.DHW);
+            d.period_planes = quad_period_planes(s.DHW);
+            d.by_period = make_fastdiv(d.period);
+            d.planes_per_cta = flat_planes_per_cta(4u * per_block, s.DHW);
+            d.slice = s.HW;
+            d.tiles = s.Hb * s.Wb;
+            d.by_slice = make_fastdiv(s.HW);
+            const dim3 grid((d.qps + per_block - 1) / per_block, s.N);
+            return dispatch_q(desc->qbits, [&](auto q) -> div_status {
+                return launch_pdl(decompress_flat_kernel<XT, LT, decltype(q)::value, FLAT_QPT, DecFlat3>, grid, 256,
+                                  flat_smem_bytes(4u * per_block, s.DHW, s.TPV), stream, (const LT*)(blob + lo.lfc_off),
+                                  (const uint32_t*)(blob + lo.packed_off), (const float*)(blob + lo.stats_off), (XT*)xhat_dev, d);
             });
         }
         return dispatch_q(desc->qbits, [&](auto q) -> div_status {

@@ -54,6 +54,9 @@ CASES = [
     ((7, 3, 3, 5, 12), 8, 8, "f32", "bf16"), ((2, 2, 17, 9, 40), 8, 2, "bf16", "f32"),
     # decompress by slices: rows that are no whole sectors, ragged heights and depths, a block of 16, a block per slice
     ((2, 3, 12, 20, 28), 16, 4, "f32", "f32"), ((2, 3, 9, 13, 20), 8, 1, "bf16", "bf16"), ((3, 2, 33, 3, 8), 4, 8, "f32", "f32"),
+    # flat decompress: table periods of one, two and four volumes, a CTA's share of many volumes and of part of one, widest volume taken
+    ((2, 40, 4, 7, 7), 8, 2, "f32", "f32"), ((3, 6, 5, 3, 6), 4, 4, "bf16", "bf16"), ((2, 8, 13, 13, 13), 8, 8, "f32", "bf16"),
+    ((1, 3, 32, 14, 14), 4, 2, "f32", "f32"), ((2, 2, 8, 31, 33), 8, 1, "f32", "f32"),
 ]
 
 
