@@ -389,11 +389,21 @@ struct DecRows {
     uint32_t bands;          // most bands that a CTA touches
     uint32_t step_rows, step_cols;      // 1024 elements = step_rows rows and step_cols columns
     FastDiv by_w, by_h, by_b;
+    __device__ __forceinline__ uint32_t lfc_row(uint32_t band) const { return band; }
 };
-template <typename XT, typename LT, int Q, int QPT>
+// 3-D maps, slices for planes: the bands of the B slices of a block have the same low-frequency values
+struct DecRows3 : DecRows {
+    uint32_t D, Db;
+    FastDiv by_hb, by_depth;
+    __device__ __forceinline__ uint32_t lfc_row(uint32_t band) const {
+        const uint32_t slice = fdiv(band, by_hb), vol = fdiv(slice, by_depth);
+        return (vol * Db + fdiv(slice - vol * D, by_b)) * Hb + (band - slice * Hb);
+    }
+};
+template <typename XT, typename LT, int Q, int QPT, typename GEOM>
 __global__ void __launch_bounds__(256)
 decompress_rows_kernel(const LT* lfc, const uint32_t* packed,
-                       const float* stats, XT* xhat, const DecRows d) {
+                       const float* stats, XT* xhat, const GEOM d) {
     extern __shared__ __align__(16) float rows_smem[];
     __shared__ DeqTable<Q> table;
     const uint32_t n = blockIdx.y;
@@ -408,12 +418,11 @@ decompress_rows_kernel(const LT* lfc, const uint32_t* packed,
     const uint32_t first_row = fdiv(blockIdx.x * (1024u * QPT), d.by_w);
     const uint32_t first_plane = fdiv(first_row, d.by_h);
     const uint32_t band0 = first_plane * d.Hb + fdiv(first_row - first_plane * d.H, d.by_b);      // bands counted through the sample
-    const LT* src = lfc + (uint64_t)n * d.tiles + (uint64_t)band0 * d.Wb;
-    const uint32_t left = d.tiles - band0 * d.Wb;
+    const LT* src = lfc + (uint64_t)n * d.tiles;
     for (uint32_t i = threadIdx.x; i < d.bands * d.W; i += 256u) {
         const uint32_t b = fdiv(i, d.by_w);
-        const uint32_t t = b * d.Wb + fdiv(i - b * d.W, d.by_b);
-        rows_smem[i] = t < left ? Elem<LT>::load(src + t) : 0.f;
+        const uint32_t t = d.lfc_row(band0 + b) * d.Wb + fdiv(i - b * d.W, d.by_b);
+        rows_smem[i] = t < d.tiles ? Elem<LT>::load(src + t) : 0.f;
     }
     __syncthreads();
     uint32_t row = fdiv(4u * q0, d.by_w);

@@ -57,6 +57,9 @@ CASES = [
     # flat decompress: table periods of one, two and four volumes, a CTA's share of many volumes and of part of one, widest volume taken
     ((2, 40, 4, 7, 7), 8, 2, "f32", "f32"), ((3, 6, 5, 3, 6), 4, 4, "bf16", "bf16"), ((2, 8, 13, 13, 13), 8, 8, "f32", "bf16"),
     ((1, 3, 32, 14, 14), 4, 2, "f32", "f32"), ((2, 2, 8, 31, 33), 8, 1, "f32", "f32"),
+    # decompress by rows (volumes beyond the flat kernel's): quads across rows, slices and volumes, a block higher than a slice
+    ((2, 2, 34, 15, 19), 8, 2, "f32", "f32"), ((1, 4, 13, 27, 27), 4, 4, "bf16", "bf16"), ((1, 4, 70, 11, 11), 64, 8, "f32", "bf16"),
+    ((2, 4, 9, 31, 31), 3, 1, "f32", "f32"), ((1, 2, 700, 3, 5), 8, 2, "f32", "f32"),
 ]
 
 
