@@ -1004,6 +1004,35 @@ Quad3 make_quad3(const Shape3& s) {
     return g;
 }
 
+// slices as the row kernels take planes: whether they do, and how
+bool rows3(const Shape3& s, DecRows3* d) {
+    Shape sl = Shape();
+    sl.H = s.H;
+    sl.W = s.W;
+    sl.B = s.B;
+    sl.Hb = s.Hb;
+    sl.HW = s.HW;
+    const uint64_t bands = rows_bands(sl, 1024u * FLAT_QPT);
+    if (s.W < 4u || s.CDHW % 4u != 0 || s.CDHW >= (1u << 31) || s.N > 65535u || bands * s.W * 4u > 40000u) return false;
+    d->qps = s.CDHW / 4u;
+    d->tiles = s.C * s.TPV;
+    d->H = s.H;
+    d->W = s.W;
+    d->Hb = s.Hb;
+    d->Wb = s.Wb;
+    d->bands = (uint32_t)bands;
+    d->step_rows = 1024u / s.W;
+    d->step_cols = 1024u % s.W;
+    d->by_w = make_fastdiv(s.W);
+    d->by_h = make_fastdiv(s.H);
+    d->by_b = make_fastdiv(s.B);
+    d->D = s.D;
+    d->Db = s.Db;
+    d->by_hb = make_fastdiv(s.Hb);
+    d->by_depth = make_fastdiv(s.D);
+    return true;
+}
+
 void make_layout3(const div_desc3d* d, const Shape3& s, div_layout* out) {
     out->lfc_off = 0;
     out->lfc_bytes = s.tiles * dtype_bytes(d->lfc_dtype);
@@ -1110,6 +1139,22 @@ div_status div_compress_3d(const div_desc3d* desc, const void* x_dev, void* comp
             }
             return launch_status();
         }
+        // Below a million elements the few CTAs wait for their bands' values (5 x 32 x 13 x 13 x 13, B = 4: 10.4 us a thread per word, 14.8 by rows);
+        // above, both compress kernels: 11 x 88 x 8 x 50 x 50 142.4 -> 66.6 us, 13 x 88 x 8 x 13 x 13 21.9 -> 19.8, 26 random ones 1.1 to 2.1 times faster.
+        DecRows3 d;
+        if (desc->qbits != 1 && s.total >= (1u << 20) && rows3(s, &d)) {
+            const dim3 grid((d.qps + 256u * FLAT_QPT - 1) / (256u * FLAT_QPT), s.N);
+            void* packed = blob + lo.packed_off;
+            float* stats = (float*)(blob + lo.stats_off);
+            const XT* xs = (const XT*)x_dev;
+            const LT* lf = (const LT*)(blob + lo.lfc_off);
+            const size_t smem = 4u * d.bands * d.W;
+            switch (desc->qbits) {
+                case 2: return launch_pdl(quant3d_rows_kernel<XT, LT, 2, FLAT_QPT>, grid, 256, smem, stream, xs, lf, ws, packed, stats, d, seed);
+                case 4: return launch_pdl(quant3d_rows_kernel<XT, LT, 4, FLAT_QPT>, grid, 256, smem, stream, xs, lf, ws, packed, stats, d, seed);
+                default: return launch_pdl(quant3d_rows_kernel<XT, LT, 8, FLAT_QPT>, grid, 256, smem, stream, xs, lf, ws, packed, stats, d, seed);
+            }
+        }
         return dispatch_q(desc->qbits, [&](auto q) -> div_status {
             quant_pack3d_kernel<XT, LT, decltype(q)::value><<<(unsigned)g2, 256, 0, stream>>>(
                 (const XT*)x_dev, (const LT*)(blob + lo.lfc_off), ws, (uint32_t*)(blob + lo.packed_off),
@@ -1210,31 +1255,8 @@ div_status div_decompress_3d(const div_desc3d* desc, const void* comp_dev, size_
             });
         }
         // larger volumes: slices as the row kernel takes planes (4 x 48 x 32 x 50 x 50 65.6 -> 18.8 us, 16 x 16 x 16 x 64 x 21 bfloat16 32.9 -> 8.5)
-        Shape sl = Shape();
-        sl.H = s.H;
-        sl.W = s.W;
-        sl.B = s.B;
-        sl.Hb = s.Hb;
-        sl.HW = s.HW;
-        const uint64_t bands = rows_bands(sl, 1024u * FLAT_QPT);
-        if (s.W >= 4u && s.CDHW % 4u == 0 && s.CDHW < (1u << 31) && s.N <= 65535u && bands * s.W * 4u <= 40000u) {
-            DecRows3 d;
-            d.qps = s.CDHW / 4u;
-            d.tiles = s.C * s.TPV;
-            d.H = s.H;
-            d.W = s.W;
-            d.Hb = s.Hb;
-            d.Wb = s.Wb;
-            d.bands = (uint32_t)bands;
-            d.step_rows = 1024u / s.W;
-            d.step_cols = 1024u % s.W;
-            d.by_w = make_fastdiv(s.W);
-            d.by_h = make_fastdiv(s.H);
-            d.by_b = make_fastdiv(s.B);
-            d.D = s.D;
-            d.Db = s.Db;
-            d.by_hb = make_fastdiv(s.Hb);
-            d.by_depth = make_fastdiv(s.D);
+        DecRows3 d;
+        if (rows3(s, &d)) {
             const dim3 grid((d.qps + 256u * FLAT_QPT - 1) / (256u * FLAT_QPT), s.N);
             return dispatch_q(desc->qbits, [&](auto q) -> div_status {
                 return launch_pdl(decompress_rows_kernel<XT, LT, decltype(q)::value, FLAT_QPT, DecRows3>, grid, 256, 4u * d.bands * d.W, stream,

@@ -489,6 +489,78 @@ quant3d_quad_kernel(const XT* __restrict__ x, const LT* lfc, const uint32_t* ws,
     }
 }
 
+// Quantise half for any width from 4 on, any block and Q in {2,4,8}: decompress_rows_kernel the other way round.  A CTA takes 1024 * QPT
+// consecutive elements, from the end of the tensor backwards (what the statistics kernel read last is still in the L2); the
+// low-frequency values of the bands that it touches stand in shared memory, W values per band.  In the place of a thread per packed word
+// that walks position by position, with its loads of x 4 * 32 / Q elements apart.
+template <typename XT, typename LT, int Q, int QPT>
+__global__ void __launch_bounds__(256)
+quant3d_rows_kernel(const XT* __restrict__ x, const LT* lfc, const uint32_t* ws, void* __restrict__ packed_v,
+                    float* __restrict__ stats, const DecRows3 d, uint64_t seed) {
+    typedef typename PackedUnit<Q>::type OutT;
+    extern __shared__ __align__(16) float rows_smem[];
+    const uint32_t n = gridDim.y - 1u - blockIdx.y, block = gridDim.x - 1u - blockIdx.x;
+    const uint64_t sample_quad0 = (uint64_t)n * d.qps;
+    const uint32_t q0 = block * (256u * QPT) + threadIdx.x;
+    uint64_t xy[QPT], zw[QPT];
+    griddep_wait();
+    griddep_launch();
+#pragma unroll
+    for (int k = 0; k < QPT; ++k) {
+        const uint32_t q = q0 + k * 256u;
+        xy[k] = 0ull;
+        zw[k] = 0ull;
+        if (q < d.qps) StripRow2<XT>::load(reinterpret_cast<const unsigned char*>(x + (sample_quad0 + q) * 4u), xy[k], zw[k]);
+    }
+    const uint32_t* slot = ws + WS_HEADER_WORDS + (size_t)n * WS_SLOT_WORDS;
+    const QParams qp = make_qparams(key_float(~slot[0]), key_float(slot[1]), Q);
+    if (block == 0 && threadIdx.x == 0) {
+        stats[2 * (size_t)n + 0] = qp.delta;
+        stats[2 * (size_t)n + 1] = qp.step;
+    }
+    const uint32_t first_row = fdiv(block * (1024u * QPT), d.by_w);
+    const uint32_t first_plane = fdiv(first_row, d.by_h);
+    const uint32_t band0 = first_plane * d.Hb + fdiv(first_row - first_plane * d.H, d.by_b);      // bands counted through the sample
+    const LT* src = lfc + (uint64_t)n * d.tiles;
+    for (uint32_t i = threadIdx.x; i < d.bands * d.W; i += 256u) {
+        const uint32_t b = fdiv(i, d.by_w);
+        const uint32_t t = d.lfc_row(band0 + b) * d.Wb + fdiv(i - b * d.W, d.by_b);
+        rows_smem[i] = t < d.tiles ? Elem<LT>::load(src + t) : 0.f;
+    }
+    __syncthreads();
+    const uint64_t delta2 = pk2(qp.delta, qp.delta), scale2 = pk2(qp.scale, qp.scale);
+    const uint64_t base = rng_sample_base(seed, n);
+    OutT* out = reinterpret_cast<OutT*>(packed_v) + sample_quad0;
+    uint32_t row = fdiv(4u * q0, d.by_w);
+    uint32_t w = 4u * q0 - row * d.W;
+    uint32_t plane = fdiv(row, d.by_h);
+    uint32_t h = row - plane * d.H;
+#pragma unroll
+    for (int k = 0; k < QPT; ++k) {
+        const uint32_t q = q0 + k * 256u;
+        if (q < d.qps) {
+            const uint32_t band = fdiv(h, d.by_b);
+            const uint32_t at = (plane * d.Hb + band - band0) * d.W + w;
+            // where the next row lies in the same band the walk along the row starts over, else it goes on into the next band
+            const uint32_t back = (h + 1u != d.H && fdiv(h + 1u, d.by_b) == band) ? d.W : 0u;
+            float lf[4];
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) lf[i] = rows_smem[at + i - (w + i >= d.W ? back : 0u)];
+            out[q] = (OutT)quant_row<Q>(sub2_rn(xy[k], pk2(lf[0], lf[1])), sub2_rn(zw[k], pk2(lf[2], lf[3])), 0ull, delta2, scale2, rng_group(base, q));
+        }
+        w += d.step_cols;
+        h += d.step_rows;
+        if (w >= d.W) {
+            w -= d.W;
+            ++h;
+        }
+        while (h >= d.H) {
+            h -= d.H;
+            ++plane;
+        }
+    }
+}
+
 template <typename XT, typename LT, int Q, int QPT>
 __global__ void __launch_bounds__(256)
 decompress3d_quad_kernel(const LT* lfc, const uint32_t* packed,

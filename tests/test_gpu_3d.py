@@ -60,6 +60,8 @@ CASES = [
     # decompress by rows (volumes beyond the flat kernel's): quads across rows, slices and volumes, a block higher than a slice
     ((2, 2, 34, 15, 19), 8, 2, "f32", "f32"), ((1, 4, 13, 27, 27), 4, 4, "bf16", "bf16"), ((1, 4, 70, 11, 11), 64, 8, "f32", "bf16"),
     ((2, 4, 9, 31, 31), 3, 1, "f32", "f32"), ((1, 2, 700, 3, 5), 8, 2, "f32", "f32"),
+    # quantise by rows (from 2^20 elements on): quads across rows, slices and samples' ends, many bands a CTA
+    ((2, 8, 16, 64, 65), 8, 2, "f32", "f32"), ((3, 7, 13, 62, 66), 4, 4, "bf16", "bf16"), ((1, 600, 16, 11, 11), 8, 8, "f32", "bf16"),
 ]
 
 
