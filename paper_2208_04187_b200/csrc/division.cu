@@ -1140,7 +1140,7 @@ div_status div_compress_3d(const div_desc3d* desc, const void* x_dev, void* comp
             return launch_status();
         }
         // Below a million elements the few CTAs wait for their bands' values (5 x 32 x 13 x 13 x 13, B = 4: 10.4 us a thread per word, 14.8 by rows);
-        // above, both compress kernels: 11 x 88 x 8 x 50 x 50 142.4 -> 66.6 us, 13 x 88 x 8 x 13 x 13 21.9 -> 19.8, 26 random ones 1.1 to 2.1 times faster.
+        // above, both compress kernels: 11 x 88 x 8 x 50 x 50 142.4 -> 66.6 us, 13 x 88 x 8 x 13 x 13 21.9 -> 19.8, 28 random ones 1.1 to 2.1 times faster.
         DecRows3 d;
         if (desc->qbits != 1 && s.total >= (1u << 20) && rows3(s, &d)) {
             const dim3 grid((d.qps + 256u * FLAT_QPT - 1) / (256u * FLAT_QPT), s.N);

@@ -8,8 +8,9 @@
 //   lfc_stats3d_strip_kernel, quant3d_strip_kernel
 //                        W % 4 == 0 and B = 4 or 8: a lane per strip of 4 adjacent columns of one block (16-byte
 //                        accesses), the default for such shapes
+//   quant3d_rows_kernel  other widths, from a million elements on: consecutive elements, low-frequency values in shared memory
 //   quant_pack3d_kernel  one thread per packed 32-bit word
-//   decompress3d_kernel  one thread per packed 32-bit word
+//   decompress3d_kernel  one thread per packed 32-bit word, for what the kernels of decompress.cuh do not take slice by slice
 // x is read twice by compress (the second time from L2 when the tensor fits).
 #pragma once
 
