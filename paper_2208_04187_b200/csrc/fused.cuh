@@ -438,6 +438,7 @@ inline uint32_t gcd_u32(uint32_t a, uint32_t b) {
     }
     return a;
 }
+inline uint32_t lcm_u32(uint32_t a, uint32_t b) { return a / gcd_u32(a, b) * b; }
 
 constexpr int FUSED_CONSUMER_WARPS = 8;
 constexpr int FUSED_THREADS = 32 * (1 + FUSED_CONSUMER_WARPS);

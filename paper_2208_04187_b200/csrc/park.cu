@@ -31,7 +31,9 @@
 // Why no wait can last: take the first sample that is not complete and one of its units that has not been reduced, chunk c of CTA Y, worker w.
 // w can be stuck on the parameters of a chunk that is at least PARK_DEPTH * sets before c; a CTA has at most that many chunks of one
 // sample (plan_park), so that chunk's sample is an earlier one, which is complete.  Or chunk c has not landed because its stage is
-// still being read: by a worker that is stuck in the same way, on a chunk even further back.
+// still being read: by a worker that is stuck in the same way, on a chunk even further back.  Or chunk c has not been asked for because
+// chunk c - ahead has not landed, which nothing holds up: a record has not been filled again by then (ahead <= stages < PARK_CHUNKS; a
+// parity tells a fill from the next and no more).
 // Chunk records are reused after PARK_CHUNKS chunks: while chunk a is not quantised its worker does not read chunk a + PARK_DEPTH * sets,
 // so that nothing beyond the PARK_MAX_STAGES chunks from there on is on its way.
 #include "halves.cuh"
@@ -55,25 +57,6 @@ struct ParkParams {
     uint32_t expected_chunks;
     uint32_t tail_rows;
     float inv_cnt[4], cnt[4];
-};
-
-// what the producer posts for a chunk
-struct ParkDesc {
-    uint64_t lfc0;                 // its first tile in the tensor
-    uint64_t quad0;                // its first group of 4 elements in the tensor
-    uint64_t ctr0;                 // counter of the random stream of that group
-    uint32_t ntiles;
-    uint32_t n;                    // sample
-};
-struct ParkCtl {
-    uint64_t full[PARK_CHUNKS];    // the chunk has landed
-    uint64_t folded[PARK_CHUNKS];  // all its units are reduced
-    uint64_t par[PARK_CHUNKS];     // its sample's parameters are there
-    uint64_t empty[PARK_MAX_STAGES];
-    ParkDesc desc[PARK_CHUNKS];
-    float delta[PARK_CHUNKS], scale[PARK_CHUNKS];
-    uint32_t kmin[PARK_CHUNKS], kmax[PARK_CHUNKS];
-    uint32_t failed, tmem;
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -486,65 +469,6 @@ park_kernel(const __grid_constant__ ParkParams p) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-bool plan_park(const div_desc* d, const Shape& s, ParkPlan* out) {
-    const uint32_t sx = d->x_dtype == DIV_F32 ? 4u : 2u;
-    if (s.W % 4 != 0 || !(s.B == 4 || s.B == 8) || s.P2 != s.B || d->qbits == 1) return false;
-    // bulk copies start on 16-byte boundaries and move multiples of 16 bytes
-    if (((uint64_t)s.CHW * sx) % 16u != 0 || ((uint64_t)s.HW * sx) % 16u != 0 || ((uint64_t)s.B * s.W * sx) % 16u != 0) return false;
-    const DeviceInfo di = device_info();
-    if (!di.ok || di.sms < 1) return false;
-    ParkPlan pl = ParkPlan();
-    pl.spb = s.W / 4u;
-    pl.paired = (s.P2 == 8u && (pl.spb & 1u)) ? 1u : 0u;
-    const uint64_t bands = (uint64_t)s.C * s.Hb;
-    if (bands >= (1ull << 31)) return false;
-    pl.bands_per_sample = (uint32_t)bands;
-    pl.uniform = (s.H % s.B == 0) ? 1u : 0u;
-    const uint32_t per_unit = 32u * (8u / s.P2);
-    const uint32_t geo1 = pl.uniform ? 1u : s.Hb;
-    const uint32_t geo = (pl.paired && (geo1 & 1u)) ? 2u * geo1 : geo1;
-    const uint64_t geo_bytes = (pl.uniform ? (uint64_t)s.B * s.W * sx : (uint64_t)s.HW * sx) * (geo / geo1);
-    const uint32_t fill = per_unit / gcd_u32(per_unit, pl.spb);
-    const uint32_t both = lcm_u32(geo, fill);
-    const uint64_t both_bytes = geo_bytes * (both / geo);
-    const uint64_t target = (uint64_t)PARK_CHUNK_ELEMS * sx;
-    uint32_t G;
-    if (both_bytes <= target) G = (uint32_t)(target / both_bytes) * both;
-    else if (geo_bytes <= target) G = (uint32_t)(target / geo_bytes) * geo;
-    else if (geo_bytes <= PARK_MOST_BYTES) G = geo;
-    else return false;
-    const uint32_t bands_up = (pl.bands_per_sample + geo - 1u) / geo * geo;
-    if (G > bands_up) G = bands_up;
-    pl.G = G;
-    pl.slots = G * pl.spb;
-    if (pl.slots > 4096u || G * s.Wb > 2048u) return false;
-    pl.nf = (pl.slots + per_unit - 1u) / per_unit;
-    pl.chunk_elems = pl.uniform ? G * s.B * s.W : (G / s.Hb) * s.HW;
-    if (pl.chunk_elems >= (1u << 15)) return false;
-    pl.chunks_per_sample = (pl.bands_per_sample + G - 1u) / G;
-    pl.stage_bytes = (pl.chunk_elems * sx + 127u) & ~127u;
-    const uint32_t fixed = pl.nf * per_unit * 4u + (uint32_t)sizeof(ParkCtl) + 128u;
-    if ((uint32_t)di.smem_optin < fixed + 2u * pl.stage_bytes) return false;
-    pl.stages = ((uint32_t)di.smem_optin - fixed) / pl.stage_bytes;
-    if (pl.stages > (uint32_t)PARK_MAX_STAGES) pl.stages = PARK_MAX_STAGES;
-    pl.smem_bytes = pl.stages * pl.stage_bytes + fixed;
-    pl.ahead = PARK_AHEAD_BYTES / pl.stage_bytes;
-    if (pl.ahead < 2u) pl.ahead = 2u;
-    const uint64_t total = (uint64_t)pl.chunks_per_sample * s.N;
-    if (total >= (1ull << 30)) return false;
-    pl.total_chunks = (uint32_t)total;
-    pl.grid = total < (uint64_t)di.sms ? (uint32_t)total : (uint32_t)di.sms;
-    if (pl.nf > PARK_WORKERS) return false;
-    pl.sets = PARK_WORKERS / pl.nf;
-    if (pl.sets > PARK_MAX_SETS) pl.sets = PARK_MAX_SETS;
-    // a CTA's units of one sample are all parked at once
-    const uint32_t per_cta = (pl.chunks_per_sample - 1u) / pl.grid + 1u;
-    pl.per_cta = per_cta;
-    if (per_cta > PARK_DEPTH * pl.sets) return false;
-    *out = pl;
-    return true;
-}
-
 template <typename XT, typename LT, int P2, int Q>
 static div_status launch_park(const ParkParams& prm, cudaStream_t st) {
     auto kern = park_kernel<XT, LT, P2, Q>;

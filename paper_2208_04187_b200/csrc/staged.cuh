@@ -717,7 +717,6 @@ staged_kernel(const SParams p) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-inline uint32_t lcm_u32(uint32_t a, uint32_t b) { return a / gcd_u32(a, b) * b; }
 
 inline div_status plan_staged(const div_desc* d, const Shape& s, SPlan* out) {
     const uint32_t sx = d->x_dtype == DIV_F32 ? 4u : 2u;

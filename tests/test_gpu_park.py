@@ -50,6 +50,20 @@ def test_parking_kernel_matches_the_two_pass_kernels(case):
     assert plan.fused == 6 and plan.threads == 1024 and plan.lag == 0
 
 
+# More chunks a CTA than it has records for them (from 64 on), twice over for the small samples: stages of 128 to 640 bytes, a
+# unit per chunk; then as many units per chunk as there are workers.
+MANY_ROUNDS = [(20000, c, 4, 4, 4, 2, "f32", "f32") for c in (2, 4, 6, 8, 10)] + [
+    (20000, 2, 8, 8, 8, 2, "f32", "f32"), (20000, 4, 8, 8, 8, 4, "bf16", "bf16"), (1024, 512, 2, 64, 8, 2, "f32", "f32")]
+
+
+@pytest.mark.parametrize("flags", [0, STAGED], ids=["default", "staged"])
+@pytest.mark.parametrize("case", MANY_ROUNDS, ids=lambda c: "x".join(map(str, c)))
+def test_many_rounds(case, flags):
+    plan = same_bytes(case, flags)
+    if flags and torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert plan.threads == 1024 and plan.lag == 0 and case[0] * plan.chunks_per_sample > 64 * plan.grid
+
+
 # the last one's planes are more than a chunk
 @pytest.mark.parametrize("case", [(64, 64, 112, 112, 8, 2, "f32", "f32"), (128, 160, 32, 32, 4, 4, "bf16", "bf16"), (64, 24, 100, 112, 8, 2, "f32", "f32")], ids=lambda c: "x".join(map(str, c)))
 def test_parking_kernel_by_default(case):
