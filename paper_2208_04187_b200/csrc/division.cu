@@ -317,12 +317,21 @@ bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPl
 // 1.3 times faster in the geometric mean there (50 x 2048 x 16 x 16 with B = 4 49.5 -> 27.8 us, 96 x 432 x 15 x 56 with B = 4 74.9 -> 37.2 us).
 // The strip kernel's time is fitted once more over its small maps (1 x 56 x 112 x 112 5.9 against 7.2 us, 4.8 MB on the parking kernel's).
 // The staged kernel keeps samples of which less than two and a half fit the parked units (8 x 1840 x 56 x 56 58.5 against 68.1 us).
+// 1-D maps stay with the line kernels, whose second read of x is from the L1 or L2 and whose units hold whole rows (here a strip has one
+// row of four or eight): of 21 random ones up to 8 MB none is faster here and the geometric mean 1.33 times slower (355 x 45 x 64 bfloat16
+// 8.3 against 14.5 us, 4 x 936 x 512 with B = 4 10.5 against 13.4 us).  (The general kernels run no map that plan_park accepts.)
 bool choose_park(const div_desc* d, const Shape& s, uint32_t flags, const ClusterPlan* cl, int code, ParkPlan* out) {
     if (flags != 0u) return code == 6 && plan_park(d, s, out);
     if ((cl && cl->turns64 <= 64u) || !plan_park(d, s, out)) return false;
     if (cl) return out->sets >= 2u && park_ns(*out) <= cluster_ns(s, *cl);      // (a chunk at a time: 96 x 16 x 100 x 100 bfloat16 21.8 -> 24.6 us)
-    if (code == 6) return 5u * out->per_cta <= 2u * PARK_DEPTH * out->sets && park_ns(*out) <= other_ns(s, code);
-    return park_ns(*out) <= (code == 2 ? 4600u + s.total * 155u / 100000u : other_ns(s, code));
+    switch (code) {
+        case 6: return 5u * out->per_cta <= 2u * PARK_DEPTH * out->sets && park_ns(*out) <= other_ns(s, code);
+        case 2: return park_ns(*out) <= 4600u + s.total * 155u / 100000u;
+        case 3:
+        case 4:
+        case 7: return park_ns(*out) <= other_ns(s, code);
+    }
+    return false;
 }
 
 // What runs a descriptor: the parking kernel, clusters, or kernel ch.code (which also follows where one of the others is refused).

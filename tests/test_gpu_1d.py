@@ -66,6 +66,14 @@ def test_line_kernels_match_the_checker(shape, block, q, xd, ld):
     assert_parity(tokens(*shape, 21, xd), block, q, 5, xd, ld, flags=binding.DIV_FLAG_TWO_LAUNCH_PLANES, expect=5)
 
 
+@pytest.mark.parametrize("shape,block,q,xd,ld", LINE + [((355, 45, 64), 8, 2, "bf16", "bf16"), ((4, 936, 512), 4, 4, "f32", "f32"),
+                                                         ((3, 1, 768), 4, 2, "f32", "f32"), ((32, 512, 768), 8, 4, "f32", "f32")])
+def test_line_kernels_run_by_default(shape, block, q, xd, ld):
+    """`fused` names what would run if another kernel's launch were refused; the threads are those of what runs."""
+    plan = binding.Codec(shape[0], shape[1], 1, shape[2], block, q, xd, ld).plan()
+    assert plan.fused == 8 and plan.on_chip == 0 and plan.threads == 256
+
+
 @pytest.mark.parametrize("shape,block,q,xd,ld", LINE + OTHER)
 @pytest.mark.parametrize("flags", [NO_LINE, TWO_PASS])
 def test_other_paths_match_the_checker_on_1d_maps(shape, block, q, xd, ld, flags):
