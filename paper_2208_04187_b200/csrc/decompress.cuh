@@ -387,7 +387,7 @@ struct DecRows {
     uint32_t tiles;          // low-frequency values of a sample
     uint32_t H, W, Hb, Wb;
     uint32_t bands;          // most bands that a CTA touches
-    uint32_t step_rows, step_cols;      // 1024 elements = step_rows rows and step_cols columns
+    uint32_t step_planes, step_rows, step_cols;      // 1024 elements: whole planes, rows (fewer than a plane's) and columns (fewer than a row's)
     FastDiv by_w, by_h, by_b;
     __device__ __forceinline__ uint32_t lfc_row(uint32_t band) const { return band; }
 };
@@ -453,11 +453,12 @@ decompress_rows_kernel(const LT* lfc, const uint32_t* packed,
         }
         w += d.step_cols;
         h += d.step_rows;
+        plane += d.step_planes;
         if (w >= d.W) {
             w -= d.W;
             ++h;
         }
-        while (h >= d.H) {
+        if (h >= d.H) {
             h -= d.H;
             ++plane;
         }

@@ -551,11 +551,12 @@ quant3d_rows_kernel(const XT* __restrict__ x, const LT* lfc, const uint32_t* ws,
         }
         w += d.step_cols;
         h += d.step_rows;
+        plane += d.step_planes;
         if (w >= d.W) {
             w -= d.W;
             ++h;
         }
-        while (h >= d.H) {
+        if (h >= d.H) {
             h -= d.H;
             ++plane;
         }

@@ -62,6 +62,8 @@ CASES = [
     ((2, 4, 9, 31, 31), 3, 1, "f32", "f32"), ((1, 2, 700, 3, 5), 8, 2, "f32", "f32"),
     # quantise by rows (from 2^20 elements on): quads across rows, slices and samples' ends, many bands a CTA
     ((2, 8, 16, 64, 65), 8, 2, "f32", "f32"), ((3, 7, 13, 62, 66), 4, 4, "bf16", "bf16"), ((1, 600, 16, 11, 11), 8, 8, "f32", "bf16"),
+    # ... steps of whole slices: slices of one row (from 2^21 elements on), of two, of several that do not divide the step
+    ((2, 64, 1640, 1, 10), 3, 2, "f32", "f32"), ((3, 32, 1366, 2, 9), 4, 4, "bf16", "bf16"), ((1, 32, 2000, 3, 6), 16, 8, "f32", "bf16"),
 ]
 
 
