@@ -311,27 +311,37 @@ bool choose_cluster(const div_desc* d, const Shape& s, uint32_t flags, ClusterPl
     return best != ~0ull && cluster_pays(d, s, *out);
 }
 
-// Does the parking kernel take a descriptor that the rules above give to clusters (cl) or to kernel `code`?  Measured against both on 800
+// Estimated times beside the parking kernel's, in ns.  To the fits above, which are for maps of samples that the device works on together,
+// comes what many small samples cost: a sample of the strip and staged kernels (13520 x 5 x 14 x 16 bfloat16 with B = 4 70 us, 38306 x 13 x
+// 8 x 8 with B = 8 484 us), a unit of the lagged kernel (57675 x 4 x 4 x 16 110 us), and a turn of the clusters beyond two.  The kernels for planes
+// a warp wide are only asked where clusters do not pay, on maps that they take half as long again for (1 x 1282 x 124 x 32 27 us).
+uint64_t beside_park_ns(const Shape& s, const ClusterPlan* cl, const Choice& ch) {
+    if (cl) return cluster_ns(s, *cl) + (cl->turns64 > 128u ? (cl->turns64 - 128u) * 1000ull / 64u : 0u);
+    switch (ch.code) {
+        case 2: return 4600u + s.total * 155u / 100000u + 4ull * s.N;
+        case 3: return other_ns(s, 3) + ch.lp.total_units * 12u / 10u;
+        case 6: return other_ns(s, 6) + s.N * 97ull / 10u;
+        case 4:
+        case 7: return other_ns(s, 7) * 3u / 2u;
+    }
+    return 0u;
+}
+// Does the parking kernel take a descriptor that the rules above give to clusters (cl) or to kernel ch.code?  Measured against both on 800
 // random maps (0.1 to 205 MB, both types, all blocks and bit widths that it takes): clusters in one turn are not asked to give way
 // (0.8 of its time in the geometric mean); clusters in turns and the kernels that read x twice where the estimated time is shorter:
 // 1.3 times faster in the geometric mean there (50 x 2048 x 16 x 16 with B = 4 49.5 -> 27.8 us, 96 x 432 x 15 x 56 with B = 4 74.9 -> 37.2 us).
-// The strip kernel's time is fitted once more over its small maps (1 x 56 x 112 x 112 5.9 against 7.2 us, 4.8 MB on the parking kernel's).
+// Of 600 more, half of them batches of 150 to 60000 small samples, it takes 175: 0.67 of the others' time in the geometric mean, two of them 4 and 10 %
+// slower; what it leaves it would mostly need longer for (2169 x 4 x 14 x 16 13.4 against 16.6 us).
 // The staged kernel keeps samples of which less than two and a half fit the parked units (8 x 1840 x 56 x 56 58.5 against 68.1 us).
 // 1-D maps stay with the line kernels, whose second read of x is from the L1 or L2 and whose units hold whole rows (here a strip has one
-// row of four or eight): of 21 random ones up to 8 MB none is faster here and the geometric mean 1.33 times slower (355 x 45 x 64 bfloat16
+// row of four or eight): of 21 random ones up to 8 MB none is faster here and the geometric mean 1.34 times slower (355 x 45 x 64 bfloat16
 // 8.3 against 14.5 us, 4 x 936 x 512 with B = 4 10.5 against 13.4 us).  (The general kernels run no map that plan_park accepts.)
-bool choose_park(const div_desc* d, const Shape& s, uint32_t flags, const ClusterPlan* cl, int code, ParkPlan* out) {
-    if (flags != 0u) return code == 6 && plan_park(d, s, out);
+bool choose_park(const div_desc* d, const Shape& s, uint32_t flags, const ClusterPlan* cl, const Choice& ch, ParkPlan* out) {
+    if (flags != 0u) return ch.code == 6 && plan_park(d, s, out);
     if ((cl && cl->turns64 <= 64u) || !plan_park(d, s, out)) return false;
-    if (cl) return out->sets >= 2u && park_ns(*out) <= cluster_ns(s, *cl);      // (a chunk at a time: 96 x 16 x 100 x 100 bfloat16 21.8 -> 24.6 us)
-    switch (code) {
-        case 6: return 5u * out->per_cta <= 2u * PARK_DEPTH * out->sets && park_ns(*out) <= other_ns(s, code);
-        case 2: return park_ns(*out) <= 4600u + s.total * 155u / 100000u;
-        case 3:
-        case 4:
-        case 7: return park_ns(*out) <= other_ns(s, code);
-    }
-    return false;
+    if (cl && out->sets < 2u) return false;               // (a chunk at a time: 96 x 16 x 100 x 100 bfloat16 21.8 -> 24.6 us)
+    if (!cl && ch.code == 6 && 5u * out->per_cta > 2u * PARK_DEPTH * out->sets) return false;
+    return park_ns(*out) <= beside_park_ns(s, cl, ch);
 }
 
 // What runs a descriptor: the parking kernel, clusters, or kernel ch.code (which also follows where one of the others is refused).
@@ -346,7 +356,7 @@ void choose_route(const div_desc* d, const Shape& s, uint32_t flags, Route* r) {
     if (r->cluster && r->cl.turns64 <= 64u) return;
     Choice ch;
     choose_compress(d, s, flags, &ch);
-    r->park = choose_park(d, s, flags, r->cluster ? &r->cl : nullptr, ch.code, &r->pk);
+    r->park = choose_park(d, s, flags, r->cluster ? &r->cl : nullptr, ch, &r->pk);
 }
 
 bool decompress_fast_ok(const Shape& s) {

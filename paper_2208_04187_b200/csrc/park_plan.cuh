@@ -40,11 +40,12 @@ struct ParkPlan {
     uint32_t chunk_elems, chunks_per_sample, bands_per_sample, total_chunks, stage_bytes;
 };
 
-// Its time in ns, fitted to 550 maps of 4 to 205 MB (within 10 % for nine in ten): the units of an SM, how often its workers go round, the
-// bytes, and how far a sample is spread.
+// Its time in ns, fitted to 550 maps of 4 to 205 MB and 124 of small samples: the units of an SM, how often its workers go round (no oftener than
+// the watcher learns of a chunk, two in about 0.9 us), the bytes, and how far a sample is spread.
 inline uint64_t park_ns(const ParkPlan& pl) {
     const uint64_t rounds = (pl.total_chunks + pl.grid - 1u) / pl.grid;
-    return 6640u + 34u * rounds * pl.nf + 1930u * rounds / pl.sets + rounds * pl.stage_bytes * 148u / 29700u + 420u * pl.chunks_per_sample / 148u;
+    const uint64_t turn = 1930u / pl.sets > 450u ? 1930u / pl.sets : 450u;
+    return 7640u + (34u * pl.nf + turn) * rounds + rounds * pl.stage_bytes * 148u / 29700u + 420u * pl.chunks_per_sample / 148u;
 }
 
 // what the producer posts for a chunk

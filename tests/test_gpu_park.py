@@ -87,3 +87,18 @@ def test_a_nan_reaches_the_sample_as_it_does_in_the_two_pass_kernels():
         rebuilt.append(codec.decompress().clone())
     assert codec.plan(STAGED).lag == 0
     torch.testing.assert_close(rebuilt[0], rebuilt[1], rtol=0, atol=0, equal_nan=True)
+
+
+def test_small_samples_go_where_they_are_faster():
+    """Batches of samples of a chunk or two: those that were measured 10 % faster or more on one side run there."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the figures are those of 148 SMs")
+
+    def parked(*a):
+        plan = binding.div_plan_query(binding.make_desc(*a))
+        return plan.threads == 1024 and plan.lag == 0
+    for others in ((3913, 2, 12, 68, 8, 4), (442, 4, 80, 80, 4, 2), (17746, 2, 13, 16, 4, 2), (9814, 12, 8, 8, 8, 2), (2140, 4, 60, 60, 8, 8),
+                   (2273, 3, 16, 16, 8, 4, "bf16", "bf16")):
+        assert not parked(*others), others
+    for here in ((38306, 13, 8, 8, 8, 2, "f32", "bf16"), (18465, 2, 20, 20, 8, 4), (9395, 15, 7, 16, 8, 2), (24230, 2, 102, 8, 4, 2), (1, 818, 84, 84, 4, 2)):
+        assert parked(*here), here
