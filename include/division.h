@@ -245,8 +245,8 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
 
 /*
  * Test hook for what the kernels that keep x on chip (on_chip 1) do when something goes wrong: runs the kernel that
- * div_compress_ex (workspace_dev NULL: div_planegroup_compress) would run with flags 0, with `timeout_ns` (1 ns to
- * 100 ms) as the limit of every wait, `fault` as below and 1 as the number of the call.  The status word is not cleared
+ * div_compress_ex (workspace_dev NULL: div_planegroup_compress) would run with flags 0, the parking kernel left out, with `timeout_ns`
+ * (1 ns to 100 ms) as the limit of every wait, `fault` as below and 1 as the number of the call.  The status word is not cleared
  * ahead of the kernel: what an earlier call recorded there (status, and in the word behind it the call's number) is
  * cleared by the kernel itself, unless the number is that of the call.  DIV_ERR_PARAM where no such kernel takes the
  * descriptor.  No counterpart in the paper.
@@ -255,6 +255,8 @@ div_status div_debug_compress_starved(const div_desc* desc, const void* x_dev, v
 #define DIV_FAULT_COPIES 1   /* the waits for x never end: the kernel gives up, records DIV_ERR_TIMEOUT (per-plane groups: NaN as
                                 the parameters of its planes) and returns; the rest of the blob is then unspecified */
 #define DIV_FAULT_REFUSED 2  /* the launch asks for more shared memory than the device has: the next kernel in line runs */
+#define DIV_FAULT_PARK_REFUSED 3 /* the same of the parking kernel, on descriptors that it takes (on_chip 1 or not): the kernel behind it runs
+                                as in an ordinary call */
 div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp_dev, size_t comp_capacity,
                              void* workspace_dev, size_t workspace_bytes, uint64_t seed, void* cuda_stream,
                              int32_t fault, uint64_t timeout_ns);

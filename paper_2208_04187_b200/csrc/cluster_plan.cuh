@@ -104,6 +104,7 @@ struct ShareFault {
     uint32_t more_smem;       // shared memory that the launch asks for beyond what it needs
     uint32_t number;          // the call's number (see share_record)
     uint32_t timeout_ns;      // limit of every wait
+    uint32_t no_park;         // more_smem is for the parking kernel's launch, and nothing is asked of the kernels behind it
 };
 div_status compress_cluster(const div_desc* d, const Shape& s, const div_layout& lo, const ClusterPlan& pl, const void* x, uint8_t* blob,
                             uint32_t* ws, uint64_t seed, cudaStream_t st, const ShareFault& fault = ShareFault());

@@ -392,9 +392,13 @@ div_status compress_map(const div_desc* desc, const Shape& s, const div_layout& 
         return DIV_ERR_CUDA;
     Route rt;
     choose_route(desc, s, flags, &rt);
-    if (!rt.park && rt.cluster && compress_cluster(desc, s, lo, rt.cl, x_dev, blob, ws, seed, stream, fault) == DIV_OK) return DIV_OK;
-    if (clear_scratch(ws, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
-    if (rt.park && compress_park(desc, s, lo, rt.pk, x_dev, blob, ws, seed, stream) == DIV_OK) return DIV_OK;
+    if (fault.number != 0u) rt.park = rt.park && fault.no_park;      // a test of the clusters, or of what follows a refused parking kernel
+    if (rt.park) {
+        if (clear_scratch(ws, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
+        if (compress_park(desc, s, lo, rt.pk, x_dev, blob, ws, seed, stream, 0u, 0u, fault.no_park ? fault.more_smem : 0u) == DIV_OK) return DIV_OK;
+    }
+    if (rt.cluster && compress_cluster(desc, s, lo, rt.cl, x_dev, blob, ws, seed, stream, fault.no_park ? ShareFault() : fault) == DIV_OK) return DIV_OK;
+    if (!rt.park && clear_scratch(ws, lo.workspace_bytes, stream) != DIV_OK) return DIV_ERR_CUDA;
     // The single-launch kernels need all their CTAs resident, so they are launched cooperatively; where the
     // device refuses such a launch (fewer SMs visible to the process than the device reports, for instance) the
     // next kernel in line takes the descriptor: nothing has been enqueued by the refused launch.
@@ -634,7 +638,7 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     if (!desc || !x_dev || !comp_dev) return DIV_ERR_NULL;
     const div_status st = check_desc(desc);
     if (st != DIV_OK) return st;
-    if (fault < DIV_FAULT_NONE || fault > DIV_FAULT_REFUSED || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
+    if (fault < DIV_FAULT_NONE || fault > DIV_FAULT_PARK_REFUSED || timeout_ns == 0 || timeout_ns > 100000000ull) return DIV_ERR_PARAM;
     if (!aligned16(x_dev) || !aligned16(comp_dev) || !aligned16(workspace_dev)) return DIV_ERR_ALIGN;
     const Shape s = make_shape(desc);
     const bool planes = workspace_dev == nullptr;
@@ -647,16 +651,17 @@ div_status div_debug_on_chip(const div_desc* desc, const void* x_dev, void* comp
     f.number = 1;
     f.timeout_ns = (uint32_t)timeout_ns;
     f.no_copies = fault == DIV_FAULT_COPIES;
-    f.more_smem = fault == DIV_FAULT_REFUSED ? 1u << 20 : 0u;
+    f.no_park = fault == DIV_FAULT_PARK_REFUSED;
+    f.more_smem = fault == DIV_FAULT_REFUSED || f.no_park ? 1u << 20 : 0u;
     const cudaStream_t stream = (cudaStream_t)cuda_stream;
     if (planes) {
         div_plan plan;
-        if (div_planegroup_plan_query(desc, 0u, &plan) != DIV_OK || !plan.on_chip) return DIV_ERR_PARAM;
+        if (div_planegroup_plan_query(desc, 0u, &plan) != DIV_OK || !plan.on_chip || f.no_park) return DIV_ERR_PARAM;
         return compress_planegroup(desc, s, lo, x_dev, (uint8_t*)comp_dev, seed, stream, 0u, f);
     }
     Route rt;
     choose_route(desc, s, 0u, &rt);
-    if (rt.park || !rt.cluster) return DIV_ERR_PARAM;
+    if (!(f.no_park ? rt.park : rt.cluster)) return DIV_ERR_PARAM;
     return compress_map(desc, s, lo, x_dev, (uint8_t*)comp_dev, (uint32_t*)workspace_dev, seed, stream, 0u, f);
 }
 

@@ -484,10 +484,11 @@ static div_status launch_park_q(const ParkParams& prm, int qbits, cudaStream_t s
 }
 
 div_status compress_park(const div_desc* d, const Shape& s, const div_layout& lo, const ParkPlan& pl, const void* x, uint8_t* blob, uint32_t* ws,
-                         uint64_t seed, cudaStream_t st, uint32_t expected_chunks, uint64_t timeout_ns) {
+                         uint64_t seed, cudaStream_t st, uint32_t expected_chunks, uint64_t timeout_ns, uint32_t more_smem) {
     ParkParams p;
     p.s = s;
     p.pl = pl;
+    p.pl.smem_bytes += more_smem;
     p.by_S = host_fastdiv(pl.chunks_per_sample);
     p.by_stages = host_fastdiv(pl.stages);
     p.x = x;

@@ -128,6 +128,6 @@ inline bool plan_park(const div_desc* d, const Shape& s, ParkPlan* out) {
 }
 
 div_status compress_park(const div_desc* d, const Shape& s, const div_layout& lo, const ParkPlan& pl, const void* x, uint8_t* blob, uint32_t* ws,
-                         uint64_t seed, cudaStream_t st, uint32_t expected_chunks = 0, uint64_t timeout_ns = 0);
+                         uint64_t seed, cudaStream_t st, uint32_t expected_chunks = 0, uint64_t timeout_ns = 0, uint32_t more_smem = 0);
 
 }  // namespace divk

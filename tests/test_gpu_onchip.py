@@ -264,6 +264,34 @@ def test_a_refused_cluster_launch_leaves_the_map_to_the_next_kernel(case):
     assert bool((codec.workspace[64:80] != 0xFF).any())        # the slots were cleared and used: another kernel ran
 
 
+# Maps that the parking kernel takes before clusters in turns, and before a kernel that reads x twice.
+PARKED = [(128, 160, 32, 32, 4, 4, "bf16", "bf16"), (50, 2048, 16, 16, 4, 2, "f32", "f32"), (64, 64, 112, 112, 8, 2, "f32", "f32")]
+
+
+@pytest.mark.parametrize("case", PARKED, ids=lambda c: "x".join(map(str, c)))
+def test_a_refused_parking_launch_leaves_the_map_to_the_kernel_that_the_plan_names(case):
+    """... over a workspace full of leftovers.  The cluster kernel leaves the slots as they were cleared, the others use them."""
+    n, c, h, w, block, q, xd, ld = case
+    x = torch.randn((n, c, h, w), device="cuda", generator=torch.Generator("cuda").manual_seed(4)).to(binding.torch_dtype(xd))
+    codec = binding.Codec(*case)
+    plan = codec.plan()
+    assert plan.threads == 1024 and plan.lag == 0
+    want = codec.compress(x, seed=5).clone()
+    codec.workspace.fill_(0xFF)
+    codec.blob.zero_()
+    assert debug_call(codec, x, 3, 100_000_000) == binding.DIV_OK
+    assert codec.device_status() == binding.DIV_OK and torch.equal(codec.blob, want)
+    assert bool((codec.workspace[64:] == 0).all()) == bool(plan.on_chip)
+    if not plan.on_chip:
+        assert debug_call(codec, x, 0, 100_000_000) == binding.DIV_ERR_PARAM
+        return
+    # the hook's other faults are the clusters', whoever comes before them
+    for fault, status in ((0, binding.DIV_OK), (1, binding.DIV_ERR_TIMEOUT), (2, binding.DIV_OK)):
+        codec.blob.zero_()
+        assert debug_call(codec, x, fault, 1_000_000 if fault == 1 else 100_000_000) == binding.DIV_OK
+        assert codec.device_status() == status and (status != binding.DIV_OK or torch.equal(codec.blob, want))
+
+
 def test_a_refused_plane_share_launch_leaves_the_map_to_the_general_kernel():
     x_np = make((2, 8, 75, 75), "bn", 17, "f32")
     x = torch.from_numpy(x_np).cuda()
