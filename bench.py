@@ -54,7 +54,7 @@ def ncu_traffic(kernel: str, map_label: str):
 
 
 def compress_name(names, plan):
-    if plan.threads == 1024 and plan.lag == 0:
+    if plan.parked:
         return "park_kernel"
     return "cluster_kernel" if plan.on_chip else names[int(plan.fused)]
 

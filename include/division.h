@@ -93,9 +93,9 @@ typedef struct div_layout {
 /* How div_compress will run a descriptor (introspection for tests and benchmarks). */
 typedef struct div_plan {
     int32_t fused;          /* for W%4==0, B in {4,8}, Q in {2,4,8}, one launch:
-                               6: bulk copies into shared-memory rings (first choice from 56 MB up with B = 8): x read once, its
-                                  residuals wait in tensor memory (parking kernel, lag 0), or, where the parts of a sample do
-                                  not fit there, x read from HBM once and re-read from L2 a little later (staged kernel);
+                               6: x read from HBM once and re-read from L2 a little later, both reads staged through
+                                  shared-memory rings by bulk copies (staged kernel; first choice from 56 MB up
+                                  with B = 8);
                                3: as 6, with plain global loads (lagged kernel; first choice from 20 MB up);
                                2: chunks wait in a shared-memory ring (strip ring kernel; first choice below 20 MB);
                                7: small planes of any width (tile side 4, 8 or 16 after padding, at most 32 lanes per
@@ -129,10 +129,11 @@ typedef struct div_plan {
                                thread-block cluster per sample).  grid, threads and smem_bytes are then those of its launch,
                                chunks_per_sample the CTAs of a cluster, chunk_elems the elements of a CTA's share and stages the
                                times that the device has to be filled; fused names the kernel that runs where the device
-                               refuses the launch.  0: all fields describe what runs.
-                               Either way threads 1024 and lag 0 say that the parking kernel (see fused, 6) takes the
-                               descriptor before all others: grid, threads, smem_bytes, chunk_elems and chunks_per_sample are
-                               those of its launch (with on_chip 0 stages too), fused and on_chip name what runs where the
+                               refuses the launch.  0: all fields describe what runs */
+    int32_t parked;         /* 1: the parking kernel takes the descriptor before all others (W%4==0, B in {4,8}, Q in {2,4,8}:
+                               x is read once, by bulk copies, and its residuals wait in tensor memory).  grid, threads
+                               (1024), smem_bytes, chunk_elems and chunks_per_sample are then those of its launch, lag is 0, and
+                               with on_chip 0 stages is the depth of its ring; fused and on_chip name what runs where the
                                device refuses it */
 } div_plan;
 
@@ -144,6 +145,8 @@ typedef struct div_plan {
 #define DIV_FLAG_NO_LINE_KERNELS 16u /* never take the pair of kernels for 1-D maps          */
 #define DIV_FLAG_NO_STAGED_KERNEL 32u/* never take the staged (bulk-copy rings) kernel       */
 #define DIV_FLAG_TWO_LAUNCH_PLANES 64u /* small planes and 1-D maps: the pair of kernels, not the fused one */
+#define DIV_FLAG_NO_PARK_KERNEL 256u /* never take the parking kernel, which otherwise runs before the staged kernel and, without
+                                        other flags, before clusters and any of the kernels above */
 
 /*
  * Sizes of the cached tuple (H^L, V^H, Delta, delta) of Sec. 4.1 in the blob layout above:

@@ -23,6 +23,7 @@ DIV_FLAG_NO_PLANE_KERNELS = 8
 DIV_FLAG_NO_LINE_KERNELS = 16
 DIV_FLAG_NO_STAGED_KERNEL = 32
 DIV_FLAG_TWO_LAUNCH_PLANES = 64
+DIV_FLAG_NO_PARK_KERNEL = 256
 DTYPE_CODES = {"f32": DIV_F32, "bf16": DIV_BF16}
 
 EXPORTED_SYMBOLS = (
@@ -55,7 +56,7 @@ class DivLayout(ctypes.Structure):
 class DivPlan(ctypes.Structure):
     _fields_ = [("fused", c_int32), ("grid", c_int32), ("threads", c_int32), ("stages", c_int32),
                 ("lag", c_int32), ("smem_bytes", c_int32), ("chunk_elems", c_int64),
-                ("chunks_per_sample", c_int64), ("decompress_fast", c_int32), ("on_chip", c_int32)]
+                ("chunks_per_sample", c_int64), ("decompress_fast", c_int32), ("on_chip", c_int32), ("parked", c_int32)]
 
 
 class DivisionError(RuntimeError):

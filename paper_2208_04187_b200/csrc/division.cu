@@ -29,7 +29,7 @@ typedef __nv_bfloat16 bf16;
 constexpr uint64_t SECTION_ALIGN = 128;
 constexpr uint32_t DIV_FLAG_ALL = DIV_FLAG_FORCE_TWO_PASS | DIV_FLAG_NO_STRIP_KERNEL | DIV_FLAG_NO_LAGGED_KERNEL |
                                   DIV_FLAG_NO_PLANE_KERNELS | DIV_FLAG_NO_LINE_KERNELS | DIV_FLAG_NO_STAGED_KERNEL |
-                                  DIV_FLAG_TWO_LAUNCH_PLANES;
+                                  DIV_FLAG_TWO_LAUNCH_PLANES | DIV_FLAG_NO_PARK_KERNEL;
 
 inline uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
 inline uint32_t dtype_bytes(int32_t dt) { return dt == DIV_F32 ? 4u : 2u; }
@@ -351,9 +351,10 @@ struct Route {
     ClusterPlan cl;
 };
 void choose_route(const div_desc* d, const Shape& s, uint32_t flags, Route* r) {
-    r->cluster = choose_cluster(d, s, flags, &r->cl);
+    const uint32_t pins = flags & ~DIV_FLAG_NO_PARK_KERNEL;       // that flag leaves the others' order as it is
+    r->cluster = choose_cluster(d, s, pins, &r->cl);
     r->park = false;
-    if (r->cluster && r->cl.turns64 <= 64u) return;
+    if (pins != flags || (r->cluster && r->cl.turns64 <= 64u)) return;
     Choice ch;
     choose_compress(d, s, flags, &ch);
     r->park = choose_park(d, s, flags, r->cluster ? &r->cl : nullptr, ch, &r->pk);
@@ -553,6 +554,7 @@ div_status div_plan_query(const div_desc* desc, uint32_t flags, div_plan* out) {
     Route rt;
     choose_route(desc, s, flags, &rt);
     out->on_chip = rt.cluster ? 1 : 0;
+    out->parked = rt.park ? 1 : 0;
     if (rt.park) {
         out->grid = (int32_t)rt.pk.grid;
         out->threads = PARK_THREADS;

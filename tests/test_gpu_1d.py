@@ -69,9 +69,9 @@ def test_line_kernels_match_the_checker(shape, block, q, xd, ld):
 @pytest.mark.parametrize("shape,block,q,xd,ld", LINE + [((355, 45, 64), 8, 2, "bf16", "bf16"), ((4, 936, 512), 4, 4, "f32", "f32"),
                                                          ((3, 1, 768), 4, 2, "f32", "f32"), ((32, 512, 768), 8, 4, "f32", "f32")])
 def test_line_kernels_run_by_default(shape, block, q, xd, ld):
-    """`fused` names what would run if another kernel's launch were refused; the threads are those of what runs."""
+    """`fused` names what would run if another kernel's launch were refused; on_chip and parked say that none comes before it."""
     plan = binding.Codec(shape[0], shape[1], 1, shape[2], block, q, xd, ld).plan()
-    assert plan.fused == 8 and plan.on_chip == 0 and plan.threads == 256
+    assert plan.fused == 8 and plan.on_chip == 0 and plan.parked == 0 and plan.threads == 256
 
 
 @pytest.mark.parametrize("shape,block,q,xd,ld", LINE + OTHER)

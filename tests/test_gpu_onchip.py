@@ -275,7 +275,7 @@ def test_a_refused_parking_launch_leaves_the_map_to_the_kernel_that_the_plan_nam
     x = torch.randn((n, c, h, w), device="cuda", generator=torch.Generator("cuda").manual_seed(4)).to(binding.torch_dtype(xd))
     codec = binding.Codec(*case)
     plan = codec.plan()
-    assert plan.threads == 1024 and plan.lag == 0
+    assert plan.parked
     want = codec.compress(x, seed=5).clone()
     codec.workspace.fill_(0xFF)
     codec.blob.zero_()

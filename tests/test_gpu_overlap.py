@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 LAGGED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_STAGED_KERNEL
 RING = binding.DIV_FLAG_NO_LAGGED_KERNEL | binding.DIV_FLAG_NO_STAGED_KERNEL
-STAGED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL
+PARKED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL
+STAGED = PARKED | binding.DIV_FLAG_NO_PARK_KERNEL
 NO_STRIPS = STAGED | binding.DIV_FLAG_NO_STAGED_KERNEL
 PAIR = binding.DIV_FLAG_TWO_LAUNCH_PLANES
 
@@ -48,6 +49,8 @@ KINDS = {
     "cluster": (lambda: binding.Codec(16, 128, 14, 14, 8, 2), 0, (1, None)),
     "cluster, several turns": (lambda: binding.Codec(40, 64, 75, 75, 8, 2, "f32", "bf16"), 0, (1, None)),
     "cluster, in place": (lambda: binding.Codec(16, 64, 32, 32, 8, 4, "bf16", "bf16"), 0, (1, None)),
+    "parking": (lambda: binding.Codec(8, 64, 56, 56, 8, 2), PARKED, (0, 6)),
+    "parking, before clusters": (lambda: binding.Codec(128, 160, 32, 32, 4, 4, "bf16", "bf16"), 0, (1, None)),
     "staged": (lambda: binding.Codec(8, 64, 56, 56, 8, 2), STAGED, (0, 6)),
     "lagged": (lambda: binding.Codec(8, 64, 56, 56, 8, 2), LAGGED, (0, 3)),
     "strip ring": (lambda: binding.Codec(8, 64, 56, 56, 8, 2), RING, (0, 2)),
@@ -71,6 +74,7 @@ def make(kind):
     if want is not None:
         plan = codec.plan(flags)
         assert plan.on_chip == want[0] and want[1] in (None, plan.fused), (plan.on_chip, plan.fused)
+        assert plan.parked == kind.startswith("parking"), kind
     return codec, flags
 
 
@@ -129,7 +133,8 @@ def test_calls_in_a_row_and_in_a_captured_graph(kind):
 
 
 @pytest.mark.parametrize("kinds", [("cluster, several turns", "staged", "lines", "per plane, share"), ("strip ring", "planes", "cluster", "volume"),
-                                   ("lagged", "cluster, in place", "general ring", "per plane, small"), ("staged", "staged", "cluster", "cluster")],
+                                   ("lagged", "cluster, in place", "general ring", "per plane, small"), ("staged", "staged", "cluster", "cluster"),
+                                   ("parking", "parking", "staged", "cluster"), ("parking, before clusters", "parking", "lines", "volume")],
                          ids=lambda k: " + ".join(k))
 def test_threads_on_streams_of_their_own(kinds):
     """Kernels whose CTAs wait for one another stay whole beside others of their sort."""
@@ -171,7 +176,7 @@ def test_one_workspace_for_kernels_in_turn():
     status words alone and clears nothing else, the others clear it for themselves."""
     codec = binding.Codec(8, 64, 28, 28, 8, 2)
     x, = inputs(codec, 1, 3)
-    order = [0, RING, LAGGED, 0, STAGED, NO_STRIPS, 0, PAIR | NO_STRIPS, binding.DIV_FLAG_FORCE_TWO_PASS, LAGGED, RING, STAGED, 0]
+    order = [0, RING, LAGGED, 0, STAGED, PARKED, NO_STRIPS, 0, PARKED, PAIR | NO_STRIPS, binding.DIV_FLAG_FORCE_TWO_PASS, LAGGED, RING, PARKED, STAGED, 0]
     assert [codec.plan(f).on_chip for f in order] == [int(f == 0) for f in order]
     assert {codec.plan(f).fused for f in order if f} == {2, 3, 6, 7, 4, 0}
     codec.compress(x, seed=2)

@@ -16,10 +16,11 @@ from paper_2208_04187_b200 import binding, build, synth
 pytestmark = pytest.mark.gpu
 
 TWO_PASS = binding.DIV_FLAG_FORCE_TWO_PASS
-# the three single-launch kernels for W % 4 == 0: each flag set leaves exactly one of them in line
+# the single-launch kernels for W % 4 == 0: each flag set leaves exactly one of them in line
 LAGGED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_STAGED_KERNEL
 RING = binding.DIV_FLAG_NO_LAGGED_KERNEL | binding.DIV_FLAG_NO_STAGED_KERNEL
-STAGED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL
+PARKED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL     # the parking kernel, staged where a sample is too large for it
+STAGED = PARKED | binding.DIV_FLAG_NO_PARK_KERNEL
 NO_SPECIAL = STAGED | binding.DIV_FLAG_NO_STAGED_KERNEL                     # small-plane kernels, else general ring
 PLANES_PAIR = NO_SPECIAL | binding.DIV_FLAG_TWO_LAUNCH_PLANES               # the small-plane pair instead of the fused kernel
 NO_STRIP = NO_SPECIAL | binding.DIV_FLAG_NO_PLANE_KERNELS                   # general ring, else two-pass
@@ -131,8 +132,8 @@ def small_input(n, c, h, w, x_dtype, seed):
 
 
 @pytest.mark.parametrize("case", SMALL, ids=lambda c: "x".join(map(str, c)))
-@pytest.mark.parametrize("flags", [0, RING, LAGGED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS],
-                         ids=["default", "strip_ring", "lagged", "staged", "planes", "planes_pair", "general_ring", "two_pass"])
+@pytest.mark.parametrize("flags", [0, RING, LAGGED, PARKED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS],
+                         ids=["default", "strip_ring", "lagged", "parking", "staged", "planes", "planes_pair", "general_ring", "two_pass"])
 def test_small_cases_match_the_checker(case, flags):
     n, c, h, w, block, q, xd, ld = case
     x = small_input(n, c, h, w, xd, seed=n + c + h + w + block + q)
@@ -195,6 +196,7 @@ def test_fused_path_is_taken_where_expected():
         assert binding.div_plan_query(d, LAGGED).fused == (3 if spec.w % 4 == 0 else 7), spec.label()
         assert binding.div_plan_query(d, RING).fused == (2 if spec.w % 4 == 0 else 7), spec.label()
         assert binding.div_plan_query(d, STAGED).fused == (6 if spec.w % 4 == 0 else 7), spec.label()
+        assert [binding.div_plan_query(d, f).parked for f in (PARKED, STAGED)] == [int(spec.w % 4 == 0), 0], spec.label()
         assert binding.div_plan_query(d).decompress_fast == (1 if spec.w % 4 == 0 else 2)
 
 
@@ -212,7 +214,7 @@ def test_cluster_kernel_is_the_default_where_a_sample_is_whole_16_byte_groups():
         takes = q != 1 and p2 in (4, 8, 16) and (c * h * w * (4 if xd == "f32" else 2)) % 16 == 0 and not lines
         d = binding.make_desc(*case)
         assert binding.div_plan_query(d).on_chip == int(takes), case
-        for flags in (RING, LAGGED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS):
+        for flags in (RING, LAGGED, PARKED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS):
             assert binding.div_plan_query(d, flags).on_chip == 0
         count += takes
     assert count >= 20
@@ -233,7 +235,7 @@ def test_decompress_reads_a_checker_blob():
 def test_degenerate_inputs():
     # constant tensor: residual identically zero, Delta = 0, exact reconstruction
     x = np.full((2, 4, 16, 16), 1.7, dtype=np.float32)
-    for flags in (0, RING, LAGGED, STAGED, TWO_PASS):
+    for flags in (0, RING, LAGGED, PARKED, STAGED, TWO_PASS):
         codec, blob, xhat = run_gpu(x, 8, 2, 3, flags=flags)
         lfc, words, stats = split_blob(blob, codec.layout, "f32")
         assert not words.any() and not stats.any()
@@ -266,7 +268,7 @@ def test_same_seed_same_bytes_other_seed_other_codes():
     assert (wa != wc).mean() > 0.5
 
 
-@pytest.mark.parametrize("flags", [RING, LAGGED, STAGED, NO_SPECIAL], ids=["strip_ring", "lagged", "staged", "planes_fused"])
+@pytest.mark.parametrize("flags", [RING, LAGGED, PARKED, STAGED, NO_SPECIAL], ids=["strip_ring", "lagged", "parking", "staged", "planes_fused"])
 def test_a_wait_that_cannot_end_gives_up_and_reports_it(flags):
     """Failure detection without a fault: the kernel waits for arrivals that never come, its 2 ms limit
     runs out, it records the timeout in the status word and returns; the context stays usable."""
@@ -276,7 +278,7 @@ def test_a_wait_that_cannot_end_gives_up_and_reports_it(flags):
         spec = synth.TensorSpec(0, 0, 8, 64, 14, 14, "relu", "f32", "f32", 8, 2)      # a small-plane map
     x = to_device(synth.make_input(spec), "f32")
     codec = binding.Codec(*spec.shape, spec.block, spec.qbits)
-    assert codec.plan(flags).fused == {RING: 2, LAGGED: 3, STAGED: 6, NO_SPECIAL: 7}[flags]
+    assert codec.plan(flags).fused == {RING: 2, LAGGED: 3, PARKED: 6, STAGED: 6, NO_SPECIAL: 7}[flags] and codec.plan(flags).parked == (flags == PARKED)
     st = binding.lib().div_debug_compress_starved(
         ctypes.byref(codec.desc), ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(codec.blob.data_ptr()), codec.blob.numel(),
         ctypes.c_void_p(codec.workspace.data_ptr()), codec.workspace.numel(), 0, ctypes.c_void_p(binding.current_stream_handle()),
@@ -298,7 +300,7 @@ def test_guard_bands_stay_untouched():
     for case in [(2, 8, 14, 14, 8, 2, "f32", "f32"), (3, 4, 32, 32, 8, 2, "f32", "f32"), (3, 5, 7, 9, 4, 1, "f32", "f32"),
                  (2, 8, 32, 32, 8, 2, "bf16", "bf16")]:
         n, c, h, w, block, q, xd, ld = case
-        for flags in (0, RING, LAGGED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS):
+        for flags in (0, RING, LAGGED, PARKED, STAGED, NO_SPECIAL, PLANES_PAIR, NO_STRIP, TWO_PASS):
             x = small_input(n, c, h, w, xd, seed=7)
             codec = binding.Codec(n, c, h, w, block, q, xd, ld)
             pad = 4096
@@ -351,7 +353,7 @@ def assert_sampled_parity(spec, seed, sample_ids, flags=0):
 def test_config0_full():
     spec = synth.config0()[0]
     x = synth.make_input(spec)
-    for flags in (0, RING, LAGGED, STAGED, NO_SPECIAL, NO_STRIP, TWO_PASS):
+    for flags in (0, RING, LAGGED, PARKED, STAGED, NO_SPECIAL, NO_STRIP, TWO_PASS):
         assert_full_parity(x, spec.block, spec.qbits, 0, flags=flags)
 
 
@@ -367,14 +369,14 @@ def test_config2_resnet50_imagenet(spec):
     assert_sampled_parity(spec, 0, range(spec.n) if spec.index < 2 else [0, 31, 63])
 
 
-@pytest.mark.parametrize("flags,code", [(0, 6), (LAGGED, 3), (RING, 2)], ids=["staged", "lagged", "strip_ring"])
+@pytest.mark.parametrize("flags,code", [(0, 6), (STAGED, 6), (LAGGED, 3), (RING, 2)], ids=["parking", "staged", "lagged", "strip_ring"])
 def test_full_size_output_does_not_depend_on_timing(flags, code):
     """The single-launch kernels hand out work by timing (claim counters, whoever closes a chunk last); the output
     must not depend on it: the same call twice on a full-size map gives byte-identical blobs."""
     spec = synth.config2()[1]
     x = to_device(synth.make_input(spec), spec.x_dtype)
     codec = binding.Codec(*spec.shape, spec.block, spec.qbits)
-    assert codec.plan(flags).fused == code
+    assert codec.plan(flags).fused == code and codec.plan(flags).parked == (flags == 0)
     first = codec.compress(x, seed=3, flags=flags).clone()
     second = codec.compress(x, seed=3, flags=flags).clone()
     third = codec.compress(x.clone(), seed=3, flags=flags)
@@ -394,7 +396,7 @@ def test_block_sum_order_on_every_path():
     x[0, 0, 0:8, 0:8] = tile
     x[1, 7, 8:16, 24:32] = tile
     x[2, 15, 24:32, 16:24] = tile.T
-    for flags in (0, RING, LAGGED, STAGED, NO_SPECIAL, NO_STRIP, TWO_PASS):
+    for flags in (0, RING, LAGGED, PARKED, STAGED, NO_SPECIAL, NO_STRIP, TWO_PASS):
         codec = assert_full_parity(x, 8, 2, seed=5, flags=flags)
         lfc, _, _ = split_blob(codec.blob.cpu().numpy(), codec.layout, "f32")
         assert lfc.reshape(3, 16, 4, 4)[0, 0, 0, 0] == np.float32(3.0 / 64.0)
@@ -405,6 +407,7 @@ def test_config2_other_paths_on_one_tensor():
     assert_sampled_parity(synth.config2()[2], 0, [0, 63], flags=NO_STRIP)
     assert_sampled_parity(synth.config2()[2], 0, [0, 63], flags=LAGGED)
     assert_sampled_parity(synth.config2()[2], 0, [0, 63], flags=RING)
+    assert_sampled_parity(synth.config2()[2], 0, [0, 63], flags=PARKED)
     assert_sampled_parity(synth.config2()[2], 0, [0, 63], flags=STAGED)
     assert_sampled_parity(synth.config2()[3], 0, [0, 63], flags=PLANES_PAIR)
     assert_sampled_parity(synth.config2()[4], 0, [0, 63], flags=PLANES_PAIR)

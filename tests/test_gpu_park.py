@@ -1,6 +1,6 @@
 """The compress kernel that parks residuals in tensor memory: the same bytes as the kernels with a pass per half, where its tilings end
 (last chunks, short bands, narrow tiles, planes larger than a chunk) and where a sample just fits what is parked, or just does not.
-(Small maps of every form against the CPU checker: test_gpu_parity, flags that leave the staged kernels alone.)"""
+(Small maps of every form against the CPU checker: test_gpu_parity, the same flags.)"""
 import pytest
 import torch
 
@@ -8,7 +8,7 @@ from paper_2208_04187_b200 import binding, build
 
 pytestmark = pytest.mark.gpu
 
-STAGED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL
+PARKED = binding.DIV_FLAG_NO_STRIP_KERNEL | binding.DIV_FLAG_NO_LAGGED_KERNEL
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -46,8 +46,8 @@ PARK = [  # n, c, h, w, block, q, x, lfc
 
 @pytest.mark.parametrize("case", PARK, ids=lambda c: "x".join(map(str, c)))
 def test_parking_kernel_matches_the_two_pass_kernels(case):
-    plan = same_bytes(case, STAGED)
-    assert plan.fused == 6 and plan.threads == 1024 and plan.lag == 0
+    plan = same_bytes(case, PARKED)
+    assert plan.fused == 6 and plan.parked and plan.threads == 1024 and plan.lag == 0
 
 
 # More chunks a CTA than it has records for them (from 64 on), twice over for the small samples: stages of 128 to 640 bytes, a
@@ -56,12 +56,12 @@ MANY_ROUNDS = [(20000, c, 4, 4, 4, 2, "f32", "f32") for c in (2, 4, 6, 8, 10)] +
     (20000, 2, 8, 8, 8, 2, "f32", "f32"), (20000, 4, 8, 8, 8, 4, "bf16", "bf16"), (1024, 512, 2, 64, 8, 2, "f32", "f32")]
 
 
-@pytest.mark.parametrize("flags", [0, STAGED], ids=["default", "staged"])
+@pytest.mark.parametrize("flags", [0, PARKED], ids=["default", "pinned"])
 @pytest.mark.parametrize("case", MANY_ROUNDS, ids=lambda c: "x".join(map(str, c)))
 def test_many_rounds(case, flags):
     plan = same_bytes(case, flags)
     if flags and torch.cuda.get_device_properties(0).multi_processor_count == 148:
-        assert plan.threads == 1024 and plan.lag == 0 and case[0] * plan.chunks_per_sample > 64 * plan.grid
+        assert plan.parked and case[0] * plan.chunks_per_sample > 64 * plan.grid
 
 
 # the last one's planes are more than a chunk
@@ -69,12 +69,12 @@ def test_many_rounds(case, flags):
 def test_parking_kernel_by_default(case):
     plan = same_bytes(case, 0)
     if torch.cuda.get_device_properties(0).multi_processor_count == 148:
-        assert plan.lag == 0 and plan.threads == 1024 and plan.grid == 148
+        assert plan.parked and plan.lag == 0 and plan.threads == 1024 and plan.grid == 148
 
 
 def test_samples_that_do_not_fit_go_to_the_staged_kernel():
-    plan = same_bytes((2, 64, 400, 400, 8, 2, "f32", "f32"), STAGED)          # 41 MB a sample, 38 MB of tensor memory
-    assert plan.fused == 6 and plan.lag > 0
+    plan = same_bytes((2, 64, 400, 400, 8, 2, "f32", "f32"), PARKED)          # 41 MB a sample, 38 MB of tensor memory
+    assert plan.fused == 6 and plan.lag > 0 and not plan.parked
 
 
 def test_a_nan_reaches_the_sample_as_it_does_in_the_two_pass_kernels():
@@ -82,10 +82,10 @@ def test_a_nan_reaches_the_sample_as_it_does_in_the_two_pass_kernels():
     x[1, 7, 30, 50] = float("nan")
     codec = binding.Codec(5, 64, 112, 112, 8, 2, "f32", "f32")
     rebuilt = []
-    for f in (STAGED, binding.DIV_FLAG_FORCE_TWO_PASS):
+    for f in (PARKED, binding.DIV_FLAG_FORCE_TWO_PASS):
         codec.compress(x, seed=11, flags=f)
         rebuilt.append(codec.decompress().clone())
-    assert codec.plan(STAGED).lag == 0
+    assert codec.plan(PARKED).parked
     torch.testing.assert_close(rebuilt[0], rebuilt[1], rtol=0, atol=0, equal_nan=True)
 
 
@@ -95,10 +95,21 @@ def test_small_samples_go_where_they_are_faster():
         pytest.skip("the figures are those of 148 SMs")
 
     def parked(*a):
-        plan = binding.div_plan_query(binding.make_desc(*a))
-        return plan.threads == 1024 and plan.lag == 0
+        return binding.div_plan_query(binding.make_desc(*a)).parked
     for others in ((3913, 2, 12, 68, 8, 4), (442, 4, 80, 80, 4, 2), (17746, 2, 13, 16, 4, 2), (9814, 12, 8, 8, 8, 2), (2140, 4, 60, 60, 8, 8),
                    (2273, 3, 16, 16, 8, 4, "bf16", "bf16")):
         assert not parked(*others), others
     for here in ((38306, 13, 8, 8, 8, 2, "f32", "bf16"), (18465, 2, 20, 20, 8, 4), (9395, 15, 7, 16, 8, 2), (24230, 2, 102, 8, 4, 2), (1, 818, 84, 84, 4, 2)):
         assert parked(*here), here
+
+
+def test_the_flag_that_excludes_it_leaves_the_others_in_their_order():
+    NO_PARK = binding.DIV_FLAG_NO_PARK_KERNEL
+    for case in PARK + MANY_ROUNDS + [(64, 64, 112, 112, 8, 2, "f32", "f32"), (128, 160, 32, 32, 4, 4, "bf16", "bf16"), (8, 64, 1, 768, 8, 4), (3, 5, 7, 9, 4, 1)]:
+        desc = binding.make_desc(*case)
+        for flags in (0, PARKED, binding.DIV_FLAG_NO_STAGED_KERNEL, binding.DIV_FLAG_FORCE_TWO_PASS):
+            with_it, without = binding.div_plan_query(desc, flags), binding.div_plan_query(desc, flags | NO_PARK)
+            assert (without.fused, without.on_chip, without.parked) == (with_it.fused, with_it.on_chip, 0), case
+            assert with_it.parked or all(getattr(with_it, f) == getattr(without, f) for f, _ in binding.DivPlan._fields_), case
+    plan = same_bytes((128, 160, 32, 32, 4, 4, "bf16", "bf16"), NO_PARK)
+    assert plan.on_chip == 1 and plan.threads in (256, 384, 512)

@@ -59,12 +59,12 @@ def _assert_equals_checker(blob, layout, x_np, block, qbits, seed, samples):
 def test_static_scratch_matches_the_checker_and_div_compress_on_calls_in_a_row():
     stream = binding.current_stream_handle()
     # four maps of different shapes, named after the kernels that take them where clusters are not to be had (the next test has
-    # a map for each kernel that keeps state in the scratch); the large one is the staged kernel's
+    # a map for each kernel that keeps state in the scratch); the large one is the parking kernel's
     cases = [
         ("strip ring kernel", synth.activation_map(8, 16, 64, 64, "relu", 4246), 8, 2, 2),           # planes too wide for the small-plane kernel
         ("fused small-plane kernel", synth.activation_map(5, 24, 14, 14, "relu", 4242), 8, 2, 7),
         ("lagged kernel", synth.activation_map(8, 64, 112, 112, "relu", 4243), 8, 2, 3),             # 25.7 MB
-        ("staged kernel", synth.activation_map(20, 64, 112, 112, "relu", 4244), 8, 2, 6),            # 64.2 MB
+        ("parking kernel", synth.activation_map(20, 64, 112, 112, "relu", 4244), 8, 2, 6),            # 64.2 MB
     ]
     prepared = []
     for name, x_np, block, qbits, plan_code in cases:
@@ -103,8 +103,8 @@ def test_static_scratch_matches_the_checker_and_div_compress_on_calls_in_a_row()
 # large that their number of CTAs is what decides (on 148 SMs).
 BY_DEFAULT = [
     ("strip ring kernel", (1, 64, 112, 112), "bf16", 0, 2), ("cluster kernel", (16, 64, 14, 14), "f32", 1, None),
-    ("lagged kernel", (16, 64, 128, 128), "bf16", 0, 3), ("fused small-plane kernel", (24, 2048, 17, 17), "f32", 0, 7),
-    ("staged kernel", (20, 64, 112, 112), "f32", 0, 6), ("line kernel", (8, 64, 1, 768), "f32", 0, 8),
+    ("lagged kernel", (20, 65, 99, 100), "bf16", 0, 3), ("fused small-plane kernel", (24, 2048, 17, 17), "f32", 0, 7),
+    ("parking kernel", (20, 64, 112, 112), "f32", 0, 6), ("staged kernel", (8, 1840, 56, 56), "f32", 0, 6), ("line kernel", (8, 64, 1, 768), "f32", 0, 8),
 ]
 
 
@@ -118,7 +118,7 @@ def test_static_scratch_between_the_kernels_that_keep_state_in_it():
         x = torch.randn(shape, device="cuda", generator=torch.Generator("cuda").manual_seed(8)).to(binding.torch_dtype(xd))
         codec, want = _reference_blob(x, (*shape, 8, 2, xd, "f32"), seed=11)
         plan = codec.plan()
-        assert plan.on_chip == on_chip and code in (None, plan.fused), name
+        assert plan.on_chip == on_chip and code in (None, plan.fused) and plan.parked == (name == "parking kernel"), name
         two_pass = binding.Codec(*shape, 8, 2, xd, "f32")
         two_pass.compress(x, seed=11, flags=binding.DIV_FLAG_FORCE_TWO_PASS)
         for g, w in zip(_sections(want, codec.layout), _sections(two_pass.blob, codec.layout)):
