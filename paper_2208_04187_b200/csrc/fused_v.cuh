@@ -442,14 +442,11 @@ fused_v_kernel(const VParams p) {
                 __threadfence_block();
                 sts_volatile(&ctl->issued[st], it + 1u);
             }
-            if (it < n_my || lds_volatile(&ctl->failed)) {
-                // a wait gave up somewhere: let the copies still in flight land before the CTA may exit
-                const uint32_t first = it > K ? it - K : 0u;
-                for (uint32_t j = first; j < it; ++j) {
-                    const uint32_t round = fdiv(j, p.by_K);
-                    uint32_t polls = 0;
-                    while (!mbar_try_wait(&ctl->full[j - round * K], round & 1) && ++polls < (1u << 20)) {
-                    }
+            // the copies on their way land before the CTA may exit, whoever gives up meanwhile
+            for (uint32_t j = it > K ? it - K : 0u; j < it; ++j) {
+                const uint32_t round = fdiv(j, p.by_K);
+                uint32_t polls = 0;
+                while (!mbar_try_wait(&ctl->full[j - round * K], round & 1) && ++polls < (1u << 20)) {
                 }
             }
         }

@@ -342,16 +342,12 @@ park_kernel(const __grid_constant__ ParkParams p) {
             const uint64_t policy = l2_policy_release();
             const uint32_t ahead = p.pl.ahead;
             uint32_t it = 0;
-            bool ok = true;
             for (; it < n_my; ++it) {
                 const uint32_t turn = fdiv(it, p.by_stages), st = it - turn * K, slot = it % PARK_CHUNKS;
                 const uint32_t j = blockIdx.x + it * grid;
                 const uint32_t n = fdiv(j, p.by_S), k = j - n * S;
                 if ((it >= K && !p_wait(&ctl->empty[st], (turn - 1u) & 1u, p, ctl, 0x80000002u)) ||
-                    (it >= ahead && !p_wait(&ctl->full[(it - ahead) % PARK_CHUNKS], ((it - ahead) / PARK_CHUNKS) & 1u, p, ctl, 0x80000005u))) {
-                    ok = false;
-                    break;
-                }
+                    (it >= ahead && !p_wait(&ctl->full[(it - ahead) % PARK_CHUNKS], ((it - ahead) / PARK_CHUNKS) & 1u, p, ctl, 0x80000005u))) break;
                 const uint32_t e0 = k * p.pl.chunk_elems;
                 const uint32_t bytes = min(p.pl.chunk_elems, s.CHW - e0) * (uint32_t)sizeof(XT);
                 ParkDesc d;
@@ -364,11 +360,10 @@ park_kernel(const __grid_constant__ ParkParams p) {
                 mbar_arrive_expect_tx(&ctl->full[slot], bytes);
                 bulk_load_hint(ring + (size_t)st * p.pl.stage_bytes, reinterpret_cast<const XT*>(p.x) + d.quad0 * 4u, bytes, &ctl->full[slot], policy);
             }
-            if (!ok || lds_volatile(&ctl->failed)) {
-                for (uint32_t t = it > K ? it - K : 0u; t < it; ++t) {
-                    uint32_t polls = 0;
-                    while (!mbar_try_wait(&ctl->full[t % PARK_CHUNKS], (t / PARK_CHUNKS) & 1u) && ++polls < (1u << 20)) {
-                    }
+            // the copies on their way land before the CTA may exit, whoever gives up meanwhile (the workers need them all in any case)
+            for (uint32_t t = it > K ? it - K : 0u; t < it; ++t) {
+                uint32_t polls = 0;
+                while (!mbar_try_wait(&ctl->full[t % PARK_CHUNKS], (t / PARK_CHUNKS) & 1u) && ++polls < (1u << 20)) {
                 }
             }
         }

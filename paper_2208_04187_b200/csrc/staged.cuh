@@ -511,14 +511,11 @@ staged_kernel(const SParams p) {
             __threadfence_block();
             sts_volatile(&desc[st].seq, it + 1u);
         }
-        if (!ok || lds_volatile(&ctl->failed)) {
-            // a wait gave up somewhere: let the copies still in flight land before the CTA may exit
-            const uint32_t first = it > K ? it - K : 0u;
-            for (uint32_t t = first; t < it; ++t) {
-                const uint32_t round = fdiv(t, by_K);
-                uint32_t polls = 0;
-                while (!mbar_try_wait(&full[t - round * K], round & 1u) && ++polls < (1u << 20)) {
-                }
+        // the copies on their way land before the CTA may exit, whoever gives up meanwhile
+        for (uint32_t t = it > K ? it - K : 0u; t < it; ++t) {
+            const uint32_t round = fdiv(t, by_K);
+            uint32_t polls = 0;
+            while (!mbar_try_wait(&full[t - round * K], round & 1u) && ++polls < (1u << 20)) {
             }
         }
         return;

@@ -1,6 +1,8 @@
 """The compress kernel that parks residuals in tensor memory: the same bytes as the kernels with a pass per half, where its tilings end
 (last chunks, short bands, narrow tiles, planes larger than a chunk) and where a sample just fits what is parked, or just does not.
 (Small maps of every form against the CPU checker: test_gpu_parity, the same flags.)"""
+import ctypes
+
 import pytest
 import torch
 
@@ -113,3 +115,27 @@ def test_the_flag_that_excludes_it_leaves_the_others_in_their_order():
             assert with_it.parked or all(getattr(with_it, f) == getattr(without, f) for f, _ in binding.DivPlan._fields_), case
     plan = same_bytes((128, 160, 32, 32, 4, 4, "bf16", "bf16"), NO_PARK)
     assert plan.on_chip == 1 and plan.threads in (256, 384, 512)
+
+
+RING = binding.DIV_FLAG_NO_LAGGED_KERNEL | binding.DIV_FLAG_NO_STAGED_KERNEL
+
+
+@pytest.mark.parametrize("flags", [PARKED, PARKED | binding.DIV_FLAG_NO_PARK_KERNEL, RING], ids=["parking", "staged", "strip ring"])
+@pytest.mark.parametrize("shape", [(4, 64, 56, 56), (3, 64, 112, 112)], ids=lambda s: "x".join(map(str, s)))
+def test_giving_up_at_once_leaves_nothing_behind(flags, shape):
+    """A limit of 1 ns runs out while copies may still be on their way: they land before their CTAs leave, nothing behind the blob is
+    written, and the calls after it, on the SMs that were left, write what they always do."""
+    x = torch.randn(shape, device="cuda", generator=torch.Generator("cuda").manual_seed(4))
+    codec = binding.Codec(*shape, 8, 2)
+    size = codec.blob.numel()
+    room = torch.full((size + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    codec.blob = room[:size]
+    want = codec.compress(x, seed=5, flags=flags).clone()
+    for _ in range(20):
+        assert binding.lib().div_debug_compress_starved(
+            ctypes.byref(codec.desc), ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(codec.blob.data_ptr()), size, ctypes.c_void_p(codec.workspace.data_ptr()),
+            codec.workspace.numel(), 0, ctypes.c_void_p(binding.current_stream_handle()), flags, 1) == binding.DIV_OK
+        assert codec.device_status() == binding.DIV_ERR_TIMEOUT
+        codec.compress(x, seed=5, flags=flags)
+        assert codec.device_status() == binding.DIV_OK and torch.equal(codec.blob, want)
+    assert bool((room[size:] == 0xA5).all())
