@@ -62,7 +62,9 @@ struct ParkParams {
 // ------------------------------------------------------------------------------------------------
 // tensor memory: 32 columns (numbers of a lane) of the quarter that the warp may touch
 // ------------------------------------------------------------------------------------------------
+// (all lanes of the warp together: what is before may have parted them)
 __device__ __forceinline__ void tmem_store32(uint32_t at, const uint32_t (&v)[32]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
         "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(at),
@@ -75,6 +77,7 @@ __device__ __forceinline__ void tmem_store32(uint32_t at, const uint32_t (&v)[32
 }
 // (the wait names the registers: nothing may touch them between the two)
 __device__ __forceinline__ void tmem_load32(uint32_t at, uint32_t (&v)[32]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
         "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -458,6 +461,7 @@ park_kernel(const __grid_constant__ ParkParams p) {
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
+    __syncwarp();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(ctl->tmem));
 }
 
