@@ -21,8 +21,9 @@ static_assert(PARK_MAX_STAGES < PARK_CHUNKS, "a record is not filled again while
 constexpr uint32_t PARK_MAX_SETS = (PARK_CHUNKS - 1 - PARK_MAX_STAGES) / PARK_DEPTH;
 constexpr uint32_t PARK_CHUNK_ELEMS = 7168;    // of a full chunk, about: 7 units (half of it: 64 x 64 x 112 x 112 44 -> 52 us)
 constexpr uint32_t PARK_MOST_BYTES = 64 * 1024;// planes up to which chunks may be larger, where a chunk has to be whole planes
-// Bytes of copies on their way to an SM at once.  The words by which the CTAs meet come back behind them: 64 x 64 x 112 x 112 with 28, 56,
-// 84, 112 KB and all of the ring 57.5, 45.5, 47.4, 49.6, 50.9 us.
+// Bytes of copies on their way to an SM at once, in whole chunks, of which at least two are (56 KB for full fp32 chunks, up to 128 KB where a
+// chunk is a large plane).  The words by which the CTAs meet come back behind them: 64 x 64 x 112 x 112 with 28, 56, 84, 112 KB and all of
+// the ring 57.5, 45.5, 47.4, 49.6, 50.9 us.
 constexpr uint32_t PARK_AHEAD_BYTES = 48 * 1024;
 
 struct ParkPlan {
